@@ -190,7 +190,7 @@ typedef enum agzo_kernel_class {
   AGZO_KC_RMW = 1,        /* the in-place low-rank pass                                    */
   AGZO_KC_XT_T = 2,       /* Y = X^T T, CUDA-core kernel                                   */
   AGZO_KC_X_Q = 3,        /* T = X Q, CUDA-core kernel                                     */
-  AGZO_KC_PANEL_QR = 4,   /* the three kernels of qr(Y) as one unit                        */
+  AGZO_KC_PANEL_QR = 4,   /* qr(Y)                                                         */
   AGZO_KC_TC_XT_T = 5,    /* Y = X^T T, tensor-core kernel                                 */
   AGZO_KC_TC_X_Q = 6,     /* T = X Q, tensor-core kernel                                   */
   AGZO_KC_OMEGA = 7,      /* Gaussian test matrix fill                                     */

@@ -216,13 +216,11 @@ size_t layer_scratch(const agzo_layer& a, bool tc, bool long_slabs, bool with_pa
   slab_shape(a, tc, long_slabs, &slabs, &slab_rows);
   if (slabs < y_parts_min) slabs = y_parts_min;
   const size_t r = (size_t)a.r, d = (size_t)a.d_in, m = (size_t)a.m;
-  const size_t gch = (d + 127) / 128;
   size_t b = 0;
   b += align_up(m * r * 4);                 // T
   b += align_up((size_t)slabs * r * d * 4); // Ypart
   b += align_up(r * d * 4);                 // Y
-  b += align_up(gch * r * r * 8);           // Gpart
-  b += align_up(r * r * 8);                 // M
+  b += align_up(panel_gram_bytes(a.d_in, a.r));   // Gpart
   if (tc && with_panels) b += tc_layer_scratch(a);
   return b;
 }
@@ -416,8 +414,7 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
           D.T = reinterpret_cast<float*>(p);      p += align_up(m * r * 4);
           const size_t parts = (size_t)(slabs > y_parts_min(a) ? slabs : y_parts_min(a));
           D.Ypart = reinterpret_cast<float*>(p);  p += align_up(parts * r * d * 4);
-          D.Gpart = reinterpret_cast<double*>(p); p += align_up(gch * r * r * 8);
-          D.M = reinterpret_cast<double*>(p);     p += align_up(r * r * 8);
+          D.Gpart = reinterpret_cast<double*>(p); p += align_up(panel_gram_bytes(a.d_in, a.r));
         }
         if (tc) {
           int row0 = 0;
@@ -880,9 +877,9 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
       if (w.max_m == 0 || P.wave_region[wv] < 0) continue;
       cudaStream_t ws = forked ? ctx->aux[P.wave_region[wv]] : s;
       DevStatus* dst = dev_status(ctx);
-      auto panel_qr = [&]() -> cudaError_t {
-        Timed t(ctx, AGZO_KC_PANEL_QR, ws, 3);
-        return launch_panel_qr(w, dst, ws);
+      auto panel_qr = [&](bool last) -> cudaError_t {
+        Timed t(ctx, AGZO_KC_PANEL_QR, ws, panel_qr_launches(w.max_r));
+        return launch_panel_qr(w, last, dst, ws);
       };
       // token-sharded run: Y = sum over ranks of X_p^T T_p, all panels of the wave in one call
       auto sum_over_ranks = [&]() -> agzo_status {
@@ -926,7 +923,7 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
       CU(ctx, xt_t(false));                    // Y <- H Omega
       for (int k = 0; k < K; ++k) {
         if ((sr = sum_over_ranks()) != AGZO_OK) return sr;
-        CU(ctx, panel_qr());                   // Q <- qr(Y)
+        CU(ctx, panel_qr(false));              // Q <- qr(Y)
         if (fz_classes) {
           CU(ctx, power_fused());
           w.after_fused = 1;                   // their partial sums are now one per share, not one per slab
@@ -937,7 +934,7 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
         }
       }
       if ((sr = sum_over_ranks()) != AGZO_OK) return sr;
-      CU(ctx, panel_qr());                     // A <- qr(Y)
+      CU(ctx, panel_qr(true));                 // A <- qr(Y)
     }
     return AGZO_OK;
   };

@@ -1,0 +1,685 @@
+// qr(Y) of Algorithm 1 for the panels of a wave: Q = Y R^-1 with the unique R that has a positive diagonal
+// (S = Y^T Y = R^T R).  With the Gram matrix and the factor in double this is as accurate in fp32 as a Householder QR
+// for cond(Y) well below 1e7.
+//
+// Up to rank 32 (panel_qr_kernel) one launch per round, a thread-block cluster of C CTAs per layer, CTA c owning a
+// contiguous slice of the columns d of Y (r x d_in):
+//   load    Y = sum of the partial sums that the last product left, in order, into shared memory
+//   gram    the slice's share of S on the FP64 tensor cores (mma.sync m8n8k4: true double multiply-adds; tcgen05
+//           has no FP64 form), the warps splitting the columns, partial sums added in a fixed order
+//   -- cluster barrier: every CTA adds the C shares, read through distributed shared memory, in rank order --
+//   factor  Cholesky and M = R^-1, by every CTA for itself (what it costs is a dependent chain, so doing it C
+//           times takes no longer than doing it once and saves a second exchange)
+//   apply   Q = Y M on the FP64 tensor cores, from the slice that is still in shared memory, and out: V (fp32) after
+//           the last round, the bf16 hi/lo operand panel of the next product before it
+// What bounds it is the latency of that chain (load, gram, exchange, r pivots).  The three kernels it replaced (Gram per
+// 512 columns, one factorisation block per layer, apply per 128 columns) handed Y, the Gram shares and M over through
+// global memory: r = 8, d_in = 1024, one layer 24 -> 10.3 us per round; r = 16, d_in = 4096 44 -> 20 us.
+//
+// Above rank 32 the FP64 products (r^2 d_in multiply-adds each) weigh more than the chain and layers of a wave differ
+// in d_in, so three launches cut the work evenly: Gram per 512 columns, factorisation per layer, apply per 128 columns.
+#include "agzo_ptx.cuh"
+
+#include "agzo_common.cuh"
+
+namespace agzo {
+
+namespace {
+
+using namespace ptx;
+
+constexpr int kQrThreads = 256;
+constexpr int kQrWarps = kQrThreads / 32;
+constexpr int kQrChunk = 128;            // columns of Y that are staged together
+constexpr int kQrMaxCluster = 8;
+constexpr int kBlk = 8;                  // block of the factorisation = tile of the FP64 tensor cores
+// up to here the slice stays in shared memory from load to apply, with two CTAs per SM
+constexpr size_t kQrResidentSmem = 112 * 1024;
+
+__device__ __forceinline__ void dmma_m8n8k4(double& c0, double& c1, double a, double b) {
+  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
+               : "+d"(c0), "+d"(c1) : "d"(a), "d"(b));
+}
+__device__ __forceinline__ double ld_cluster_f64(uint32_t addr) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
+  return v;
+}
+
+// Sizes of an instantiation.  NT: 8-row tiles of the panel (the wave's largest rank, rounded up).
+template <int NT>
+struct QrCfg {
+  static constexpr int r8 = 8 * NT;
+  static constexpr int tiles = NT * (NT + 1) / 2;          // 8 x 8 tiles of the upper triangle of S
+  static constexpr int my_tiles = NT <= 4 ? tiles : 10;    // ... of them per warp, at most
+  static constexpr int ksplit = NT <= 4 ? kQrWarps : 2;    // warps that split the columns (eight tile rows: four sets of tiles)
+  static constexpr int ap = r8 + 1;                        // pitch of S / R in doubles
+  static constexpr int mp = (r8 + 15) / 16 * 16 + 4;       // pitch of M in doubles
+  static constexpr size_t g_bytes = (size_t)tiles * 64 * 8;
+  static constexpr size_t am_bytes = (size_t)r8 * (ap + mp) * 8;
+  static constexpr size_t p_bytes = NT <= 4 ? (size_t)kQrWarps * tiles * 64 * 8 : 0;
+  static constexpr size_t u_bytes = am_bytes > p_bytes ? am_bytes : p_bytes;   // warps' partial sums, then S/R and M
+  static constexpr size_t fixed = g_bytes + u_bytes;
+};
+// pitch of the staged columns in floats: 12 beyond a multiple of 32, so that the 8 x 4 elements of a Gram fragment
+// fall into 32 banks and an apply fragment's into 28
+__host__ __device__ inline int qr_pitch(int cols) { return cols + 12; }
+
+// Which tiles of the upper triangle a warp of set H works on.  Eight tile rows are split into four sets that touch few
+// different tile rows each (a fragment is converted to double once per set): the two triangles of ten tiles and the
+// two halves, eight tiles each, of the square between them.
+template <int NT, int H>
+__device__ constexpr bool qr_tile_mine(int bi, int bj) {
+  return NT <= 4 ? true
+                 : (H == 0 ? bj < 4 : H == 3 ? bi >= 4 : (bi < 4 && bj >= 4 && (bi < 2) == (H == 1)));
+}
+template <int NT, int H>
+__device__ constexpr bool qr_row_used(int b) {
+  return NT <= 4 ? true : (H == 0 ? b < 4 : H == 3 ? b >= 4 : (b >= 4 || (b < 2) == (H == 1)));
+}
+
+// Gram products of `steps` groups of four columns, this warp taking every ksplit-th group.  Fragments (PTX ISA, m8n8k4
+// .f64): lane l holds A[l / 4][l % 4], B[l % 4][l / 4] and D[l / 4][2 (l % 4) + {0, 1}]; with A = Y[8 bi ..][c ..] and
+// B = Y[8 bj ..][c ..]^T both operands are the element (l / 4, l % 4) of a row block of the staged columns.
+template <int NT, int H>
+__device__ __forceinline__ void qr_gram(const float* sY, int pitch, int steps, int k0, double (&acc)[QrCfg<NT>::my_tiles][2]) {
+  const int lane = threadIdx.x & 31, fr = lane >> 2, fc = lane & 3;
+  const float* base = sY + fr * pitch + fc;
+#pragma unroll 2
+  for (int ks = k0; ks < steps; ks += QrCfg<NT>::ksplit) {
+    double f[NT];
+#pragma unroll
+    for (int b = 0; b < NT; ++b)
+      if (qr_row_used<NT, H>(b)) f[b] = (double)base[8 * b * pitch + 4 * ks];
+    int t = 0;
+#pragma unroll
+    for (int bi = 0; bi < NT; ++bi)
+#pragma unroll
+      for (int bj = bi; bj < NT; ++bj)
+        if (qr_tile_mine<NT, H>(bi, bj)) { dmma_m8n8k4(acc[t][0], acc[t][1], f[bi], f[bj]); ++t; }
+  }
+}
+
+// adds this warp's sums to a Gram share (this lane's two elements of every tile of the warp)
+template <int NT, int H>
+__device__ __forceinline__ void qr_add_share(double* g, const double (&acc)[QrCfg<NT>::my_tiles][2], bool first) {
+  int t = 0, n = 0;
+#pragma unroll
+  for (int bi = 0; bi < NT; ++bi)
+#pragma unroll
+    for (int bj = bi; bj < NT; ++bj, ++t)
+      if (qr_tile_mine<NT, H>(bi, bj)) {
+        double2* p = reinterpret_cast<double2*>(g + t * 64);
+        double2 v = first ? make_double2(0.0, 0.0) : *p;
+        v.x += acc[n][0]; v.y += acc[n][1];
+        *p = v;
+        ++n;
+      }
+}
+
+// Stages columns [d0, d0 + ncols) of Y (ncols a multiple of 128; zero beyond d_in and beyond row r) into sY.
+// from_y: read L.Y as it is; else the sum of the partial sums, which is also written to L.Y when `keep` is set.
+__device__ __forceinline__ void qr_load(const DevLayer& L, float* sY, int pitch, int r8, int d0, int ncols, int nparts,
+                                        bool from_y, bool keep) {
+  const int r = L.r, d_in = L.d_in;
+  const long long part = (long long)r * d_in;
+  const float* src0 = from_y ? L.Y : L.Ypart;
+  const int np = from_y ? 1 : nparts;
+  if ((d_in & 3) == 0) {
+    const int vrow = ncols >> 2, nvec = r8 * vrow;
+    constexpr int U = 4, P = 4;                      // 16 independent loads before the first use
+    for (int i0 = threadIdx.x; i0 < nvec; i0 += U * kQrThreads) {
+      float4 v[U];
+      const float* src[U];
+      bool live[U];
+      int at[U], col[U], row[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * kQrThreads;
+        row[u] = i / vrow;
+        col[u] = d0 + 4 * (i - row[u] * vrow);
+        at[u] = row[u] * pitch + (col[u] - d0);
+        live[u] = i < nvec && row[u] < r && col[u] < d_in;
+        src[u] = src0 + (long long)row[u] * d_in + col[u];
+        v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+      for (int s0 = 0; s0 < np; s0 += P) {
+        float4 t[U][P];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int s = 0; s < P; ++s)
+            t[u][s] = live[u] && s0 + s < np ? __ldcg(reinterpret_cast<const float4*>(src[u] + (s0 + s) * part))
+                                             : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int s = 0; s < P; ++s) { v[u].x += t[u][s].x; v[u].y += t[u][s].y; v[u].z += t[u][s].z; v[u].w += t[u][s].w; }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (i0 + u * kQrThreads >= nvec) continue;
+        *reinterpret_cast<float4*>(sY + at[u]) = v[u];
+        if (keep && live[u]) *reinterpret_cast<float4*>(L.Y + (long long)row[u] * d_in + col[u]) = v[u];
+      }
+    }
+  } else {
+    for (int i = threadIdx.x; i < r8 * ncols; i += kQrThreads) {
+      const int k = i / ncols, c = i - k * ncols, d = d0 + c;
+      float y = 0.f;
+      if (k < r && d < d_in) {
+        for (int s = 0; s < np; ++s) y += __ldcg(src0 + s * part + (long long)k * d_in + d);
+        if (keep) L.Y[(long long)k * d_in + d] = y;
+      }
+      sY[k * pitch + c] = y;
+    }
+  }
+}
+
+// Diagonal block kb (8 x 8) of the factorisation by one warp, every lane on the whole block in registers: the chain is
+// then four times (rsqrt, multiply, multiply-add) with no exchange between lanes.  D = R_kk^-1 goes to the block of M
+// (zero below the diagonal): lane j takes column j.
+// A pivot with R_kk <= kRankTol * ||y_k|| (what is left of column k after the columns before it are projected out,
+// against the column's own length) marks a dependent column, which becomes zero.  The test is scale-free per column: the
+// columns of Y = H (H^T Q) carry squared singular values, so a short column is normal and says nothing about dependence.
+template <int NT>
+__device__ __forceinline__ void qr_factor_block(const double* A, double* M, const double* own, int kb, int r, DevStatus* status,
+                                                bool report) {
+  constexpr int ap = QrCfg<NT>::ap, mp = QrCfg<NT>::mp;
+  const int lane = threadIdx.x & 31, j = lane & 7;
+  const int o = kb * kBlk;
+  double a[kBlk][kBlk], rinv[kBlk];          // the upper triangle is used
+#pragma unroll
+  for (int i = 0; i < kBlk; ++i)
+#pragma unroll
+    for (int c = i; c < kBlk; ++c) a[i][c] = A[(o + i) * ap + o + c];
+  bool any_bad = false;
+  // two pivots at a time: with d1 = a_kk and det = d1 a_22 - a_12^2 both reciprocal roots start together
+  // (1 / R_22 = sqrt(d1) / sqrt(det)); what a subtraction loses in det it loses in a_22 - R_12^2 as well
+#pragma unroll
+  for (int k = 0; k < kBlk; k += 2) {
+    const double d1 = a[k][k], a12 = a[k][k + 1], a22 = a[k + 1][k + 1];
+    const double det = fma(d1, a22, -(a12 * a12));
+    const double r1 = rsqrt(d1), rd = rsqrt(det);
+    const bool live1 = o + k < r, live2 = o + k + 1 < r;
+    const bool bad1 = !(d1 > 0.0) || d1 <= kRankTol * kRankTol * own[o + k];
+    const double i1 = (live1 && !bad1) ? r1 : 0.0;
+    const double d2 = bad1 ? a22 : det * (r1 * r1);
+    const bool bad2 = !(d2 > 0.0) || d2 <= kRankTol * kRankTol * own[o + k + 1];
+    double i2 = (d1 * r1) * rd;
+    if (bad1) i2 = rsqrt(a22);
+    if (!live2 || bad2) i2 = 0.0;
+    any_bad = any_bad || (live1 && bad1) || (live2 && bad2);
+    rinv[k] = i1;
+    rinv[k + 1] = i2;
+#pragma unroll
+    for (int c = k + 1; c < kBlk; ++c) a[k][c] *= i1;
+#pragma unroll
+    for (int c = k + 2; c < kBlk; ++c) a[k + 1][c] = (a[k + 1][c] - a[k][k + 1] * a[k][c]) * i2;
+#pragma unroll
+    for (int i = k + 2; i < kBlk; ++i)
+#pragma unroll
+      for (int c = i; c < kBlk; ++c) a[i][c] = (a[i][c] - a[k][i] * a[k][c]) - a[k + 1][i] * a[k + 1][c];
+  }
+  if (any_bad && report && lane == 0) atomicExch(&status->rank_deficient, 1);
+  // column j of the inverse from the bottom up, the sums kept running
+  double acc[kBlk];
+#pragma unroll
+  for (int i = 0; i < kBlk; ++i) acc[i] = 0.0;
+#pragma unroll
+  for (int i = kBlk - 1; i >= 0; --i) {
+    const double x = i == j ? rinv[i] : (i < j ? -acc[i] * rinv[i] : 0.0);
+    acc[i] = x;
+#pragma unroll
+    for (int l = 0; l < i; ++l) acc[l] += a[l][i] * x;
+  }
+  if (lane < kBlk) {
+#pragma unroll
+    for (int i = 0; i < kBlk; ++i) M[(o + i) * mp + o + j] = acc[i];
+  }
+}
+
+// One 8 x 8 tile  C += sign P Q  of doubles in shared memory, k from 0 to kdim - 1:
+// element (i, k) of P at p[k * pk + i * pi], element (k, j) of Q at q[k * qk + j].
+__device__ __forceinline__ void dtile(double& c0, double& c1, const double* p, int pk, int pi, const double* q, int qk, int kdim,
+                                      double sign) {
+  const int lane = threadIdx.x & 31, fr = lane >> 2, fc = lane & 3;
+#pragma unroll 2
+  for (int k = 0; k < kdim; k += 4) dmma_m8n8k4(c0, c1, sign * p[(k + fc) * pk + fr * pi], q[(k + fc) * qk + fr]);
+}
+
+// Block (i, j), i < j, of M = R^-1 by one warp, the blocks of M left of column j and D_j being known:
+// M_ij = -(sum_{i <= l < j} M_il R_lj) D_j.  The sum passes through the block (j, i) below the diagonal of A, which nothing
+// else uses.
+template <int NT>
+__device__ __forceinline__ void qr_inverse_block(double* A, double* M, int i, int j) {
+  constexpr int ap = QrCfg<NT>::ap, mp = QrCfg<NT>::mp;
+  const int lane = threadIdx.x & 31, fr = lane >> 2, fc = lane & 3;
+  double* t = A + kBlk * j * ap + kBlk * i;
+  double c0 = 0.0, c1 = 0.0;
+  dtile(c0, c1, M + kBlk * i * mp + kBlk * i, 1, mp, A + kBlk * i * ap + kBlk * j, ap, kBlk * (j - i), 1.0);
+  t[fr * ap + 2 * fc] = c0; t[fr * ap + 2 * fc + 1] = c1;
+  __syncwarp();
+  c0 = c1 = 0.0;
+  dtile(c0, c1, t, 1, ap, M + kBlk * j * mp + kBlk * j, mp, kBlk, -1.0);
+  double* m = M + (kBlk * i + fr) * mp + kBlk * j + 2 * fc;
+  m[0] = c0; m[1] = c1;
+}
+
+// S (upper triangle in A) -> M = R^-1 (upper triangle) in blocks of 8: one warp factors the diagonal block, the rest of
+// the block row, the trailing update and the off-diagonal blocks of M are tiles on the FP64 tensor cores.  Column kb - 1
+// of M is made by the other warps while warp 0 factors block kb.  Up to 16 columns one warp does it all.  (One thread
+// arrangement over the whole matrix with a barrier per pivot, the form before this one, took 63 us at r = 64; this 15.)
+template <int NT>
+__device__ __forceinline__ void qr_factor(double* A, double* M, const double* own, int r, DevStatus* status, bool report) {
+  constexpr int ap = QrCfg<NT>::ap, mp = QrCfg<NT>::mp;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, fr = lane >> 2, fc = lane & 3;
+  const int nb = (r + kBlk - 1) / kBlk;
+  constexpr bool kOneWarp = NT <= 2;
+  if (kOneWarp && warp != 0) { __syncthreads(); return; }
+  const int me = kOneWarp ? 0 : warp, workers = kOneWarp ? 1 : kQrWarps;
+  auto sync = [&]() { if (kOneWarp) __syncwarp(); else __syncthreads(); };
+  for (int kb = 0; kb < nb; ++kb) {
+    const int o = kb * kBlk;
+    if (warp == 0) qr_factor_block<NT>(A, M, own, kb, r, status, report);
+    if (!kOneWarp && warp > 0)
+      for (int i = warp - 1; i < kb - 1; i += kQrWarps - 1) qr_inverse_block<NT>(A, M, i, kb - 1);
+    sync();
+    const int ntr = nb - 1 - kb;                            // tiles to the right of the block
+    for (int t = me; t < ntr; t += workers) {               // R_k. = R_kk^-T A_k. in place, a tile per warp
+      double* p = A + o * ap + o + kBlk * (t + 1);
+      double c0 = 0.0, c1 = 0.0;
+      dtile(c0, c1, M + o * mp + o, mp, 1, p, ap, kBlk, 1.0);
+      __syncwarp();
+      p[fr * ap + 2 * fc] = c0; p[fr * ap + 2 * fc + 1] = c1;
+    }
+    sync();
+    int t = 0;                                              // A_ij -= R_ki^T R_kj on the tiles of the upper triangle
+    for (int bi = 0; bi < ntr; ++bi)
+      for (int bj = bi; bj < ntr; ++bj, ++t) {
+        if (t % workers != me) continue;
+        double* p = A + (o + kBlk * (bi + 1) + fr) * ap + o + kBlk * (bj + 1) + 2 * fc;
+        double c0 = p[0], c1 = p[1];
+        dtile(c0, c1, A + o * ap + o + kBlk * (bi + 1), ap, 1, A + o * ap + o + kBlk * (bj + 1), ap, kBlk, -1.0);
+        p[0] = c0; p[1] = c1;
+      }
+    sync();
+  }
+  for (int i = me; i < nb - 1; i += workers) qr_inverse_block<NT>(A, M, i, nb - 1);
+  __syncthreads();
+}
+
+// Q = Y M in place on `ncols` staged columns: Q^T (r x 8 columns) = M^T Y in 8 x 8 tiles, A[k][j] = M[j][k], K = j up
+// to the tile's last k (M is upper triangular).  A warp owns whole 8-column strips, so it may overwrite them.
+template <int NT>
+__device__ __forceinline__ void qr_apply(float* sY, int pitch, const double* M, int ncols) {
+  constexpr int mp = QrCfg<NT>::mp;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, fr = lane >> 2, fc = lane & 3;
+  constexpr int kSp = 2;                          // strips at a time: independent chains for the FP64 pipe
+  for (int s0 = warp * kSp; s0 < ncols / 8; s0 += kQrWarps * kSp) {
+    double acc[kSp][NT][2];
+#pragma unroll
+    for (int sp = 0; sp < kSp; ++sp)
+#pragma unroll
+      for (int kt = 0; kt < NT; ++kt) acc[sp][kt][0] = acc[sp][kt][1] = 0.0;
+#pragma unroll
+    for (int j0 = 0; j0 < 8 * NT; j0 += 4) {
+      double b[kSp];
+#pragma unroll
+      for (int sp = 0; sp < kSp; ++sp) b[sp] = (double)sY[(j0 + fc) * pitch + 8 * (s0 + sp) + fr];
+      const double* ma = M + (j0 + fc) * mp + fr;
+#pragma unroll
+      for (int kt = 0; kt < NT; ++kt)
+        if (8 * kt + 7 >= j0) {
+          const double a = ma[8 * kt];
+#pragma unroll
+          for (int sp = 0; sp < kSp; ++sp) dmma_m8n8k4(acc[sp][kt][0], acc[sp][kt][1], a, b[sp]);
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int sp = 0; sp < kSp; ++sp)
+#pragma unroll
+      for (int kt = 0; kt < NT; ++kt)
+        *reinterpret_cast<float2*>(sY + (8 * kt + fr) * pitch + 8 * (s0 + sp) + 2 * fc) =
+            make_float2((float)acc[sp][kt][0], (float)acc[sp][kt][1]);
+  }
+}
+
+// Q of columns [d0, d0 + ncols) out: V rows (fp32) and / or the bf16 hi/lo rows of the next product's operand
+__device__ __forceinline__ void qr_store(const DevLayer& L, const float* sY, int pitch, int d0, int ncols, bool to_v, bool to_qb) {
+  const int r = L.r, d_in = L.d_in;
+  const int rows = to_qb ? L.NP : r;               // the panel's padding rows are zero, as Q's are
+  if ((d_in & 3) == 0 && (L.ldv & 3) == 0 && (reinterpret_cast<uintptr_t>(L.V) & 15u) == 0) {
+    const int vrow = ncols >> 2;
+    for (int i = threadIdx.x; i < rows * vrow; i += kQrThreads) {
+      const int k = i / vrow, c = 4 * (i - k * vrow), d = d0 + c;
+      if (d >= d_in) continue;
+      const float4 q = *reinterpret_cast<const float4*>(sY + k * pitch + c);
+      if (to_v && k < r) *reinterpret_cast<float4*>(L.V + (long long)k * L.ldv + d) = q;
+      if (to_qb) {
+        const __nv_bfloat162 h0 = __floats2bfloat162_rn(q.x, q.y), h1 = __floats2bfloat162_rn(q.z, q.w);
+        const __nv_bfloat162 l0 = __floats2bfloat162_rn(q.x - __low2float(h0), q.y - __high2float(h0));
+        const __nv_bfloat162 l1 = __floats2bfloat162_rn(q.z - __low2float(h1), q.w - __high2float(h1));
+        uint2 h, l;
+        h.x = *reinterpret_cast<const uint32_t*>(&h0); h.y = *reinterpret_cast<const uint32_t*>(&h1);
+        l.x = *reinterpret_cast<const uint32_t*>(&l0); l.y = *reinterpret_cast<const uint32_t*>(&l1);
+        *reinterpret_cast<uint2*>(L.Qb + (long long)k * d_in + d) = h;
+        *reinterpret_cast<uint2*>(L.Qb + (long long)(L.NP + k) * d_in + d) = l;
+      }
+    }
+  } else {
+    for (int i = threadIdx.x; i < rows * ncols; i += kQrThreads) {
+      const int k = i / ncols, c = i - k * ncols, d = d0 + c;
+      if (d >= d_in) continue;
+      const float q = sY[k * pitch + c];
+      if (to_v && k < r) L.V[(long long)k * L.ldv + d] = q;
+      if (to_qb) {
+        const __nv_bfloat16 hi = __float2bfloat16_rn(q);
+        L.Qb[(long long)k * d_in + d] = hi;
+        L.Qb[(long long)(L.NP + k) * d_in + d] = __float2bfloat16_rn(q - __bfloat162float(hi));
+      }
+    }
+  }
+}
+
+// kResident: the CTA's whole slice stays in shared memory from load to apply; otherwise it is staged 128 columns at
+// a time and read a second time (from L.Y, through L2) for the apply.
+template <int NT, bool kResident>
+__global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer* __restrict__ layers, int l0, int C, int pitch,
+                                                                 int y_reduced, int after_fused, int last, DevStatus* status) {
+  static_assert(NT <= 4, "larger ranks take the three launches");
+  using Cfg = QrCfg<NT>;
+  const DevLayer& L = layers[l0 + (int)blockIdx.x / C];
+  const int rank = (int)cluster_ctarank();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  extern __shared__ __align__(16) unsigned char qr_smem[];
+  double* sU = reinterpret_cast<double*>(qr_smem);                       // warps' partial sums, then S / R and M
+  double* sG = reinterpret_cast<double*>(qr_smem + Cfg::u_bytes);        // this CTA's share of S, [tile][8][8]
+  float* sY = reinterpret_cast<float*>(qr_smem + Cfg::fixed);            // [r8][pitch]
+  double* A = sU;
+  double* M = sU + Cfg::r8 * Cfg::ap;
+  __shared__ double own[AGZO_MAX_RANK];
+  const int r = L.r, nparts = y_parts(L, after_fused);
+  const int cpc = (L.gchunks + C - 1) / C;
+  const int ch0 = rank * cpc, nch = max(0, min(cpc, L.gchunks - ch0));
+  const int d0 = ch0 * kQrChunk;
+
+  double acc[Cfg::my_tiles][2];
+#pragma unroll
+  for (int t = 0; t < Cfg::my_tiles; ++t) acc[t][0] = acc[t][1] = 0.0;
+  if (kResident) {
+    qr_load(L, sY, pitch, Cfg::r8, d0, nch * kQrChunk, nparts, y_reduced != 0, false);
+    __syncthreads();
+    qr_gram<NT, 0>(sY, pitch, nch * kQrChunk / 4, warp, acc);
+  } else {
+    for (int ch = 0; ch < nch; ++ch) {
+      __syncthreads();
+      qr_load(L, sY, pitch, Cfg::r8, d0 + ch * kQrChunk, kQrChunk, nparts, y_reduced != 0, y_reduced == 0);
+      __syncthreads();
+      qr_gram<NT, 0>(sY, pitch, kQrChunk / 4, warp, acc);
+    }
+  }
+  // the warps' sums into this CTA's share of S, in warp order; fragment element (l / 4, 2 (l % 4) + x) of a tile
+  const int el = (lane >> 2) * 8 + 2 * (lane & 3);
+#pragma unroll
+  for (int t = 0; t < Cfg::tiles; ++t)
+    *reinterpret_cast<double2*>(sU + (warp * Cfg::tiles + t) * 64 + el) = make_double2(acc[t][0], acc[t][1]);
+  __syncthreads();
+  for (int i = tid; i < Cfg::tiles * 64; i += kQrThreads) {
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < kQrWarps; ++w) s += sU[w * Cfg::tiles * 64 + i];
+    sG[i] = s;
+  }
+  __syncwarp();
+  cluster_sync_all();                       // every CTA's share is in its shared memory
+  for (int i = tid; i < Cfg::tiles * 64; i += kQrThreads) {
+    double v[kQrMaxCluster], sum = 0.0;
+#pragma unroll
+    for (int c = 0; c < kQrMaxCluster; ++c) v[c] = c < C ? ld_cluster_f64(mapa_shared(smem_u32(sG + i), (uint32_t)c)) : 0.0;
+#pragma unroll
+    for (int c = 0; c < kQrMaxCluster; ++c) sum += v[c];
+    int t = i >> 6, bi = 0;
+    while (t >= NT - bi) { t -= NT - bi; ++bi; }
+    const int row = 8 * bi + ((i & 63) >> 3), col = 8 * (bi + t) + (i & 7);
+    A[row * Cfg::ap + col] = sum;
+    if (row == col) own[row] = sum;
+  }
+  __syncthreads();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // done with the peers' shares
+  qr_factor<NT>(A, M, own, r, status, rank == 0);
+
+  const bool to_v = last || !L.Qb, to_qb = !last && L.Qb;
+  if (kResident) {
+    qr_apply<NT>(sY, pitch, M, nch * kQrChunk);
+    __syncthreads();
+    qr_store(L, sY, pitch, d0, nch * kQrChunk, to_v, to_qb);
+  } else {
+    for (int ch = 0; ch < nch; ++ch) {
+      __syncthreads();
+      qr_load(L, sY, pitch, Cfg::r8, d0 + ch * kQrChunk, kQrChunk, nparts, true, false);
+      __syncthreads();
+      qr_apply<NT>(sY, pitch, M, kQrChunk);
+      __syncthreads();
+      qr_store(L, sY, pitch, d0 + ch * kQrChunk, kQrChunk, to_v, to_qb);
+    }
+  }
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // nobody leaves while a peer may read its share
+}
+
+// ------------------------------------------------------------------ ranks above 32: three launches
+constexpr int kGramGroup = 4;            // 128-column chunks per CTA of the Gram launch
+
+// In global memory a share of S is the nt (nt + 1) / 2 tiles of the layer's own rank (nt = r / 8, rounded up), row by
+// row; M, once it is known, takes the place of the first share.
+__host__ __device__ inline int qr_share_elems(int r) { const int nt = (r + 7) >> 3; return nt * (nt + 1) / 2 * 64; }
+__device__ __forceinline__ void qr_tile_of(int t, int nt, int* bi, int* bj) {
+  int b = 0;
+  while (t >= nt - b) { t -= nt - b; ++b; }
+  *bi = b; *bj = b + t;
+}
+
+// Gram share of up to 512 columns of a layer, and their Y = sum of the partial sums.  Two warps split the columns of
+// each of the four tile sets; a scheduler's two warps have 18 tiles between them.
+__global__ void __launch_bounds__(kQrThreads, 2) panel_gram_kernel(const DevLayer* __restrict__ layers, int l0, int y_reduced,
+                                                                   int after_fused) {
+  using Cfg = QrCfg<8>;
+  const DevLayer& L = layers[l0 + blockIdx.y];
+  const int ch0 = blockIdx.x * kGramGroup;
+  if (ch0 >= L.gchunks) return;
+  const int nch = min(kGramGroup, L.gchunks - ch0), nparts = y_parts(L, after_fused);
+  extern __shared__ __align__(16) unsigned char qr_smem[];
+  float* sY = reinterpret_cast<float*>(qr_smem);           // [64][pitch], then the share of S
+  const int pitch = qr_pitch(kQrChunk);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int set = (warp + 2 * (warp >> 2)) & 3, turn0 = warp >> 2;
+  double acc[Cfg::my_tiles][2];
+#pragma unroll
+  for (int t = 0; t < Cfg::my_tiles; ++t) acc[t][0] = acc[t][1] = 0.0;
+  for (int ch = 0; ch < nch; ++ch) {
+    __syncthreads();
+    qr_load(L, sY, pitch, Cfg::r8, (ch0 + ch) * kQrChunk, kQrChunk, nparts, y_reduced != 0, y_reduced == 0);
+    __syncthreads();
+    if (set == 0) qr_gram<8, 0>(sY, pitch, kQrChunk / 4, turn0, acc);
+    else if (set == 1) qr_gram<8, 1>(sY, pitch, kQrChunk / 4, turn0, acc);
+    else if (set == 2) qr_gram<8, 2>(sY, pitch, kQrChunk / 4, turn0, acc);
+    else qr_gram<8, 3>(sY, pitch, kQrChunk / 4, turn0, acc);
+  }
+  static_assert(Cfg::g_bytes <= (size_t)Cfg::r8 * (kQrChunk + 12) * 4, "the share of S fits the staging buffer");
+  double* sG = reinterpret_cast<double*>(qr_smem);
+  const int el = (lane >> 2) * 8 + 2 * (lane & 3);
+  __syncthreads();                        // the staged columns have been used: their place takes the sums
+  for (int turn = 0; turn < Cfg::ksplit; ++turn) {
+    if (turn0 == turn) {
+      if (set == 0) qr_add_share<8, 0>(sG + el, acc, turn == 0);
+      else if (set == 1) qr_add_share<8, 1>(sG + el, acc, turn == 0);
+      else if (set == 2) qr_add_share<8, 2>(sG + el, acc, turn == 0);
+      else qr_add_share<8, 3>(sG + el, acc, turn == 0);
+    }
+    __syncthreads();
+  }
+  const int nt = (L.r + 7) >> 3, n2 = qr_share_elems(L.r) / 2;
+  double2* out = reinterpret_cast<double2*>(L.Gpart) + (size_t)blockIdx.x * n2;
+  for (int i = tid; i < n2; i += kQrThreads) {
+    int bi, bj;
+    qr_tile_of(i >> 5, nt, &bi, &bj);
+    out[i] = reinterpret_cast<const double2*>(sG)[(bi * 8 - bi * (bi - 1) / 2 + bj - bi) * 32 + (i & 31)];
+  }
+}
+
+// One CTA per layer: S = sum of its shares in order, factorisation, M out
+__global__ void __launch_bounds__(kQrThreads) panel_factor_kernel(const DevLayer* __restrict__ layers, int l0, DevStatus* status) {
+  using Cfg = QrCfg<8>;
+  const DevLayer& L = layers[l0 + blockIdx.x];
+  extern __shared__ __align__(16) unsigned char qr_smem[];
+  double* A = reinterpret_cast<double*>(qr_smem);
+  double* M = A + Cfg::r8 * Cfg::ap;
+  __shared__ double own[AGZO_MAX_RANK];
+  const int tid = threadIdx.x, r = L.r;
+  const int nsh = (L.gchunks + kGramGroup - 1) / kGramGroup;
+  const int nt = (r + 7) >> 3, ne = qr_share_elems(r);
+  constexpr int kPer = (Cfg::tiles * 64 + kQrThreads - 1) / kQrThreads;
+  double sum[kPer];
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) sum[u] = 0.0;
+  for (int s0 = 0; s0 < nsh; s0 += 2) {
+    double v[2][kPer];
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) {
+        const int i = tid + u * kQrThreads;
+        v[s][u] = s0 + s < nsh && i < ne ? __ldcg(L.Gpart + (size_t)(s0 + s) * ne + i) : 0.0;
+      }
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) sum[u] += v[s][u];
+  }
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const int i = tid + u * kQrThreads;
+    if (i >= ne) break;
+    int bi, bj;
+    qr_tile_of(i >> 6, nt, &bi, &bj);
+    const int row = 8 * bi + ((i & 63) >> 3), col = 8 * bj + (i & 7);
+    A[row * Cfg::ap + col] = sum[u];
+    if (row == col) own[row] = sum[u];
+  }
+  __syncthreads();
+  qr_factor<8>(A, M, own, r, status, true);
+  for (int i = tid; i < ne; i += kQrThreads) {
+    int bi, bj;
+    qr_tile_of(i >> 6, nt, &bi, &bj);
+    L.Gpart[i] = M[(8 * bi + ((i & 63) >> 3)) * Cfg::mp + 8 * bj + (i & 7)];
+  }
+}
+
+// Q = Y M on 128 columns of a layer
+__global__ void __launch_bounds__(kQrThreads, 2) panel_apply_kernel(const DevLayer* __restrict__ layers, int l0, int last) {
+  using Cfg = QrCfg<8>;
+  const DevLayer& L = layers[l0 + blockIdx.y];
+  const int d0 = blockIdx.x * kQrChunk;
+  if (d0 >= L.d_in) return;
+  extern __shared__ __align__(16) unsigned char qr_smem[];
+  double* M = reinterpret_cast<double*>(qr_smem);
+  float* sY = reinterpret_cast<float*>(M + Cfg::r8 * Cfg::mp);
+  const int pitch = qr_pitch(kQrChunk);
+  for (int i = threadIdx.x; i < Cfg::r8 * Cfg::mp; i += kQrThreads) M[i] = 0.0;   // tiles below the diagonal, rows beyond r
+  __syncthreads();
+  const int nt = (L.r + 7) >> 3, n2 = qr_share_elems(L.r) / 2;
+  constexpr int kPer = (Cfg::tiles * 32 + kQrThreads - 1) / kQrThreads;
+  double2 v[kPer];
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const int i = threadIdx.x + u * kQrThreads;
+    v[u] = i < n2 ? __ldcg(reinterpret_cast<const double2*>(L.Gpart) + i) : make_double2(0.0, 0.0);
+  }
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const int i = threadIdx.x + u * kQrThreads;
+    if (i >= n2) break;
+    int bi, bj;
+    qr_tile_of(i >> 5, nt, &bi, &bj);
+    *reinterpret_cast<double2*>(M + (8 * bi + ((i & 31) >> 2)) * Cfg::mp + 8 * bj + 2 * (i & 3)) = v[u];
+  }
+  qr_load(L, sY, pitch, Cfg::r8, d0, kQrChunk, 1, true, false);
+  __syncthreads();
+  qr_apply<8>(sY, pitch, M, kQrChunk);
+  __syncthreads();
+  qr_store(L, sY, pitch, d0, kQrChunk, last || !L.Qb, !last && L.Qb);
+}
+
+// CTAs per layer: eight while the launch is a chain of latencies; with so many layers that eight each would queue for
+// the SMs (two CTAs each), four or two, since every CTA repeats the factorisation (r = 8, d_in = 2048, 196 layers: 44.5 /
+// 27.7 / 26.1 us with 8 / 4 / 2; r = 16, d_in = 4096, 70 layers: 43.5 / 28.3 / 55.1 us; 35 layers 28.7 / 27.4 / 51.5)
+int qr_cluster(const ExtractWave& w) {
+  const int nl = w.l1 - w.l0;
+  const int most = nl <= 40 ? 8 : nl <= 80 ? 4 : 2;
+  return w.max_gchunks < most ? w.max_gchunks : most;
+}
+
+template <int NT>
+cudaError_t launch_qr(const ExtractWave& w, bool last, DevStatus* d_status, cudaStream_t s) {
+  using Cfg = QrCfg<NT>;
+  const int C = qr_cluster(w);
+  const int slice = (w.max_gchunks + C - 1) / C * kQrChunk;
+  const size_t whole = Cfg::fixed + (size_t)Cfg::r8 * qr_pitch(slice) * sizeof(float);
+  const bool resident = whole <= kQrResidentSmem;
+  const int pitch = qr_pitch(resident ? slice : kQrChunk);
+  const size_t smem = Cfg::fixed + (size_t)Cfg::r8 * pitch * sizeof(float);
+  auto kernel = resident ? panel_qr_kernel<NT, true> : panel_qr_kernel<NT, false>;
+  if (smem > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQrResidentSmem);
+    if (e != cudaSuccess) return e;
+  }
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)C;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)(C * (w.l1 - w.l0)));
+  cfg.blockDim = dim3(kQrThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, w.d_layers, w.l0, C, pitch, w.y_reduced, w.after_fused, last ? 1 : 0, d_status);
+}
+
+cudaError_t launch_qr_large(const ExtractWave& w, bool last, DevStatus* d_status, cudaStream_t s) {
+  using Cfg = QrCfg<8>;
+  const unsigned nl = (unsigned)(w.l1 - w.l0);
+  const size_t stage = (size_t)Cfg::r8 * qr_pitch(kQrChunk) * sizeof(float);
+  const size_t factor = Cfg::am_bytes, apply = (size_t)Cfg::r8 * Cfg::mp * sizeof(double) + stage;
+  cudaError_t e = cudaFuncSetAttribute(panel_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)factor);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(panel_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply);
+  if (e != cudaSuccess) return e;
+  panel_gram_kernel<<<dim3((unsigned)((w.max_gchunks + kGramGroup - 1) / kGramGroup), nl), kQrThreads, stage, s>>>(
+      w.d_layers, w.l0, w.y_reduced, w.after_fused);
+  panel_factor_kernel<<<nl, kQrThreads, factor, s>>>(w.d_layers, w.l0, d_status);
+  panel_apply_kernel<<<dim3((unsigned)w.max_gchunks, nl), kQrThreads, apply, s>>>(w.d_layers, w.l0, last ? 1 : 0);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+int panel_qr_launches(int max_r) { return max_r > 32 ? 3 : 1; }
+
+// Scratch of a layer for the three-launch form, which a wave with a larger rank takes for all its layers
+size_t panel_gram_bytes(int d_in, int r) {
+  const size_t groups = (size_t)((d_in + kGramGroup * kQrChunk - 1) / (kGramGroup * kQrChunk));
+  return groups * qr_share_elems(r) * sizeof(double);
+}
+
+cudaError_t launch_panel_qr(const ExtractWave& w, bool last, DevStatus* d_status, cudaStream_t s) {
+  if (w.max_r <= 8) return launch_qr<1>(w, last, d_status, s);
+  if (w.max_r <= 16) return launch_qr<2>(w, last, d_status, s);
+  if (w.max_r <= 32) return launch_qr<4>(w, last, d_status, s);
+  return launch_qr_large(w, last, d_status, s);
+}
+
+}  // namespace agzo

@@ -99,8 +99,7 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
   rec.T = reinterpret_cast<float*>(p);      p += up256(M * R * 4);
   rec.Ypart = reinterpret_cast<float*>(p);  p += up256((size_t)slabs * R * D * 4);
   rec.Y = reinterpret_cast<float*>(p);      p += up256(R * D * 4);
-  rec.Gpart = reinterpret_cast<double*>(p); p += up256(gch * R * R * 8);
-  rec.M = reinterpret_cast<double*>(p);
+  rec.Gpart = reinterpret_cast<double*>(p);     // never more than the two terms in r^2 of the limit above
   static_assert(sizeof(DevLayer) <= 384, "layer record must fit its slot");
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -114,11 +113,11 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
   if (launch_fill_omega(w, seed, s) != cudaSuccess) return AGZO_ERR_CUDA;     // Omega
   if (launch_xt_t(w, s) != cudaSuccess) return AGZO_ERR_CUDA;                 // Y <- H Omega
   for (int k = 0; k < K; ++k) {
-    if (launch_panel_qr(w, d_status, s) != cudaSuccess) return AGZO_ERR_CUDA;  // Q <- qr(Y)
+    if (launch_panel_qr(w, false, d_status, s) != cudaSuccess) return AGZO_ERR_CUDA;  // Q <- qr(Y)
     if (launch_x_q(w, s) != cudaSuccess) return AGZO_ERR_CUDA;
     if (launch_xt_t(w, s) != cudaSuccess) return AGZO_ERR_CUDA;               // Y <- H (H^T Q)
   }
-  if (launch_panel_qr(w, d_status, s) != cudaSuccess) return AGZO_ERR_CUDA;    // A <- qr(Y)
+  if (launch_panel_qr(w, true, d_status, s) != cudaSuccess) return AGZO_ERR_CUDA;    // A <- qr(Y)
   if (d_rank_deficient) {
     static_end_kernel<<<1, 1, 0, s>>>(d_status, d_rank_deficient);
     if (cudaGetLastError() != cudaSuccess) return AGZO_ERR_CUDA;

@@ -1,0 +1,47 @@
+"""qr(Y) at the edges of its dispatch: ranks around the tiles of eight, the change of form above rank 32, slices that
+stay in shared memory and slices that do not, every cluster size (layers per launch), panels without 16-byte rows.
+
+Tolerances: orthonormality 1e-5 (Q is rounded to fp32: r entries of 2^-24 relative error each, with the Gram matrix and
+the factor in double); projectors 1e-3 as everywhere (the fp32 product before the factorisation)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import agzo_oracle as O
+from paper_2601_17261_b200 import binding as B
+from paper_2601_17261_b200 import workloads as WL
+
+from gpu_helpers import DEV, Ctx, projector_distance, to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+
+def check(m, dims, r, K, bf16, n_layers=1):
+    Xs = [WL.planted_activations(m, d, min(16, d), seed=7 + d, bf16=bf16) for d in dims]
+    devs = [to_dev(X, bf16)[0] for X in Xs]
+    pick = [i % len(dims) for i in range(n_layers)]
+    Vs = [torch.full((r, dims[p]), 7.0, device=DEV) for p in pick]
+    layers = [B.make_layer(X=devs[p], V=V, r=r, layer_id=i) for i, (p, V) in enumerate(zip(pick, Vs))]
+    with Ctx(layers) as ctx:
+        B.agzo_extract_subspace(ctx, layers, 5, K)
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+    for i in sorted({0, n_layers // 2, n_layers - 1}):
+        Vg = to_host(Vs[i])
+        assert np.abs(Vg.astype(np.float64) @ Vg.T - np.eye(r)).max() <= 1e-5, i
+        assert projector_distance(Vg, O.extract_subspace(Xs[pick[i]], r, K, 5, i)) <= 1e-3, i
+
+
+@pytest.mark.parametrize("r", [1, 7, 8, 9, 16, 17, 32, 33, 40, 41, 64])
+@pytest.mark.parametrize("d_in", [67, 130, 1160])
+def test_ranks_and_columns(r, d_in):
+    check(300, [d_in], r, 1, bf16=False)
+
+
+@pytest.mark.parametrize("r,dims", [(16, [12288]), (16, [12416]), (32, [4096]), (8, [24704])])
+def test_slices_in_and_out_of_shared_memory(r, dims):
+    check(256, dims, r, 1, bf16=True)
+
+
+@pytest.mark.parametrize("n_layers", [40, 41, 80, 81])
+def test_layers_per_launch(n_layers):
+    check(256, [1032, 128, 3080], 12, 1, bf16=True, n_layers=n_layers)
