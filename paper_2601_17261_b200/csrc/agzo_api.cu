@@ -187,22 +187,26 @@ bool same_input(const agzo_layer& a, const agzo_layer& b) {
   return a.X == b.X && a.ldx == b.ldx && a.m == b.m && a.d_in == b.d_in && a.x_dtype == b.x_dtype;
 }
 
-// Token slabs of the X^T T product.  CUDA-core kernels: 32 slabs at most.  Tensor-core
-// kernels: slabs of 2048 tokens (32 pipeline steps per CTA) when the layer has that many.  When
+// Token slabs of the X^T T product.  CUDA-core kernels: cc_slab_rows.  Tensor-core kernels: slabs of 2048 tokens (32 pipeline steps per CTA) when the layer has that many.  When
 // the call's layers fill the grid by their column blocks alone (long_slabs), a slab is up to
 // 16384 tokens: every slab costs a partial Y (r x d_in floats written, and read again by the
 // panel QR), and the CTAs' pipelines start and drain less often.
 constexpr int kLongSlabColumnBlocks = 1024;   // 128-column blocks over all layers from which slabs are long
-void slab_shape(const agzo_layer& a, bool tc, bool long_slabs, int* slabs, int* slab_rows) {
+// cc_blocks: 128-column blocks over the call's layers on the CUDA-core path; 0 = the most slabs the layer can get (sizing).
+void slab_shape(const agzo_layer& a, bool tc, bool long_slabs, long long cc_blocks, int* slabs, int* slab_rows) {
   int rows;
   if (tc) {
     rows = a.m >= 8192 ? (long_slabs ? (a.m < 16384 ? a.m : 16384) : 2048) : (a.m + 3) / 4;
     rows = (rows + 127) / 128 * 128;      // whole tiles of every tensor-core kernel (64 or 128 tokens)
+    if (rows < 256) rows = 256;
+  } else if (cc_blocks > 0) {
+    rows = cc_slab_rows(a.m, cc_blocks);
   } else {
-    rows = (a.m + 31) / 32;
-    rows = (rows + 31) / 32 * 32;
+    const int most = (a.m + kCcMinSlabRows - 1) / kCcMinSlabRows;
+    *slabs = most < kCcMaxSlabs ? most : kCcMaxSlabs;
+    *slab_rows = 0;
+    return;
   }
-  if (rows < 256) rows = 256;
   *slab_rows = rows;
   *slabs = (a.m + rows - 1) / rows;
 }
@@ -210,10 +214,11 @@ void slab_shape(const agzo_layer& a, bool tc, bool long_slabs, int* slabs, int* 
 // scratch bytes one layer needs for extraction (0 when it has no X)
 // y_parts_min: room for at least that many partial sums of Y (the fused power step leaves one per share of
 // its launch that meets the layer, which can be more than the slabs of X^T T)
-size_t layer_scratch(const agzo_layer& a, bool tc, bool long_slabs, bool with_panels = true, int y_parts_min = 0) {
+size_t layer_scratch(const agzo_layer& a, bool tc, bool long_slabs, long long cc_blocks, bool with_panels = true,
+                     int y_parts_min = 0) {
   if (!has_x(a)) return 0;
   int slabs, slab_rows;
-  slab_shape(a, tc, long_slabs, &slabs, &slab_rows);
+  slab_shape(a, tc, long_slabs, cc_blocks, &slabs, &slab_rows);
   if (slabs < y_parts_min) slabs = y_parts_min;
   const size_t r = (size_t)a.r, d = (size_t)a.d_in, m = (size_t)a.m;
   size_t b = 0;
@@ -347,10 +352,10 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     return opts.extract_fused && extract_path != 1 && extract_path != 3 && tc_available && tc_eligible(a) &&
            fused_eligible(opts.fused_caps, a, opts.extract_fused == 2) && (opts.extract_fused == 2 || !shares_input((int)(&a - L)));
   };
-  long long column_blocks = 0;
+  long long column_blocks = 0, cc_blocks = 0;
   for (int k = 0; k < n; ++k)
-    if (has_x(L[k]) && extract_path != 1 && tc_available && tc_eligible(L[k]))
-      column_blocks += (L[k].d_in + 127) / 128;
+    if (has_x(L[k]))
+      (extract_path != 1 && tc_available && tc_eligible(L[k]) ? column_blocks : cc_blocks) += (L[k].d_in + 127) / 128;
   const bool long_slabs_any = column_blocks >= kLongSlabColumnBlocks;
   auto long_slabs_for = [&](const agzo_layer&) { return long_slabs_any; };
   auto y_parts_min = [&](const agzo_layer& a) {
@@ -385,7 +390,8 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
       }
       auto unit_need = [&](int len, int nrows) {
         size_t b = 0;
-        for (int g = 0; g < len; ++g) b += layer_scratch(L[j + g], tc, long_slabs_for(L[j + g]), false, y_parts_min(L[j + g]));
+        for (int g = 0; g < len; ++g)
+          b += layer_scratch(L[j + g], tc, long_slabs_for(L[j + g]), ws ? cc_blocks : 0, false, y_parts_min(L[j + g]));
         if (tc) b += tc_panel_bytes(L[j], nrows);
         return b;
       };
@@ -407,7 +413,7 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
           DevLayer& D = plan->dev[j + g];
           const agzo_layer& a = L[j + g];
           int slabs, slab_rows;
-          slab_shape(a, tc, long_slabs_for(a), &slabs, &slab_rows);
+          slab_shape(a, tc, long_slabs_for(a), cc_blocks, &slabs, &slab_rows);
           const size_t r = (size_t)a.r, d = (size_t)a.d_in, m = (size_t)a.m;
           const size_t gch = (d + 127) / 128;
           D.slabs = slabs; D.slab_rows = slab_rows; D.gchunks = (int)gch;

@@ -37,117 +37,255 @@ cudaError_t launch_fill_omega(const ExtractWave& w, uint64_t seed, cudaStream_t 
   return cudaGetLastError();
 }
 
-__device__ __forceinline__ float load_x(const DevLayer& L, long long t, int d) {
-  return L.x_dtype == AGZO_BF16
-             ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(L.X)[t * L.ldx + d])
-             : reinterpret_cast<const float*>(L.X)[t * L.ldx + d];
+// ------------------------------------------------------------------ four consecutive columns of one row of X
+// kind of access a layer's X allows: 16-byte fp32, 8-byte bf16, or element by element
+enum XKind : int { X_F32_VEC = 0, X_BF16_VEC = 1, X_SCALAR = 2 };
+__device__ __forceinline__ int x_kind(const DevLayer& L) {
+  const uintptr_t p = reinterpret_cast<uintptr_t>(L.X);
+  if ((L.d_in & 3) != 0 || (L.ldx & 3) != 0) return X_SCALAR;
+  if (L.x_dtype == AGZO_F32) return (p & 15u) == 0 ? X_F32_VEC : X_SCALAR;
+  return (p & 7u) == 0 ? X_BF16_VEC : X_SCALAR;
+}
+// zero beyond d_in; `ok` false: zeros
+template <int KIND>
+__device__ __forceinline__ float4 load_x4(const DevLayer& L, long long t, int d, bool ok) {
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (!ok || d >= L.d_in) return v;
+  if constexpr (KIND == X_F32_VEC) {
+    return __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(L.X) + t * L.ldx + d));
+  } else if constexpr (KIND == X_BF16_VEC) {
+    const uint2 u = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(L.X) + t * L.ldx + d));
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                       __uint_as_float(u.y & 0xFFFF0000u));
+  } else {
+    float e[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const long long at = t * L.ldx + d + c;
+      e[c] = d + c >= L.d_in ? 0.f
+             : L.x_dtype == AGZO_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(L.X)[at])
+                                      : reinterpret_cast<const float*>(L.X)[at];
+    }
+    return make_float4(e[0], e[1], e[2], e[3]);
+  }
 }
 
+constexpr int kXThreads = 256, kXWarps = kXThreads / 32;
+constexpr int kXCols = 128;              // columns of one row that a warp reads at a time, four per lane
+
 // ------------------------------------------------------------------ Ypart[s][k][d] = sum_{t in slab s} X[t][d] T[t][k]
-// block: 256 threads = 256 columns d; grid (d chunks, slabs, layers).  Rank handled in chunks of 16.
-constexpr int kXtTokens = 32;
-__global__ void __launch_bounds__(256) xt_t_kernel(const DevLayer* __restrict__ layers, int l0) {
-  const DevLayer& L = layers[l0 + blockIdx.z];
-  const int slab = blockIdx.y;
-  if (slab >= L.slabs) return;
-  const int d0 = blockIdx.x * 256;
-  if (d0 >= L.d_in) return;
-  const int d = d0 + threadIdx.x;
-  const bool d_ok = d < L.d_in;
-  const int t_begin = slab * L.slab_rows;
-  const int t_end = min(L.m, t_begin + L.slab_rows);
-  __shared__ float sT[kXtTokens][16];
-  const int r = L.r;
-  for (int k0 = 0; k0 < r; k0 += 16) {
-    const int kc = min(16, r - k0);
-    float acc[16];
+// CTA = 128 columns x token slab; a lane keeps 4 columns x RC ranks in registers, the eight warps split the tokens of
+// the slab (their sums are added pairwise at the end, in a fixed order), T comes from shared memory as broadcasts.
+// Ranks above RC are further passes over the slab, from L2.
+// Bound by X (HBM, or L2 where neighbouring layers read the same buffer) for RC <= 8.  The form before this one gave a
+// thread one column and all tokens of the slab, one 2- or 4-byte load at a time, and always 16 ranks: 14 fp32 layers of 4000
+// tokens (328 MB), r = 8: 289 us per product, now 115; one 512 x 256 layer, r = 4: 60 us, now 3.4.
+constexpr int kXtTokens = 128;           // tokens of T staged at a time
+template <int RC, int KIND>
+__device__ __forceinline__ void xt_t_body(const DevLayer& L, float* sT, float* sRed, int d0, int slab) {
+  constexpr int U = 4;                   // tokens in flight per warp
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int d = d0 + 4 * lane, r = L.r;
+  const int t_begin = slab * L.slab_rows, t_end = min(L.m, t_begin + L.slab_rows);
+  for (int k0 = 0; k0 < r; k0 += RC) {
+    const int kc = min(RC, r - k0);
+    float acc[RC][4];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) acc[k] = 0.f;
+    for (int k = 0; k < RC; ++k)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[k][c] = 0.f;
     for (int tb = t_begin; tb < t_end; tb += kXtTokens) {
+      float4 x[U];                       // the first rows of the chunk are on their way while T is staged
+      const int n = min(kXtTokens, t_end - tb);
+#pragma unroll
+      for (int u = 0; u < U; ++u) x[u] = load_x4<KIND>(L, tb + warp + u * kXWarps, d, warp + u * kXWarps < n);
       __syncthreads();
-      for (int i = threadIdx.x; i < kXtTokens * 16; i += 256) {
-        const int tt = i >> 4, k = i & 15;
-        sT[tt][k] = (tb + tt < t_end && k < kc) ? L.T[(long long)(tb + tt) * r + k0 + k] : 0.f;
+      for (int i = threadIdx.x; i < n * RC; i += kXThreads) {
+        const int tt = i / RC, k = i - tt * RC;
+        sT[i] = k < kc ? L.T[(long long)(tb + tt) * r + k0 + k] : 0.f;
       }
       __syncthreads();
-      if (d_ok) {
-        const int nt = min(kXtTokens, t_end - tb);
-        for (int tt = 0; tt < nt; ++tt) {
-          const float x = load_x(L, tb + tt, d);
+      for (int t0 = warp; t0 < n; t0 += U * kXWarps) {
+        float4 nx[U];
 #pragma unroll
-          for (int k = 0; k < 16; ++k) acc[k] = fmaf(x, sT[tt][k], acc[k]);
+        for (int u = 0; u < U; ++u) {
+          const int t = t0 + (U + u) * kXWarps;
+          nx[u] = load_x4<KIND>(L, tb + t, d, t < n);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int t = min(t0 + u * kXWarps, n - 1);          // x is zero beyond n
+#pragma unroll
+          for (int k4 = 0; k4 < RC; k4 += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(sT + t * RC + k4);
+            const float tv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              acc[k4 + k][0] = fmaf(x[u].x, tv[k], acc[k4 + k][0]);
+              acc[k4 + k][1] = fmaf(x[u].y, tv[k], acc[k4 + k][1]);
+              acc[k4 + k][2] = fmaf(x[u].z, tv[k], acc[k4 + k][2]);
+              acc[k4 + k][3] = fmaf(x[u].w, tv[k], acc[k4 + k][3]);
+            }
+          }
+          x[u] = nx[u];
         }
       }
     }
-    if (d_ok) {
+    // the warps' sums, halving: 4..7 onto 0..3, 2..3 onto 0..1, 1 onto 0
+#pragma unroll
+    for (int half = kXWarps / 2; half >= 1; half >>= 1) {
+      __syncthreads();
+      if (warp >= half && warp < 2 * half) {
+#pragma unroll
+        for (int k = 0; k < RC; ++k)
+          *reinterpret_cast<float4*>(sRed + (((warp - half) * RC + k) * 32 + lane) * 4) =
+              make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
+      }
+      __syncthreads();
+      if (warp < half) {
+#pragma unroll
+        for (int k = 0; k < RC; ++k) {
+          const float4 v = *reinterpret_cast<const float4*>(sRed + ((warp * RC + k) * 32 + lane) * 4);
+          acc[k][0] += v.x; acc[k][1] += v.y; acc[k][2] += v.z; acc[k][3] += v.w;
+        }
+      }
+    }
+    if (warp == 0) {
       float* out = L.Ypart + ((long long)slab * r + k0) * L.d_in + d;
-      for (int k = 0; k < kc; ++k) out[(long long)k * L.d_in] = acc[k];
+#pragma unroll
+      for (int k = 0; k < RC; ++k) {
+        if (k >= kc) break;
+        if (KIND != X_SCALAR) {
+          if (d < L.d_in)
+            *reinterpret_cast<float4*>(out + (long long)k * L.d_in) = make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
+        } else {
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (d + c < L.d_in) out[(long long)k * L.d_in + c] = acc[k][c];
+        }
+      }
     }
   }
 }
 
+template <int RC>
+__global__ void __launch_bounds__(kXThreads, 2) xt_t_kernel(const DevLayer* __restrict__ layers, int l0) {
+  const DevLayer& L = layers[l0 + blockIdx.z];
+  const int slab = blockIdx.y, d0 = blockIdx.x * kXCols;
+  if (slab >= L.slabs || d0 >= L.d_in) return;
+  __shared__ __align__(16) float sT[kXtTokens * RC];
+  __shared__ __align__(16) float sRed[kXWarps / 2 * RC * kXCols];
+  const int kind = x_kind(L);
+  if (kind == X_F32_VEC) xt_t_body<RC, X_F32_VEC>(L, sT, sRed, d0, slab);
+  else if (kind == X_BF16_VEC) xt_t_body<RC, X_BF16_VEC>(L, sT, sRed, d0, slab);
+  else xt_t_body<RC, X_SCALAR>(L, sT, sRed, d0, slab);
+}
+
 cudaError_t launch_xt_t(const ExtractWave& w, cudaStream_t s) {
-  dim3 grid((w.max_din + 255) / 256, w.max_slabs, w.l1 - w.l0);
-  xt_t_kernel<<<grid, 256, 0, s>>>(w.d_layers, w.l0);
+  const dim3 grid((w.max_din + kXCols - 1) / kXCols, w.max_slabs, w.l1 - w.l0);
+  if (w.max_r <= 4) xt_t_kernel<4><<<grid, kXThreads, 0, s>>>(w.d_layers, w.l0);
+  else if (w.max_r <= 8) xt_t_kernel<8><<<grid, kXThreads, 0, s>>>(w.d_layers, w.l0);
+  else xt_t_kernel<16><<<grid, kXThreads, 0, s>>>(w.d_layers, w.l0);
   return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ T[t][k] = sum_d X[t][d] Q[k][d]   (Q = rows of V)
-// one warp per token; Q streamed through shared memory in column chunks.
-constexpr int kXqCols = 256;
-constexpr int kXqWarps = 8;
-__global__ void __launch_bounds__(256) x_q_kernel(const DevLayer* __restrict__ layers, int l0) {
-  const DevLayer& L = layers[l0 + blockIdx.y];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tokens_per_block = kXqWarps * 4;
-  const int t0 = blockIdx.x * tokens_per_block;
-  if (t0 >= L.m) return;
-  __shared__ float sQ[16][kXqCols + 1];
-  const int r = L.r;
-  for (int k0 = 0; k0 < r; k0 += 16) {
-    const int kc = min(16, r - k0);
-    float acc[4][16];
+// A warp takes four tokens, its lanes four columns each; Q passes through shared memory 512 columns at a time, so that
+// a 16-byte read of it serves 16 multiply-adds (as many cycles of the FMA pipes as the read takes of shared memory).
+// The lanes' sums are added by halving exchanges (a lane ends up with RC / 8 of them).  Same bound as X^T T; before: one column per lane and load, 16 ranks always, 713 us and 15 us
+// on the two examples above, now 95 and 3.1.
+constexpr int kXqChunk = 512, kXqTokens = 4;
+template <int RC, int KIND>
+__device__ __forceinline__ void x_q_body(const DevLayer& L, float* sQ, int t0) {
+  constexpr int TOK = kXqTokens;
+  const int lane = threadIdx.x & 31, r = L.r, d_in = L.d_in;
+  const bool v_vec = (d_in & 3) == 0 && (L.ldv & 3) == 0 && (reinterpret_cast<uintptr_t>(L.V) & 15u) == 0;
+  for (int k0 = 0; k0 < r; k0 += RC) {
+    const int kc = min(RC, r - k0);
+    float acc[TOK * RC];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < TOK * RC; ++i) acc[i] = 0.f;
+    for (int c0 = 0; c0 < d_in; c0 += kXqChunk) {
+      const int nc = min(kXqChunk, d_in - c0);
+      float4 x[TOK];                     // the first columns of the chunk are on their way while Q is staged
 #pragma unroll
-      for (int k = 0; k < 16; ++k) acc[i][k] = 0.f;
-    for (int c0 = 0; c0 < L.d_in; c0 += kXqCols) {
+      for (int t = 0; t < TOK; ++t) x[t] = load_x4<KIND>(L, t0 + t, c0 + 4 * lane, t0 + t < L.m);
       __syncthreads();
-      for (int i = threadIdx.x; i < 16 * kXqCols; i += 256) {
-        const int k = i / kXqCols, c = i - k * kXqCols;
-        sQ[k][c] = (k < kc && c0 + c < L.d_in) ? L.V[(long long)(k0 + k) * L.ldv + c0 + c] : 0.f;
-      }
-      __syncthreads();
-      const int nc = min(kXqCols, L.d_in - c0);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int t = t0 + warp * 4 + i;
-        if (t < L.m) {
-          for (int c = lane; c < nc; c += 32) {
-            const float x = load_x(L, t, c0 + c);
-#pragma unroll
-            for (int k = 0; k < 16; ++k) acc[i][k] = fmaf(x, sQ[k][c], acc[i][k]);
-          }
+      if (v_vec) {
+        for (int i = threadIdx.x; i < RC * (kXqChunk / 4); i += kXThreads) {
+          const int k = i / (kXqChunk / 4), c = 4 * (i - k * (kXqChunk / 4));
+          *reinterpret_cast<float4*>(sQ + k * kXqChunk + c) =
+              k < kc && c < nc ? *reinterpret_cast<const float4*>(L.V + (long long)(k0 + k) * L.ldv + c0 + c)
+                               : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      } else {
+        for (int i = threadIdx.x; i < RC * kXqChunk; i += kXThreads) {
+          const int k = i / kXqChunk, c = i - k * kXqChunk;
+          sQ[i] = k < kc && c < nc ? L.V[(long long)(k0 + k) * L.ldv + c0 + c] : 0.f;
         }
       }
+      __syncthreads();
+      for (int c = 4 * lane; c - 4 * lane < nc; c += kXCols) {
+        float4 nx[TOK];
+        const bool more = c - 4 * lane + kXCols < nc;
+#pragma unroll
+        for (int t = 0; t < TOK; ++t) nx[t] = load_x4<KIND>(L, t0 + t, c0 + c + kXCols, more && t0 + t < L.m);
+#pragma unroll
+        for (int k = 0; k < RC; ++k) {
+          const float4 q = *reinterpret_cast<const float4*>(sQ + k * kXqChunk + c);
+#pragma unroll
+          for (int t = 0; t < TOK; ++t)
+            acc[t * RC + k] = fmaf(x[t].w, q.w, fmaf(x[t].z, q.z, fmaf(x[t].y, q.y, fmaf(x[t].x, q.x, acc[t * RC + k]))));
+        }
+#pragma unroll
+        for (int t = 0; t < TOK; ++t) x[t] = nx[t];
+      }
     }
+    int at = 0;                          // first of the sums this lane keeps
+    constexpr int N = TOK * RC;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int t = t0 + warp * 4 + i;
+    for (int o = 16, n = N / 2; o >= 1; o >>= 1, n >>= 1) {
+      const bool up = (lane & o) != 0;
+      if (n >= 1) {
 #pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        float v = acc[i][k];
+        for (int i = 0; i < N / 2; ++i)
+          if (i < n) {
+            const float send = up ? acc[i] : acc[i + n], keep = up ? acc[i + n] : acc[i];
+            acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+          }
+        at += up ? n : 0;
+      } else {
+        acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+      }
+    }
+    constexpr int kKeep = N >= 32 ? N / 32 : 1;
+    if (N >= 32 || (lane & (32 / (N < 32 ? N : 32) - 1)) == 0) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0 && t < L.m && k < kc) L.T[(long long)t * r + k0 + k] = v;
+      for (int i = 0; i < kKeep; ++i) {
+        const int t = t0 + (at + i) / RC, k = (at + i) % RC;
+        if (t < L.m && k < kc) L.T[(long long)t * r + k0 + k] = acc[i];
       }
     }
   }
 }
 
+template <int RC>
+__global__ void __launch_bounds__(kXThreads, 2) x_q_kernel(const DevLayer* __restrict__ layers, int l0) {
+  const DevLayer& L = layers[l0 + blockIdx.y];
+  if ((int)blockIdx.x * kXWarps * kXqTokens >= L.m) return;
+  __shared__ __align__(16) float sQ[RC * kXqChunk];
+  const int t0 = ((int)blockIdx.x * kXWarps + (threadIdx.x >> 5)) * kXqTokens;
+  const int kind = x_kind(L);
+  if (kind == X_F32_VEC) x_q_body<RC, X_F32_VEC>(L, sQ, t0);
+  else if (kind == X_BF16_VEC) x_q_body<RC, X_BF16_VEC>(L, sQ, t0);
+  else x_q_body<RC, X_SCALAR>(L, sQ, t0);
+}
+
 cudaError_t launch_x_q(const ExtractWave& w, cudaStream_t s) {
-  dim3 grid((w.max_m + kXqWarps * 4 - 1) / (kXqWarps * 4), w.l1 - w.l0);
-  x_q_kernel<<<grid, 256, 0, s>>>(w.d_layers, w.l0);
+  const dim3 grid((w.max_m + kXWarps * kXqTokens - 1) / (kXWarps * kXqTokens), w.l1 - w.l0);
+  if (w.max_r <= 4) x_q_kernel<4><<<grid, kXThreads, 0, s>>>(w.d_layers, w.l0);
+  else if (w.max_r <= 8) x_q_kernel<8><<<grid, kXThreads, 0, s>>>(w.d_layers, w.l0);
+  else x_q_kernel<16><<<grid, kXThreads, 0, s>>>(w.d_layers, w.l0);
   return cudaGetLastError();
 }
 

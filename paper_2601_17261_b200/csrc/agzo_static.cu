@@ -73,16 +73,22 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
   if ((reinterpret_cast<uintptr_t>(X) & (es - 1)) || (reinterpret_cast<uintptr_t>(V) & 3u))
     return AGZO_ERR_INVALID_ARG;
 
-  // token slabs of the X^T T product (same rule as the workspace planner)
+  // token slabs of the X^T T product.  What the array admits is decided with slabs of at least 256 tokens; inside that
+  // limit the slabs are as short as the room left over allows, down to what fills the GPU.
   int slab_rows = (m + 31) / 32;
   slab_rows = (slab_rows + 31) / 32 * 32;
   if (slab_rows < 256) slab_rows = 256;
-  const int slabs = (m + slab_rows - 1) / slab_rows;
+  int slabs = (m + slab_rows - 1) / slab_rows;
   const size_t gch = ((size_t)d_in + 127) / 128;
   const size_t R = (size_t)r, D = (size_t)d_in, M = (size_t)m;
   const size_t need = 512 + up256(M * R * 4) + up256((size_t)slabs * R * D * 4) + up256(R * D * 4) +
                       up256(gch * R * R * 8) + up256(R * R * 8);
   if (need > kStaticScratchBytes) return AGZO_ERR_WORKSPACE;   // problem too large for the fixed array
+  for (int rows = cc_slab_rows(m, (long long)gch); rows < slab_rows; rows += 32) {
+    const int n = (m + rows - 1) / rows;
+    const size_t more = up256((size_t)n * R * D * 4) - up256((size_t)slabs * R * D * 4);
+    if (n > slabs && need + more <= kStaticScratchBytes) { slab_rows = rows; slabs = n; break; }
+  }
 
   int dev = -1;
   unsigned char* base = nullptr;
