@@ -34,7 +34,9 @@ struct Plan {
   std::vector<size_t> wave_y_count;   // floats, alignment gaps included
   int regions = 1;
   int total_tiles = 0;
+  int tile_rows = kRmwMaxTileRows;
   int max_r = 0;
+  int cc_max_r = 0;                // largest rank among layers of the CUDA-core pass
   int fast_mode_mask = 0;          // storage modes present among layers on the vector path
   bool any_slow = false;           // some layer needs the scalar kernel
   bool has_extract = false;
@@ -61,6 +63,7 @@ struct PlanOpts {
   bool share_inputs;     // consecutive layers with the same X are served by one sweep
   int extract_regions;   // 1: waves run one after another; 2: alternate waves use two scratch regions
                          // and two helper streams, so one wave's small kernels overlap the other's sweeps
+  int sm_count;          // of the device; when sizing without one, any number will do
   const FusedCaps* fused_caps;   // what the device holds of the fused kernel; null when sizing without a device
 };
 
@@ -254,6 +257,7 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
   const int regions = opts.extract_regions == 2 ? 2 : 1;
   plan->regions = regions;
   plan->max_r = 0;
+  plan->cc_max_r = 0;
   plan->fast_mode_mask = 0;
   plan->any_slow = false;
   plan->has_extract = false;
@@ -270,9 +274,17 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
   // Which layers take the tensor-core pass, and whether their R operands are staged in scratch
   // (ranks above 16): the operand image of every 128-row tile of every such layer, laid out from
   // the start of the scratch area (which extraction uses at other times).
+  // 16-byte accesses possible for every operand of the CUDA-core pass
+  auto vector_rows = [&](const agzo_layer& a) {
+    const size_t es = a.w_dtype == AGZO_BF16 ? 2 : 4;
+    bool vec = a.W && aligned16(a.W) && (a.ldw * es) % 16 == 0 && a.d_in % 8 == 0 && aligned16(a.V) && a.ldv % 4 == 0;
+    if (a.W16) vec = vec && aligned16(a.W16) && (a.ldw16 * 2) % 16 == 0;
+    return vec;
+  };
   auto takes_tc_rmw = [&](const agzo_layer& a) {
+    // from rank 3 on the element-by-element kernel is no alternative where the vector kernels cannot run
     return tc_available && opts.rmw_path != 1 && rmw_tc_eligible(a) &&
-           (opts.rmw_path == 2 || a.r >= opts.rmw_tc_min_rank);
+           (opts.rmw_path == 2 || a.r >= opts.rmw_tc_min_rank || (a.r >= 3 && !vector_rows(a)));
   };
   {
     size_t img = 0;
@@ -289,6 +301,13 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     plan->max_row_tiles = max_tiles;
     plan->image_bytes = want ? img : 0;
   }
+  {
+    long long strips = 0;
+    for (int i = 0; i < n; ++i)
+      if (L[i].W && !takes_tc_rmw(L[i]))
+        strips += (long long)((L[i].d_in + kRmwTileCols - 1) / kRmwTileCols) * ((L[i].d_out + kRmwMinTileRows - 1) / kRmwMinTileRows);
+    plan->tile_rows = rmw_tile_rows(strips, opts.sm_count);
+  }
   size_t img_off = 0;
   int tiles = 0;
   long long items = 0;
@@ -301,10 +320,7 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     D.d_out = a.d_out; D.d_in = a.d_in; D.m = a.m; D.r = a.r;
     D.layer_id = a.layer_id;
     D.rmw_mode = a.W16 ? RMW_PAIR_COMPUTE : (a.w_dtype == AGZO_BF16 ? RMW_BF16 : RMW_F32);
-    const size_t es = a.w_dtype == AGZO_BF16 ? 2 : 4;
-    bool vec = a.W && aligned16(a.W) && (a.ldw * es) % 16 == 0 && a.d_in % 8 == 0 &&
-               aligned16(a.V) && a.ldv % 4 == 0;
-    if (a.W16) vec = vec && aligned16(a.W16) && (a.ldw16 * 2) % 16 == 0;
+    const bool vec = vector_rows(a);
     D.vec_ok = vec ? 1 : 0;
     // bf16 weights of sufficient rank go through the tensor-core pass and get no CUDA-core tiles
     const bool tc_rmw = takes_tc_rmw(a);
@@ -324,10 +340,11 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
       if (ws) D.wmap = ws + maps_offset(n) + (size_t)i * kMapBytes + 384;
     } else if (a.W) {
       if (vec) plan->fast_mode_mask |= 1 << D.rmw_mode; else plan->any_slow = true;
+      plan->cc_max_r = std::max(plan->cc_max_r, a.r);
     }
     D.tile0 = tiles;
-    D.tiles_c = (a.d_in + 511) / 512;
-    D.tiles_r = (a.W && !tc_rmw) ? (a.d_out + 255) / 256 : 0;
+    D.tiles_c = (a.d_in + kRmwTileCols - 1) / kRmwTileCols;
+    D.tiles_r = (a.W && !tc_rmw) ? (a.d_out + plan->tile_rows - 1) / plan->tile_rows : 0;
     plan->tile_start[i] = tiles;
     const long long nt = (long long)D.tiles_c * D.tiles_r;
     if (tiles + nt > 0x7fffffff) return AGZO_ERR_INVALID_ARG;
@@ -508,7 +525,7 @@ agzo_status prepare(agzo_ctx* c, const agzo_layer* L, int n, cudaStream_t s) {
   PlanOpts opts{c->wave_bytes, c->extract_path, c->rmw_path, c->rmw_tc_min_rank, c->rmw_tc_panels, c->rmw_stage_r,
                 c->tc.available, c->extract_fused, c->share_inputs != 0,
                 c->allreduce ? 1 : c->extract_streams,    // the ranks' sums run in wave order on the caller's stream
-                &c->tc.fused};
+                c->sm_count, &c->tc.fused};
   agzo_status st = build_plan(L, n, c->ws, c->ws_bytes, opts, &plan, nullptr);
   if (st == AGZO_ERR_WORKSPACE && opts.extract_regions == 2) {   // a workspace sized for one region
     opts.extract_regions = 1;
@@ -581,7 +598,7 @@ agzo_status rmw_pass(agzo_ctx* c, const agzo_layer* L, int n, uint64_t seed, flo
   }
   if (c->plan.total_tiles > 0) {
     Timed t(c, AGZO_KC_RMW, s);
-    CU(c, launch_rmw(dev_layers(c), dev_tiles(c, n), n, c->plan.total_tiles, c->plan.max_r,
+    CU(c, launch_rmw(dev_layers(c), dev_tiles(c, n), n, c->plan.total_tiles, c->plan.tile_rows, c->plan.cc_max_r,
                      c->plan.fast_mode_mask, c->plan.any_slow, seed, coef, d_coef, pair_update,
                      c->sm_count, s));
   }
@@ -618,13 +635,13 @@ agzo_status agzo_workspace_bytes(const agzo_layer* h_layers, int n, size_t* h_by
   // the CUDA-core kernels, whose slabs are shaped differently)
   Plan plan;
   size_t scratch = 0, scratch_cc = 0;
-  st = build_plan(h_layers, n, nullptr, 0, PlanOpts{kDefaultWaveBytes, 0, 0, 3, 0, 0, true, 0, false, 2, nullptr}, &plan, &scratch);
+  st = build_plan(h_layers, n, nullptr, 0, PlanOpts{kDefaultWaveBytes, 0, 0, 3, 0, 0, true, 0, false, 2, 148, nullptr}, &plan, &scratch);
   if (st != AGZO_OK) return st;
-  st = build_plan(h_layers, n, nullptr, 0, PlanOpts{kDefaultWaveBytes, 1, 1, 0, 1, 1, false, 0, false, 2, nullptr}, &plan, &scratch_cc);
+  st = build_plan(h_layers, n, nullptr, 0, PlanOpts{kDefaultWaveBytes, 1, 1, 0, 1, 1, false, 0, false, 2, 148, nullptr}, &plan, &scratch_cc);
   if (st != AGZO_OK) return st;
   if (scratch_cc > scratch) scratch = scratch_cc;
   // ... and for the fused power step, whose layers keep room for one partial sum of Y per share of a launch
-  st = build_plan(h_layers, n, nullptr, 0, PlanOpts{kDefaultWaveBytes, 0, 0, 3, 0, 0, true, 2, false, 2, nullptr}, &plan, &scratch_cc);
+  st = build_plan(h_layers, n, nullptr, 0, PlanOpts{kDefaultWaveBytes, 0, 0, 3, 0, 0, true, 2, false, 2, 148, nullptr}, &plan, &scratch_cc);
   if (st != AGZO_OK) return st;
   if (scratch_cc > scratch) scratch = scratch_cc;
   *h_bytes = kHeaderBytes + table_bytes(n) + scratch + kAlign;
@@ -649,7 +666,8 @@ agzo_status agzo_create(agzo_ctx** out, int device, void* workspace, size_t work
   c->last_cuda = 0;
   c->extract_path = 0;
   c->rmw_path = 0;
-  c->rmw_tc_min_rank = 3;   // measured: from r = 3 on the tensor-core pass is the faster one
+  c->rmw_tc_min_rank = 5;   // 8B shapes, six blocks, one pass, CUDA cores / tensor cores: r = 1 736 / 786 us, r = 4 732 / 783,
+                            // r = 6 822 / 780, r = 8 823 / 783, r = 16 1471 / 770; 0.6B shapes r = 4 282 / 302, r = 6 331 / 316
   c->rmw_tc_slots = 0;
   c->rmw_tc_inflight = 0;
   c->rmw_tc_panels = 0;

@@ -1,20 +1,38 @@
 // In-place low-rank passes of Algorithm 2: W <- W + c * R A^T with R regenerated from the
 // Philox counter inside the kernel (Eq. agzo-perturb).  One grouped launch covers every
-// layer of the call; a tile is kTileRows x kTileCols of one layer's W.
+// layer of the call; a tile is tile_rows x kTileCols of one layer's W.
 //
-// HBM-bound for r <= 16: each weight is read once and written once (16-byte accesses, eight
-// rows in flight per thread); R for the tile's rows is generated once into shared memory
+// HBM-bound for r <= 16: each weight is read once and written once (16-byte accesses, 128 bytes
+// in flight per thread at all times); R for the tile's rows is generated once into shared memory
 // and the tile's slice of A^T lives in registers, so neither R nor Delta ever reaches DRAM.
+// Measured (one pass over six 8B-shaped blocks, bf16, 4.6 GB, copy rate 6541 GB/s): r = 1 6289 GB/s (6182 with loads
+// issued a sub-block at a time and after R), r = 4 6326 (5614), r = 8 5625 (4740); 28 0.6B-shaped blocks r = 4 6246 (5317), fp32
+// r = 8 6194 (4448); eight 1024 x 1024 master/compute pairs, r = 8: 37 -> 13 us; one fp32 256 x 256 layer 16 -> 4 us.
 #include "agzo_common.cuh"
 
 namespace agzo {
 
 constexpr int kRmwThreads = 256;
-constexpr int kTileCols = 512;   // 64 threads x 8 consecutive columns
-constexpr int kTileRows = 256;
+constexpr int kTileCols = kRmwTileCols;   // 64 threads x 8 consecutive columns
+constexpr int kTileRows = kRmwMaxTileRows;   // largest tile (shared memory is sized for it)
 constexpr int kRowLanes = 4;     // thread groups that take different rows
 constexpr int kRowsInFlight = 8; // rows per thread per sub-block
 constexpr int kSubRows = kRowLanes * kRowsInFlight;
+// rows whose loads a thread keeps in flight: 128 bytes
+template <int MODE> constexpr int rows_ahead() { return MODE == RMW_BF16 ? 8 : 4; }
+
+// two fp32 multiply-adds per instruction, each rounded like fmaf
+__device__ __forceinline__ uint64_t pack_f32x2(float a, float b) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ void unpack_f32x2(uint64_t d, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(d)); }
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
 
 __device__ __forceinline__ float bf16lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf16hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
@@ -74,7 +92,9 @@ __device__ __forceinline__ void store8(const DevLayer& L, long long row, int col
 }
 
 // ------------------------------------------------------------------ R for the rows of a tile
-// sG[row_local * RS + k] = R[row0 + row_local][k]; columns r..RS-1 are zero.
+// sG[DUP * (row_local * RS + k)] = R[row0 + row_local][k], DUP = 2: twice, side by side (an operand of the packed
+// multiply-adds); columns r..RS-1 are zero.
+template <int DUP>
 __device__ __forceinline__ void generate_G(float* sG, int RS, int r, long long row0, int nrows,
                                            uint32_t layer_id, uint64_t seed) {
   const long long e_first = row0 * r;
@@ -91,7 +111,9 @@ __device__ __forceinline__ void generate_G(float* sG, int RS, int r, long long r
       if (e >= e_first && e < e_last) {
         const int local = (int)(e - e_first);
         const int rl = local / r;
-        sG[rl * RS + (local - rl * r)] = gv[lane];
+        const int at = rl * RS + (local - rl * r);
+        if (DUP == 2) *reinterpret_cast<float2*>(sG + 2 * at) = make_float2(gv[lane], gv[lane]);
+        else sG[at] = gv[lane];
       }
     }
   }
@@ -99,74 +121,80 @@ __device__ __forceinline__ void generate_G(float* sG, int RS, int r, long long r
     const int pad = RS - r;
     for (int i = threadIdx.x; i < nrows * pad; i += kRmwThreads) {
       const int rl = i / pad;
-      sG[rl * RS + r + (i - rl * pad)] = 0.f;
+      const int at = rl * RS + r + (i - rl * pad);
+      if (DUP == 2) *reinterpret_cast<float2*>(sG + 2 * at) = make_float2(0.f, 0.f);
+      else sG[at] = 0.f;
     }
   }
 }
 
 // ------------------------------------------------------------------ r <= 16: A^T slice in registers
+// A thread's weights of a tile: eight columns, rows ry, ry + 4, ...  The loads of the first rows are issued before R is
+// generated, and every row that has been written is followed by the load of the row `rows_ahead` further on.
 template <int RC, int MODE>
-__device__ __forceinline__ void tile_body_reg(const DevLayer& L, const float* sG, int row0,
-                                              int nrows, int col0, float coef) {
-  const int cx = threadIdx.x & 63;
-  const int ry = threadIdx.x >> 6;
-  const int col = col0 + cx * 8;
-  if (col >= L.d_in) return;   // d_in is a multiple of 8 on this path
+struct TileReg {
+  static constexpr int kAhead = rows_ahead<MODE>();
+  uint64_t v[RC][4];
+  Raw8<MODE> raw[kAhead];
+  int col, ry;
+  bool live;
 
-  float v[RC][8];
+  __device__ __forceinline__ void begin(const DevLayer& L, int row0, int nrows, int col0) {
+    col = col0 + (threadIdx.x & 63) * 8;
+    ry = threadIdx.x >> 6;
+    live = col < L.d_in;                 // d_in is a multiple of 8 on this path
+    if (!live) return;
 #pragma unroll
-  for (int k = 0; k < RC; ++k) {
-    if (k < L.r) {
-      const float* p = L.V + (long long)k * L.ldv + col;
-      const float4 a = __ldg(reinterpret_cast<const float4*>(p));
-      const float4 b = __ldg(reinterpret_cast<const float4*>(p) + 1);
-      v[k][0] = a.x; v[k][1] = a.y; v[k][2] = a.z; v[k][3] = a.w;
-      v[k][4] = b.x; v[k][5] = b.y; v[k][6] = b.z; v[k][7] = b.w;
-    } else {
+    for (int j = 0; j < kAhead; ++j)
+      if (ry + j * kRowLanes < nrows) load8<MODE>(L, (long long)(row0 + ry + j * kRowLanes), col, raw[j]);
 #pragma unroll
-      for (int c = 0; c < 8; ++c) v[k][c] = 0.f;
+    for (int k = 0; k < RC; ++k) {
+      float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+      if (k < L.r) {
+        const float* p = L.V + (long long)k * L.ldv + col;
+        a = __ldg(reinterpret_cast<const float4*>(p));
+        b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+      }
+      v[k][0] = pack_f32x2(a.x, a.y); v[k][1] = pack_f32x2(a.z, a.w);
+      v[k][2] = pack_f32x2(b.x, b.y); v[k][3] = pack_f32x2(b.z, b.w);
     }
   }
 
-  for (int sb = 0; sb < nrows; sb += kSubRows) {
-    Raw8<MODE> raw[kRowsInFlight];
+  __device__ __forceinline__ void run(const DevLayer& L, const float* sG, int row0, int nrows, float coef) {
+    if (!live) return;
+    const uint64_t c2 = pack_f32x2(coef, coef);
+    for (int sb = ry; sb < nrows; sb += kAhead * kRowLanes) {
 #pragma unroll
-    for (int j = 0; j < kRowsInFlight; ++j) {
-      const int rl = sb + ry + j * kRowLanes;
-      if (rl < nrows) load8<MODE>(L, (long long)(row0 + rl), col, raw[j]);
-    }
+      for (int j = 0; j < kAhead; ++j) {
+        const int rl = sb + j * kRowLanes;
+        if (rl >= nrows) break;
+        uint64_t z[4] = {0, 0, 0, 0};
+        const float* g = sG + 2 * rl * RC;
+        if constexpr (RC == 1) {
+          const uint64_t g2 = *reinterpret_cast<const uint64_t*>(g);
 #pragma unroll
-    for (int j = 0; j < kRowsInFlight; ++j) {
-      const int rl = sb + ry + j * kRowLanes;
-      if (rl < nrows) {
-        float w[8];
-        unpack8<MODE>(raw[j], w);
-        const float* g = sG + rl * RC;
-        float gk[RC];
-        if (RC >= 4) {
-#pragma unroll
-          for (int k4 = 0; k4 < RC / 4; ++k4) {
-            const float4 g4 = *reinterpret_cast<const float4*>(g + 4 * k4);
-            gk[(4 * k4 + 0) % RC] = g4.x; gk[(4 * k4 + 1) % RC] = g4.y;
-            gk[(4 * k4 + 2) % RC] = g4.z; gk[(4 * k4 + 3) % RC] = g4.w;
-          }
+          for (int c = 0; c < 4; ++c) z[c] = fma_f32x2(g2, v[0][c], z[c]);
         } else {
 #pragma unroll
-          for (int k = 0; k < RC; ++k) gk[k] = g[k];
-        }
-        float o[8];
+          for (int k = 0; k < RC; k += 2) {          // k ascending, fixed order
+            const ulonglong2 g2 = *reinterpret_cast<const ulonglong2*>(g + 2 * k);
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          float z = 0.f;
+            for (int c = 0; c < 4; ++c) z[c] = fma_f32x2(g2.x, v[k][c], z[c]);
 #pragma unroll
-          for (int k = 0; k < RC; ++k) z = fmaf(gk[k], v[k][c], z);   // k ascending, fixed order
-          o[c] = fmaf(coef, z, w[c]);
+            for (int c = 0; c < 4; ++c) z[c] = fma_f32x2(g2.y, v[k + 1][c], z[c]);
+          }
         }
+        float w[8], o[8];
+        unpack8<MODE>(raw[j], w);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) unpack_f32x2(fma_f32x2(c2, z[c], pack_f32x2(w[2 * c], w[2 * c + 1])), o[2 * c], o[2 * c + 1]);
         store8<MODE>(L, (long long)(row0 + rl), col, o);
+        const int next = rl + kAhead * kRowLanes;
+        if (next < nrows) load8<MODE>(L, (long long)(row0 + next), col, raw[j]);
       }
     }
   }
-}
+};
 
 // ------------------------------------------------------------------ 16 < r <= 64: A^T slice in shared memory
 template <int MODE>
@@ -222,13 +250,27 @@ __device__ __forceinline__ void tile_body_smem(const DevLayer& L, const float* s
   }
 }
 
+// the layer of a tile: the last entry of the prefix that is <= tile.  A warp looks at 32 entries at a time (a binary
+// search is a chain of log2(layers) dependent loads, paid by every tile); all 32 lanes must call it.
 __device__ __forceinline__ int find_layer(const int* tile_start, int n_layers, int tile) {
-  int lo = 0, hi = n_layers - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (__ldg(tile_start + mid) <= tile) lo = mid; else hi = mid - 1;
+  const int lane = threadIdx.x & 31;
+  int lo = 0, n = n_layers;
+  while (n > 1) {
+    const int step = (n + 31) >> 5;
+    const int at = lo + lane * step;
+    const unsigned le = __ballot_sync(0xffffffffu, lane * step < n && __ldg(tile_start + at) <= tile);
+    const int last = 31 - __clz(le);           // entry `lo` always qualifies
+    n = min(step, n - last * step);
+    lo += last * step;
   }
   return lo;
+}
+
+// one 16-byte piece of the record per thread
+__device__ __forceinline__ void fetch_layer(DevLayer* dst, const DevLayer* src) {
+  static_assert(sizeof(DevLayer) % 16 == 0 && sizeof(DevLayer) / 16 <= kRmwThreads, "one piece per thread");
+  if (threadIdx.x < sizeof(DevLayer) / 16)
+    reinterpret_cast<uint4*>(dst)[threadIdx.x] = reinterpret_cast<const uint4*>(src)[threadIdx.x];
 }
 
 __device__ __forceinline__ int effective_mode(const DevLayer& L, int pair_update) {
@@ -241,7 +283,7 @@ __device__ __forceinline__ int effective_mode(const DevLayer& L, int pair_update
 template <int RC, int MODE>
 __global__ void __launch_bounds__(kRmwThreads, (RC <= 8 ? 2 : 1))
 rmw_reg_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ tile_start,
-               int n_layers, int total_tiles, uint64_t seed, float coef_imm,
+               int n_layers, int total_tiles, int tile_rows, uint64_t seed, float coef_imm,
                const float* __restrict__ d_coef, int pair_update) {
   extern __shared__ __align__(16) float smem[];
   __shared__ DevLayer sL;
@@ -250,24 +292,26 @@ rmw_reg_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ tile
   for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
     const int li = find_layer(tile_start, n_layers, tile);
     __syncthreads();   // previous tile is done with sG and sL
-    if (threadIdx.x == 0) sL = layers[li];
+    fetch_layer(&sL, layers + li);
     __syncthreads();
     const DevLayer& L = sL;
     if (!L.vec_ok || effective_mode(L, pair_update) != MODE) continue;
     const int t = tile - L.tile0;
     const int tr = t / L.tiles_c, tc = t - tr * L.tiles_c;
-    const int row0 = tr * kTileRows, col0 = tc * kTileCols;
-    const int nrows = min(kTileRows, L.d_out - row0);
-    generate_G(sG, RC, L.r, row0, nrows, L.layer_id, seed);
+    const int row0 = tr * tile_rows, col0 = tc * kTileCols;
+    const int nrows = min(tile_rows, L.d_out - row0);
+    TileReg<RC, MODE> body;
+    body.begin(L, row0, nrows, col0);
+    generate_G<2>(sG, RC, L.r, row0, nrows, L.layer_id, seed);
     __syncthreads();
-    tile_body_reg<RC, MODE>(L, sG, row0, nrows, col0, coef);
+    body.run(L, sG, row0, nrows, coef);
   }
 }
 
 template <int MODE>
 __global__ void __launch_bounds__(kRmwThreads, 1)
 rmw_smem_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ tile_start,
-                int n_layers, int total_tiles, int max_rs, uint64_t seed, float coef_imm,
+                int n_layers, int total_tiles, int tile_rows, int max_rs, uint64_t seed, float coef_imm,
                 const float* __restrict__ d_coef, int pair_update) {
   extern __shared__ __align__(16) float smem[];
   __shared__ DevLayer sL;
@@ -277,16 +321,16 @@ rmw_smem_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ til
   for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
     const int li = find_layer(tile_start, n_layers, tile);
     __syncthreads();
-    if (threadIdx.x == 0) sL = layers[li];
+    fetch_layer(&sL, layers + li);
     __syncthreads();
     const DevLayer& L = sL;
     if (!L.vec_ok || effective_mode(L, pair_update) != MODE) continue;
     const int RS = (L.r + 3) & ~3;
     const int t = tile - L.tile0;
     const int tr = t / L.tiles_c, tc = t - tr * L.tiles_c;
-    const int row0 = tr * kTileRows, col0 = tc * kTileCols;
-    const int nrows = min(kTileRows, L.d_out - row0);
-    generate_G(sG, RS, L.r, row0, nrows, L.layer_id, seed);
+    const int row0 = tr * tile_rows, col0 = tc * kTileCols;
+    const int nrows = min(tile_rows, L.d_out - row0);
+    generate_G<1>(sG, RS, L.r, row0, nrows, L.layer_id, seed);
     for (int i = threadIdx.x; i < RS * kTileCols; i += kRmwThreads) {
       const int k = i / kTileCols, c = i - k * kTileCols;
       sV[i] = (k < L.r && col0 + c < L.d_in) ? __ldg(L.V + (long long)k * L.ldv + col0 + c) : 0.f;
@@ -300,7 +344,7 @@ rmw_smem_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ til
 // the layers the vector kernels cannot take.
 __global__ void __launch_bounds__(kRmwThreads)
 rmw_generic_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ tile_start,
-                   int n_layers, int total_tiles, uint64_t seed, float coef_imm,
+                   int n_layers, int total_tiles, int tile_rows, uint64_t seed, float coef_imm,
                    const float* __restrict__ d_coef, int pair_update) {
   __shared__ float sG[32 * AGZO_MAX_RANK];
   __shared__ DevLayer sL;
@@ -308,7 +352,7 @@ rmw_generic_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ 
   for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
     const int li = find_layer(tile_start, n_layers, tile);
     __syncthreads();
-    if (threadIdx.x == 0) sL = layers[li];
+    fetch_layer(&sL, layers + li);
     __syncthreads();
     const DevLayer& L = sL;
     if (L.vec_ok) continue;
@@ -316,12 +360,12 @@ rmw_generic_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ 
     const int r = L.r;
     const int t = tile - L.tile0;
     const int tr = t / L.tiles_c, tc = t - tr * L.tiles_c;
-    const int row0 = tr * kTileRows, col0 = tc * kTileCols;
-    const int nrows = min(kTileRows, L.d_out - row0);
+    const int row0 = tr * tile_rows, col0 = tc * kTileCols;
+    const int nrows = min(tile_rows, L.d_out - row0);
     for (int sb = 0; sb < nrows; sb += 32) {
       const int nr = min(32, nrows - sb);
       __syncthreads();
-      generate_G(sG, r, r, row0 + sb, nr, L.layer_id, seed);
+      generate_G<1>(sG, r, r, row0 + sb, nr, L.layer_id, seed);
       __syncthreads();
       for (int c = threadIdx.x; c < kTileCols; c += kRmwThreads) {
         const int col = col0 + c;
@@ -345,7 +389,7 @@ rmw_generic_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ 
 }
 
 struct RmwArgs {
-  const DevLayer* d_layers; const int* d_tile_start; int n_layers, total_tiles;
+  const DevLayer* d_layers; const int* d_tile_start; int n_layers, total_tiles, tile_rows;
   uint64_t seed; float coef; const float* d_coef; int pair_update; int sm_count;
 };
 
@@ -353,10 +397,10 @@ template <int RC, int MODE>
 static cudaError_t launch_reg(const RmwArgs& a, cudaStream_t s) {
   const int per_sm = RC <= 8 ? 2 : 1;
   const int grid = a.total_tiles < a.sm_count * per_sm ? a.total_tiles : a.sm_count * per_sm;
-  const size_t smem = (size_t)kTileRows * RC * sizeof(float);
+  const size_t smem = (size_t)a.tile_rows * RC * 2 * sizeof(float);
   rmw_reg_kernel<RC, MODE><<<grid, kRmwThreads, smem, s>>>(a.d_layers, a.d_tile_start, a.n_layers,
-                                                           a.total_tiles, a.seed, a.coef, a.d_coef,
-                                                           a.pair_update);
+                                                           a.total_tiles, a.tile_rows, a.seed, a.coef,
+                                                           a.d_coef, a.pair_update);
   return cudaGetLastError();
 }
 
@@ -374,17 +418,17 @@ static cudaError_t launch_mode(const RmwArgs& a, int max_r, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const int grid = a.total_tiles < a.sm_count ? a.total_tiles : a.sm_count;
   rmw_smem_kernel<MODE><<<grid, kRmwThreads, smem, s>>>(a.d_layers, a.d_tile_start, a.n_layers,
-                                                        a.total_tiles, max_rs, a.seed, a.coef,
+                                                        a.total_tiles, a.tile_rows, max_rs, a.seed, a.coef,
                                                         a.d_coef, a.pair_update);
   return cudaGetLastError();
 }
 
 cudaError_t launch_rmw(const DevLayer* d_layers, const int* d_tile_start, int n_layers,
-                       int total_tiles, int max_r, int fast_mode_mask, bool any_slow,
+                       int total_tiles, int tile_rows, int max_r, int fast_mode_mask, bool any_slow,
                        uint64_t seed, float coef, const float* d_coef, bool pair_update,
                        int sm_count, cudaStream_t s) {
   if (total_tiles <= 0) return cudaSuccess;
-  RmwArgs a{d_layers, d_tile_start, n_layers, total_tiles, seed, coef, d_coef, pair_update ? 1 : 0, sm_count};
+  RmwArgs a{d_layers, d_tile_start, n_layers, total_tiles, tile_rows, seed, coef, d_coef, pair_update ? 1 : 0, sm_count};
   cudaError_t e = cudaSuccess;
   if (pair_update && (fast_mode_mask & (1 << RMW_PAIR_COMPUTE)))
     fast_mode_mask = (fast_mode_mask & ~(1 << RMW_PAIR_COMPUTE)) | (1 << RMW_PAIR_UPDATE);
@@ -395,7 +439,7 @@ cudaError_t launch_rmw(const DevLayer* d_layers, const int* d_tile_start, int n_
   if (e == cudaSuccess && any_slow) {
     const int grid = total_tiles < sm_count * 4 ? total_tiles : sm_count * 4;
     rmw_generic_kernel<<<grid, kRmwThreads, 0, s>>>(d_layers, d_tile_start, n_layers, total_tiles,
-                                                    seed, coef, d_coef, pair_update ? 1 : 0);
+                                                    tile_rows, seed, coef, d_coef, pair_update ? 1 : 0);
     e = cudaGetLastError();
   }
   return e;

@@ -3,7 +3,8 @@
 //
 // The CUDA-core kernel (agzo_rmw.cu) spends r + 1 fp32 FMAs per weight; from r = 16 on that is
 // more arithmetic than the FP32 pipes can do in the time HBM needs to stream the weight once in
-// and once out, and measured it falls behind this kernel from r = 3 on.  Here the product Delta = R A^T of a 128-row tile is one small tcgen05.mma chain
+// and once out, and measured it falls behind this kernel from r = 5 on.  Here the product
+// Delta = R A^T of a 128-row tile is one small tcgen05.mma chain
 // (M = 128, N = the panel's columns, K = 4 * rp), its fp32 result waits in TMEM, and the only
 // per-weight work left for the CUDA cores is  w + c * delta  and the rounding to bf16.
 //

@@ -1,0 +1,72 @@
+"""The CUDA-core in-place pass at the edges of its tiles and of its search for a tile's layer: rows around the tile heights,
+columns around 512, every rank class and storage, one layer up to more than a thousand.
+
+Tolerances are the suite's: one bf16 step with at most 1e-3 of the elements differing, or four fp32 steps, and the
+cancellation floor of an fp32 evaluation."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import agzo_oracle as O
+from paper_2601_17261_b200 import binding as B
+from paper_2601_17261_b200 import workloads as WL
+
+from gpu_helpers import DEV, Ctx, assert_weights_match, cancellation_floor, to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+
+def one(d_out, d_in, r, kind, lid=0):
+    W0 = WL.gaussian_weights(d_out, d_in, 0.02, seed=lid + d_out, bf16=kind == "bf16")
+    Vh = O.extract_subspace(WL.plain_activations(max(2 * r, 32), d_in, seed=d_in), r, 1, 3, lid)
+    Wd, _ = to_dev(W0, kind == "bf16")
+    W16 = Wd.to(torch.bfloat16) if kind == "pair" else None
+    Vd, _ = to_dev(Vh, False)
+    return W0, Vh, Wd, W16, (Vd, B.make_layer(W=Wd, W16=W16, V=Vd, r=r, layer_id=lid))
+
+
+def verify(W0, Vh, Wd, W16, kind, c, seed, lid):
+    store = "f32" if kind == "f32" else "bf16"
+    got = to_host(W16 if kind == "pair" else Wd)
+    assert_weights_match(got, O.apply_direction(W0, Vh, seed, lid, np.float32(c), store), store,
+                         floor=cancellation_floor(W0, c, seed, lid, Vh))
+
+
+@pytest.mark.parametrize("kind", ["bf16", "f32", "pair"])
+@pytest.mark.parametrize("r", [1, 2, 3, 4, 5, 8, 9, 16])
+@pytest.mark.parametrize("d_out,d_in", [(1, 16), (31, 512), (33, 520), (257, 1032), (300, 8 * 67)])
+def test_tiles(kind, r, d_out, d_in):
+    W0, Vh, Wd, W16, (_, layer) = one(d_out, d_in, r, kind)
+    with Ctx([layer]) as ctx:
+        B.agzo_set_option(ctx, "rmw_path", 1)
+        B.agzo_perturb(ctx, [layer], 11, 1e-3)
+        torch.cuda.synchronize()
+    verify(W0, Vh, Wd, W16, kind, 1e-3, 11, 0)
+
+
+@pytest.mark.parametrize("n", [2, 32, 33, 1025])
+def test_layer_of_a_tile(n):
+    made = [one(40 + 8 * (i % 7), 16 + 8 * (i % 5), 1 + i % 4, ("bf16", "f32")[i % 2], lid=i) for i in range(n)]
+    layers = [m[4][1] for m in made]
+    with Ctx(layers) as ctx:
+        B.agzo_perturb(ctx, layers, 5, 2e-3)
+        torch.cuda.synchronize()
+    for i in sorted({0, 1, n // 2, n - 2, n - 1}):
+        verify(*made[i][:4], ("bf16", "f32")[i % 2], 2e-3, 5, i)
+
+
+def test_tall_tiles():
+    # enough rows for tiles of 256, with a remainder in both directions
+    W0, Vh, Wd, W16, (_, layer) = one(60000, 520, 4, "bf16")
+    rows = np.r_[0:300, 29800:30100, 59700:60000]
+    with Ctx([layer]) as ctx:
+        for seed in range(2):
+            B.agzo_perturb(ctx, [layer], seed, 1e-3)
+        torch.cuda.synchronize()
+    want = W0
+    for seed in range(2):
+        want = O.apply_direction(want, Vh, seed, 0, np.float32(1e-3), "bf16")
+    # two passes: one bf16 step each
+    got = to_host(Wd)[rows]
+    assert np.abs(got - want[rows]).max() <= 2 * 2.0 ** -7 * np.abs(W0).max()
+    assert (got != want[rows]).mean() <= 2e-3
