@@ -3,6 +3,8 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -116,6 +118,24 @@ struct agzo_ctx {
 };
 
 namespace {
+
+// What is asked of a device and set for its kernels is the same for every context: done once per device.
+cudaError_t device_init(int device, TcState* tc) {
+  static std::mutex mu;
+  static std::map<int, TcState> known;
+  std::lock_guard<std::mutex> lock(mu);
+  auto it = known.find(device);
+  if (it == known.end()) {
+    TcState st;
+    cudaError_t e = panel_qr_init();
+    if (e == cudaSuccess) e = rmw_init();
+    if (e == cudaSuccess) e = tc_init(&st, device);
+    if (e != cudaSuccess) return e;
+    it = known.emplace(device, st).first;
+  }
+  *tc = it->second;
+  return cudaSuccess;
+}
 
 #define CU(ctx, expr)                              \
   do {                                             \
@@ -704,7 +724,7 @@ agzo_status agzo_create(agzo_ctx** out, int device, void* workspace, size_t work
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMemset(c->ws, 0, kHeaderBytes);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
-  if (e == cudaSuccess) e = tc_init(&c->tc, device);
+  if (e == cudaSuccess) e = device_init(device, &c->tc);
   if (e != cudaSuccess) {
     if (c->stage_ev) cudaEventDestroy(c->stage_ev);
     if (c->fork_ev) cudaEventDestroy(c->fork_ev);

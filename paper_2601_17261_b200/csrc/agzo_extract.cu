@@ -12,6 +12,8 @@ namespace agzo {
 // Local token t is row row0 + t of the test matrix of the whole batch: element e of the stream is
 // (row0 + t) * r + k, so the Philox blocks that cover the local rows are walked, whatever row0 is.
 __global__ void fill_omega_kernel(const DevLayer* __restrict__ layers, int l0, uint64_t seed, long long row0) {
+  chain_wait();
+  if (short_launch()) chain_next();
   const DevLayer& L = layers[l0 + blockIdx.y];
   const long long n = (long long)L.m * L.r;
   const long long e0 = row0 * L.r;
@@ -33,8 +35,7 @@ cudaError_t launch_fill_omega(const ExtractWave& w, uint64_t seed, cudaStream_t 
   int gx = (int)((nb + 255) / 256);
   if (gx > 512) gx = 512;
   if (gx < 1) gx = 1;
-  fill_omega_kernel<<<dim3(gx, w.l1 - w.l0), 256, 0, s>>>(w.d_layers, w.l0, seed, w.omega_row0);
-  return cudaGetLastError();
+  return launch_chained(fill_omega_kernel, dim3(gx, w.l1 - w.l0), 256, 0, 0, s, w.d_layers, w.l0, seed, w.omega_row0);
 }
 
 // ------------------------------------------------------------------ four consecutive columns of one row of X
@@ -172,6 +173,8 @@ template <int RC>
 __global__ void __launch_bounds__(kXThreads, 2) xt_t_kernel(const DevLayer* __restrict__ layers, int l0) {
   const DevLayer& L = layers[l0 + blockIdx.z];
   const int slab = blockIdx.y, d0 = blockIdx.x * kXCols;
+  chain_wait();
+  if (short_launch()) chain_next();
   if (slab >= L.slabs || d0 >= L.d_in) return;
   __shared__ __align__(16) float sT[kXtTokens * RC];
   __shared__ __align__(16) float sRed[kXWarps / 2 * RC * kXCols];
@@ -183,10 +186,8 @@ __global__ void __launch_bounds__(kXThreads, 2) xt_t_kernel(const DevLayer* __re
 
 cudaError_t launch_xt_t(const ExtractWave& w, cudaStream_t s) {
   const dim3 grid((w.max_din + kXCols - 1) / kXCols, w.max_slabs, w.l1 - w.l0);
-  if (w.max_r <= 4) xt_t_kernel<4><<<grid, kXThreads, 0, s>>>(w.d_layers, w.l0);
-  else if (w.max_r <= 8) xt_t_kernel<8><<<grid, kXThreads, 0, s>>>(w.d_layers, w.l0);
-  else xt_t_kernel<16><<<grid, kXThreads, 0, s>>>(w.d_layers, w.l0);
-  return cudaGetLastError();
+  const auto kernel = w.max_r <= 4 ? xt_t_kernel<4> : w.max_r <= 8 ? xt_t_kernel<8> : xt_t_kernel<16>;
+  return launch_chained(kernel, grid, kXThreads, 0, 0, s, w.d_layers, w.l0);
 }
 
 // ------------------------------------------------------------------ T[t][k] = sum_d X[t][d] Q[k][d]   (Q = rows of V)
@@ -272,6 +273,8 @@ __device__ __forceinline__ void x_q_body(const DevLayer& L, float* sQ, int t0) {
 template <int RC>
 __global__ void __launch_bounds__(kXThreads, 2) x_q_kernel(const DevLayer* __restrict__ layers, int l0) {
   const DevLayer& L = layers[l0 + blockIdx.y];
+  chain_wait();
+  if (short_launch()) chain_next();
   if ((int)blockIdx.x * kXWarps * kXqTokens >= L.m) return;
   __shared__ __align__(16) float sQ[RC * kXqChunk];
   const int t0 = ((int)blockIdx.x * kXWarps + (threadIdx.x >> 5)) * kXqTokens;
@@ -283,16 +286,16 @@ __global__ void __launch_bounds__(kXThreads, 2) x_q_kernel(const DevLayer* __res
 
 cudaError_t launch_x_q(const ExtractWave& w, cudaStream_t s) {
   const dim3 grid((w.max_m + kXWarps * kXqTokens - 1) / (kXWarps * kXqTokens), w.l1 - w.l0);
-  if (w.max_r <= 4) x_q_kernel<4><<<grid, kXThreads, 0, s>>>(w.d_layers, w.l0);
-  else if (w.max_r <= 8) x_q_kernel<8><<<grid, kXThreads, 0, s>>>(w.d_layers, w.l0);
-  else x_q_kernel<16><<<grid, kXThreads, 0, s>>>(w.d_layers, w.l0);
-  return cudaGetLastError();
+  const auto kernel = w.max_r <= 4 ? x_q_kernel<4> : w.max_r <= 8 ? x_q_kernel<8> : x_q_kernel<16>;
+  return launch_chained(kernel, grid, kXThreads, 0, 0, s, w.d_layers, w.l0);
 }
 
 // Y[k][d] = sum_s Ypart[s][k][d] in slab order, on its own: token-sharded extraction sums Y over
 // the ranks before the panel QR reads it
 __global__ void __launch_bounds__(256) sum_slabs_kernel(const DevLayer* __restrict__ layers, int l0, int after_fused) {
   const DevLayer& L = layers[l0 + blockIdx.y];
+  chain_wait();
+  if (short_launch()) chain_next();
   const int nparts = y_parts(L, after_fused);
   const long long n = (long long)L.r * L.d_in;
   for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
@@ -305,8 +308,7 @@ __global__ void __launch_bounds__(256) sum_slabs_kernel(const DevLayer* __restri
 cudaError_t launch_sum_slabs(const ExtractWave& w, cudaStream_t s) {
   long long blocks = ((long long)w.max_r * w.max_din + 255) / 256;
   if (blocks > 256) blocks = 256;
-  sum_slabs_kernel<<<dim3((unsigned)blocks, w.l1 - w.l0), 256, 0, s>>>(w.d_layers, w.l0, w.after_fused);
-  return cudaGetLastError();
+  return launch_chained(sum_slabs_kernel, dim3((unsigned)blocks, w.l1 - w.l0), 256, 0, 0, s, w.d_layers, w.l0, w.after_fused);
 }
 
 }  // namespace agzo

@@ -183,6 +183,7 @@ fused_power_step_kernel(const DevLayer* __restrict__ layers, int l0, int l1, int
   cluster_sync_all();          // every CTA's barriers exist before anyone arrives on them remotely
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
+  chain_wait();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -250,6 +251,7 @@ fused_power_step_kernel(const DevLayer* __restrict__ layers, int l0, int l1, int
           }
         }
       }
+      chain_next();            // the last tile is on its way
       if (!ok) sh.failed = 1;
       if (!ok || sh.failed) {
         for (int k = ns > kRingC ? ns - kRingC : 0; k < ns; ++k) mbar_wait(&sh.xc_full[k % kRingC], (k / kRingC) & 1);
@@ -662,25 +664,10 @@ cudaError_t launch_fused_power_step(const FusedCaps& caps, const ExtractWave& w,
     }
   if (total == 0) return cudaSuccess;
   if (C < 1 || C > kMaxCluster || caps.clusters[wide][C] <= 0) return cudaErrorInvalidConfiguration;   // the planner picks no such size
-  cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)C;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.blockDim = dim3(kFzThreads);
-  cfg.dynamicSmemBytes = fz_smem_bytes(wide, small);
-  cfg.stream = s;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
   // persistent clusters, never more than can be resident at once; the same count as fused_plan_shares used
   const int nclusters = total < caps.clusters[wide][C] ? total : caps.clusters[wide][C];
-  cfg.gridDim = dim3((unsigned)(nclusters * C));
-  const DevLayer* layers = w.d_layers;
-  int l0 = w.l0, l1 = w.l1;
-  int base = total / nclusters, rem = total % nclusters;
-  void* args[] = {(void*)&layers, (void*)&l0, (void*)&l1, (void*)&C, (void*)&base, (void*)&rem, (void*)&d_status};
-  return cudaLaunchKernelExC(&cfg, (const void*)fz_kernel(wide, small), args);
+  return launch_chained(fz_kernel(wide, small), dim3((unsigned)(nclusters * C)), kFzThreads, fz_smem_bytes(wide, small), C, s,
+                        w.d_layers, w.l0, w.l1, C, total / nclusters, total % nclusters, d_status);
 }
 
 }  // namespace agzo

@@ -89,6 +89,9 @@ __global__ void __launch_bounds__(kTcThreads) tc_x_q_kernel(const DevLayer* __re
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
+  chain_wait();
+  const bool early = short_launch();
+  if (early) chain_next();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -147,6 +150,7 @@ __global__ void __launch_bounds__(kTcThreads) tc_x_q_kernel(const DevLayer* __re
     const int q = warp & 3;
     const bool ok = mbar_wait(&sh.accum, 0);
     tc_fence_after();
+    if (!early) chain_next();
     if (!ok) sh.failed = 1;
     const int t = t0 + q * 32 + lane;
     if (ok) {
@@ -215,6 +219,9 @@ __global__ void __launch_bounds__(kTcThreads) tc_xt_t_kernel(const DevLayer* __r
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
+  chain_wait();
+  const bool early = short_launch();
+  if (early) chain_next();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -261,6 +268,7 @@ __global__ void __launch_bounds__(kTcThreads) tc_xt_t_kernel(const DevLayer* __r
     const int q = warp & 3;
     const bool ok = mbar_wait(&sh.accum, 0);
     tc_fence_after();
+    if (!early) chain_next();
     if (!ok) sh.failed = 1;
     const int d = d0 + q * 32 + lane;
     if (ok) {
@@ -294,6 +302,8 @@ __global__ void __launch_bounds__(kTcThreads) tc_xt_t_kernel(const DevLayer* __r
 // test matrix (see fill_omega_kernel).
 __global__ void __launch_bounds__(256) tc_fill_omega_kernel(const DevLayer* __restrict__ layers, int l0, uint64_t seed,
                                                             long long row0) {
+  chain_wait();
+  if (short_launch()) chain_next();
   const DevLayer& L = layers[l0 + blockIdx.y];
   const int r = L.r, NP = L.NP, groups = NP >> 3;
   const long long mp = L.m_pad;
@@ -475,8 +485,7 @@ cudaError_t tc_fill_omega(const TcState&, const ExtractWave& w, const DevLayer*,
   int gx = (int)((units + 255) / 256);
   if (gx > 1024) gx = 1024;
   if (gx < 1) gx = 1;
-  tc_fill_omega_kernel<<<dim3(gx, w.l1 - w.l0), 256, 0, s>>>(w.d_layers, w.l0, seed, w.omega_row0);
-  return cudaGetLastError();
+  return launch_chained(tc_fill_omega_kernel, dim3(gx, w.l1 - w.l0), 256, 0, 0, s, w.d_layers, w.l0, seed, w.omega_row0);
 }
 
 cudaError_t tc_xt_t(const TcState&, const ExtractWave& w, const DevLayer* h_dev, DevStatus* d_status,
@@ -488,9 +497,8 @@ cudaError_t tc_xt_t(const TcState&, const ExtractWave& w, const DevLayer* h_dev,
   }
   const int stages = stages_for(max_nb);
   dim3 grid((w.max_din + 127) / 128, w.max_slabs, w.l1 - w.l0);
-  tc_xt_t_kernel<<<grid, kTcThreads, smem_for(max_nb, stages), s>>>(w.d_layers, w.l0, d_status, stages,
-                                                                    skip_fused ? 1 : 0);
-  return cudaGetLastError();
+  return launch_chained(tc_xt_t_kernel, grid, kTcThreads, smem_for(max_nb, stages), 0, s, w.d_layers, w.l0, d_status, stages,
+                        skip_fused ? 1 : 0);
 }
 
 cudaError_t tc_x_q(const TcState&, const ExtractWave& w, const DevLayer* h_dev, DevStatus* d_status,
@@ -502,9 +510,8 @@ cudaError_t tc_x_q(const TcState&, const ExtractWave& w, const DevLayer* h_dev, 
   }
   const int stages = stages_for(max_nb);
   dim3 grid((w.max_m + 127) / 128, w.l1 - w.l0);
-  tc_x_q_kernel<<<grid, kTcThreads, smem_for(max_nb, stages), s>>>(w.d_layers, w.l0, d_status, stages,
-                                                                   skip_fused ? 1 : 0);
-  return cudaGetLastError();
+  return launch_chained(tc_x_q_kernel, grid, kTcThreads, smem_for(max_nb, stages), 0, s, w.d_layers, w.l0, d_status, stages,
+                        skip_fused ? 1 : 0);
 }
 
 }  // namespace agzo

@@ -405,6 +405,8 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
   const int ch0 = rank * cpc, nch = max(0, min(cpc, L.gchunks - ch0));
   const int d0 = ch0 * kQrChunk;
 
+  chain_wait();
+  if (short_launch()) chain_next();
   double acc[Cfg::my_tiles][2];
 #pragma unroll
   for (int t = 0; t < Cfg::my_tiles; ++t) acc[t][0] = acc[t][1] = 0.0;
@@ -487,6 +489,8 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_gram_kernel(const DevLaye
                                                                    int after_fused) {
   using Cfg = QrCfg<8>;
   const DevLayer& L = layers[l0 + blockIdx.y];
+  chain_wait();
+  if (short_launch()) chain_next();
   const int ch0 = blockIdx.x * kGramGroup;
   if (ch0 >= L.gchunks) return;
   const int nch = min(kGramGroup, L.gchunks - ch0), nparts = y_parts(L, after_fused);
@@ -538,6 +542,8 @@ __global__ void __launch_bounds__(kQrThreads) panel_factor_kernel(const DevLayer
   double* M = A + Cfg::r8 * Cfg::ap;
   __shared__ double own[AGZO_MAX_RANK];
   const int tid = threadIdx.x, r = L.r;
+  chain_wait();
+  if (short_launch()) chain_next();
   const int nsh = (L.gchunks + kGramGroup - 1) / kGramGroup;
   const int nt = (r + 7) >> 3, ne = qr_share_elems(r);
   constexpr int kPer = (Cfg::tiles * 64 + kQrThreads - 1) / kQrThreads;
@@ -582,6 +588,8 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_apply_kernel(const DevLay
   using Cfg = QrCfg<8>;
   const DevLayer& L = layers[l0 + blockIdx.y];
   const int d0 = blockIdx.x * kQrChunk;
+  chain_wait();
+  if (short_launch()) chain_next();
   if (d0 >= L.d_in) return;
   extern __shared__ __align__(16) unsigned char qr_smem[];
   double* M = reinterpret_cast<double*>(qr_smem);
@@ -614,58 +622,58 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_apply_kernel(const DevLay
 
 // CTAs per layer: eight while the launch is a chain of latencies; with so many layers that eight each would queue for
 // the SMs (two CTAs each), four or two, since every CTA repeats the factorisation (r = 8, d_in = 2048, 196 layers: 44.5 /
-// 27.7 / 26.1 us with 8 / 4 / 2; r = 16, d_in = 4096, 70 layers: 43.5 / 28.3 / 55.1 us; 35 layers 28.7 / 27.4 / 51.5)
-int qr_cluster(const ExtractWave& w) {
-  const int nl = w.l1 - w.l0;
-  const int most = nl <= 40 ? 8 : nl <= 80 ? 4 : 2;
-  return w.max_gchunks < most ? w.max_gchunks : most;
-}
+// 27.7 / 26.1 us with 8 / 4 / 2; r = 16, d_in = 4096, 70 layers: 43.5 / 28.3 / 55.1 us; 35 layers 28.7 / 27.4 / 51.5), but
+// never so few that the widest layer's slice leaves shared memory where eight would keep it (the 55 us above).
+template <int NT>
+size_t qr_smem(int slice) { return QrCfg<NT>::fixed + (size_t)QrCfg<NT>::r8 * qr_pitch(slice) * sizeof(float); }
 
 template <int NT>
 cudaError_t launch_qr(const ExtractWave& w, bool last, DevStatus* d_status, cudaStream_t s) {
-  using Cfg = QrCfg<NT>;
-  const int C = qr_cluster(w);
-  const int slice = (w.max_gchunks + C - 1) / C * kQrChunk;
-  const size_t whole = Cfg::fixed + (size_t)Cfg::r8 * qr_pitch(slice) * sizeof(float);
-  const bool resident = whole <= kQrResidentSmem;
-  const int pitch = qr_pitch(resident ? slice : kQrChunk);
-  const size_t smem = Cfg::fixed + (size_t)Cfg::r8 * pitch * sizeof(float);
-  auto kernel = resident ? panel_qr_kernel<NT, true> : panel_qr_kernel<NT, false>;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQrResidentSmem);
-    if (e != cudaSuccess) return e;
-  }
-  cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)C;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3((unsigned)(C * (w.l1 - w.l0)));
-  cfg.blockDim = dim3(kQrThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, w.d_layers, w.l0, C, pitch, w.y_reduced, w.after_fused, last ? 1 : 0, d_status);
+  const int nl = w.l1 - w.l0;
+  auto slice_of = [&](int c) { return (w.max_gchunks + c - 1) / c * kQrChunk; };
+  int C = nl <= 40 ? 8 : nl <= 80 ? 4 : 2;
+  while (C < kQrMaxCluster && qr_smem<NT>(slice_of(C)) > kQrResidentSmem) C *= 2;
+  if (C > w.max_gchunks) C = w.max_gchunks;
+  const bool resident = qr_smem<NT>(slice_of(C)) <= kQrResidentSmem;
+  const int slice = resident ? slice_of(C) : kQrChunk;
+  return launch_chained(resident ? panel_qr_kernel<NT, true> : panel_qr_kernel<NT, false>, dim3((unsigned)(C * nl)), kQrThreads,
+                        qr_smem<NT>(slice), C, s, w.d_layers, w.l0, C, qr_pitch(slice), w.y_reduced, w.after_fused, last ? 1 : 0,
+                        d_status);
 }
 
+constexpr size_t kGramSmem = (size_t)64 * (kQrChunk + 12) * sizeof(float);
+constexpr size_t kFactorSmem = QrCfg<8>::am_bytes;
+constexpr size_t kApplySmem = (size_t)64 * QrCfg<8>::mp * sizeof(double) + kGramSmem;
+
 cudaError_t launch_qr_large(const ExtractWave& w, bool last, DevStatus* d_status, cudaStream_t s) {
-  using Cfg = QrCfg<8>;
   const unsigned nl = (unsigned)(w.l1 - w.l0);
-  const size_t stage = (size_t)Cfg::r8 * qr_pitch(kQrChunk) * sizeof(float);
-  const size_t factor = Cfg::am_bytes, apply = (size_t)Cfg::r8 * Cfg::mp * sizeof(double) + stage;
-  cudaError_t e = cudaFuncSetAttribute(panel_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)factor);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(panel_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply);
-  if (e != cudaSuccess) return e;
-  panel_gram_kernel<<<dim3((unsigned)((w.max_gchunks + kGramGroup - 1) / kGramGroup), nl), kQrThreads, stage, s>>>(
-      w.d_layers, w.l0, w.y_reduced, w.after_fused);
-  panel_factor_kernel<<<nl, kQrThreads, factor, s>>>(w.d_layers, w.l0, d_status);
-  panel_apply_kernel<<<dim3((unsigned)w.max_gchunks, nl), kQrThreads, apply, s>>>(w.d_layers, w.l0, last ? 1 : 0);
-  return cudaGetLastError();
+  cudaError_t e = launch_chained(panel_gram_kernel, dim3((unsigned)((w.max_gchunks + kGramGroup - 1) / kGramGroup), nl), kQrThreads,
+                                 kGramSmem, 0, s, w.d_layers, w.l0, w.y_reduced, w.after_fused);
+  if (e == cudaSuccess) e = launch_chained(panel_factor_kernel, dim3(nl), kQrThreads, kFactorSmem, 0, s, w.d_layers, w.l0, d_status);
+  if (e == cudaSuccess)
+    e = launch_chained(panel_apply_kernel, dim3((unsigned)w.max_gchunks, nl), kQrThreads, kApplySmem, 0, s, w.d_layers, w.l0,
+                       last ? 1 : 0);
+  return e;
+}
+
+template <typename K>
+cudaError_t allow_smem(K* kernel, size_t bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 }  // namespace
+
+cudaError_t panel_qr_init() {
+  cudaError_t e = allow_smem(panel_qr_kernel<1, true>, kQrResidentSmem);
+  if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<1, false>, kQrResidentSmem);
+  if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<2, true>, kQrResidentSmem);
+  if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<2, false>, kQrResidentSmem);
+  if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<4, true>, kQrResidentSmem);
+  if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<4, false>, kQrResidentSmem);
+  if (e == cudaSuccess) e = allow_smem(panel_factor_kernel, kFactorSmem);
+  if (e == cudaSuccess) e = allow_smem(panel_apply_kernel, kApplySmem);
+  return e;
+}
 
 int panel_qr_launches(int max_r) { return max_r > 32 ? 3 : 1; }
 

@@ -152,8 +152,8 @@ struct TileReg {
       float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
       if (k < L.r) {
         const float* p = L.V + (long long)k * L.ldv + col;
-        a = __ldg(reinterpret_cast<const float4*>(p));
-        b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+        a = __ldcg(reinterpret_cast<const float4*>(p));
+        b = __ldcg(reinterpret_cast<const float4*>(p) + 1);
       }
       v[k][0] = pack_f32x2(a.x, a.y); v[k][1] = pack_f32x2(a.z, a.w);
       v[k][2] = pack_f32x2(b.x, b.y); v[k][3] = pack_f32x2(b.z, b.w);
@@ -288,7 +288,9 @@ rmw_reg_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ tile
   extern __shared__ __align__(16) float smem[];
   __shared__ DevLayer sL;
   float* sG = smem;
-  const float coef = d_coef ? __ldg(d_coef) : coef_imm;
+  chain_wait();
+  if (total_tiles <= (int)gridDim.x) chain_next();
+  const float coef = d_coef ? __ldcg(d_coef) : coef_imm;
   for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
     const int li = find_layer(tile_start, n_layers, tile);
     __syncthreads();   // previous tile is done with sG and sL
@@ -317,7 +319,9 @@ rmw_smem_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ til
   __shared__ DevLayer sL;
   float* sG = smem;                              // [kTileRows][RS]
   float* sV = smem + kTileRows * max_rs;         // [RS][kTileCols]
-  const float coef = d_coef ? __ldg(d_coef) : coef_imm;
+  chain_wait();
+  if (total_tiles <= (int)gridDim.x) chain_next();
+  const float coef = d_coef ? __ldcg(d_coef) : coef_imm;
   for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
     const int li = find_layer(tile_start, n_layers, tile);
     __syncthreads();
@@ -333,7 +337,7 @@ rmw_smem_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ til
     generate_G<1>(sG, RS, L.r, row0, nrows, L.layer_id, seed);
     for (int i = threadIdx.x; i < RS * kTileCols; i += kRmwThreads) {
       const int k = i / kTileCols, c = i - k * kTileCols;
-      sV[i] = (k < L.r && col0 + c < L.d_in) ? __ldg(L.V + (long long)k * L.ldv + col0 + c) : 0.f;
+      sV[i] = (k < L.r && col0 + c < L.d_in) ? __ldcg(L.V + (long long)k * L.ldv + col0 + c) : 0.f;
     }
     __syncthreads();
     tile_body_smem<MODE>(L, sG, sV, RS, row0, nrows, col0, coef);
@@ -348,7 +352,9 @@ rmw_generic_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ 
                    const float* __restrict__ d_coef, int pair_update) {
   __shared__ float sG[32 * AGZO_MAX_RANK];
   __shared__ DevLayer sL;
-  const float coef = d_coef ? __ldg(d_coef) : coef_imm;
+  chain_wait();
+  if (total_tiles <= (int)gridDim.x) chain_next();
+  const float coef = d_coef ? __ldcg(d_coef) : coef_imm;
   for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
     const int li = find_layer(tile_start, n_layers, tile);
     __syncthreads();
@@ -373,7 +379,7 @@ rmw_generic_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ 
         for (int rl = 0; rl < nr; ++rl) {
           const long long row = row0 + sb + rl;
           float z = 0.f;
-          for (int k = 0; k < r; ++k) z = fmaf(sG[rl * r + k], __ldg(L.V + (long long)k * L.ldv + col), z);
+          for (int k = 0; k < r; ++k) z = fmaf(sG[rl * r + k], __ldcg(L.V + (long long)k * L.ldv + col), z);
           float w;
           if (mode == RMW_BF16) w = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(L.W)[row * L.ldw + col]);
           else w = reinterpret_cast<const float*>(L.W)[row * L.ldw + col];
@@ -393,15 +399,18 @@ struct RmwArgs {
   uint64_t seed; float coef; const float* d_coef; int pair_update; int sm_count;
 };
 
+// A pass of one tile per CTA may start beside its predecessor.  A longer one may not: CTAs that take their places one by
+// one while the panel QR runs out drift apart and the pass loses the locality of its row segments (rank-1 pass over eight
+// 8B-shaped blocks behind the extraction: 970 us, 1190 us when started early).
+static int starts_early(int total_tiles, int grid) { return total_tiles <= grid ? 1 : 0; }
+
 template <int RC, int MODE>
 static cudaError_t launch_reg(const RmwArgs& a, cudaStream_t s) {
   const int per_sm = RC <= 8 ? 2 : 1;
   const int grid = a.total_tiles < a.sm_count * per_sm ? a.total_tiles : a.sm_count * per_sm;
   const size_t smem = (size_t)a.tile_rows * RC * 2 * sizeof(float);
-  rmw_reg_kernel<RC, MODE><<<grid, kRmwThreads, smem, s>>>(a.d_layers, a.d_tile_start, a.n_layers,
-                                                           a.total_tiles, a.tile_rows, a.seed, a.coef,
-                                                           a.d_coef, a.pair_update);
-  return cudaGetLastError();
+  return launch_kernel(rmw_reg_kernel<RC, MODE>, dim3(grid), kRmwThreads, smem, 0, starts_early(a.total_tiles, grid), s, a.d_layers, a.d_tile_start, a.n_layers,
+                        a.total_tiles, a.tile_rows, a.seed, a.coef, a.d_coef, a.pair_update);
 }
 
 template <int MODE>
@@ -413,14 +422,9 @@ static cudaError_t launch_mode(const RmwArgs& a, int max_r, cudaStream_t s) {
   if (max_r <= 16) return launch_reg<16, MODE>(a, s);
   const int max_rs = (max_r + 3) & ~3;
   const size_t smem = ((size_t)kTileRows * max_rs + (size_t)max_rs * kTileCols) * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(rmw_smem_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(((size_t)kTileRows * 64 + (size_t)64 * kTileCols) * sizeof(float)));
-  if (e != cudaSuccess) return e;
   const int grid = a.total_tiles < a.sm_count ? a.total_tiles : a.sm_count;
-  rmw_smem_kernel<MODE><<<grid, kRmwThreads, smem, s>>>(a.d_layers, a.d_tile_start, a.n_layers,
-                                                        a.total_tiles, a.tile_rows, max_rs, a.seed, a.coef,
-                                                        a.d_coef, a.pair_update);
-  return cudaGetLastError();
+  return launch_kernel(rmw_smem_kernel<MODE>, dim3(grid), kRmwThreads, smem, 0, starts_early(a.total_tiles, grid), s, a.d_layers, a.d_tile_start, a.n_layers,
+                        a.total_tiles, a.tile_rows, max_rs, a.seed, a.coef, a.d_coef, a.pair_update);
 }
 
 cudaError_t launch_rmw(const DevLayer* d_layers, const int* d_tile_start, int n_layers,
@@ -438,10 +442,18 @@ cudaError_t launch_rmw(const DevLayer* d_layers, const int* d_tile_start, int n_
   if (e == cudaSuccess && (fast_mode_mask & (1 << RMW_PAIR_UPDATE))) e = launch_mode<RMW_PAIR_UPDATE>(a, max_r, s);
   if (e == cudaSuccess && any_slow) {
     const int grid = total_tiles < sm_count * 4 ? total_tiles : sm_count * 4;
-    rmw_generic_kernel<<<grid, kRmwThreads, 0, s>>>(d_layers, d_tile_start, n_layers, total_tiles,
-                                                    tile_rows, seed, coef, d_coef, pair_update ? 1 : 0);
-    e = cudaGetLastError();
+    e = launch_kernel(rmw_generic_kernel, dim3(grid), kRmwThreads, 0, 0, starts_early(total_tiles, grid), s, d_layers, d_tile_start, n_layers, total_tiles,
+                       tile_rows, seed, coef, d_coef, pair_update ? 1 : 0);
   }
+  return e;
+}
+
+cudaError_t rmw_init() {
+  const int smem = (int)(((size_t)kTileRows * 64 + (size_t)64 * kTileCols) * sizeof(float));
+  cudaError_t e = cudaFuncSetAttribute(rmw_smem_kernel<RMW_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(rmw_smem_kernel<RMW_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(rmw_smem_kernel<RMW_PAIR_COMPUTE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(rmw_smem_kernel<RMW_PAIR_UPDATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   return e;
 }
 
@@ -451,7 +463,9 @@ cudaError_t launch_rmw(const DevLayer* d_layers, const int* d_tile_start, int n_
 template <typename T>
 __global__ void dense_kernel(T* w, long long n, long long b_first, uint64_t seed, uint32_t layer_id, float scale,
                              const float* d_scale) {
-  const float c = d_scale ? scale * __ldg(d_scale) : scale;
+  chain_wait();
+  if (short_launch()) chain_next();
+  const float c = d_scale ? scale * __ldcg(d_scale) : scale;
   const long long nb = (n + 3) >> 2;
   for (long long b = b_first + blockIdx.x * (long long)blockDim.x + threadIdx.x; b < nb;
        b += (long long)gridDim.x * blockDim.x) {
@@ -472,7 +486,9 @@ __global__ void dense_kernel(T* w, long long n, long long b_first, uint64_t seed
 template <typename T>
 __global__ void __launch_bounds__(256) dense_vec_kernel(T* w, long long n8, uint64_t seed, uint32_t layer_id, float scale,
                                                         const float* d_scale) {
-  const float c = d_scale ? scale * __ldg(d_scale) : scale;
+  chain_wait();
+  if (short_launch()) chain_next();
+  const float c = d_scale ? scale * __ldcg(d_scale) : scale;
   for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < n8; g += (long long)gridDim.x * blockDim.x) {
     const float4 ga = gaussian_block((uint64_t)(2 * g), layer_id, kTagDense, seed);
     const float4 gb = gaussian_block((uint64_t)(2 * g + 1), layer_id, kTagDense, seed);
@@ -507,15 +523,13 @@ cudaError_t launch_dense_t(T* w, long long n, uint64_t seed, uint32_t layer_id, 
   if ((reinterpret_cast<uintptr_t>(w) & 15u) == 0) n8 = n >> 3;
   if (n8 > 0) {
     const int grid = (int)((n8 + 255) / 256 < cap ? (n8 + 255) / 256 : cap);
-    dense_vec_kernel<T><<<grid, 256, 0, s>>>(w, n8, seed, layer_id, scale, d_scale);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_chained(dense_vec_kernel<T>, dim3(grid), 256, 0, 0, s, w, n8, seed, layer_id, scale, d_scale);
     if (e != cudaSuccess) return e;
   }
   if (8 * n8 < n) {                                    // the rest: blocks from 2 n8 on
     const long long nb = ((n + 3) >> 2) - 2 * n8;
     const int grid = (int)((nb + 255) / 256 < cap ? (nb + 255) / 256 : cap);
-    dense_kernel<T><<<grid, 256, 0, s>>>(w, n, 2 * n8, seed, layer_id, scale, d_scale);
-    return cudaGetLastError();
+    return launch_chained(dense_kernel<T>, dim3(grid), 256, 0, 0, s, w, n, 2 * n8, seed, layer_id, scale, d_scale);
   }
   return cudaSuccess;
 }
@@ -530,6 +544,8 @@ cudaError_t launch_dense(void* w, long long n, int dtype, uint64_t seed, uint32_
 
 // ------------------------------------------------------------------ Gaussian right factor (LOZO comparison)
 __global__ void fill_basis_kernel(const DevLayer* __restrict__ layers, uint64_t seed) {
+  chain_wait();
+  chain_next();
   const DevLayer& L = layers[blockIdx.y];
   const long long n = (long long)L.r * L.d_in;
   const long long nb = (n + 3) >> 2;
@@ -553,28 +569,29 @@ cudaError_t launch_fill_basis(const DevLayer* d_layers, int n_layers, int max_el
   int gx = (max_elems / 4 + 255) / 256;
   if (gx < 1) gx = 1;
   if (gx > 64) gx = 64;
-  fill_basis_kernel<<<dim3((unsigned)gx, (unsigned)n_layers), 256, 0, s>>>(d_layers, seed);
-  return cudaGetLastError();
+  return launch_chained(fill_basis_kernel, dim3((unsigned)gx, (unsigned)n_layers), 256, 0, 0, s, d_layers, seed);
 }
 
 // ------------------------------------------------------------------ scalars (Algorithm 2, step 3)
 __global__ void ghat_kernel(const double* fp, const double* fo, float eps, int mode, float* g) {
+  chain_wait();
+  chain_next();
   const double d = *fp - *fo;
   *g = (float)(mode == 0 ? d / (2.0 * (double)eps) : d / (double)eps);
 }
 cudaError_t launch_ghat(const double* fp, const double* fo, float eps, int mode, float* g, cudaStream_t s) {
-  ghat_kernel<<<1, 1, 0, s>>>(fp, fo, eps, mode, g);
-  return cudaGetLastError();
+  return launch_chained(ghat_kernel, dim3(1), 1, 0, 0, s, fp, fo, eps, mode, g);
 }
 
 // kind 0: eps - lr*g   kind 1: -(eps + lr*g)   kind 2: -lr*g
 __global__ void coef_kernel(const float* g, float eps, float lr, int kind, float* out) {
+  chain_wait();
+  chain_next();
   const double lg = (double)lr * (double)*g;
   *out = (float)(kind == 0 ? (double)eps - lg : kind == 1 ? -((double)eps + lg) : -lg);
 }
 cudaError_t launch_coef(const float* g, float eps, float lr, int kind, float* d_coef, cudaStream_t s) {
-  coef_kernel<<<1, 1, 0, s>>>(g, eps, lr, kind, d_coef);
-  return cudaGetLastError();
+  return launch_chained(coef_kernel, dim3(1), 1, 0, 0, s, g, eps, lr, kind, d_coef);
 }
 
 // ------------------------------------------------------------------ test exports

@@ -208,6 +208,7 @@ rmw_tc_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ item_
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
+  chain_wait();
 
   if (warp == kWarpLoader) {
     if (lane == 0) {
@@ -233,6 +234,7 @@ rmw_tc_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ item_
           }
         }
       }
+      chain_next();             // the last weights are on their way
       if (!ok) sh.failed = 1;
       if (!ok || sh.failed) {   // leaving early: the copies in flight must land before the CTA goes away
         for (int k = n > slots ? n - slots : 0; k < n; ++k) mbar_wait(&sh.full_w[k % slots], (k / slots) & 1);
@@ -329,7 +331,7 @@ rmw_tc_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ item_
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           const int k = 8 * g + u;
-          v[u] = (k < r && col < L.d_in) ? __ldg(L.V + (long long)k * L.ldv + col) : 0.f;
+          v[u] = (k < r && col < L.d_in) ? __ldcg(L.V + (long long)k * L.ldv + col) : 0.f;
         }
         uint4 hi, lo;
         split8(v, &hi, &lo);
@@ -378,7 +380,7 @@ rmw_tc_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ item_
     const int q = warp & 3;            // TMEM lanes 32q .. 32q+31 belong to this warp
     const int h = e >> 2;              // which half of a box's 64 columns
     const int i = q * 32 + lane;       // row inside the tile
-    const float coef = d_coef ? __ldg(d_coef) : coef_imm;
+    const float coef = d_coef ? __ldcg(d_coef) : coef_imm;
     uint32_t off[4];                   // this thread's four 16-byte chunks inside any box
 #pragma unroll
     for (int c = 0; c < 4; ++c) off[c] = swz(i, h * 4 + c);
@@ -440,6 +442,8 @@ rmw_tc_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ item_
 // scratch exactly as rmw_tc_kernel lays it out in shared memory (K atoms of [128 rows][128 bytes],
 // 128-byte swizzle), so the pass can bulk-copy it.
 __global__ void __launch_bounds__(256) rmw_tc_fill_r_kernel(const DevLayer* __restrict__ layers, uint64_t seed) {
+  chain_wait();
+  if (short_launch()) chain_next();
   const DevLayer& L = layers[blockIdx.y];
   if (!L.rimg) return;
   const int rb = blockIdx.x;
@@ -512,8 +516,7 @@ cudaError_t launch_rmw_tc(const DevLayer* d_layers, const int* d_item_start, int
                           float coef, const float* d_coef, DevStatus* d_status, int sm_count, cudaStream_t s) {
   if (total_items <= 0) return cudaSuccess;
   if (staged && fill) {
-    rmw_tc_fill_r_kernel<<<dim3((unsigned)max_row_tiles, (unsigned)n_layers), 256, 0, s>>>(d_layers, seed);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_chained(rmw_tc_fill_r_kernel, dim3((unsigned)max_row_tiles, (unsigned)n_layers), 256, 0, 0, s, d_layers, seed);
     if (e != cudaSuccess) return e;
   }
   const int katoms = rtc_katoms(max_rp);
@@ -531,9 +534,8 @@ cudaError_t launch_rmw_tc(const DevLayer* d_layers, const int* d_item_start, int
   // bandwidth (4 to 5 boxes of 16 KiB); more only lengthens the queues in front of the stores
   if (inflight < 1) inflight = max_r <= 8 ? 4 : 5;
   if (inflight > slots) inflight = slots;
-  rmw_tc_kernel<<<grid, threads, smem, s>>>(d_layers, d_item_start, n_layers, total_items, a_bufs, a_buf_bytes,
-                                             max_b_bytes, slots, inflight, staged ? 1 : 0, seed, coef, d_coef, d_status);
-  return cudaGetLastError();
+  return launch_chained(rmw_tc_kernel, dim3(grid), threads, smem, 0, s, d_layers, d_item_start, n_layers, total_items, a_bufs,
+                        a_buf_bytes, max_b_bytes, slots, inflight, staged ? 1 : 0, seed, coef, d_coef, d_status);
 }
 
 }  // namespace agzo

@@ -32,6 +32,7 @@ cudaError_t scratch_of_current_device(int* dev_out, unsigned char** out) {
   if (!g_scratch_addr[dev]) {
     void* p = nullptr;
     e = cudaGetSymbolAddress(&p, g_static_scratch);   // once per device, with that device current
+    if (e == cudaSuccess) e = agzo::panel_qr_init();
     if (e != cudaSuccess) return e;
     g_scratch_addr[dev] = p;
   }
@@ -46,6 +47,8 @@ inline size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 // rewritten and the status word cleared here; every other slice is fully overwritten by the
 // kernels before it is read.
 __global__ void static_begin_kernel(agzo::DevLayer rec, agzo::DevLayer* dst, agzo::DevStatus* st) {
+  agzo::chain_wait();      // an earlier call may still read the record; the kernels after it read it before they wait,
+                           // so they are not allowed to start early (no chain_next)
   *dst = rec;
   st->rank_deficient = 0;
   st->timeout = 0;
@@ -54,6 +57,7 @@ __global__ void static_begin_kernel(agzo::DevLayer rec, agzo::DevLayer* dst, agz
 }
 
 __global__ void static_end_kernel(const agzo::DevStatus* st, int32_t* flag) {
+  agzo::chain_wait();
   *flag = st->rank_deficient;
 }
 
@@ -109,8 +113,7 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
   static_assert(sizeof(DevLayer) <= 384, "layer record must fit its slot");
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  static_begin_kernel<<<1, 1, 0, s>>>(rec, d_rec, d_status);
-  if (cudaGetLastError() != cudaSuccess) return AGZO_ERR_CUDA;
+  if (launch_chained(static_begin_kernel, dim3(1), 1, 0, 0, s, rec, d_rec, d_status) != cudaSuccess) return AGZO_ERR_CUDA;
 
   ExtractWave w{};
   w.d_layers = d_rec;
@@ -125,8 +128,7 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
   }
   if (launch_panel_qr(w, true, d_status, s) != cudaSuccess) return AGZO_ERR_CUDA;    // A <- qr(Y)
   if (d_rank_deficient) {
-    static_end_kernel<<<1, 1, 0, s>>>(d_status, d_rank_deficient);
-    if (cudaGetLastError() != cudaSuccess) return AGZO_ERR_CUDA;
+    if (launch_chained(static_end_kernel, dim3(1), 1, 0, 0, s, d_status, d_rank_deficient) != cudaSuccess) return AGZO_ERR_CUDA;
   }
   return AGZO_OK;
 }

@@ -1,0 +1,71 @@
+"""Kernels that may start while their predecessor runs out: whole iterations issued back to back give bit for bit what
+they give when the device is idle before every call (whatever a kernel read too early would differ)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2601_17261_b200 import binding as B
+from paper_2601_17261_b200 import workloads as WL
+
+from gpu_helpers import DEV, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+def build(shapes, m, r, bf16):
+    out = []
+    for i, (d_in, d_out) in enumerate(shapes):
+        X, _ = to_dev(WL.planted_activations(m, d_in, min(16, d_in), seed=i, bf16=bf16), bf16)
+        W, _ = to_dev(WL.gaussian_weights(d_out, d_in, 0.02, seed=i, bf16=bf16), bf16)
+        V = torch.zeros(r, d_in, device=DEV)
+        out.append((X, W, V, B.make_layer(X=X, W=W, V=V, r=r, layer_id=i)))
+    return out
+
+
+def iterate(sets, sync, streams=(None,)):
+    ctxs = [B.agzo_create([t[3] for t in s], 0) for s in sets]
+    losses = torch.tensor([1.0, 0.999], dtype=torch.float64, device=DEV)
+    ghats = [torch.zeros(1, device=DEV) for _ in sets]
+    torch.cuda.synchronize()
+    wait = torch.cuda.synchronize if sync else (lambda: None)
+    for seed in range(4):
+        for j, (s, ctx) in enumerate(zip(sets, ctxs)):
+            st = streams[j % len(streams)]
+            L = [t[3] for t in s]
+            B.agzo_extract_subspace(ctx, L, seed, 2, stream=st); wait()
+            B.agzo_perturb(ctx, L, seed, 1e-2, stream=st); wait()
+            B.agzo_perturb(ctx, L, seed, -2e-2, stream=st); wait()
+            B.agzo_ghat(ctx, losses[0:1], losses[1:2], 1e-2, 0, ghats[j], stream=st); wait()
+            B.agzo_restore_update(ctx, L, seed, 1e-2, 1e-1, 0, ghats[j], stream=st); wait()
+            B.agzo_perturb_dense(ctx, s[0][1], seed, 7, 1e-3, stream=st); wait()
+    torch.cuda.synchronize()
+    for ctx in ctxs:
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+        B.agzo_destroy(ctx)
+    return [t[k].clone() for s in sets for t in s for k in (1, 2)]
+
+
+@pytest.mark.parametrize("n_streams", [1, 2])
+@pytest.mark.parametrize("r,bf16", [(3, False), (4, True), (8, True), (24, True), (40, True)])
+def test_back_to_back_equals_one_by_one(r, bf16, n_streams):
+    shapes = [[(256, 64)], [(1024, 300), (512, 96)], [(1160, 40)] * 3]
+    streams = [torch.cuda.Stream() for _ in range(n_streams)]
+    a = iterate([build(s, 600, r, bf16) for s in shapes], sync=True)
+    b = iterate([build(s, 600, r, bf16) for s in shapes], sync=False, streams=streams)
+    for x, y in zip(a, b):
+        assert torch.equal(x, y)
+
+
+def test_workspace_free_calls_back_to_back():
+    Xs = [to_dev(WL.planted_activations(m, d, 8, seed=m, bf16=False), False)[0] for m, d in ((300, 200), (1000, 512), (64, 128))]
+    got = []
+    for sync in (True, False):
+        Vs = [torch.zeros(8, X.shape[1], device=DEV) for X in Xs for _ in range(2)]
+        for i, V in enumerate(Vs):
+            B.agzo_extract_subspace_static(Xs[i // 2], V, 8, 2, i, i)
+            if sync:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        got.append(Vs)
+    for x, y in zip(*got):
+        assert torch.equal(x, y)
