@@ -126,16 +126,25 @@ def _check(status: int, what: str, allow: Sequence[int] = ()) -> int:
     return status
 
 
+_DTYPE_CODES = {torch.bfloat16: AGZO_BF16, torch.float32: AGZO_F32}
+
+
 def _dtype_code(t: torch.Tensor) -> int:
-    if t.dtype == torch.bfloat16:
-        return AGZO_BF16
-    if t.dtype == torch.float32:
-        return AGZO_F32
-    raise TypeError(f"unsupported dtype {t.dtype}")
+    code = _DTYPE_CODES.get(t.dtype)
+    if code is None:
+        raise TypeError(f"unsupported dtype {t.dtype}")
+    return code
+
+
+# the current stream's handle without building a Stream object (a few hundred nanoseconds instead of microseconds: the
+# smallest calls are host-bound); torch versions without it take the public way
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream_ptr(stream) -> int:
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
@@ -146,33 +155,33 @@ def make_layer(*, V: torch.Tensor, r: int, layer_id: int, W: Optional[torch.Tens
                X: Optional[torch.Tensor] = None, W16: Optional[torch.Tensor] = None,
                d_in: Optional[int] = None) -> agzo_layer:
     """Descriptor from 2-D torch tensors (last dimension contiguous); keeps no reference."""
-    L = agzo_layer()
-    if V.dim() != 2 or V.stride(1) != 1 or V.dtype != torch.float32:
+    v_stride = V.stride()
+    if len(v_stride) != 2 or v_stride[1] != 1 or V.dtype != torch.float32:
         raise ValueError("V must be [r][ldv] fp32 with unit inner stride")
-    L.V, L.ldv, L.r, L.layer_id, L.reserved = V.data_ptr(), V.stride(0), int(r), int(layer_id), 0
     if d_in is None:
-        d_in = W.shape[1] if W is not None else X.shape[1]
-    L.d_in = int(d_in)
+        d_in = (W if W is not None else X).shape[1]
+    w = w16 = x = None
+    ldw = ldw16 = ldx = w_dtype = x_dtype = d_out = m = 0
     if W is not None:
-        if W.dim() != 2 or W.stride(1) != 1:
+        w_stride = W.stride()
+        if len(w_stride) != 2 or w_stride[1] != 1:
             raise ValueError("W must be 2-D with unit inner stride")
-        L.W, L.ldw, L.w_dtype, L.d_out = W.data_ptr(), W.stride(0), _dtype_code(W), W.shape[0]
+        w, ldw, w_dtype, d_out = W.data_ptr(), w_stride[0], _dtype_code(W), W.shape[0]
     if W16 is not None:
         if W16.dtype != torch.bfloat16 or W16.stride(1) != 1:
             raise ValueError("W16 must be bf16 with unit inner stride")
-        L.W16, L.ldw16 = W16.data_ptr(), W16.stride(0)
+        w16, ldw16 = W16.data_ptr(), W16.stride(0)
     if X is not None:
-        if X.dim() != 2 or X.stride(1) != 1:
+        x_stride = X.stride()
+        if len(x_stride) != 2 or x_stride[1] != 1:
             raise ValueError("X must be 2-D with unit inner stride")
-        L.X, L.ldx, L.x_dtype, L.m = X.data_ptr(), X.stride(0), _dtype_code(X), X.shape[0]
-    return L
+        x, ldx, x_dtype, m = X.data_ptr(), x_stride[0], _dtype_code(X), X.shape[0]
+    return agzo_layer(w, ldw, w16, ldw16, x, ldx, V.data_ptr(), v_stride[0], w_dtype, x_dtype, d_out, int(d_in), m, int(r),
+                      int(layer_id), 0)
 
 
 def layer_array(layers: Sequence[agzo_layer]):
-    arr = (agzo_layer * max(1, len(layers)))()
-    for i, l in enumerate(layers):
-        arr[i] = l
-    return arr
+    return (agzo_layer * max(1, len(layers)))(*layers)
 
 
 # ---------------------------------------------------------------- thin wrappers, same names

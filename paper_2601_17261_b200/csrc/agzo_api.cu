@@ -102,9 +102,11 @@ struct agzo_ctx {
   std::vector<agzo_layer> cached;
   bool cached_valid;
   Plan plan;
-  // pinned staging for the upload
+  // the tables as they were built, and pinned staging for those too large for a kernel's parameters
+  std::vector<char> h_tables;
   void* h_stage;
   size_t h_stage_bytes;
+  bool h_stage_busy;       // a copy out of h_stage may still be under way (stage_ev tells)
   cudaEvent_t stage_ev;
   bool stage_pending;
   cudaStream_t stage_stream;  // stream of the last table upload: a call on another stream waits for stage_ev
@@ -532,6 +534,32 @@ int* dev_items(agzo_ctx* c, int n) { return dev_tiles(c, n) + (n + 1); }
 DevStatus* dev_status(agzo_ctx* c) { return reinterpret_cast<DevStatus*>(c->ws); }
 float* dev_coef(agzo_ctx* c) { return reinterpret_cast<float*>(c->ws + kCoefOffset); }
 
+// Tables of up to 30 KiB (36 layers) travel as the parameters of a kernel that writes them to the workspace: the launch
+// takes its copy, so the host neither waits for an earlier upload nor keeps a buffer, and the stream stays a chain of
+// kernels.  A forward hook that extracts one group of layers per call uploads once per call; with a pinned buffer the host
+// waited there for the previous call's kernels.  The kernels after it read the tables before they wait for their
+// predecessor, so this one does not let them start early.
+constexpr int kTableThreads = 256, kTableCtas = 8;
+template <int BYTES> struct TableBlob { uint4 d[BYTES / 16]; };
+template <int BYTES>
+__global__ void __launch_bounds__(kTableThreads) table_kernel(const __grid_constant__ TableBlob<BYTES> blob, uint4* dst, int n16) {
+  chain_wait();
+  for (int i = blockIdx.x * kTableThreads + threadIdx.x; i < n16; i += gridDim.x * kTableThreads) dst[i] = blob.d[i];
+}
+template <int BYTES>
+cudaError_t launch_table(const std::vector<char>& t, char* dst, cudaStream_t s) {
+  TableBlob<BYTES> blob;
+  std::memcpy(&blob, t.data(), t.size());
+  const int n16 = (int)(t.size() / 16), ctas = std::min(kTableCtas, (n16 + kTableThreads - 1) / kTableThreads);
+  return launch_chained(table_kernel<BYTES>, dim3((unsigned)ctas), kTableThreads, 0, 0, s, blob, reinterpret_cast<uint4*>(dst), n16);
+}
+constexpr size_t kTableParamBytes = 30 * 1024;
+cudaError_t upload_as_parameters(const std::vector<char>& t, char* dst, cudaStream_t s) {
+  if (t.size() <= 3 * 1024) return launch_table<3 * 1024>(t, dst, s);
+  if (t.size() <= 10 * 1024) return launch_table<10 * 1024>(t, dst, s);
+  return launch_table<(int)kTableParamBytes>(t, dst, s);
+}
+
 // Makes the device tables describe `L`; uploads only when the descriptors changed.
 agzo_status prepare(agzo_ctx* c, const agzo_layer* L, int n, cudaStream_t s) {
   if (same_layers(c, L, n)) {
@@ -554,21 +582,10 @@ agzo_status prepare(agzo_ctx* c, const agzo_layer* L, int n, cudaStream_t s) {
   if (st != AGZO_OK) return st;
   const size_t lb = align_up((size_t)n * sizeof(DevLayer));
   const size_t tb = prefix_bytes(n) + (size_t)n * kMapBytes;
-  if (c->stage_pending) {
-    CU(c, cudaEventSynchronize(c->stage_ev));
-    c->stage_pending = false;
-  }
-  if (lb + tb > c->h_stage_bytes) {
-    if (c->h_stage) CU(c, cudaFreeHost(c->h_stage));
-    c->h_stage = nullptr;
-    c->h_stage_bytes = 0;
-    CU(c, cudaMallocHost(&c->h_stage, (lb + tb) * 2));
-    c->h_stage_bytes = (lb + tb) * 2;
-  }
   if (n > 0) {
-    std::memcpy(c->h_stage, plan.dev.data(), (size_t)n * sizeof(DevLayer));
-    char* hs = static_cast<char*>(c->h_stage);
-    std::memset(hs + lb, 0, tb);
+    c->h_tables.assign(lb + tb, 0);      // both multiples of 16
+    char* hs = c->h_tables.data();
+    std::memcpy(hs, plan.dev.data(), (size_t)n * sizeof(DevLayer));
     std::memcpy(hs + lb, plan.tile_start.data(), (size_t)(n + 1) * sizeof(int));
     std::memcpy(hs + lb + (size_t)(n + 1) * sizeof(int), plan.item_start.data(), (size_t)(n + 1) * sizeof(int));
     char* hmaps = hs + lb + prefix_bytes(n);
@@ -579,7 +596,24 @@ agzo_status prepare(agzo_ctx* c, const agzo_layer* L, int n, cudaStream_t s) {
       if (plan.dev[i].wmap && !rmw_tc_encode_map(c->tc, plan.dev[i], hmaps + (size_t)i * kMapBytes + 384))
         return AGZO_ERR_UNSUPPORTED;
     }
-    CU(c, cudaMemcpyAsync(c->ws + kHeaderBytes, c->h_stage, lb + tb, cudaMemcpyHostToDevice, s));
+    c->cached_valid = false;             // until the upload is on its way
+    if (lb + tb <= kTableParamBytes) {
+      c->launches += 1;
+      CU(c, upload_as_parameters(c->h_tables, c->ws + kHeaderBytes, s));
+    } else {
+      if (c->h_stage_busy) CU(c, cudaEventSynchronize(c->stage_ev));
+      c->h_stage_busy = false;
+      if (lb + tb > c->h_stage_bytes) {
+        if (c->h_stage) CU(c, cudaFreeHost(c->h_stage));
+        c->h_stage = nullptr;
+        c->h_stage_bytes = 0;
+        CU(c, cudaMallocHost(&c->h_stage, (lb + tb) * 2));
+        c->h_stage_bytes = (lb + tb) * 2;
+      }
+      std::memcpy(c->h_stage, hs, lb + tb);
+      CU(c, cudaMemcpyAsync(c->ws + kHeaderBytes, c->h_stage, lb + tb, cudaMemcpyHostToDevice, s));
+      c->h_stage_busy = true;
+    }
     CU(c, cudaEventRecord(c->stage_ev, s));
     c->stage_pending = true;
     c->stage_stream = s;
@@ -708,6 +742,7 @@ agzo_status agzo_create(agzo_ctx** out, int device, void* workspace, size_t work
   c->cached_valid = false;
   c->h_stage = nullptr;
   c->h_stage_bytes = 0;
+  c->h_stage_busy = false;
   c->stage_pending = false;
   c->stage_ev = nullptr;
   c->time_class = 0;

@@ -69,3 +69,31 @@ def test_workspace_free_calls_back_to_back():
         got.append(Vs)
     for x, y in zip(*got):
         assert torch.equal(x, y)
+
+
+def test_layer_lists_alternate_without_waiting():
+    # lists on both sides of every way their tables are uploaded (in a kernel's parameters of three sizes, from pinned memory)
+    X, _ = to_dev(WL.planted_activations(70, 64, 8, seed=1, bf16=True), True)
+    counts = (3, 4, 11, 12, 36, 37, 60)
+    got = []
+    for sync in (True, False):
+        Ws = [to_dev(WL.gaussian_weights(24, 64, 0.02, seed=i, bf16=True), True)[0] for i in range(sum(counts))]
+        Vs = [torch.zeros(4, 64, device=DEV) for _ in Ws]
+        layers = [B.make_layer(X=X, W=W, V=V, r=4, layer_id=i) for i, (W, V) in enumerate(zip(Ws, Vs))]
+        ctx = B.agzo_create(layers, 0)
+        torch.cuda.synchronize()
+        for seed in range(3):
+            at = 0
+            for n in counts:
+                B.agzo_extract_subspace(ctx, layers[at:at + n], seed, 1)
+                if sync:
+                    torch.cuda.synchronize()
+                B.agzo_perturb(ctx, layers[at:at + n], seed, 1e-2)
+                if sync:
+                    torch.cuda.synchronize()
+                at += n
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+        B.agzo_destroy(ctx)
+        got.append(Ws + Vs)
+    for x, y in zip(*got):
+        assert torch.equal(x, y)
