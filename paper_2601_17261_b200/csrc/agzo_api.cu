@@ -236,25 +236,6 @@ void slab_shape(const agzo_layer& a, bool tc, bool long_slabs, long long cc_bloc
   *slabs = (a.m + rows - 1) / rows;
 }
 
-// scratch bytes one layer needs for extraction (0 when it has no X)
-// y_parts_min: room for at least that many partial sums of Y (the fused power step leaves one per share of
-// its launch that meets the layer, which can be more than the slabs of X^T T)
-size_t layer_scratch(const agzo_layer& a, bool tc, bool long_slabs, long long cc_blocks, bool with_panels = true,
-                     int y_parts_min = 0) {
-  if (!has_x(a)) return 0;
-  int slabs, slab_rows;
-  slab_shape(a, tc, long_slabs, cc_blocks, &slabs, &slab_rows);
-  if (slabs < y_parts_min) slabs = y_parts_min;
-  const size_t r = (size_t)a.r, d = (size_t)a.d_in, m = (size_t)a.m;
-  size_t b = 0;
-  b += align_up(m * r * 4);                 // T
-  b += align_up((size_t)slabs * r * d * 4); // Ypart
-  b += align_up(r * d * 4);                 // Y
-  b += align_up(panel_gram_bytes(a.d_in, a.r));   // Gpart
-  if (tc && with_panels) b += tc_layer_scratch(a);
-  return b;
-}
-
 constexpr size_t kMapBytes = 512;   // four TMA descriptors per layer
 // device tables after the header: layer records | tile prefix and item prefix (n + 1 ints each) | TMA descriptors
 size_t prefix_bytes(int n) { return align_up((size_t)2 * (n + 1) * sizeof(int)); }
@@ -380,25 +361,25 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
 
   // extraction waves: consecutive layers whose activations fit the wave budget and whose
   // scratch fits the workspace
-  // A layer that shares its X with a neighbour stays with the two-sweep kernels unless fusing is forced: one
-  // sweep serves the whole group there, which moves fewer bytes per layer than one fused pass per layer.
-  auto shares_input = [&](int k) {
-    if (!opts.share_inputs) return false;
-    return (k > 0 && has_x(L[k - 1]) && tc_eligible(L[k - 1]) && same_input(L[k - 1], L[k])) ||
-           (k + 1 < n && has_x(L[k + 1]) && tc_eligible(L[k + 1]) && same_input(L[k], L[k + 1]));
-  };
-  auto runs_fused = [&](const agzo_layer& a) {
-    return opts.extract_fused && extract_path != 1 && extract_path != 3 && tc_available && tc_eligible(a) &&
-           fused_eligible(opts.fused_caps, a, opts.extract_fused == 2) && (opts.extract_fused == 2 || !shares_input((int)(&a - L)));
+  auto on_tc = [&](const agzo_layer& a) { return extract_path != 1 && tc_available && tc_eligible(a); };
+  // the fused power step for a layer, or for layers on one X taken as one layer of `ranks` ranks
+  auto with_ranks = [](agzo_layer a, int ranks) { a.r = ranks; return a; };
+  auto fuses = [&](const agzo_layer& a, int ranks) {
+    return opts.extract_fused && extract_path != 3 && on_tc(a) && ranks <= 16 &&
+           fused_eligible(opts.fused_caps, with_ranks(a, ranks), opts.extract_fused == 2);
   };
   long long column_blocks = 0, cc_blocks = 0;
   for (int k = 0; k < n; ++k)
     if (has_x(L[k]))
-      (extract_path != 1 && tc_available && tc_eligible(L[k]) ? column_blocks : cc_blocks) += (L[k].d_in + 127) / 128;
+      (on_tc(L[k]) ? column_blocks : cc_blocks) += (L[k].d_in + 127) / 128;
   const bool long_slabs_any = column_blocks >= kLongSlabColumnBlocks;
-  auto long_slabs_for = [&](const agzo_layer&) { return long_slabs_any; };
-  auto y_parts_min = [&](const agzo_layer& a) {
-    return runs_fused(a) ? fused_parts_bound(a, fused_cluster_size(opts.fused_caps, a, opts.extract_fused == 2)) : 0;
+  // partial sums of Y that a unit's last product can leave: slabs, or shares of a fused launch
+  auto parts_of = [&](const agzo_layer& a, bool tc, bool fused, int ranks) {
+    int slabs, slab_rows;
+    slab_shape(a, tc, long_slabs_any, ws ? cc_blocks : 0, &slabs, &slab_rows);
+    if (!fused) return slabs;
+    const int C = ws ? fused_cluster_size(opts.fused_caps, with_ranks(a, ranks), opts.extract_fused == 2) : fused_min_cluster(a);
+    return std::max(slabs, fused_parts_bound(a, C));
   };
   int i = 0;
   while (i < n) {
@@ -413,34 +394,46 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     size_t used = 0, used_y = 0;    // scratch of the wave so far; the part of it that is Y panels
     int64_t xbytes = 0;
     int j = i;
-    const bool wave_tc = extract_path != 1 && tc_available && tc_eligible(L[i]);
+    const bool wave_tc = on_tc(L[i]);
     while (j < n && has_x(L[j])) {
-      const bool tc = extract_path != 1 && tc_available && tc_eligible(L[j]);
+      const bool tc = on_tc(L[j]);
       if (tc != wave_tc) break;      // a wave runs on one kind of kernel
-      // a unit is one layer, or a run of consecutive layers that read the same X (one sweep serves all)
-      int glen = 1, rows = tc ? tc_operand_rows(L[j].r) : 0;
-      if (tc && opts.share_inputs && !runs_fused(L[j])) {
-        while (j + glen < n && has_x(L[j + glen]) && same_input(L[j], L[j + glen]) && tc_eligible(L[j + glen]) &&
-               !runs_fused(L[j + glen]) &&
-               rows + tc_operand_rows(L[j + glen].r) <= 256) {
-          rows += tc_operand_rows(L[j + glen].r);
-          ++glen;
+      // A unit is one layer, or a run of consecutive layers that read the same X.  A run of at most 16 ranks in all takes
+      // the fused power step as one layer of that many ranks; a larger one the two sweeps, which serve it with two
+      // reads of X per step where fusing it layer by layer would read X once for each (unless fusing is forced).
+      int glen = 1, ranks = L[j].r;
+      bool fused = tc && fuses(L[j], ranks);
+      if (tc && opts.share_inputs) {
+        int run = 1, all = ranks;
+        while (j + run < n && has_x(L[j + run]) && same_input(L[j], L[j + run])) all += L[j + run++].r;
+        if (run > 1 && fuses(L[j], all)) {
+          glen = run; ranks = all; fused = true;
+        } else if (run > 1 && !(fused && opts.extract_fused == 2)) {
+          fused = false;
+          while (glen < run && tc_operand_rows(ranks + L[j + glen].r) <= 256 &&
+                 !(opts.extract_fused == 2 && fuses(L[j + glen], L[j + glen].r)))
+            ranks += L[j + glen++].r;
         }
       }
-      auto unit_need = [&](int len, int nrows) {
-        size_t b = 0;
-        for (int g = 0; g < len; ++g)
-          b += layer_scratch(L[j + g], tc, long_slabs_for(L[j + g]), ws ? cc_blocks : 0, false, y_parts_min(L[j + g]));
-        if (tc) b += tc_panel_bytes(L[j], nrows);
+      auto unit_need = [&]() {
+        size_t b = align_up((size_t)parts_of(L[j], tc, fused, ranks) * ranks * (size_t)L[j].d_in * 4);      // Ypart
+        for (int g = 0; g < glen; ++g) {
+          const agzo_layer& a = L[j + g];
+          if (!tc) b += align_up((size_t)a.m * a.r * 4);        // T
+          b += align_up((size_t)a.r * a.d_in * 4);              // Y
+          b += align_up(panel_gram_bytes(a.d_in, a.r));         // Gpart
+        }
+        if (tc) b += tc_panel_bytes(L[j], ranks);
         return b;
       };
-      size_t need = unit_need(glen, rows);
+      size_t need = unit_need();
       const int64_t xb = (int64_t)L[j].m * L[j].d_in * (L[j].x_dtype == AGZO_BF16 ? 2 : 4);
       if (j > i && (used + need > scratch_cap || xbytes + xb > wave_bytes)) break;
       if (used + need > scratch_cap && glen > 1) {   // the group alone does not fit: fall back to single layers
         glen = 1;
-        rows = tc_operand_rows(L[j].r);
-        need = unit_need(glen, rows);
+        ranks = L[j].r;
+        fused = false;
+        need = unit_need();
       }
       if (used + need > scratch_cap) return AGZO_ERR_WORKSPACE;
       // carve
@@ -448,34 +441,31 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
       for (int g = 0; g < glen; ++g) need_y += align_up((size_t)L[j + g].r * (size_t)L[j + g].d_in * 4);
       if (ws) {
         char* p = ws + base + (size_t)region * scratch_cap + (used - used_y);
+        float* ypart = reinterpret_cast<float*>(p);
+        p += align_up((size_t)parts_of(L[j], tc, fused, ranks) * ranks * (size_t)L[j].d_in * 4);
+        int off = 0;
         for (int g = 0; g < glen; ++g) {
           DevLayer& D = plan->dev[j + g];
           const agzo_layer& a = L[j + g];
-          int slabs, slab_rows;
-          slab_shape(a, tc, long_slabs_for(a), cc_blocks, &slabs, &slab_rows);
-          const size_t r = (size_t)a.r, d = (size_t)a.d_in, m = (size_t)a.m;
-          const size_t gch = (d + 127) / 128;
-          D.slabs = slabs; D.slab_rows = slab_rows; D.gchunks = (int)gch;
-          D.T = reinterpret_cast<float*>(p);      p += align_up(m * r * 4);
-          const size_t parts = (size_t)(slabs > y_parts_min(a) ? slabs : y_parts_min(a));
-          D.Ypart = reinterpret_cast<float*>(p);  p += align_up(parts * r * d * 4);
+          slab_shape(a, tc, long_slabs_any, cc_blocks, &D.slabs, &D.slab_rows);
+          D.gchunks = (a.d_in + 127) / 128;
+          D.Ypart = ypart + (size_t)off * a.d_in;
+          D.ypart_stride = (long long)ranks * a.d_in;
+          off += a.r;
+          if (!tc) { D.T = reinterpret_cast<float*>(p); p += align_up((size_t)a.m * a.r * 4); }
           D.Gpart = reinterpret_cast<double*>(p); p += align_up(panel_gram_bytes(a.d_in, a.r));
         }
-        if (tc) {
-          int row0 = 0;
-          for (int g = 0; g < glen; ++g) {
-            DevLayer& D = plan->dev[j + g];
-            const agzo_layer& a = L[j + g];
-            tc_set_panels(a, &D, p, rows, row0);
-            row0 += tc_operand_rows(a.r);
-            D.grp_role = glen == 1 ? 0 : (g == 0 ? 1 : 2);
-            D.grp_n = g == 0 ? glen : 0;
-            D.grp_NB = g == 0 ? rows : 0;
-            D.tmaps = ws + maps_offset(n) + (size_t)(j + g) * kMapBytes;
-            // the power steps of this layer run fused (X read once per step) where its shape allows
-            D.fz_C = runs_fused(a) ? fused_cluster_size(opts.fused_caps, a, opts.extract_fused == 2) : 0;
-            D.fz_slice = fused_slice_cols(opts.fused_caps, a, opts.extract_fused == 2);
-          }
+        off = 0;
+        for (int g = 0; tc && g < glen; ++g) {
+          DevLayer& D = plan->dev[j + g];
+          tc_set_panels(L[j + g], &D, p, ranks, off, g == glen - 1);
+          off += L[j + g].r;
+          D.grp_role = glen == 1 ? 0 : (g == 0 ? 1 : 2);
+          D.tmaps = ws + maps_offset(n) + (size_t)(j + g) * kMapBytes;
+          // the power steps of this unit run fused (X read once per step) where its shape allows
+          const agzo_layer all = with_ranks(L[j], ranks);
+          D.fz_C = fused ? fused_cluster_size(opts.fused_caps, all, opts.extract_fused == 2) : 0;
+          D.fz_slice = fused ? fused_slice_cols(opts.fused_caps, all, opts.extract_fused == 2) : 0;
         }
       }
       used += need;

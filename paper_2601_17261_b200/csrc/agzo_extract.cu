@@ -152,7 +152,7 @@ __device__ __forceinline__ void xt_t_body(const DevLayer& L, float* sT, float* s
       }
     }
     if (warp == 0) {
-      float* out = L.Ypart + ((long long)slab * r + k0) * L.d_in + d;
+      float* out = L.Ypart + slab * L.ypart_stride + (long long)k0 * L.d_in + d;
 #pragma unroll
       for (int k = 0; k < RC; ++k) {
         if (k >= kc) break;
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(256) sum_slabs_kernel(const DevLayer* __restri
   const long long n = (long long)L.r * L.d_in;
   for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
     float y = 0.f;
-    for (int s = 0; s < nparts; ++s) y += L.Ypart[(long long)s * n + i];
+    for (int s = 0; s < nparts; ++s) y += L.Ypart[s * L.ypart_stride + i];
     L.Y[i] = y;
   }
 }

@@ -118,7 +118,7 @@ struct FzWalk {
   __device__ bool next(const DevLayer* layers, int l1, int C, int cluster, FzItem* it) {
     for (; l < l1; ++l) {
       const DevLayer* L = layers + l;
-      if (L->fz_C != C) continue;
+      if (L->fz_C != C || L->grp_role == 2) continue;
       const int nt = (L->m + kTT - 1) / kTT;
       const int b = max(lo, L->fz_tile0), e = min(hi, L->fz_tile0 + nt);
       if (b >= e) continue;
@@ -371,7 +371,7 @@ fused_power_step_kernel(const DevLayer* __restrict__ layers, int l0, int l1, int
     FzItem it;
     for (FzWalk walk(l0, cluster, share_base, share_rem); ok && walk.next(layers, l1, C, cluster, &it); ++ic) {
       const DevLayer& L = *it.L;
-      const int NB = L.NB, NP = L.NP, r = L.r;
+      const int NB = L.NB, NP = L.NP, r = L.pr;
       const int col0 = rank * L.fz_slice;
       const int live = min(L.fz_slice, L.d_in - col0);
       const int mb = (live + 127) / 128;
@@ -484,7 +484,7 @@ fused_power_step_kernel(const DevLayer* __restrict__ layers, int l0, int l1, int
       tc_fence_after();
       for (int b = 0; b < mb; ++b) {
         const int d = col0 + b * 128 + q * 32 + lane;
-        float* out = L.Ypart + (long long)it.part * r * L.d_in + d;
+        float* out = L.Ypart + it.part * L.ypart_stride + d;
         for (int k0 = 0; k0 < NP; k0 += 8) {
           float hi[8], lo[8];
           tmem_ld8(tmem + lane_off + (uint32_t)(b * NB + k0), hi);
@@ -609,6 +609,8 @@ int fused_parts_bound(const agzo_layer& a, int C) {
   return nt < shares ? nt : shares;
 }
 
+int fused_min_cluster(const agzo_layer& a) { return (a.d_in + kWideSliceCols - 1) / kWideSliceCols; }
+
 // The arithmetic of the work split on plain arrays (also what the host-side test export runs): layer i has
 // tiles[i] tiles; with `clusters` resident clusters there are G = min(total, clusters) shares.  Writes each
 // layer's first tile in the list, the first share that meets it and the number of shares that do; returns G
@@ -634,7 +636,7 @@ void fused_plan_shares(const FusedCaps& caps, DevLayer* dev, int l0, int l1, int
   std::vector<int> idx, tiles;
   bool wide = C > 8;
   for (int i = l0; i < l1; ++i)
-    if (dev[i].fz_C == C) {
+    if (dev[i].fz_C == C && dev[i].grp_role != 2) {
       idx.push_back(i);
       tiles.push_back((dev[i].m + kTT - 1) / kTT);
       wide = wide || dev[i].fz_slice > kSliceCols;
@@ -648,6 +650,8 @@ void fused_plan_shares(const FusedCaps& caps, DevLayer* dev, int l0, int l1, int
     dev[idx[k]].fz_tile0 = tile0[k];
     dev[idx[k]].fz_first = first[k];
     dev[idx[k]].fz_parts = parts[k];
+    for (int i = idx[k] + 1; dev[idx[k]].grp_role == 1 && i < l1 && dev[i].grp_role == 2; ++i)
+      dev[i].fz_parts = parts[k];        // the group's layers read the partial sums that their leader's pieces leave
   }
 }
 
@@ -657,7 +661,7 @@ cudaError_t launch_fused_power_step(const FusedCaps& caps, const ExtractWave& w,
   int total = 0;
   bool wide = C > 8, small = true;
   for (int i = w.l0; i < w.l1; ++i)
-    if (h_dev[i].fz_C == C) {
+    if (h_dev[i].fz_C == C && h_dev[i].grp_role != 2) {
       total += (h_dev[i].m + kTT - 1) / kTT;
       if (h_dev[i].fz_slice > kSliceCols) wide = true;
       if (h_dev[i].NB > 16) small = false;

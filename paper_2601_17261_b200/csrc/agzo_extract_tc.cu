@@ -65,8 +65,7 @@ __global__ void __launch_bounds__(kTcThreads) tc_x_q_kernel(const DevLayer* __re
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   __shared__ TcShared sh;
-  const int NB = L.grp_role == 1 ? L.grp_NB : L.NB;   // operand rows: the whole group's for a leader
-  const int nmem = L.grp_role == 1 ? L.grp_n : 1;
+  const int NB = L.NB;                                // operand rows: the whole group's for a leader
   const int a_bytes = 2 * kTileBytes;                 // [128 tokens][64 d]
   const int b_bytes = NB * kBoxK * 2;                 // [NB][64 d]
   const int stage_bytes = a_bytes + ((b_bytes + 1023) & ~1023);
@@ -154,23 +153,20 @@ __global__ void __launch_bounds__(kTcThreads) tc_x_q_kernel(const DevLayer* __re
     if (!ok) sh.failed = 1;
     const int t = t0 + q * 32 + lane;
     if (ok) {
-      for (int mi = 0; mi < nmem; ++mi) {               // the layers this CTA serves
-        const DevLayer& M = layers[li + mi];
-        const int NP = M.NP, off = L.grp_role == 1 ? M.grp_off : 0;
-        __nv_bfloat16* Tt = M.Tb;
-        const long long mp = M.m_pad;
-        for (int k0 = 0; k0 < NP; k0 += 8) {
-          float hi[8], lo[8];
-          tmem_ld8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(off + k0), hi);
-          tmem_ld8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(off + NP + k0), lo);
-          if (t < L.m) {
+      const int NP = L.NP;
+      __nv_bfloat16* Tt = L.Tb;
+      const long long mp = L.m_pad;
+      for (int k0 = 0; k0 < NP; k0 += 8) {
+        float hi[8], lo[8];
+        tmem_ld8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)k0, hi);
+        tmem_ld8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(NP + k0), lo);
+        if (t < L.m) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              __nv_bfloat16 h, l;
-              split_bf16(hi[j] + lo[j], &h, &l);
-              Tt[(long long)(k0 + j) * mp + t] = h;
-              Tt[(long long)(NP + k0 + j) * mp + t] = l;
-            }
+          for (int j = 0; j < 8; ++j) {
+            __nv_bfloat16 h, l;
+            split_bf16(hi[j] + lo[j], &h, &l);
+            Tt[(long long)(k0 + j) * mp + t] = h;
+            Tt[(long long)(NP + k0 + j) * mp + t] = l;
           }
         }
       }
@@ -193,8 +189,7 @@ __global__ void __launch_bounds__(kTcThreads) tc_xt_t_kernel(const DevLayer* __r
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   __shared__ TcShared sh;
-  const int NB = L.grp_role == 1 ? L.grp_NB : L.NB;
-  const int nmem = L.grp_role == 1 ? L.grp_n : 1;
+  const int NB = L.NB;
   const int a_bytes = 2 * kTileBytes;                 // two [64 tokens][64 d] boxes: d0.., d0+64..
   const int b_bytes = NB * kBoxK * 2;                 // [NB][64 tokens]
   const int stage_bytes = a_bytes + ((b_bytes + 1023) & ~1023);
@@ -272,19 +267,16 @@ __global__ void __launch_bounds__(kTcThreads) tc_xt_t_kernel(const DevLayer* __r
     if (!ok) sh.failed = 1;
     const int d = d0 + q * 32 + lane;
     if (ok) {
-      for (int mi = 0; mi < nmem; ++mi) {               // the layers this CTA serves (same slabs: same m)
-        const DevLayer& M = layers[l0 + blockIdx.z + mi];
-        const int r = M.r, NP = M.NP, off = L.grp_role == 1 ? M.grp_off : 0;
-        float* out = M.Ypart + (long long)slab * r * L.d_in + d;
-        for (int k0 = 0; k0 < NP; k0 += 8) {
-          float hi[8], lo[8];
-          tmem_ld8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(off + k0), hi);
-          tmem_ld8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(off + NP + k0), lo);
-          if (d < L.d_in) {
+      const int r = L.pr, NP = L.NP;
+      float* out = L.Ypart + slab * L.ypart_stride + d;
+      for (int k0 = 0; k0 < NP; k0 += 8) {
+        float hi[8], lo[8];
+        tmem_ld8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)k0, hi);
+        tmem_ld8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(NP + k0), lo);
+        if (d < L.d_in) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-              if (k0 + j < r) out[(long long)(k0 + j) * L.d_in] = hi[j] + lo[j];
-          }
+          for (int j = 0; j < 8; ++j)
+            if (k0 + j < r) out[(long long)(k0 + j) * L.d_in] = hi[j] + lo[j];
         }
       }
     }
@@ -305,7 +297,9 @@ __global__ void __launch_bounds__(256) tc_fill_omega_kernel(const DevLayer* __re
   chain_wait();
   if (short_launch()) chain_next();
   const DevLayer& L = layers[l0 + blockIdx.y];
-  const int r = L.r, NP = L.NP, groups = NP >> 3;
+  const int r = L.r, NP = L.NP, rows = L.prow_n, groups = (rows + 7) >> 3;
+  __nv_bfloat16* hi_rows = L.Tb + (long long)L.grp_off * L.m_pad;
+  __nv_bfloat16* lo_rows = hi_rows + (long long)NP * L.m_pad;
   const long long mp = L.m_pad;
   const long long units = (long long)L.m * groups;
   for (long long unit = blockIdx.x * 256ll + threadIdx.x; unit < units; unit += (long long)gridDim.x * 256) {
@@ -338,8 +332,10 @@ __global__ void __launch_bounds__(256) tc_fill_omega_kernel(const DevLayer* __re
     for (int u = 0; u < 8; ++u) {
       __nv_bfloat16 h, l;
       split_bf16(v[u], &h, &l);
-      L.Tb[(long long)(8 * g + u) * mp + t] = h;
-      L.Tb[(long long)(NP + 8 * g + u) * mp + t] = l;
+      if (8 * g + u < rows) {
+        hi_rows[(long long)(8 * g + u) * mp + t] = h;
+        lo_rows[(long long)(8 * g + u) * mp + t] = l;
+      }
     }
   }
 }
@@ -447,21 +443,20 @@ bool tc_eligible(const agzo_layer& a) {
 
 int tc_operand_rows(int r) { return 2 * np_of(r); }
 
-size_t tc_panel_bytes(const agzo_layer& a, int rows) {
-  return up256((size_t)rows * (size_t)a.d_in * 2) + up256((size_t)rows * (size_t)mpad_of(a.m) * 2);
+size_t tc_panel_bytes(const agzo_layer& a, int ranks) {
+  const size_t rows = (size_t)tc_operand_rows(ranks);
+  return up256(rows * (size_t)a.d_in * 2) + up256(rows * (size_t)mpad_of(a.m) * 2);
 }
 
-size_t tc_layer_scratch(const agzo_layer& a) { return tc_panel_bytes(a, tc_operand_rows(a.r)); }
-
-void tc_set_panels(const agzo_layer& a, DevLayer* D, char* p, int rows, int row0) {
-  D->NP = np_of(a.r);
+void tc_set_panels(const agzo_layer& a, DevLayer* D, char* p, int ranks, int off, bool last) {
+  D->NP = np_of(ranks);
   D->NB = 2 * D->NP;
   D->m_pad = mpad_of(a.m);
-  __nv_bfloat16* qb = reinterpret_cast<__nv_bfloat16*>(p);
-  __nv_bfloat16* tb = reinterpret_cast<__nv_bfloat16*>(p + up256((size_t)rows * (size_t)a.d_in * 2));
-  D->Qb = qb + (size_t)row0 * a.d_in;
-  D->Tb = tb + (size_t)row0 * D->m_pad;
-  D->grp_off = row0;
+  D->Qb = reinterpret_cast<__nv_bfloat16*>(p);
+  D->Tb = reinterpret_cast<__nv_bfloat16*>(p + up256((size_t)D->NB * (size_t)a.d_in * 2));
+  D->pr = ranks;
+  D->grp_off = off;
+  D->prow_n = last ? D->NP - off : a.r;
 }
 
 bool tc_encode_maps(const TcState& st, const DevLayer& D, void* host_maps) {
@@ -469,8 +464,7 @@ bool tc_encode_maps(const TcState& st, const DevLayer& D, void* host_maps) {
   uint8_t* out = static_cast<uint8_t*>(host_maps);
   // X [m][ldx]: inner = d_in, outer = m; one box = 64 columns x 64 tokens
   if (!encode_2d(st.encode_fn, out, D.X, (uint64_t)D.d_in, (uint64_t)D.m, (uint64_t)D.ldx * 2, 64, 64)) return false;
-  // a group leader's descriptors cover the operand rows of the whole group
-  const uint32_t nb = D.grp_role == 1 ? (uint32_t)D.grp_NB : (uint32_t)D.NB;
+  const uint32_t nb = (uint32_t)D.NB;       // a group leader's descriptors cover the panel of the whole group
   // Qb [nb][d_in]: box = 64 columns x nb rows
   if (!encode_2d(st.encode_fn, out + 128, D.Qb, (uint64_t)D.d_in, (uint64_t)nb, (uint64_t)D.d_in * 2, 64, nb))
     return false;
@@ -481,7 +475,7 @@ bool tc_encode_maps(const TcState& st, const DevLayer& D, void* host_maps) {
 }
 
 cudaError_t tc_fill_omega(const TcState&, const ExtractWave& w, const DevLayer*, uint64_t seed, cudaStream_t s) {
-  const long long units = (long long)w.max_m * ((w.max_r + 7) >> 3);
+  const long long units = (long long)w.max_m * ((w.max_r + 14) >> 3);   // a layer's rows, padding rows of its panel included
   int gx = (int)((units + 255) / 256);
   if (gx > 1024) gx = 1024;
   if (gx < 1) gx = 1;
@@ -492,7 +486,7 @@ cudaError_t tc_xt_t(const TcState&, const ExtractWave& w, const DevLayer* h_dev,
                     bool skip_fused, cudaStream_t s) {
   int max_nb = 0;
   for (int i = w.l0; i < w.l1; ++i) {
-    const int nb = h_dev[i].grp_role == 1 ? h_dev[i].grp_NB : h_dev[i].NB;
+    const int nb = h_dev[i].NB;
     max_nb = nb > max_nb ? nb : max_nb;
   }
   const int stages = stages_for(max_nb);
@@ -505,7 +499,7 @@ cudaError_t tc_x_q(const TcState&, const ExtractWave& w, const DevLayer* h_dev, 
                    bool skip_fused, cudaStream_t s) {
   int max_nb = 0;
   for (int i = w.l0; i < w.l1; ++i) {
-    const int nb = h_dev[i].grp_role == 1 ? h_dev[i].grp_NB : h_dev[i].NB;
+    const int nb = h_dev[i].NB;
     max_nb = nb > max_nb ? nb : max_nb;
   }
   const int stages = stages_for(max_nb);

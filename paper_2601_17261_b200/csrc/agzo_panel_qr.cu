@@ -122,7 +122,7 @@ __device__ __forceinline__ void qr_add_share(double* g, const double (&acc)[QrCf
 __device__ __forceinline__ void qr_load(const DevLayer& L, float* sY, int pitch, int r8, int d0, int ncols, int nparts,
                                         bool from_y, bool keep) {
   const int r = L.r, d_in = L.d_in;
-  const long long part = (long long)r * d_in;
+  const long long part = L.ypart_stride;
   const float* src0 = from_y ? L.Y : L.Ypart;
   const int np = from_y ? 1 : nparts;
   if ((d_in & 3) == 0) {
@@ -349,13 +349,15 @@ __device__ __forceinline__ void qr_apply(float* sY, int pitch, const double* M, 
 // Q of columns [d0, d0 + ncols) out: V rows (fp32) and / or the bf16 hi/lo rows of the next product's operand
 __device__ __forceinline__ void qr_store(const DevLayer& L, const float* sY, int pitch, int d0, int ncols, bool to_v, bool to_qb) {
   const int r = L.r, d_in = L.d_in;
-  const int rows = to_qb ? L.NP : r;               // the panel's padding rows are zero, as Q's are
+  const int rows = to_qb ? L.prow_n : r;
+  __nv_bfloat16* hi_rows = L.Qb + (long long)L.grp_off * d_in;
+  __nv_bfloat16* lo_rows = hi_rows + (long long)L.NP * d_in;
   if ((d_in & 3) == 0 && (L.ldv & 3) == 0 && (reinterpret_cast<uintptr_t>(L.V) & 15u) == 0) {
     const int vrow = ncols >> 2;
     for (int i = threadIdx.x; i < rows * vrow; i += kQrThreads) {
       const int k = i / vrow, c = 4 * (i - k * vrow), d = d0 + c;
       if (d >= d_in) continue;
-      const float4 q = *reinterpret_cast<const float4*>(sY + k * pitch + c);
+      const float4 q = k < r ? *reinterpret_cast<const float4*>(sY + k * pitch + c) : make_float4(0.f, 0.f, 0.f, 0.f);
       if (to_v && k < r) *reinterpret_cast<float4*>(L.V + (long long)k * L.ldv + d) = q;
       if (to_qb) {
         const __nv_bfloat162 h0 = __floats2bfloat162_rn(q.x, q.y), h1 = __floats2bfloat162_rn(q.z, q.w);
@@ -364,20 +366,20 @@ __device__ __forceinline__ void qr_store(const DevLayer& L, const float* sY, int
         uint2 h, l;
         h.x = *reinterpret_cast<const uint32_t*>(&h0); h.y = *reinterpret_cast<const uint32_t*>(&h1);
         l.x = *reinterpret_cast<const uint32_t*>(&l0); l.y = *reinterpret_cast<const uint32_t*>(&l1);
-        *reinterpret_cast<uint2*>(L.Qb + (long long)k * d_in + d) = h;
-        *reinterpret_cast<uint2*>(L.Qb + (long long)(L.NP + k) * d_in + d) = l;
+        *reinterpret_cast<uint2*>(hi_rows + (long long)k * d_in + d) = h;
+        *reinterpret_cast<uint2*>(lo_rows + (long long)k * d_in + d) = l;
       }
     }
   } else {
     for (int i = threadIdx.x; i < rows * ncols; i += kQrThreads) {
       const int k = i / ncols, c = i - k * ncols, d = d0 + c;
       if (d >= d_in) continue;
-      const float q = sY[k * pitch + c];
+      const float q = k < r ? sY[k * pitch + c] : 0.f;
       if (to_v && k < r) L.V[(long long)k * L.ldv + d] = q;
       if (to_qb) {
         const __nv_bfloat16 hi = __float2bfloat16_rn(q);
-        L.Qb[(long long)k * d_in + d] = hi;
-        L.Qb[(long long)(L.NP + k) * d_in + d] = __float2bfloat16_rn(q - __bfloat162float(hi));
+        hi_rows[(long long)k * d_in + d] = hi;
+        lo_rows[(long long)k * d_in + d] = __float2bfloat16_rn(q - __bfloat162float(hi));
       }
     }
   }

@@ -107,6 +107,7 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
   rec.x_dtype = x_dtype; rec.d_in = d_in; rec.m = m; rec.r = r; rec.layer_id = layer_id;
   rec.slabs = slabs; rec.slab_rows = slab_rows; rec.gchunks = (int)gch;
   rec.T = reinterpret_cast<float*>(p);      p += up256(M * R * 4);
+  rec.ypart_stride = (long long)r * d_in;
   rec.Ypart = reinterpret_cast<float*>(p);  p += up256((size_t)slabs * R * D * 4);
   rec.Y = reinterpret_cast<float*>(p);      p += up256(R * D * 4);
   rec.Gpart = reinterpret_cast<double*>(p);     // never more than the two terms in r^2 of the limit above

@@ -23,12 +23,11 @@ struct TcState {
 cudaError_t tc_init(TcState* st, int device);
 // true when the layer's activations can go through the tensor-core kernels
 bool tc_eligible(const agzo_layer& a);
-size_t tc_layer_scratch(const agzo_layer& a);
-// operand rows of one layer (hi + lo parts of r rounded up to 8) and bytes of panels with `rows` rows
-int tc_operand_rows(int r);
-size_t tc_panel_bytes(const agzo_layer& a, int rows);   // Qb [rows][d_in] + Tb [rows][m_pad], each 256-byte padded
-// points D at rows [row0, row0 + its operand rows) of panels that start at p and have `rows` rows
-void tc_set_panels(const agzo_layer& a, DevLayer* D, char* p, int rows, int row0);
+// operand rows of a panel of `ranks` ranks (hi + lo parts, ranks rounded up to 8) and the bytes of the two panels
+int tc_operand_rows(int ranks);
+size_t tc_panel_bytes(const agzo_layer& a, int ranks);   // Qb [rows][d_in] + Tb [rows][m_pad], each 256-byte padded
+// points D at panels that start at p and hold `ranks` ranks, this layer's from `off` on; last: it is the panel's last layer
+void tc_set_panels(const agzo_layer& a, DevLayer* D, char* p, int ranks, int off, bool last);
 
 // writes the layer's TMA descriptors (512 bytes) into host memory; false when encoding fails
 bool tc_encode_maps(const TcState& st, const DevLayer& D, void* host_maps);
@@ -69,6 +68,7 @@ bool fused_eligible(const FusedCaps* caps, const agzo_layer& a, bool any_size);
 int fused_cluster_size(const FusedCaps* caps, const agzo_layer& a, bool any_size);
 int fused_slice_cols(const FusedCaps* caps, const agzo_layer& a, bool any_size);   // columns of X per CTA of the cluster, 0 = not eligible
 int fused_parts_bound(const agzo_layer& a, int C);              // partial sums of Y a power step can leave, at most
+int fused_min_cluster(const agzo_layer& a);                     // the smallest C that any device or rank can lead to
 void fused_plan_shares(const FusedCaps& caps, DevLayer* dev, int l0, int l1, int C);   // fills fz_tile0 / fz_first / fz_parts of a wave's layers of size C
 int fused_resident_clusters(const FusedCaps& caps, int C);      // clusters of C CTAs the device holds at once
 // the split on plain arrays and the first tile of share k (host; the kernel walks the same shares)
