@@ -27,10 +27,19 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kTcThreads = 192;        // warp 0: TMA producer, warp 1: MMA issuer, warps 2..5: epilogue
+// Threads of a CTA that works on MB blocks of 128 rows: warp 0 TMA producer, warp 1 MMA issuer, then four epilogue warps
+// per block.
+constexpr int tc_threads(int mb) { return 64 + 128 * mb; }
 constexpr int kBoxK = 64;              // elements per 128-byte swizzle row
 constexpr int kTileBytes = 64 * kBoxK * 2;   // one [64 rows][64 elems] bf16 box = 8 KiB
-constexpr size_t kMinSmem = 80 * 1024;  // keeps at most 2 CTAs per SM: 2 * 128 TMEM columns fit
+constexpr size_t kMinSmem = 80 * 1024;  // keeps at most 2 CTAs per SM: 2 * 256 TMEM columns fit
+
+// One block per CTA (two CTAs per SM) while the operand panel is small.  A panel of NB rows is fetched through L2 once per
+// block of X, NB / 128 bytes per byte of X; from about one byte per byte on, the path from L2 into the SMs is what the
+// sweep waits for (r = 64, q + k in one panel of 256 rows: 5.1 TB/s of X, 11.7 TB/s into the SMs).  Two blocks per CTA (one
+// CTA per SM) then share each fetch.  Extraction, one / two blocks: four 8B-shaped blocks with shared inputs r = 24 4174 / 3751 us,
+// r = 64 5920 / 5272; 20 0.6B-shaped blocks r = 16 1808 / 1670; panels of up to 64 rows 3005 / 3001 (r = 16 without shared inputs).
+constexpr int kTwoBlockRows = 96;      // panel rows from which a launch takes two blocks per CTA
 
 struct TcShared {
   uint64_t full[8];
@@ -52,29 +61,53 @@ __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16* hi, __nv_bflo
   *lo = __float2bfloat16_rn(v - __bfloat162float(h));
 }
 
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+
+// Eight ranks k0 .. k0 + 7 of token t of T out, as bf16 hi and lo parts (Tt is [NB][m_pad], tokens contiguous)
+__device__ __forceinline__ void put_t8(const DevLayer& L, int k0, int t, const float (&v)[8]) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    __nv_bfloat16 h, l;
+    split_bf16(v[j], &h, &l);
+    L.Tb[(long long)(k0 + j) * L.m_pad + t] = h;
+    L.Tb[(long long)(L.NP + k0 + j) * L.m_pad + t] = l;
+  }
+}
+
 // ---------------------------------------------------------------- T = X Q  (Tt = T^T as bf16 hi/lo)
-// One CTA per 128-token tile of one layer.  grid = (max token tiles, layers in the wave).
-__global__ void __launch_bounds__(kTcThreads) tc_x_q_kernel(const DevLayer* __restrict__ layers, int l0,
-                                                            DevStatus* status, int stages, int skip_fused) {
+// One cluster of CK CTAs per tile of 128 * MB tokens of one layer; grid = (max token tiles * CK, layers in the wave).
+// CK > 1 (MB = 1 only): launches with fewer token tiles than the device has room for split the columns over the CTAs of a
+// cluster; their sums of T meet through distributed shared memory, CTA c adding (in rank order) and writing the ranks
+// 8 c .. 8 c + 7, 8 (c + CK) ...  Four 0.6B-shaped blocks, 613 tokens, r = 8, a call per group: 1465 -> 1186 us.
+template <int MB>
+__global__ void __launch_bounds__(tc_threads(MB)) tc_x_q_kernel(const DevLayer* __restrict__ layers, int l0, DevStatus* status,
+                                                                int stages, int skip_fused, int CK) {
   // CTA rows are handed out in the order the scheduler starts them: the layers with the longest
   // token rows (largest d_in, longest CTAs) go first so that the wave does not end on them
   const int li = l0 + layers[l0 + blockIdx.y].xq_order;
   const DevLayer& L = layers[li];
-  const int t0 = blockIdx.x * 128;
+  const int rank = CK > 1 ? (int)cluster_ctarank() : 0;
+  const int t0 = ((int)blockIdx.x / CK) * 128 * MB;
   if (t0 >= L.m || (skip_fused && L.fz_C) || L.grp_role == 2) return;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   __shared__ TcShared sh;
-  const int NB = L.NB;                                // operand rows: the whole group's for a leader
-  const int a_bytes = 2 * kTileBytes;                 // [128 tokens][64 d]
+  const int NB = L.NB, NP = L.NP;                     // operand rows: the whole group's for a leader
+  const int a_bytes = 2 * MB * kTileBytes;            // [128 MB tokens][64 d]
   const int b_bytes = NB * kBoxK * 2;                 // [NB][64 d]
   const int stage_bytes = a_bytes + ((b_bytes + 1023) & ~1023);
-  const int nk = (L.d_in + kBoxK - 1) / kBoxK;
+  const int nk_all = (L.d_in + kBoxK - 1) / kBoxK;
+  const int kb = rank * nk_all / CK, nk = (rank + 1) * nk_all / CK - kb;   // this CTA's k-steps
+  const int nblk = min(MB, (L.m - t0 + 127) / 128);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint8_t* maps = reinterpret_cast<const uint8_t*>(L.tmaps);
   const void* map_x = maps;            // X  [m][d_in], box 64 x 64
   const void* map_q = maps + 128;      // Qb [NB][d_in], box 64 x NB
-  const uint32_t ncols = pow2_cols(NB);
+  const uint32_t ncols = pow2_cols(MB * NB);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
@@ -112,12 +145,12 @@ __global__ void __launch_bounds__(kTcThreads) tc_x_q_kernel(const DevLayer* __re
           if (kk >= stages && !mbar_wait(&sh.empty[s], ((kk / stages) - 1) & 1)) { sh.failed = 1; ok = false; break; }
           a[u] = tiles + (size_t)s * stage_bytes;
           bar[u] = &sh.full[s];
-          mbar_expect_tx(bar[u], a_bytes + b_bytes);
+          mbar_expect_tx(bar[u], nblk * 2 * kTileBytes + b_bytes);
         }
         if (!ok) break;
-        for (int u = 0; u < n2; ++u) tma_load_2d(a[u], map_x, (k + u) * kBoxK, t0, bar[u]);
-        for (int u = 0; u < n2; ++u) tma_load_2d(a[u] + kTileBytes, map_x, (k + u) * kBoxK, t0 + 64, bar[u]);
-        for (int u = 0; u < n2; ++u) tma_load_2d(a[u] + a_bytes, map_q, (k + u) * kBoxK, 0, bar[u]);
+        for (int x = 0; x < 2 * nblk; ++x)
+          for (int u = 0; u < n2; ++u) tma_load_2d(a[u] + x * kTileBytes, map_x, (kb + k + u) * kBoxK, t0 + 64 * x, bar[u]);
+        for (int u = 0; u < n2; ++u) tma_load_2d(a[u] + a_bytes, map_q, (kb + k + u) * kBoxK, 0, bar[u]);
         issued = k + n2;
       }
       if (!ok || sh.failed) {    // leaving early: the copies in flight must land before the CTA goes away
@@ -125,52 +158,73 @@ __global__ void __launch_bounds__(kTcThreads) tc_x_q_kernel(const DevLayer* __re
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = instr_desc(128, NB, 0, 0);
-      bool ok = true;
-      for (int k = 0; k < nk && ok; ++k) {
-        const int s = k % stages;
-        if (!mbar_wait(&sh.full[s], (k / stages) & 1)) { sh.failed = 1; ok = false; break; }
-        tc_fence_after();
-        const uint32_t a = smem_u32(tiles + (size_t)s * stage_bytes);
-        const uint32_t b = a + a_bytes;
+    // all lanes run the loop and one elected lane issues: the descriptors stay warp-uniform (see mma_bf16_if)
+    const uint32_t go = elect_one();
+    const uint32_t idesc = instr_desc(128, NB, 0, 0), tiles_addr = smem_u32(tiles);
+    uint32_t s = 0, par = 0, acc = 0u;
+    for (int k = 0; k < nk; ++k) {
+      if (!mbar_wait_warp(&sh.full[s], par)) { sh.failed = 1; break; }
+      tc_fence_after();
+      const uint32_t a = tiles_addr + s * (uint32_t)stage_bytes;
+      const uint64_t bd = smem_desc(a + (uint32_t)a_bytes, 0, 1024);
 #pragma unroll
-        for (int kk = 0; kk < kBoxK / 16; ++kk) {
-          const uint64_t ad = smem_desc(a + kk * 32, 0, 1024);
-          const uint64_t bd = smem_desc(b + kk * 32, 0, 1024);
-          mma_bf16(tmem, ad, bd, idesc, (k > 0 || kk > 0) ? 1u : 0u);
-        }
-        mma_commit(&sh.empty[s]);      // the stage is free once these MMAs have read it
+      for (int x = 0; x < MB; ++x) {
+        if (x >= nblk) break;
+        const uint64_t ad = smem_desc(a + (uint32_t)(x * 2 * kTileBytes), 0, 1024);
+#pragma unroll
+        for (int kk = 0; kk < kBoxK / 16; ++kk)          // 16 columns = 32 bytes = 2 descriptor units further
+          mma_bf16_if(go, tmem + (uint32_t)(x * NB), ad + (uint64_t)(2 * kk), bd + (uint64_t)(2 * kk), idesc, kk > 0 ? 1u : acc);
       }
-      mma_commit(&sh.accum);           // arrives when every MMA issued so far is done
+      acc = 1u;
+      mma_commit_if(go, &sh.empty[s]);       // the stage is free once these MMAs have read it
+      if (++s == (uint32_t)stages) { s = 0; par ^= 1u; }
     }
+    mma_commit_if(go, &sh.accum);            // arrives when every MMA issued so far is done
   } else {
-    // epilogue: TMEM lane i of this warp's quarter = token t0 + 32*q + lane
-    const int q = warp & 3;
+    // epilogue: TMEM lane i of this warp's quarter = token 32 q + lane of the block
+    const int q = warp & 3, blk = (warp - 2) >> 2;
     const bool ok = mbar_wait(&sh.accum, 0);
     tc_fence_after();
     if (!early) chain_next();
     if (!ok) sh.failed = 1;
-    const int t = t0 + q * 32 + lane;
-    if (ok) {
-      const int NP = L.NP;
-      __nv_bfloat16* Tt = L.Tb;
-      const long long mp = L.m_pad;
+    const int row = q * 32 + lane, t = t0 + 128 * blk + row;
+    if (ok && blk < nblk) {
       for (int k0 = 0; k0 < NP; k0 += 8) {
         float hi[8], lo[8];
-        tmem_ld8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)k0, hi);
-        tmem_ld8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(NP + k0), lo);
-        if (t < L.m) {
+        const uint32_t col = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(blk * NB + k0);
+        tmem_ld8(col, hi);
+        tmem_ld8(col + (uint32_t)NP, lo);
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            __nv_bfloat16 h, l;
-            split_bf16(hi[j] + lo[j], &h, &l);
-            Tt[(long long)(k0 + j) * mp + t] = h;
-            Tt[(long long)(NP + k0 + j) * mp + t] = l;
-          }
+        for (int j = 0; j < 8; ++j) hi[j] += lo[j];
+        if (CK > 1) {            // the pipeline's stages are idle: they take the partial sums, [rank group][token][8]
+          float4* p = reinterpret_cast<float4*>(tiles) + ((k0 >> 3) * 128 + row) * 2;
+          p[0] = make_float4(hi[0], hi[1], hi[2], hi[3]);
+          p[1] = make_float4(hi[4], hi[5], hi[6], hi[7]);
+        } else if (t < L.m) {
+          put_t8(L, k0, t, hi);
         }
       }
     }
+  }
+  if (MB == 1 && CK > 1) {
+    __syncwarp();
+    cluster_sync_all();          // every CTA's partial sums are in its shared memory
+    const int q = warp & 3, row = q * 32 + lane, t = t0 + row;
+    if (warp >= 2 && t < L.m) {
+      for (int g = rank; g < NP / 8; g += CK) {
+        float v[8] = {};
+        const uint32_t at = smem_u32(tiles) + (uint32_t)((g * 128 + row) * 32);
+        for (int c = 0; c < CK; ++c) {
+          const uint32_t src = mapa_shared(at, (uint32_t)c);
+          const float4 x = ld_cluster_f4(src), y = ld_cluster_f4(src + 16);
+          v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
+          v[4] += y.x; v[5] += y.y; v[6] += y.z; v[7] += y.w;
+        }
+        put_t8(L, 8 * g, t, v);
+      }
+    }
+    __syncwarp();
+    cluster_sync_all();          // nobody leaves while a peer reads its sums
   }
   tc_fence_before();
   __syncthreads();
@@ -179,20 +233,22 @@ __global__ void __launch_bounds__(kTcThreads) tc_x_q_kernel(const DevLayer* __re
 }
 
 // ---------------------------------------------------------------- Ypart[s] = X_s^T T_s
-// One CTA per (128 columns of X, token slab) of one layer.  grid = (column chunks, slabs, layers).
-__global__ void __launch_bounds__(kTcThreads) tc_xt_t_kernel(const DevLayer* __restrict__ layers, int l0,
-                                                             DevStatus* status, int stages, int skip_fused) {
+// One CTA per (128 * MB columns of X, token slab) of one layer.  grid = (column chunks, slabs, layers).
+template <int MB>
+__global__ void __launch_bounds__(tc_threads(MB)) tc_xt_t_kernel(const DevLayer* __restrict__ layers, int l0, DevStatus* status,
+                                                                 int stages, int skip_fused) {
   const DevLayer& L = layers[l0 + blockIdx.z];
-  const int d0 = blockIdx.x * 128;
+  const int d0 = blockIdx.x * 128 * MB;
   const int slab = blockIdx.y;
   if (d0 >= L.d_in || slab >= L.slabs || (skip_fused && L.fz_C) || L.grp_role == 2) return;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   __shared__ TcShared sh;
   const int NB = L.NB;
-  const int a_bytes = 2 * kTileBytes;                 // two [64 tokens][64 d] boxes: d0.., d0+64..
+  const int a_bytes = 2 * MB * kTileBytes;            // two [64 tokens][64 d] boxes per block of 128 columns
   const int b_bytes = NB * kBoxK * 2;                 // [NB][64 tokens]
   const int stage_bytes = a_bytes + ((b_bytes + 1023) & ~1023);
+  const int nblk = min(MB, (L.d_in - d0 + 127) / 128);
   const int t_begin = slab * L.slab_rows;
   const int t_end = min(L.m, t_begin + L.slab_rows);
   const int nk = (t_end - t_begin + kBoxK - 1) / kBoxK;
@@ -200,7 +256,7 @@ __global__ void __launch_bounds__(kTcThreads) tc_xt_t_kernel(const DevLayer* __r
   const uint8_t* maps = reinterpret_cast<const uint8_t*>(L.tmaps);
   const void* map_x = maps;            // X  [m][d_in], box 64 x 64
   const void* map_t = maps + 256;      // Tt [NB][m],   box 64 x NB
-  const uint32_t ncols = pow2_cols(NB);
+  const uint32_t ncols = pow2_cols(MB * NB);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
@@ -228,9 +284,8 @@ __global__ void __launch_bounds__(kTcThreads) tc_xt_t_kernel(const DevLayer* __r
         if (k >= stages && !mbar_wait(&sh.empty[s], ((k / stages) - 1) & 1)) { sh.failed = 1; break; }
         uint8_t* a = tiles + (size_t)s * stage_bytes;
         const int tk = t_begin + k * kBoxK;
-        mbar_expect_tx(&sh.full[s], a_bytes + b_bytes);
-        tma_load_2d(a, map_x, d0, tk, &sh.full[s]);
-        tma_load_2d(a + kTileBytes, map_x, d0 + 64, tk, &sh.full[s]);
+        mbar_expect_tx(&sh.full[s], nblk * 2 * kTileBytes + b_bytes);
+        for (int x = 0; x < 2 * nblk; ++x) tma_load_2d(a + x * kTileBytes, map_x, d0 + 64 * x, tk, &sh.full[s]);
         tma_load_2d(a + a_bytes, map_t, tk, 0, &sh.full[s]);
         issued = k + 1;
       }
@@ -239,40 +294,43 @@ __global__ void __launch_bounds__(kTcThreads) tc_xt_t_kernel(const DevLayer* __r
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = instr_desc(128, NB, 1, 0);     // A is MN-major: the X tile as X^T
-      bool ok = true;
-      for (int k = 0; k < nk && ok; ++k) {
-        const int s = k % stages;
-        if (!mbar_wait(&sh.full[s], (k / stages) & 1)) { sh.failed = 1; ok = false; break; }
-        tc_fence_after();
-        const uint32_t a = smem_u32(tiles + (size_t)s * stage_bytes);
-        const uint32_t b = a + a_bytes;
+    const uint32_t go = elect_one();
+    const uint32_t idesc = instr_desc(128, NB, 1, 0), tiles_addr = smem_u32(tiles);     // A is MN-major: the X tile as X^T
+    uint32_t s = 0, par = 0, acc = 0u;
+    for (int k = 0; k < nk; ++k) {
+      if (!mbar_wait_warp(&sh.full[s], par)) { sh.failed = 1; break; }
+      tc_fence_after();
+      const uint32_t a = tiles_addr + s * (uint32_t)stage_bytes;
+      const uint64_t bd = smem_desc(a + (uint32_t)a_bytes, 0, 1024);
 #pragma unroll
-        for (int kk = 0; kk < kBoxK / 16; ++kk) {
-          // 16 tokens = two 8-row swizzle atoms = 2048 bytes further down the X boxes
-          const uint64_t ad = smem_desc(a + kk * 2048, kTileBytes, 1024);
-          const uint64_t bd = smem_desc(b + kk * 32, 0, 1024);
-          mma_bf16(tmem, ad, bd, idesc, (k > 0 || kk > 0) ? 1u : 0u);
-        }
-        mma_commit(&sh.empty[s]);
+      for (int x = 0; x < MB; ++x) {
+        if (x >= nblk) break;
+        const uint64_t ad = smem_desc(a + (uint32_t)(x * 2 * kTileBytes), kTileBytes, 1024);
+#pragma unroll
+        for (int kk = 0; kk < kBoxK / 16; ++kk)
+          // 16 tokens = two 8-row swizzle atoms = 2048 bytes = 128 descriptor units further down the X boxes
+          mma_bf16_if(go, tmem + (uint32_t)(x * NB), ad + (uint64_t)(128 * kk), bd + (uint64_t)(2 * kk), idesc, kk > 0 ? 1u : acc);
       }
-      mma_commit(&sh.accum);
+      acc = 1u;
+      mma_commit_if(go, &sh.empty[s]);
+      if (++s == (uint32_t)stages) { s = 0; par ^= 1u; }
     }
+    mma_commit_if(go, &sh.accum);
   } else {
-    const int q = warp & 3;
+    const int q = warp & 3, blk = (warp - 2) >> 2;
     const bool ok = mbar_wait(&sh.accum, 0);
     tc_fence_after();
     if (!early) chain_next();
     if (!ok) sh.failed = 1;
-    const int d = d0 + q * 32 + lane;
-    if (ok) {
+    const int d = d0 + 128 * blk + q * 32 + lane;
+    if (ok && blk < nblk) {
       const int r = L.pr, NP = L.NP;
       float* out = L.Ypart + slab * L.ypart_stride + d;
       for (int k0 = 0; k0 < NP; k0 += 8) {
         float hi[8], lo[8];
-        tmem_ld8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)k0, hi);
-        tmem_ld8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(NP + k0), lo);
+        const uint32_t col = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(blk * NB + k0);
+        tmem_ld8(col, hi);
+        tmem_ld8(col + (uint32_t)NP, lo);
         if (d < L.d_in) {
 #pragma unroll
           for (int j = 0; j < 8; ++j)
@@ -380,17 +438,35 @@ int np_of(int r) { return (r + 7) & ~7; }
 long long mpad_of(int m) { return ((long long)m + 7) & ~7ll; }
 size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 
-int stages_for(int NB) {
-  const int stage = 2 * kTileBytes + ((NB * kBoxK * 2 + 1023) & ~1023);
-  int s = (int)((96 * 1024) / stage);
+int stage_bytes(int NB, int mb) { return mb * 2 * kTileBytes + ((NB * kBoxK * 2 + 1023) & ~1023); }
+int stages_for(int NB, int mb) {
+  int s = (mb == 1 ? 96 : 220) * 1024 / stage_bytes(NB, mb);
   if (s > 8) s = 8;
   if (s < 2) s = 2;
   return s;
 }
-size_t smem_for(int NB, int stages) {
-  const size_t stage = 2 * kTileBytes + ((NB * kBoxK * 2 + 1023) & ~1023);
-  size_t b = stage * stages + 1024;
-  return b < kMinSmem ? kMinSmem : b;
+size_t smem_for(int NB, int mb, int stages) {
+  const size_t b = (size_t)stage_bytes(NB, mb) * stages + 1024, least = mb == 1 ? kMinSmem : 120 * 1024;   // two, one CTA per SM
+  return b < least ? least : b;
+}
+
+// What a product's launch has to serve: the layers that stand for themselves or lead a group
+struct ProductShape {
+  int max_nb = 0, min_nk = 1 << 30;
+  long long tiles = 0;      // blocks of 128 tokens, or of 128 columns times slabs
+};
+template <typename F>
+ProductShape product_shape(const ExtractWave& w, const DevLayer* h_dev, bool skip_fused, F tiles_of) {
+  ProductShape p;
+  for (int i = w.l0; i < w.l1; ++i) {
+    const DevLayer& D = h_dev[i];
+    if (D.grp_role == 2 || (skip_fused && D.fz_C)) continue;
+    p.max_nb = D.NB > p.max_nb ? D.NB : p.max_nb;
+    const int nk = (D.d_in + kBoxK - 1) / kBoxK;
+    p.min_nk = nk < p.min_nk ? nk : p.min_nk;
+    p.tiles += tiles_of(D);
+  }
+  return p;
 }
 
 }  // namespace
@@ -417,9 +493,9 @@ cudaError_t tc_init(TcState* st, int device) {
   st->encode_fn = fn;
   st->available = major == 10;
   if (st->available) {
-    e = cudaFuncSetAttribute(tc_x_q_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(tc_xt_t_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    for (const void* k : {(const void*)tc_x_q_kernel<1>, (const void*)tc_x_q_kernel<2>, (const void*)tc_xt_t_kernel<1>,
+                          (const void*)tc_xt_t_kernel<2>})
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
     if (e == cudaSuccess) e = rmw_tc_init();
     if (e == cudaSuccess) {
       int sms = 0;
@@ -484,28 +560,24 @@ cudaError_t tc_fill_omega(const TcState&, const ExtractWave& w, const DevLayer*,
 
 cudaError_t tc_xt_t(const TcState&, const ExtractWave& w, const DevLayer* h_dev, DevStatus* d_status,
                     bool skip_fused, cudaStream_t s) {
-  int max_nb = 0;
-  for (int i = w.l0; i < w.l1; ++i) {
-    const int nb = h_dev[i].NB;
-    max_nb = nb > max_nb ? nb : max_nb;
-  }
-  const int stages = stages_for(max_nb);
-  dim3 grid((w.max_din + 127) / 128, w.max_slabs, w.l1 - w.l0);
-  return launch_chained(tc_xt_t_kernel, grid, kTcThreads, smem_for(max_nb, stages), 0, s, w.d_layers, w.l0, d_status, stages,
-                        skip_fused ? 1 : 0);
+  const ProductShape p = product_shape(w, h_dev, skip_fused, [](const DevLayer& D) { return (long long)D.gchunks * D.slabs; });
+  const int mb = p.max_nb >= kTwoBlockRows && p.tiles >= 2 * 148 * 2 ? 2 : 1;
+  const int stages = stages_for(p.max_nb, mb);
+  const dim3 grid((w.max_din + 128 * mb - 1) / (128 * mb), w.max_slabs, w.l1 - w.l0);
+  return launch_chained(mb == 1 ? tc_xt_t_kernel<1> : tc_xt_t_kernel<2>, grid, tc_threads(mb), smem_for(p.max_nb, mb, stages), 0, s,
+                        w.d_layers, w.l0, d_status, stages, skip_fused ? 1 : 0);
 }
 
 cudaError_t tc_x_q(const TcState&, const ExtractWave& w, const DevLayer* h_dev, DevStatus* d_status,
                    bool skip_fused, cudaStream_t s) {
-  int max_nb = 0;
-  for (int i = w.l0; i < w.l1; ++i) {
-    const int nb = h_dev[i].NB;
-    max_nb = nb > max_nb ? nb : max_nb;
-  }
-  const int stages = stages_for(max_nb);
-  dim3 grid((w.max_m + 127) / 128, w.l1 - w.l0);
-  return launch_chained(tc_x_q_kernel, grid, kTcThreads, smem_for(max_nb, stages), 0, s, w.d_layers, w.l0, d_status, stages,
-                        skip_fused ? 1 : 0);
+  const ProductShape p = product_shape(w, h_dev, skip_fused, [](const DevLayer& D) { return (long long)(D.m + 127) / 128; });
+  const int mb = p.max_nb >= kTwoBlockRows && p.tiles >= 2 * 148 * 2 ? 2 : 1;
+  int ck = 1;       // CTAs per token tile: up to two per SM, and at least two k-steps each
+  while (mb == 1 && ck < 8 && p.tiles * ck * 2 <= 296 && p.min_nk >= 4 * ck) ck *= 2;
+  const int stages = stages_for(p.max_nb, mb);
+  const dim3 grid((w.max_m + 128 * mb - 1) / (128 * mb) * ck, w.l1 - w.l0);
+  return launch_chained(mb == 1 ? tc_x_q_kernel<1> : tc_x_q_kernel<2>, grid, tc_threads(mb), smem_for(p.max_nb, mb, stages),
+                        ck > 1 ? ck : 0, s, w.d_layers, w.l0, d_status, stages, skip_fused ? 1 : 0, ck);
 }
 
 }  // namespace agzo

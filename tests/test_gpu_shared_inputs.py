@@ -39,3 +39,41 @@ def test_groups(fused, ranks, m, d_in):
                 Vg = to_host(Vs[i])
                 assert np.abs(Vg.astype(np.float64) @ Vg.T - np.eye(r)).max() <= 1e-5, (K, i)
                 assert projector_distance(Vg, O.extract_subspace(src[i][0], r, K, 9, i)) <= 1e-3, (K, i)
+
+
+@pytest.mark.parametrize("r", [1, 8, 24, 48, 64])
+@pytest.mark.parametrize("m,d_in", [(256, 128), (300, 520), (613, 1024), (1300, 1480), (4000, 264)])
+def test_columns_split_over_a_cluster(r, m, d_in):
+    # few token tiles: T = X Q splits the columns over 2, 4 or 8 CTAs, with steps left over
+    X = WL.planted_activations(m, d_in, 16, seed=m, bf16=True)
+    Xd = to_dev(X, True)[0]
+    V = torch.zeros(r, d_in, device=DEV)
+    layers = [B.make_layer(X=Xd, V=V, r=r, layer_id=2)]
+    with Ctx(layers) as ctx:
+        B.agzo_set_option(ctx, "extract_path", 3)
+        B.agzo_extract_subspace(ctx, layers, 4, 2)
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+    Vg = to_host(V)
+    assert np.abs(Vg.astype(np.float64) @ Vg.T - np.eye(r)).max() <= 1e-5
+    assert projector_distance(Vg, O.extract_subspace(X, r, 2, 4, 2)) <= 1e-3
+
+
+@pytest.mark.parametrize("ranks", [(48,), (24, 24), (64, 64)])
+def test_two_blocks_per_cta(ranks):
+    # enough tiles for two blocks of 128 rows per CTA; ragged tokens and columns leave half-empty pairs
+    shapes = [(8300, 1160)] * 6 + [(8300, 904)] * 6
+    Xs = {s: WL.planted_activations(*s, 16, seed=s[1], bf16=True) for s in set(shapes)}
+    Xd = [to_dev(Xs[s], True)[0] for s in shapes]
+    Vs, layers = [], []
+    for i, s in enumerate(shapes):
+        for r in ranks:
+            Vs.append((s, r, torch.zeros(r, s[1], device=DEV)))
+            layers.append(B.make_layer(X=Xd[i], V=Vs[-1][2], r=r, layer_id=len(layers)))
+    with Ctx(layers) as ctx:
+        B.agzo_extract_subspace(ctx, layers, 4, 1)
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+    for i in (0, len(Vs) - 1):
+        s, r, V = Vs[i]
+        Vg = to_host(V)
+        assert np.abs(Vg.astype(np.float64) @ Vg.T - np.eye(r)).max() <= 1e-5
+        assert projector_distance(Vg, O.extract_subspace(Xs[s], r, 1, 4, i)) <= 1e-3
