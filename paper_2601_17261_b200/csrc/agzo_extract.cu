@@ -47,28 +47,37 @@ __device__ __forceinline__ int x_kind(const DevLayer& L) {
   if (L.x_dtype == AGZO_F32) return (p & 15u) == 0 ? X_F32_VEC : X_SCALAR;
   return (p & 7u) == 0 ? X_BF16_VEC : X_SCALAR;
 }
-// zero beyond d_in; `ok` false: zeros
+// Row t (below m), columns d .. d + 3.  The vector kinds read four columns inside the row whatever d is: for uses where what
+// they are multiplied with is zero there, or the product is not stored.  The scalar kind returns zeros beyond d_in.
 template <int KIND>
-__device__ __forceinline__ float4 load_x4(const DevLayer& L, long long t, int d, bool ok) {
+__device__ __forceinline__ float4 load_x4_at(const DevLayer& L, int t, int d) {
   float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (!ok || d >= L.d_in) return v;
+  if constexpr (KIND != X_SCALAR) d = min(d, L.d_in - 4);
+  const long long at = (long long)t * L.ldx + d;
   if constexpr (KIND == X_F32_VEC) {
-    return __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(L.X) + t * L.ldx + d));
+    const float* p = reinterpret_cast<const float*>(L.X) + at;
+    asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
   } else if constexpr (KIND == X_BF16_VEC) {
-    const uint2 u = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(L.X) + t * L.ldx + d));
-    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
-                       __uint_as_float(u.y & 0xFFFF0000u));
+    const __nv_bfloat16* p = reinterpret_cast<const __nv_bfloat16*>(L.X) + at;
+    uint2 u;
+    asm("ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(u.x), "=r"(u.y) : "l"(p));
+    v = make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                    __uint_as_float(u.y & 0xFFFF0000u));
   } else {
     float e[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const long long at = t * L.ldx + d + c;
+    for (int c = 0; c < 4; ++c)
       e[c] = d + c >= L.d_in ? 0.f
-             : L.x_dtype == AGZO_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(L.X)[at])
-                                      : reinterpret_cast<const float*>(L.X)[at];
-    }
-    return make_float4(e[0], e[1], e[2], e[3]);
+             : L.x_dtype == AGZO_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(L.X)[at + c])
+                                      : reinterpret_cast<const float*>(L.X)[at + c];
+    v = make_float4(e[0], e[1], e[2], e[3]);
   }
+  return v;
+}
+// zeros beyond d_in, and where `ok` is false
+template <int KIND>
+__device__ __forceinline__ float4 load_x4(const DevLayer& L, int t, int d, bool ok) {
+  return ok && d < L.d_in ? load_x4_at<KIND>(L, t, d) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 constexpr int kXThreads = 256, kXWarps = kXThreads / 32;
@@ -80,56 +89,96 @@ constexpr int kXCols = 128;              // columns of one row that a warp reads
 // Ranks above RC are further passes over the slab, from L2.
 // Bound by X (HBM, or L2 where neighbouring layers read the same buffer) for RC <= 8.  The form before this one gave a
 // thread one column and all tokens of the slab, one 2- or 4-byte load at a time, and always 16 ranks: 14 fp32 layers of 4000
-// tokens (328 MB), r = 8: 289 us per product, now 115; one 512 x 256 layer, r = 4: 60 us, now 3.4.
+// tokens (328 MB), r = 8: 289 us per product, now 71; one 512 x 256 layer, r = 4: 60 us, now 3.4.
 constexpr int kXtTokens = 128;           // tokens of T staged at a time
 template <int RC, int KIND>
 __device__ __forceinline__ void xt_t_body(const DevLayer& L, float* sT, float* sRed, int d0, int slab) {
-  constexpr int U = 4;                   // tokens in flight per warp
+  constexpr int U = RC <= 8 ? 8 : 4;     // tokens in flight per warp
+  // Above rank 8 the pass is bound by its multiply-adds: two columns per instruction, T side by side twice as their operand
+  // (4096 x 2048, r = 16: 38 -> 29 us per product; at r = 8 the wider operand reads cost more than they save: 71 -> 78 us)
+  constexpr bool kPacked = RC > 8;
+  constexpr int kDup = kPacked ? 2 : 1;
+  constexpr int kStage = kXtTokens * RC / kXThreads;     // values of T per thread and chunk
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int d = d0 + 4 * lane, r = L.r;
   const int t_begin = slab * L.slab_rows, t_end = min(L.m, t_begin + L.slab_rows);
   for (int k0 = 0; k0 < r; k0 += RC) {
     const int kc = min(RC, r - k0);
     float acc[RC][4];
+    uint64_t acc2[kPacked ? RC : 1][2];
 #pragma unroll
-    for (int k = 0; k < RC; ++k)
+    for (int k = 0; k < RC; ++k) {
 #pragma unroll
       for (int c = 0; c < 4; ++c) acc[k][c] = 0.f;
-    for (int tb = t_begin; tb < t_end; tb += kXtTokens) {
-      float4 x[U];                       // the first rows of the chunk are on their way while T is staged
-      const int n = min(kXtTokens, t_end - tb);
+      if (kPacked) acc2[k][0] = acc2[k][1] = 0;
+    }
+    // Both streams run ahead: a chunk's T is fetched into registers while the chunk before it is worked on, and the next U
+    // rows of X while the current ones are used, across chunks too; T is zero beyond the slab, where X is read at its last row.
+    float tv[kStage];
+    auto fetch_t = [&](int tb) {
 #pragma unroll
-      for (int u = 0; u < U; ++u) x[u] = load_x4<KIND>(L, tb + warp + u * kXWarps, d, warp + u * kXWarps < n);
+      for (int j = 0; j < kStage; ++j) {
+        const int i = threadIdx.x + j * kXThreads, tt = i / RC, k = i - tt * RC;
+        tv[j] = tb + tt < t_end && k < kc ? L.T[(long long)(tb + tt) * r + k0 + k] : 0.f;
+      }
+    };
+    float4 x[U];
+    fetch_t(t_begin);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int t = t_begin + warp + u * kXWarps;
+      x[u] = load_x4_at<KIND>(L, min(t, t_end - 1), d);
+    }
+    for (int tb = t_begin; tb < t_end; tb += kXtTokens) {
       __syncthreads();
-      for (int i = threadIdx.x; i < n * RC; i += kXThreads) {
-        const int tt = i / RC, k = i - tt * RC;
-        sT[i] = k < kc ? L.T[(long long)(tb + tt) * r + k0 + k] : 0.f;
+#pragma unroll
+      for (int j = 0; j < kStage; ++j) {
+        const int i = threadIdx.x + j * kXThreads;
+        if (kPacked) *reinterpret_cast<float2*>(sT + 2 * i) = make_float2(tv[j], tv[j]);
+        else sT[i] = tv[j];
       }
       __syncthreads();
-      for (int t0 = warp; t0 < n; t0 += U * kXWarps) {
-        float4 nx[U];
+      if (tb + kXtTokens < t_end) fetch_t(tb + kXtTokens);
+      const int rounds = (min(kXtTokens, t_end - tb) + kXWarps - 1) / kXWarps;
+#pragma unroll 1
+      for (int i0 = 0; i0 < rounds; i0 += U) {        // rows warp + 8 (i0 + u) of the chunk
+        const float* st = sT + kDup * (warp + i0 * kXWarps) * RC;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const int t = t0 + (U + u) * kXWarps;
-          nx[u] = load_x4<KIND>(L, tb + t, d, t < n);
-        }
+          const float4 xu = x[u];
+          const int next = tb + warp + (i0 + U + u) * kXWarps;     // zero beyond the slab
+          x[u] = load_x4_at<KIND>(L, min(next, t_end - 1), d);
+          if constexpr (kPacked) {
+            const uint64_t xa = pack_f32x2(xu.x, xu.y), xb = pack_f32x2(xu.z, xu.w);
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int t = min(t0 + u * kXWarps, n - 1);          // x is zero beyond n
+            for (int k = 0; k < RC; k += 2) {
+              const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(st + 2 * (u * kXWarps * RC + k));
+              acc2[k][0] = fma_f32x2(xa, v.x, acc2[k][0]);
+              acc2[k][1] = fma_f32x2(xb, v.x, acc2[k][1]);
+              acc2[k + 1][0] = fma_f32x2(xa, v.y, acc2[k + 1][0]);
+              acc2[k + 1][1] = fma_f32x2(xb, v.y, acc2[k + 1][1]);
+            }
+          } else
 #pragma unroll
           for (int k4 = 0; k4 < RC; k4 += 4) {
-            const float4 v = *reinterpret_cast<const float4*>(sT + t * RC + k4);
-            const float tv[4] = {v.x, v.y, v.z, v.w};
+            const float4 v = *reinterpret_cast<const float4*>(st + u * kXWarps * RC + k4);
+            const float tk[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              acc[k4 + k][0] = fmaf(x[u].x, tv[k], acc[k4 + k][0]);
-              acc[k4 + k][1] = fmaf(x[u].y, tv[k], acc[k4 + k][1]);
-              acc[k4 + k][2] = fmaf(x[u].z, tv[k], acc[k4 + k][2]);
-              acc[k4 + k][3] = fmaf(x[u].w, tv[k], acc[k4 + k][3]);
+              acc[k4 + k][0] = fmaf(xu.x, tk[k], acc[k4 + k][0]);
+              acc[k4 + k][1] = fmaf(xu.y, tk[k], acc[k4 + k][1]);
+              acc[k4 + k][2] = fmaf(xu.z, tk[k], acc[k4 + k][2]);
+              acc[k4 + k][3] = fmaf(xu.w, tk[k], acc[k4 + k][3]);
             }
           }
-          x[u] = nx[u];
         }
+      }
+    }
+    if (kPacked) {
+#pragma unroll
+      for (int k = 0; k < RC; ++k) {
+        unpack_f32x2(acc2[k][0], acc[k][0], acc[k][1]);
+        unpack_f32x2(acc2[k][1], acc[k][2], acc[k][3]);
       }
     }
     // the warps' sums, halving: 4..7 onto 0..3, 2..3 onto 0..1, 1 onto 0
@@ -176,7 +225,7 @@ __global__ void __launch_bounds__(kXThreads, 2) xt_t_kernel(const DevLayer* __re
   chain_wait();
   if (short_launch()) chain_next();
   if (slab >= L.slabs || d0 >= L.d_in) return;
-  __shared__ __align__(16) float sT[kXtTokens * RC];
+  __shared__ __align__(16) float sT[kXtTokens * RC * (RC > 8 ? 2 : 1)];
   __shared__ __align__(16) float sRed[kXWarps / 2 * RC * kXCols];
   const int kind = x_kind(L);
   if (kind == X_F32_VEC) xt_t_body<RC, X_F32_VEC>(L, sT, sRed, d0, slab);
@@ -191,56 +240,57 @@ cudaError_t launch_xt_t(const ExtractWave& w, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------------ T[t][k] = sum_d X[t][d] Q[k][d]   (Q = rows of V)
-// A warp takes four tokens, its lanes four columns each; Q passes through shared memory 512 columns at a time, so that
-// a 16-byte read of it serves 16 multiply-adds (as many cycles of the FMA pipes as the read takes of shared memory).
-// The lanes' sums are added by halving exchanges (a lane ends up with RC / 8 of them).  Same bound as X^T T; before: one column per lane and load, 16 ranks always, 713 us and 15 us
-// on the two examples above, now 95 and 3.1.
-constexpr int kXqChunk = 512, kXqTokens = 4;
-template <int RC, int KIND>
-__device__ __forceinline__ void x_q_body(const DevLayer& L, float* sQ, int t0) {
+// A warp takes four tokens, its lanes four columns each, so that a 16-byte read of Q serves 16 multiply-adds.  Q is read
+// through L1, which X passes by (no_allocate), so it is fetched about once per SM, and the warps run without barriers.  The
+// lanes' sums are added by halving exchanges (a lane ends up with RC / 8 of them).  Same bound as X^T T; with one column per
+// lane and load, and always 16 ranks: 713 us and 15 us on the two examples above, now 94 and 3.
+constexpr int kXqTokens = 4;
+template <bool VVEC>
+__device__ __forceinline__ float4 load_q4(const float* p, int left) {
+  if constexpr (VVEC) {
+    return left > 0 ? *reinterpret_cast<const float4*>(p) : make_float4(0.f, 0.f, 0.f, 0.f);
+  } else {
+    float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (left > 0) q.x = p[0];
+    if (left > 1) q.y = p[1];
+    if (left > 2) q.z = p[2];
+    if (left > 3) q.w = p[3];
+    return q;
+  }
+}
+
+// SPLIT = 2: two neighbouring warps take half of the columns each and the sums meet in sPart (launches of so few tokens
+// that the SMs would have fewer than eight warps)
+template <int RC, int SPLIT, int KIND, bool VVEC>
+__device__ __forceinline__ void x_q_body(const DevLayer& L, int t0, float* sPart) {
   constexpr int TOK = kXqTokens;
-  const int lane = threadIdx.x & 31, r = L.r, d_in = L.d_in;
-  const bool v_vec = (d_in & 3) == 0 && (L.ldv & 3) == 0 && (reinterpret_cast<uintptr_t>(L.V) & 15u) == 0;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = L.r;
+  const int half = SPLIT == 2 ? warp & 1 : 0;
+  const int blocks = (L.d_in + kXCols - 1) / kXCols;
+  const int c_begin = half * ((blocks + 1) / 2) * kXCols;
+  const int d_end = SPLIT == 2 && half == 0 ? min(L.d_in, (blocks + 1) / 2 * kXCols) : L.d_in;
   for (int k0 = 0; k0 < r; k0 += RC) {
     const int kc = min(RC, r - k0);
+    const float* V = L.V + (long long)k0 * L.ldv;
     float acc[TOK * RC];
 #pragma unroll
     for (int i = 0; i < TOK * RC; ++i) acc[i] = 0.f;
-    for (int c0 = 0; c0 < d_in; c0 += kXqChunk) {
-      const int nc = min(kXqChunk, d_in - c0);
-      float4 x[TOK];                     // the first columns of the chunk are on their way while Q is staged
+    float4 x[TOK];
 #pragma unroll
-      for (int t = 0; t < TOK; ++t) x[t] = load_x4<KIND>(L, t0 + t, c0 + 4 * lane, t0 + t < L.m);
-      __syncthreads();
-      if (v_vec) {
-        for (int i = threadIdx.x; i < RC * (kXqChunk / 4); i += kXThreads) {
-          const int k = i / (kXqChunk / 4), c = 4 * (i - k * (kXqChunk / 4));
-          *reinterpret_cast<float4*>(sQ + k * kXqChunk + c) =
-              k < kc && c < nc ? *reinterpret_cast<const float4*>(L.V + (long long)(k0 + k) * L.ldv + c0 + c)
-                               : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-      } else {
-        for (int i = threadIdx.x; i < RC * kXqChunk; i += kXThreads) {
-          const int k = i / kXqChunk, c = i - k * kXqChunk;
-          sQ[i] = k < kc && c < nc ? L.V[(long long)(k0 + k) * L.ldv + c0 + c] : 0.f;
-        }
+    for (int t = 0; t < TOK; ++t) x[t] = load_x4<KIND>(L, t0 + t, c_begin + 4 * lane, t0 + t < L.m);
+    for (int c = c_begin + 4 * lane; c - 4 * lane < d_end; c += kXCols) {
+      float4 nx[TOK];
+#pragma unroll
+      for (int t = 0; t < TOK; ++t) nx[t] = load_x4<KIND>(L, t0 + t, c + kXCols, t0 + t < L.m);
+#pragma unroll
+      for (int k = 0; k < RC; ++k) {
+        const float4 q = load_q4<VVEC>(V + (long long)min(k, kc - 1) * L.ldv + c, L.d_in - c);   // ranks beyond kc are not stored
+#pragma unroll
+        for (int t = 0; t < TOK; ++t)
+          acc[t * RC + k] = fmaf(x[t].w, q.w, fmaf(x[t].z, q.z, fmaf(x[t].y, q.y, fmaf(x[t].x, q.x, acc[t * RC + k]))));
       }
-      __syncthreads();
-      for (int c = 4 * lane; c - 4 * lane < nc; c += kXCols) {
-        float4 nx[TOK];
-        const bool more = c - 4 * lane + kXCols < nc;
 #pragma unroll
-        for (int t = 0; t < TOK; ++t) nx[t] = load_x4<KIND>(L, t0 + t, c0 + c + kXCols, more && t0 + t < L.m);
-#pragma unroll
-        for (int k = 0; k < RC; ++k) {
-          const float4 q = *reinterpret_cast<const float4*>(sQ + k * kXqChunk + c);
-#pragma unroll
-          for (int t = 0; t < TOK; ++t)
-            acc[t * RC + k] = fmaf(x[t].w, q.w, fmaf(x[t].z, q.z, fmaf(x[t].y, q.y, fmaf(x[t].x, q.x, acc[t * RC + k]))));
-        }
-#pragma unroll
-        for (int t = 0; t < TOK; ++t) x[t] = nx[t];
-      }
+      for (int t = 0; t < TOK; ++t) x[t] = nx[t];
     }
     int at = 0;                          // first of the sums this lane keeps
     constexpr int N = TOK * RC;
@@ -260,6 +310,17 @@ __device__ __forceinline__ void x_q_body(const DevLayer& L, float* sQ, int t0) {
       }
     }
     constexpr int kKeep = N >= 32 ? N / 32 : 1;
+    if constexpr (SPLIT == 2) {
+      __syncthreads();                   // the previous ranks' sums have been used
+      if (half == 1) {
+#pragma unroll
+        for (int i = 0; i < kKeep; ++i) sPart[(warp >> 1) * 32 * kKeep + i * 32 + lane] = acc[i];
+      }
+      __syncthreads();
+      if (half == 1) continue;
+#pragma unroll
+      for (int i = 0; i < kKeep; ++i) acc[i] += sPart[(warp >> 1) * 32 * kKeep + i * 32 + lane];
+    }
     if (N >= 32 || (lane & (32 / (N < 32 ? N : 32) - 1)) == 0) {
 #pragma unroll
       for (int i = 0; i < kKeep; ++i) {
@@ -270,24 +331,32 @@ __device__ __forceinline__ void x_q_body(const DevLayer& L, float* sQ, int t0) {
   }
 }
 
-template <int RC>
+template <int RC, int SPLIT>
 __global__ void __launch_bounds__(kXThreads, 2) x_q_kernel(const DevLayer* __restrict__ layers, int l0) {
   const DevLayer& L = layers[l0 + blockIdx.y];
   chain_wait();
   if (short_launch()) chain_next();
-  if ((int)blockIdx.x * kXWarps * kXqTokens >= L.m) return;
-  __shared__ __align__(16) float sQ[RC * kXqChunk];
-  const int t0 = ((int)blockIdx.x * kXWarps + (threadIdx.x >> 5)) * kXqTokens;
-  const int kind = x_kind(L);
-  if (kind == X_F32_VEC) x_q_body<RC, X_F32_VEC>(L, sQ, t0);
-  else if (kind == X_BF16_VEC) x_q_body<RC, X_BF16_VEC>(L, sQ, t0);
-  else x_q_body<RC, X_SCALAR>(L, sQ, t0);
+  constexpr int kGroups = kXWarps / SPLIT;               // token groups per CTA
+  if ((int)blockIdx.x * kGroups * kXqTokens >= L.m) return;
+  __shared__ float sPart[SPLIT == 2 ? kGroups * 32 * (RC / 8 > 1 ? RC / 8 : 1) : 1];
+  const int t0 = ((int)blockIdx.x * kGroups + (int)(threadIdx.x >> 5) / SPLIT) * kXqTokens;
+  const bool v_vec = (L.d_in & 3) == 0 && (L.ldv & 3) == 0 && (reinterpret_cast<uintptr_t>(L.V) & 15u) == 0;
+  const int kind = v_vec ? x_kind(L) : X_SCALAR;
+  if (kind == X_F32_VEC) x_q_body<RC, SPLIT, X_F32_VEC, true>(L, t0, sPart);
+  else if (kind == X_BF16_VEC) x_q_body<RC, SPLIT, X_BF16_VEC, true>(L, t0, sPart);
+  else x_q_body<RC, SPLIT, X_SCALAR, false>(L, t0, sPart);
 }
 
-cudaError_t launch_x_q(const ExtractWave& w, cudaStream_t s) {
-  const dim3 grid((w.max_m + kXWarps * kXqTokens - 1) / (kXWarps * kXqTokens), w.l1 - w.l0);
-  const auto kernel = w.max_r <= 4 ? x_q_kernel<4> : w.max_r <= 8 ? x_q_kernel<8> : x_q_kernel<16>;
+template <int SPLIT>
+cudaError_t launch_x_q_split(const ExtractWave& w, cudaStream_t s) {
+  const int per = kXWarps / SPLIT * kXqTokens;
+  const dim3 grid((w.max_m + per - 1) / per, w.l1 - w.l0);
+  const auto kernel = w.max_r <= 4 ? x_q_kernel<4, SPLIT> : w.max_r <= 8 ? x_q_kernel<8, SPLIT> : x_q_kernel<16, SPLIT>;
   return launch_chained(kernel, grid, kXThreads, 0, 0, s, w.d_layers, w.l0);
+}
+cudaError_t launch_x_q(const ExtractWave& w, cudaStream_t s) {
+  const bool few = (long long)w.max_m * (w.l1 - w.l0) <= 148ll * kXWarps * kXqTokens;
+  return few ? launch_x_q_split<2>(w, s) : launch_x_q_split<1>(w, s);
 }
 
 // Y[k][d] = sum_s Ypart[s][k][d] in slab order, on its own: token-sharded extraction sums Y over

@@ -88,10 +88,9 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
   const size_t need = 512 + up256(M * R * 4) + up256((size_t)slabs * R * D * 4) + up256(R * D * 4) +
                       up256(gch * R * R * 8) + up256(R * R * 8);
   if (need > kStaticScratchBytes) return AGZO_ERR_WORKSPACE;   // problem too large for the fixed array
-  for (int rows = cc_slab_rows(m, (long long)gch); rows < slab_rows; rows += 32) {
-    const int n = (m + rows - 1) / rows;
-    const size_t more = up256((size_t)n * R * D * 4) - up256((size_t)slabs * R * D * 4);
-    if (n > slabs && need + more <= kStaticScratchBytes) { slab_rows = rows; slabs = n; break; }
+  for (int rows = cc_slab_rows(m, (long long)gch);; rows += 32) {      // ends at 256 tokens per slab at the latest
+    const size_t n = ((size_t)m + rows - 1) / rows;
+    if (need - up256((size_t)slabs * R * D * 4) + up256(n * R * D * 4) <= kStaticScratchBytes) { slab_rows = rows; slabs = (int)n; break; }
   }
 
   int dev = -1;
