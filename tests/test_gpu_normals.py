@@ -1,0 +1,28 @@
+"""The Gaussian generator over four million consecutive elements of a stream: uniforms down to the ends of their range (logarithms of
+numbers next to 1, angles next to every quadrant boundary).
+
+Tolerance: 2e-6 max(1, |g|), the bound every stream in the suite is held to; on top of it the root mean square of the
+difference stays below 2e-7, a few units in the last place of fp32 at the size of a normal."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import agzo_oracle as O
+from paper_2601_17261_b200 import binding as B
+
+from gpu_helpers import DEV
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("seed,layer", [(1, 0), (1 << 40, 77)])
+def test_normals(seed, layer):
+    n, r = 1 << 22, 4
+    ctx = B.Context(0, 4096)
+    got = B.agzo_debug_gaussian(ctx, seed, layer, 0, 0, n).cpu().numpy().astype(np.float64)
+    want = O.gen_G(seed, layer, n // r, r).astype(np.float64).reshape(-1)
+    d = np.abs(got - want)
+    assert (d <= 2e-6 * np.maximum(1.0, np.abs(want))).all()
+    assert np.sqrt(np.mean(d * d)) <= 2e-7
+    assert np.isfinite(got).all()
+    B.agzo_destroy(ctx)
