@@ -129,7 +129,7 @@ cudaError_t device_init(int device, TcState* tc) {
   auto it = known.find(device);
   if (it == known.end()) {
     TcState st;
-    cudaError_t e = panel_qr_init();
+    cudaError_t e = panel_qr_init(&st.qr_wide);
     if (e == cudaSuccess) e = rmw_init();
     if (e == cudaSuccess) e = tc_init(&st, device);
     if (e != cudaSuccess) return e;
@@ -932,6 +932,7 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
       w.l0 = l0; w.l1 = l1;
       w.omega_row0 = ctx->allreduce ? ctx->token_offset : 0;
       w.y_reduced = ctx->allreduce ? 1 : 0;
+      w.qr_wide = ctx->tc.qr_wide ? 1 : 0;
       bool all_tc = ctx->extract_path != 1;
       for (int i = l0; i < l1; ++i) {
         const DevLayer& D = P.dev[i];

@@ -31,7 +31,7 @@ using namespace ptx;
 constexpr int kQrThreads = 256;
 constexpr int kQrWarps = kQrThreads / 32;
 constexpr int kQrChunk = 128;            // columns of Y that are staged together
-constexpr int kQrMaxCluster = 8;
+constexpr int kQrMaxCluster = 16;         // beyond the portable 8: asked for, and used only where the device grants it
 constexpr int kBlk = 8;                  // block of the factorisation = tile of the FP64 tensor cores
 // up to here the slice stays in shared memory from load to apply, with two CTAs per SM
 constexpr size_t kQrResidentSmem = 112 * 1024;
@@ -622,7 +622,8 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_apply_kernel(const DevLay
   qr_store(L, sY, pitch, d0, kQrChunk, last || !L.Qb, !last && L.Qb);
 }
 
-// CTAs per layer: eight while the launch is a chain of latencies; with so many layers that eight each would queue for
+// CTAs per layer: eight, for up to eight layers sixteen, while the launch is a chain of latencies (two 8B-shaped blocks from
+// hooks, one group per launch: 3000 -> 2848 us per iteration with sixteen); with so many layers that eight each would queue for
 // the SMs (two CTAs each), four or two, since every CTA repeats the factorisation (r = 8, d_in = 2048, 196 layers: 44.5 /
 // 27.7 / 26.1 us with 8 / 4 / 2; r = 16, d_in = 4096, 70 layers: 43.5 / 28.3 / 55.1 us; 35 layers 28.7 / 27.4 / 51.5), but
 // never so few that the widest layer's slice leaves shared memory where eight would keep it (the 55 us above).
@@ -633,8 +634,8 @@ template <int NT>
 cudaError_t launch_qr(const ExtractWave& w, bool last, DevStatus* d_status, cudaStream_t s) {
   const int nl = w.l1 - w.l0;
   auto slice_of = [&](int c) { return (w.max_gchunks + c - 1) / c * kQrChunk; };
-  int C = nl <= 40 ? 8 : nl <= 80 ? 4 : 2;
-  while (C < kQrMaxCluster && qr_smem<NT>(slice_of(C)) > kQrResidentSmem) C *= 2;
+  int C = nl <= 8 && w.qr_wide ? 16 : nl <= 40 ? 8 : nl <= 80 ? 4 : 2;
+  while (C < 8 && qr_smem<NT>(slice_of(C)) > kQrResidentSmem) C *= 2;
   if (C > w.max_gchunks) C = w.max_gchunks;
   const bool resident = qr_smem<NT>(slice_of(C)) <= kQrResidentSmem;
   const int slice = resident ? slice_of(C) : kQrChunk;
@@ -662,16 +663,36 @@ template <typename K>
 cudaError_t allow_smem(K* kernel, size_t bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
+template <typename K>
+bool allow_wide(K* kernel) {
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 16;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(16);
+  cfg.blockDim = dim3(kQrThreads);
+  cfg.dynamicSmemBytes = kQrResidentSmem;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0;
+}
 
 }  // namespace
 
-cudaError_t panel_qr_init() {
+cudaError_t panel_qr_init(bool* wide) {
   cudaError_t e = allow_smem(panel_qr_kernel<1, true>, kQrResidentSmem);
   if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<1, false>, kQrResidentSmem);
   if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<2, true>, kQrResidentSmem);
   if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<2, false>, kQrResidentSmem);
   if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<4, true>, kQrResidentSmem);
   if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<4, false>, kQrResidentSmem);
+  *wide = allow_wide(panel_qr_kernel<1, true>) && allow_wide(panel_qr_kernel<1, false>) && allow_wide(panel_qr_kernel<2, true>) &&
+              allow_wide(panel_qr_kernel<2, false>) && allow_wide(panel_qr_kernel<4, true>) && allow_wide(panel_qr_kernel<4, false>);
+  cudaGetLastError();
   if (e == cudaSuccess) e = allow_smem(panel_factor_kernel, kFactorSmem);
   if (e == cudaSuccess) e = allow_smem(panel_apply_kernel, kApplySmem);
   return e;

@@ -22,6 +22,7 @@ static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBy
 
 std::mutex g_mu;
 void* g_scratch_addr[kMaxDevices] = {};
+bool g_qr_wide[kMaxDevices] = {};
 
 cudaError_t scratch_of_current_device(int* dev_out, unsigned char** out) {
   int dev = -1;
@@ -32,7 +33,7 @@ cudaError_t scratch_of_current_device(int* dev_out, unsigned char** out) {
   if (!g_scratch_addr[dev]) {
     void* p = nullptr;
     e = cudaGetSymbolAddress(&p, g_static_scratch);   // once per device, with that device current
-    if (e == cudaSuccess) e = agzo::panel_qr_init();
+    if (e == cudaSuccess) e = agzo::panel_qr_init(&g_qr_wide[dev]);
     if (e != cudaSuccess) return e;
     g_scratch_addr[dev] = p;
   }
@@ -118,6 +119,7 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
   ExtractWave w{};
   w.d_layers = d_rec;
   w.l0 = 0; w.l1 = 1;
+  w.qr_wide = g_qr_wide[dev] ? 1 : 0;
   w.max_m = m; w.max_din = d_in; w.max_r = r; w.max_slabs = slabs; w.max_gchunks = (int)gch;
   if (launch_fill_omega(w, seed, s) != cudaSuccess) return AGZO_ERR_CUDA;     // Omega
   if (launch_xt_t(w, s) != cudaSuccess) return AGZO_ERR_CUDA;                 // Y <- H Omega

@@ -17,6 +17,7 @@ struct TcState {
   void* encode_fn = nullptr;   // cuTensorMapEncodeTiled, resolved through the runtime
   int device = -1;
   bool available = false;
+  bool qr_wide = false;        // panel_qr_init
   FusedCaps fused;
 };
 
