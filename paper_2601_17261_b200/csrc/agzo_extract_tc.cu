@@ -121,6 +121,18 @@ __global__ void __launch_bounds__(tc_threads(MB)) tc_x_q_kernel(const DevLayer* 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
+  const uint32_t step_tx = nblk * 2 * kTileBytes + b_bytes;
+  // With one row block per CTA the ring's first tiles of X are on their way before the panel that the predecessor writes
+  // is waited for (a step of small shapes through forward hooks, 613 tokens, r = 8: 1124 -> 1081 us).  With two the same
+  // was slower (eight 8B blocks, r = 64: 11.86 -> 12.07 ms at best).
+  const int pre = MB == 1 ? min(stages, nk) : 0;
+  if (MB == 1 && threadIdx.x == 0) {
+    tmap_acquire(map_x);
+    for (int k = 0; k < pre; ++k) {
+      mbar_expect_tx(&sh.full[k], step_tx);
+      for (int x = 0; x < 2 * nblk; ++x) tma_load_2d(tiles + (size_t)k * stage_bytes + x * kTileBytes, map_x, (kb + k) * kBoxK, t0 + 64 * x, &sh.full[k]);
+    }
+  }
   chain_wait();
   const bool early = short_launch();
   if (early) chain_next();
@@ -136,7 +148,10 @@ __global__ void __launch_bounds__(tc_threads(MB)) tc_x_q_kernel(const DevLayer* 
       bool ok = true;
       int issued = 0;            // k-steps whose loads have been issued
       const int group = stages >= 4 ? 2 : 1;
-      for (int k = 0; k < nk && ok; k += group) {
+      for (int k = 0; k < pre; ++k)
+        tma_load_2d(tiles + (size_t)k * stage_bytes + a_bytes, map_q, (kb + k) * kBoxK, 0, &sh.full[k]);
+      issued = pre;
+      for (int k = pre; k < nk && ok; k += group) {
         const int n2 = min(group, nk - k);
         uint8_t* a[2];
         uint64_t* bar[2];
@@ -145,7 +160,7 @@ __global__ void __launch_bounds__(tc_threads(MB)) tc_x_q_kernel(const DevLayer* 
           if (kk >= stages && !mbar_wait(&sh.empty[s], ((kk / stages) - 1) & 1)) { sh.failed = 1; ok = false; break; }
           a[u] = tiles + (size_t)s * stage_bytes;
           bar[u] = &sh.full[s];
-          mbar_expect_tx(bar[u], nblk * 2 * kTileBytes + b_bytes);
+          mbar_expect_tx(bar[u], step_tx);
         }
         if (!ok) break;
         for (int x = 0; x < 2 * nblk; ++x)
@@ -270,6 +285,15 @@ __global__ void __launch_bounds__(tc_threads(MB)) tc_xt_t_kernel(const DevLayer*
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
+  const uint32_t step_tx = nblk * 2 * kTileBytes + b_bytes;
+  const int pre = MB == 1 ? min(stages, nk) : 0;       // as in tc_x_q_kernel
+  if (MB == 1 && threadIdx.x == 0) {
+    tmap_acquire(map_x);
+    for (int k = 0; k < pre; ++k) {
+      mbar_expect_tx(&sh.full[k], step_tx);
+      for (int x = 0; x < 2 * nblk; ++x) tma_load_2d(tiles + (size_t)k * stage_bytes + x * kTileBytes, map_x, d0 + 64 * x, t_begin + k * kBoxK, &sh.full[k]);
+    }
+  }
   chain_wait();
   const bool early = short_launch();
   if (early) chain_next();
@@ -278,13 +302,15 @@ __global__ void __launch_bounds__(tc_threads(MB)) tc_xt_t_kernel(const DevLayer*
     if (lane == 0) {
       tmap_acquire(map_x);
       tmap_acquire(map_t);
-      int issued = 0;
-      for (int k = 0; k < nk; ++k) {
+      for (int k = 0; k < pre; ++k)
+        tma_load_2d(tiles + (size_t)k * stage_bytes + a_bytes, map_t, t_begin + k * kBoxK, 0, &sh.full[k]);
+      int issued = pre;
+      for (int k = pre; k < nk; ++k) {
         const int s = k % stages;
         if (k >= stages && !mbar_wait(&sh.empty[s], ((k / stages) - 1) & 1)) { sh.failed = 1; break; }
         uint8_t* a = tiles + (size_t)s * stage_bytes;
         const int tk = t_begin + k * kBoxK;
-        mbar_expect_tx(&sh.full[s], nblk * 2 * kTileBytes + b_bytes);
+        mbar_expect_tx(&sh.full[s], step_tx);
         for (int x = 0; x < 2 * nblk; ++x) tma_load_2d(a + x * kTileBytes, map_x, d0 + 64 * x, tk, &sh.full[s]);
         tma_load_2d(a + a_bytes, map_t, tk, 0, &sh.full[s]);
         issued = k + 1;

@@ -4,10 +4,11 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import agzo_oracle as O
 from paper_2601_17261_b200 import binding as B
 from paper_2601_17261_b200 import workloads as WL
 
-from gpu_helpers import DEV, to_dev
+from gpu_helpers import DEV, projector_distance, to_dev, to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -97,3 +98,32 @@ def test_layer_lists_alternate_without_waiting():
         got.append(Ws + Vs)
     for x, y in zip(*got):
         assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("r,bf16", [(4, False), (5, True), (8, True), (40, True)])
+@pytest.mark.parametrize("m,d_in", [(256, 128), (300, 200), (513, 520), (600, 1160), (2100, 264)])
+def test_activations_written_just_before_the_call(m, d_in, r, bf16):
+    # the products ask for their first tiles of X before they wait for the kernel before them: from one tile in all to
+    # more than any ring holds, in buffers that every call finds rewritten by the work queued right before it
+    src = [to_dev(WL.planted_activations(m, d_in, 16, seed=i, bf16=bf16), bf16)[0] for i in range(4)]
+    got = []
+    for sync in (True, False):
+        X = torch.zeros_like(src[0])
+        Vs = [torch.zeros(r, d_in, device=DEV) for _ in src]
+        ctx = B.agzo_create([B.make_layer(X=X, V=Vs[0], r=r, layer_id=3)], 0)
+        B.agzo_set_option(ctx, "extract_path", 3 if bf16 else 1)
+        torch.cuda.synchronize()
+        for s, V in zip(src, Vs):
+            X.copy_(s)
+            B.agzo_extract_subspace(ctx, [B.make_layer(X=X, V=V, r=r, layer_id=3)], 6, 2)
+            if sync:
+                torch.cuda.synchronize()
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+        B.agzo_destroy(ctx)
+        got.append(Vs)
+    for x, y in zip(*got):
+        assert torch.equal(x, y)
+    for i in (0, 3):
+        Vg = to_host(got[1][i])
+        assert np.abs(Vg.astype(np.float64) @ Vg.T - np.eye(r)).max() <= 1e-5
+        assert projector_distance(Vg, O.extract_subspace(to_host(src[i]), r, 2, 6, 3)) <= 1e-3
