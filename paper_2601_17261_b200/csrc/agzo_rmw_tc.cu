@@ -14,7 +14,7 @@
 // the parts, so the products are exact and summed in fp32; what is dropped is below 2^-17 of
 // each term.
 //
-// Work item = (layer, chunk of 8 or 32 row tiles, group of up to two adjacent column panels).
+// Work item = (layer, chunk of 1 to 8 row tiles, group of up to two adjacent column panels).
 // The R operand of a row tile serves every panel of the group, so R is regenerated once per
 // 128 x (2 * panel width) weights and the CTA streams up to 1 KiB of every weight row.  For
 // ranks above 16 the R operands are not regenerated at all: a fill kernel writes every tile's
@@ -315,15 +315,58 @@ rmw_tc_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ item_
       const Item it = decode_item(layers, item_start, n_layers, item);
       const DevLayer& L = *it.L;
       const int r = L.r, g8 = it.rp >> 3;
-      // B operand: row n = column col0 + n of the panel, K = [Ah | Al]
+      // B operand: row n = column col0 + n of the panel, K = [Ah | Al].  What V's rows hold is on its way before the
+      // last item's chain has let go of the operand.
+      const int b_atom = it.cw * 128;
+      const int ncols = it.np * it.cw;                   // columns of the whole group
+      const bool quads = ((L.d_in | L.ldv) & 3) == 0 && (reinterpret_cast<uintptr_t>(L.V) & 15u) == 0;
+      float4 v4[8];
+      // a unit: four columns, eight rank indices; the eight lanes of a quarter warp take neighbouring columns
+      auto unit_at = [&](int unit, int* g, int* nn) {
+        const int gq = min(4, g8), per = 8 * gq;           // g8 = 2, 4, 6 or 8
+        const int blk = unit / per, in = unit - blk * per, cb = ncols >> 5;
+        const int gb = blk / cb;
+        const int gw = min(gq, g8 - gb * gq);              // groups of this row of blocks (g8 = 6: four, then two)
+        *g = gb * gq + (in >> 3);
+        *nn = 4 * ((blk - gb * cb) * 8 + (in & 7));
+        return (in >> 3) < gw;
+      };
+      const int nblkunits = quads ? ((g8 + 3) >> 2) * min(4, g8) * (ncols >> 2) : 0;
+      auto fetch = [&](int unit) {
+        int g, nn;
+        if (unit >= nblkunits || !unit_at(unit, &g, &nn)) return;
+        const int col = it.col0 + nn;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int k = 8 * g + u;
+          v4[u] = k < r && col < L.d_in ? __ldcg(reinterpret_cast<const float4*>(L.V + (long long)k * L.ldv + col))
+                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      };
+      fetch(gt);
       if (ic > 0) {
         ok = mbar_wait(&sh.b_empty, (ic - 1) & 1);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
       }
-      const int b_atom = it.cw * 128;
-      const int ncols = it.np * it.cw;                   // columns of the whole group
-      for (int unit = gt; unit < ncols * g8; unit += gen_threads) {
+      for (int unit = gt; unit < nblkunits; unit += gen_threads) {
+        int g, nn;
+        const bool mine = unit_at(unit, &g, &nn);
+        if (mine) {
+          const int p = nn / it.cw, n = nn - p * it.cw;
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = c == 0 ? v4[u].x : c == 1 ? v4[u].y : c == 2 ? v4[u].z : v4[u].w;
+            uint4 hi, lo;
+            split8(v, &hi, &lo);
+            put_group(sB + (size_t)p * kBBytes, b_atom, n + c, g, g8, hi, lo);
+          }
+        }
+        fetch(unit + gen_threads);
+      }
+      for (int unit = gt; !quads && unit < ncols * g8; unit += gen_threads) {
         const int g = unit / ncols, nn = unit - g * ncols;
         const int p = nn / it.cw, n = nn - p * it.cw;
         const int col = it.col0 + nn;
@@ -466,7 +509,7 @@ bool rmw_tc_eligible(const agzo_layer& a) {
          (a.ldw * 2) % 16 == 0 && a.d_out >= 1 && a.d_in >= 1 && a.r >= 1 && a.r <= AGZO_MAX_RANK;
 }
 
-void rmw_tc_shape(const agzo_layer& a, int panels, bool staged, DevLayer* D) {
+void rmw_tc_shape(const agzo_layer& a, int panels, bool staged, int halvings, DevLayer* D) {
   const int rp = rtc_rank_padded(a.r);
   const int katoms = rtc_katoms(rp);                     // 1 (rp <= 32) or 2 K atoms of 64
   // panels == 0: one panel per item while R is cheap to regenerate (rp = 16: the pass is
@@ -482,9 +525,15 @@ void rmw_tc_shape(const agzo_layer& a, int panels, bool staged, DevLayer* D) {
   D->rtc_cw = cw;
   D->rtc_np = np;
   D->rtc_panels = (a.d_in + np * cw - 1) / (np * cw);   // panel groups
-  // row tiles per item: the B operand is rebuilt once per item, which stalls the MMA pipeline for a
-  // few microseconds when the rank is large, so those items are taller
-  D->rtc_chunk_blocks = rp >= 32 ? 32 : 8;
+  // Row tiles per item.  The B operand is rebuilt once per item, which the larger it is the longer stalls the
+  // chain; short items keep the CTAs of a row block together on neighbouring columns of W and share the tail out evenly.
+  // Six 8B-shaped blocks, us per pass at 8 / 4 / 2 tiles: r = 8 784 / 745 / 749, r = 16 827 / 769 / 836, r = 24
+  // 834 / 809 / 758, r = 64 819 / 842 / 999 (and 892, 870, 787 and 770 for r = 64, 24, 16 and 8 at 32, 32, 8 and 8 tiles with
+  // the B operand read an element at a time).  Equal contiguous shares of one list of tiles, a CTA walking down its panel
+  // alone, lost 6 to 35 %: neighbouring CTAs then stream different rows.
+  int chunk = rp <= 16 ? 4 : rp <= 32 && np == 1 ? 2 : 8;
+  for (int k = 0; k < halvings && chunk > 1; ++k) chunk /= 2;
+  D->rtc_chunk_blocks = chunk;
   const int nrb = (a.d_out + kRows - 1) / kRows;
   D->rtc_chunks = (nrb + D->rtc_chunk_blocks - 1) / D->rtc_chunk_blocks;
 }
@@ -530,9 +579,10 @@ cudaError_t launch_rmw_tc(const DevLayer* d_layers, const int* d_item_start, int
   const int grid = total_items < sm_count ? total_items : sm_count;
   // operand-builder warps: four keep up with the stream for r <= 8, larger ranks get eight
   const int threads = (kWarpGen0 + (max_r <= 8 ? 4 : kMaxGenWarps)) * 32;
-  // loads in flight per CTA: enough to cover the HBM latency at this SM's share of the
-  // bandwidth (4 to 5 boxes of 16 KiB); more only lengthens the queues in front of the stores
-  if (inflight < 1) inflight = max_r <= 8 ? 4 : 5;
+  // loads in flight per CTA: enough to cover the HBM latency at this SM's share of the bandwidth; more only lengthens the
+  // queues in front of the stores (six 8B-shaped blocks, us per pass with 3 / 4 / 5 / 6: r = 8 797 / 751 / 774 / 772,
+  // r = 16 823 / 748 / 767 / 780, r = 24 886 / 784 / 781 / 796, r = 64 830 / 808 / 856 / 814)
+  if (inflight < 1) inflight = 4;
   if (inflight > slots) inflight = slots;
   return launch_chained(rmw_tc_kernel, dim3(grid), threads, smem, 0, s, d_layers, d_item_start, n_layers, total_items, a_bufs,
                         a_buf_bytes, max_b_bytes, slots, inflight, staged ? 1 : 0, seed, coef, d_coef, d_status);

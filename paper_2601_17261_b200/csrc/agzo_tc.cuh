@@ -39,7 +39,8 @@ bool tc_encode_bf16_2d(const TcState& st, void* out, const void* base, uint64_t 
 
 // ---- tensor-core in-place pass (agzo_rmw_tc.cu)
 bool rmw_tc_eligible(const agzo_layer& a);
-void rmw_tc_shape(const agzo_layer& a, int panels, bool staged, DevLayer* D);   // fills the rtc_* fields except item0 / wmap
+// fills the rtc_* fields except item0 / wmap; halvings: how often the item height chosen by rank is halved
+void rmw_tc_shape(const agzo_layer& a, int panels, bool staged, int halvings, DevLayer* D);
 bool rmw_tc_encode_map(const TcState& st, const DevLayer& D, void* host_map);
 cudaError_t rmw_tc_init();
 // one block that waits on a barrier nothing completes, until the bounded wait gives up (test export)
