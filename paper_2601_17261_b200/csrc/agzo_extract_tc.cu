@@ -373,53 +373,58 @@ __global__ void __launch_bounds__(tc_threads(MB)) tc_xt_t_kernel(const DevLayer*
 
 // ---------------------------------------------------------------- Omega -> Tt (hi/lo), pads zero
 // Tt is [NB][m_pad] with the tokens contiguous, Omega's stream is row-major over (token, k): a
-// thread takes one token and eight consecutive k (at most three Philox blocks), so that for every
-// k a warp writes 32 neighbouring tokens.  Local token t is row row0 + t of the whole batch's
+// thread takes kTok neighbouring tokens and the eight consecutive k of group blockIdx.z, so that for every
+// k a warp writes 32 kTok neighbouring tokens.  Local token t is row row0 + t of the whole batch's
 // test matrix (see fill_omega_kernel).
+// Bound by the instructions of the generator: two tokens a thread make four-byte stores and independent chains, and no division
+// per unit: 196 layers, 8192 tokens, r = 8 49 -> 37 us, 50 layers, 16384 tokens, r = 16 43 -> 32;
+// one where two would leave SMs without work.
+template <int kTok>
 __global__ void __launch_bounds__(256) tc_fill_omega_kernel(const DevLayer* __restrict__ layers, int l0, uint64_t seed,
                                                             long long row0) {
   chain_wait();
   if (short_launch()) chain_next();
   const DevLayer& L = layers[l0 + blockIdx.y];
-  const int r = L.r, NP = L.NP, rows = L.prow_n, groups = (rows + 7) >> 3;
-  __nv_bfloat16* hi_rows = L.Tb + (long long)L.grp_off * L.m_pad;
-  __nv_bfloat16* lo_rows = hi_rows + (long long)NP * L.m_pad;
-  const long long mp = L.m_pad;
-  const long long units = (long long)L.m * groups;
-  for (long long unit = blockIdx.x * 256ll + threadIdx.x; unit < units; unit += (long long)gridDim.x * 256) {
-    const int g = (int)(unit / L.m);
-    const long long t = unit - (long long)g * L.m;
-    const int nv = min(8, r - 8 * g);                 // live k of this group (the rest is padding)
-    float v[8];
+  const int g = (int)blockIdx.z, r = L.r, rows = L.prow_n;
+  const int t0 = (int)(blockIdx.x * 256 + threadIdx.x) * kTok;
+  if (8 * g >= rows || t0 >= L.m) return;
+  const int nv = min(8, r - 8 * g);                 // live k of this group (the rest is padding)
+  float v[kTok][8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = 0.f;
-    if (nv > 0) {
-      const long long e_first = (row0 + t) * r + 8 * g;
-      const long long b0 = e_first >> 2;
-      const int off = (int)(e_first & 3);
-      const int nblk = (off + nv + 3) >> 2;
-      float x[12];
-      const float4 ga = gaussian_block((uint64_t)b0, L.layer_id, kTagOmega, seed);
-      float4 gb = make_float4(0.f, 0.f, 0.f, 0.f), gc = gb;
-      if (nblk > 1) gb = gaussian_block((uint64_t)(b0 + 1), L.layer_id, kTagOmega, seed);
-      if (nblk > 2) gc = gaussian_block((uint64_t)(b0 + 2), L.layer_id, kTagOmega, seed);
-      x[0] = ga.x; x[1] = ga.y; x[2] = ga.z; x[3] = ga.w;
-      x[4] = gb.x; x[5] = gb.y; x[6] = gb.z; x[7] = gb.w;
-      x[8] = gc.x; x[9] = gc.y; x[10] = gc.z; x[11] = gc.w;
+  for (int i = 0; i < kTok; ++i) {
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const float y = off == 0 ? x[u] : off == 1 ? x[u + 1] : off == 2 ? x[u + 2] : x[u + 3];
-        v[u] = u < nv ? y : 0.f;
-      }
-    }
+    for (int u = 0; u < 8; ++u) v[i][u] = 0.f;
+    if (nv <= 0 || t0 + i >= L.m) continue;
+    const long long e_first = (row0 + t0 + i) * r + 8 * g;
+    const uint64_t b0 = (uint64_t)(e_first >> 2);
+    const int off = (int)(e_first & 3);
+    const int nblk = (off + nv + 3) >> 2;           // at most three Philox blocks, two where r is a multiple of four
+    const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 ga = gaussian_block(b0, L.layer_id, kTagOmega, seed);
+    const float4 gb = nblk > 1 ? gaussian_block(b0 + 1, L.layer_id, kTagOmega, seed) : none;
+    const float4 gc = nblk > 2 ? gaussian_block(b0 + 2, L.layer_id, kTagOmega, seed) : none;
+    const float x[12] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w, gc.x, gc.y, gc.z, gc.w};
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      __nv_bfloat16 h, l;
-      split_bf16(v[u], &h, &l);
-      if (8 * g + u < rows) {
-        hi_rows[(long long)(8 * g + u) * mp + t] = h;
-        lo_rows[(long long)(8 * g + u) * mp + t] = l;
-      }
+      const float y = off == 0 ? x[u] : off == 1 ? x[u + 1] : off == 2 ? x[u + 2] : x[u + 3];
+      v[i][u] = u < nv ? y : 0.f;
+    }
+  }
+  __nv_bfloat16* hi_rows = L.Tb + (long long)(L.grp_off + 8 * g) * L.m_pad + t0;
+  __nv_bfloat16* lo_rows = hi_rows + (long long)L.NP * L.m_pad;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    if (8 * g + u >= rows) break;
+    __nv_bfloat16 h[kTok], l[kTok];
+#pragma unroll
+    for (int i = 0; i < kTok; ++i) split_bf16(v[i][u], &h[i], &l[i]);
+    const long long at = (long long)u * L.m_pad;
+    if (kTok == 2) {        // the pitch is a multiple of eight: the second token is inside the row, beyond m a zero
+      *reinterpret_cast<__nv_bfloat162*>(hi_rows + at) = __nv_bfloat162(h[0], h[kTok - 1]);
+      *reinterpret_cast<__nv_bfloat162*>(lo_rows + at) = __nv_bfloat162(l[0], l[kTok - 1]);
+    } else {
+      hi_rows[at] = h[0];
+      lo_rows[at] = l[0];
     }
   }
 }
@@ -577,11 +582,11 @@ bool tc_encode_maps(const TcState& st, const DevLayer& D, void* host_maps) {
 }
 
 cudaError_t tc_fill_omega(const TcState&, const ExtractWave& w, const DevLayer*, uint64_t seed, cudaStream_t s) {
-  const long long units = (long long)w.max_m * ((w.max_r + 14) >> 3);   // a layer's rows, padding rows of its panel included
-  int gx = (int)((units + 255) / 256);
-  if (gx > 1024) gx = 1024;
-  if (gx < 1) gx = 1;
-  return launch_chained(tc_fill_omega_kernel, dim3(gx, w.l1 - w.l0), 256, 0, 0, s, w.d_layers, w.l0, seed, w.omega_row0);
+  const unsigned nl = (unsigned)(w.l1 - w.l0), groups = (unsigned)((w.max_r + 14) >> 3);   // padding rows of a panel included
+  const bool pairs = (long long)w.max_m * groups * nl >= 2ll * 148 * 2048;
+  const unsigned per = pairs ? 512 : 256;
+  return launch_chained(pairs ? tc_fill_omega_kernel<2> : tc_fill_omega_kernel<1>, dim3(((unsigned)w.max_m + per - 1) / per, nl, groups),
+                        256, 0, 0, s, w.d_layers, w.l0, seed, w.omega_row0);
 }
 
 cudaError_t tc_xt_t(const TcState&, const ExtractWave& w, const DevLayer* h_dev, DevStatus* d_status,

@@ -9,8 +9,9 @@ import torch
 
 from oracle import agzo_oracle as O
 from paper_2601_17261_b200 import binding as B
+from paper_2601_17261_b200 import workloads as WL
 
-from gpu_helpers import DEV
+from gpu_helpers import DEV, Ctx, projector_distance, to_dev, to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -26,3 +27,21 @@ def test_normals(seed, layer):
     assert np.sqrt(np.mean(d * d)) <= 2e-7
     assert np.isfinite(got).all()
     B.agzo_destroy(ctx)
+
+
+@pytest.mark.parametrize("m", [301, 75777])
+@pytest.mark.parametrize("r", [3, 61, 64])
+def test_first_product_with_the_test_matrix(m, r):
+    # K = 0 is qr(X^T Omega): one token a thread for the short batch, two (and an odd last token) for the long one
+    d_in = 128
+    X = WL.planted_activations(m, d_in, 16, seed=m, bf16=True)
+    Xd = to_dev(X, True)[0]
+    V = torch.zeros(r, d_in, device=DEV)
+    layers = [B.make_layer(X=Xd, V=V, r=r, layer_id=4)]
+    with Ctx(layers) as ctx:
+        B.agzo_set_option(ctx, "extract_path", 2)
+        B.agzo_extract_subspace(ctx, layers, 9, 0)
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+    Vg = to_host(V)
+    assert np.abs(Vg.astype(np.float64) @ Vg.T - np.eye(r)).max() <= 1e-5
+    assert projector_distance(Vg, O.extract_subspace(X, r, 0, 9, 4)) <= 1e-3
