@@ -993,10 +993,14 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
         return all_tc ? tc_x_q(ctx->tc, w, P.dev.data(), dst, true, ws) : launch_x_q(w, ws);
       };
       auto power_fused = [&]() -> cudaError_t {              // Y <- H (H^T Q) in one pass
-        for (int C = 1; C <= 16; ++C) {
-          if (!(fz_classes & (1u << C))) continue;
+        // a launch per cluster size, the largest clusters first; they touch different layers and run into one another
+        unsigned left = fz_classes;
+        for (int C = 16; C >= 1; --C) {
+          if (!(left & (1u << C))) continue;
+          left &= ~(1u << C);
           Timed t(ctx, AGZO_KC_FUSED_POWER, ws);
-          cudaError_t e = launch_fused_power_step(ctx->tc.fused, w, P.dev.data(), C, dst, ws);
+          const bool follows = (fz_classes >> (C + 1)) != 0;
+          cudaError_t e = launch_fused_power_step(ctx->tc.fused, w, P.dev.data(), C, follows, left != 0, dst, ws);
           if (e != cudaSuccess) return e;
         }
         return cudaSuccess;

@@ -140,10 +140,14 @@ __device__ __forceinline__ uint32_t swz(int i, int j) {
 // kWide: some layer of the launch has 768-column slices (its Q slice takes 12 boxes instead of 8, so ring A
 // has one slot less, and its six Y accumulators need more than 256 TMEM columns) or the cluster has more
 // than 8 CTAs; only the wide instantiations are marked for cluster sizes beyond the portable 8.
+// follows / followed: a power step with several cluster sizes is several launches over different layers.  A followed one
+// lets the next start as soon as what it waits for itself is there, so the next one's clusters take over every SM that
+// falls free, and the next (follows) waits for it only before it ends (196 0.6B-shaped layers, 8192 tokens, r = 8, three
+// sizes: step 4710 -> 4570 us; two waves of 8B or 1.7B shapes with two sizes each: 0 to -1 %).
 template <bool kWide, bool kSmall>
 __global__ void __launch_bounds__(kFzThreads, 1)
 fused_power_step_kernel(const DevLayer* __restrict__ layers, int l0, int l1, int C, int share_base, int share_rem,
-                        DevStatus* status) {
+                        int follows, int followed, DevStatus* status) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   __shared__ FzShared sh;
@@ -183,7 +187,8 @@ fused_power_step_kernel(const DevLayer* __restrict__ layers, int l0, int l1, int
   cluster_sync_all();          // every CTA's barriers exist before anyone arrives on them remotely
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
-  chain_wait();
+  if (!follows) chain_wait();
+  if (followed) chain_next();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -251,7 +256,7 @@ fused_power_step_kernel(const DevLayer* __restrict__ layers, int l0, int l1, int
           }
         }
       }
-      chain_next();            // the last tile is on its way
+      if (!followed) chain_next();            // the last tile is on its way
       if (!ok) sh.failed = 1;
       if (!ok || sh.failed) {
         for (int k = ns > kRingC ? ns - kRingC : 0; k < ns; ++k) mbar_wait(&sh.xc_full[k % kRingC], (k / kRingC) & 1);
@@ -506,10 +511,11 @@ fused_power_step_kernel(const DevLayer* __restrict__ layers, int l0, int l1, int
   __syncthreads();
   if (sh.failed && threadIdx.x == 0) { atomicExch(&status->timeout, 1); atomicExch(&status->where, 4); }
   cluster_sync_all();          // no peer reads my exchange buffer or arrives on my barriers after this
+  if (follows) chain_wait();   // complete no earlier than the launches before: the next kernel waits for this one alone
   if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem, tmem_cols); }
 }
 
-using FzKernel = void (*)(const DevLayer*, int, int, int, int, int, DevStatus*);
+using FzKernel = void (*)(const DevLayer*, int, int, int, int, int, int, int, DevStatus*);
 FzKernel fz_kernel(bool wide, bool small) {
   return wide ? (small ? fused_power_step_kernel<true, true> : fused_power_step_kernel<true, false>)
               : (small ? fused_power_step_kernel<false, true> : fused_power_step_kernel<false, false>);
@@ -657,7 +663,7 @@ void fused_plan_shares(const FusedCaps& caps, DevLayer* dev, int l0, int l1, int
 
 // One fused power step for the layers of the wave whose cluster size is C.
 cudaError_t launch_fused_power_step(const FusedCaps& caps, const ExtractWave& w, const DevLayer* h_dev, int C,
-                                    DevStatus* d_status, cudaStream_t s) {
+                                    bool follows, bool followed, DevStatus* d_status, cudaStream_t s) {
   int total = 0;
   bool wide = C > 8, small = true;
   for (int i = w.l0; i < w.l1; ++i)
@@ -671,7 +677,8 @@ cudaError_t launch_fused_power_step(const FusedCaps& caps, const ExtractWave& w,
   // persistent clusters, never more than can be resident at once; the same count as fused_plan_shares used
   const int nclusters = total < caps.clusters[wide][C] ? total : caps.clusters[wide][C];
   return launch_chained(fz_kernel(wide, small), dim3((unsigned)(nclusters * C)), kFzThreads, fz_smem_bytes(wide, small), C, s,
-                        w.d_layers, w.l0, w.l1, C, total / nclusters, total % nclusters, d_status);
+                        w.d_layers, w.l0, w.l1, C, total / nclusters, total % nclusters, follows ? 1 : 0, followed ? 1 : 0,
+                        d_status);
 }
 
 }  // namespace agzo

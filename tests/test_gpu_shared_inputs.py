@@ -77,3 +77,32 @@ def test_two_blocks_per_cta(ranks):
         Vg = to_host(V)
         assert np.abs(Vg.astype(np.float64) @ Vg.T - np.eye(r)).max() <= 1e-5
         assert projector_distance(Vg, O.extract_subspace(Xs[s], r, 1, 4, i)) <= 1e-3
+
+
+@pytest.mark.parametrize("r", [8, 16])
+@pytest.mark.parametrize("widths", [(1024, 2048), (3072, 1024, 2048, 1024), (8192, 1024, 4096)])
+def test_power_step_of_several_cluster_sizes(widths, r):
+    # one launch per cluster size, running into one another; twice, with and without the device idle between the calls
+    m = 1500
+    Xs = [WL.planted_activations(m, d, 16, seed=i, bf16=True) for i, d in enumerate(widths)]
+    Xd = [to_dev(X, True)[0] for X in Xs]
+    runs = []
+    for sync in (True, False):
+        Vs = [[torch.zeros(r, d, device=DEV) for d in widths] for _ in range(3)]
+        sets = [[B.make_layer(X=x, V=v, r=r, layer_id=i) for i, (x, v) in enumerate(zip(Xd, V))] for V in Vs]
+        with Ctx(sets[0]) as ctx:
+            B.agzo_set_option(ctx, "extract_fused", 2)
+            assert len({c for c in B.agzo_query_fused(ctx, sets[0]) if c > 0}) >= 2
+            for k, layers in enumerate(sets):
+                B.agzo_extract_subspace(ctx, layers, k, 3)
+                if sync:
+                    torch.cuda.synchronize()
+            assert B.agzo_poll(ctx) == B.AGZO_OK
+        runs.append(Vs)
+    for a, b in zip(runs[0], runs[1]):
+        for x, y in zip(a, b):
+            assert torch.equal(x, y)
+    for i, d in enumerate(widths):
+        Vg = to_host(runs[1][2][i])
+        assert np.abs(Vg.astype(np.float64) @ Vg.T - np.eye(r)).max() <= 1e-5, i
+        assert projector_distance(Vg, O.extract_subspace(Xs[i], r, 3, 2, i)) <= 1e-3, i
