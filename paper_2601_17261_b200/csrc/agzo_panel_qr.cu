@@ -178,7 +178,8 @@ __device__ __forceinline__ void qr_load(const DevLayer& L, float* sY, int pitch,
 
 // Diagonal block kb (8 x 8) of the factorisation by one warp, every lane on the whole block in registers: the chain is
 // then four times (rsqrt, multiply, multiply-add) with no exchange between lanes.  D = R_kk^-1 goes to the block of M
-// (zero below the diagonal): lane j takes column j.
+// (zero below the diagonal): lane j takes row j, which goes through the elimination with the block instead of a back
+// substitution after it.
 // A pivot with R_kk <= kRankTol * ||y_k|| (what is left of column k after the columns before it are projected out,
 // against the column's own length) marks a dependent column, which becomes zero.  The test is scale-free per column: the
 // columns of Y = H (H^T Q) carry squared singular values, so a short column is normal and says nothing about dependence.
@@ -188,11 +189,14 @@ __device__ __forceinline__ void qr_factor_block(const double* A, double* M, cons
   constexpr int ap = QrCfg<NT>::ap, mp = QrCfg<NT>::mp;
   const int lane = threadIdx.x & 31, j = lane & 7;
   const int o = kb * kBlk;
-  double a[kBlk][kBlk], rinv[kBlk];          // the upper triangle is used
+  double a[kBlk][kBlk];                      // the upper triangle is used
+  double b[kBlk];                            // e_j under the same elimination: column j of R^-T, which is row j of D
 #pragma unroll
   for (int i = 0; i < kBlk; ++i)
 #pragma unroll
     for (int c = i; c < kBlk; ++c) a[i][c] = A[(o + i) * ap + o + c];
+#pragma unroll
+  for (int i = 0; i < kBlk; ++i) b[i] = i == j ? 1.0 : 0.0;
   bool any_bad = false;
   // two pivots at a time: with d1 = a_kk and det = d1 a_22 - a_12^2 both reciprocal roots start together
   // (1 / R_22 = sqrt(d1) / sqrt(det)); what a subtraction loses in det it loses in a_22 - R_12^2 as well
@@ -210,32 +214,23 @@ __device__ __forceinline__ void qr_factor_block(const double* A, double* M, cons
     if (bad1) i2 = rsqrt(a22);
     if (!live2 || bad2) i2 = 0.0;
     any_bad = any_bad || (live1 && bad1) || (live2 && bad2);
-    rinv[k] = i1;
-    rinv[k + 1] = i2;
 #pragma unroll
     for (int c = k + 1; c < kBlk; ++c) a[k][c] *= i1;
 #pragma unroll
     for (int c = k + 2; c < kBlk; ++c) a[k + 1][c] = (a[k + 1][c] - a[k][k + 1] * a[k][c]) * i2;
+    b[k] *= i1;
+    b[k + 1] = (b[k + 1] - a[k][k + 1] * b[k]) * i2;
 #pragma unroll
-    for (int i = k + 2; i < kBlk; ++i)
+    for (int i = k + 2; i < kBlk; ++i) {
 #pragma unroll
       for (int c = i; c < kBlk; ++c) a[i][c] = (a[i][c] - a[k][i] * a[k][c]) - a[k + 1][i] * a[k + 1][c];
+      b[i] = (b[i] - a[k][i] * b[k]) - a[k + 1][i] * b[k + 1];
+    }
   }
   if (any_bad && report && lane == 0) atomicExch(&status->rank_deficient, 1);
-  // column j of the inverse from the bottom up, the sums kept running
-  double acc[kBlk];
-#pragma unroll
-  for (int i = 0; i < kBlk; ++i) acc[i] = 0.0;
-#pragma unroll
-  for (int i = kBlk - 1; i >= 0; --i) {
-    const double x = i == j ? rinv[i] : (i < j ? -acc[i] * rinv[i] : 0.0);
-    acc[i] = x;
-#pragma unroll
-    for (int l = 0; l < i; ++l) acc[l] += a[l][i] * x;
-  }
   if (lane < kBlk) {
 #pragma unroll
-    for (int i = 0; i < kBlk; ++i) M[(o + i) * mp + o + j] = acc[i];
+    for (int i = 0; i < kBlk; ++i) M[(o + j) * mp + o + i] = b[i];
   }
 }
 
@@ -392,7 +387,14 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
                                                                  int y_reduced, int after_fused, int last, DevStatus* status) {
   static_assert(NT <= 4, "larger ranks take the three launches");
   using Cfg = QrCfg<NT>;
-  const DevLayer& L = layers[l0 + (int)blockIdx.x / C];
+  // the layer's record comes into shared memory before the wait: read in place, each of its lines would cost the chain a
+  // trip to L2 where it is first touched
+  __shared__ __align__(16) unsigned char record[sizeof(DevLayer)];
+  static_assert(sizeof(DevLayer) % 8 == 0, "copied in words of eight bytes");
+  for (int i = threadIdx.x; i < (int)(sizeof(DevLayer) / 8); i += kQrThreads)
+    reinterpret_cast<uint64_t*>(record)[i] = reinterpret_cast<const uint64_t*>(layers + l0 + (int)blockIdx.x / C)[i];
+  __syncthreads();
+  const DevLayer& L = *reinterpret_cast<const DevLayer*>(record);
   const int rank = (int)cluster_ctarank();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   extern __shared__ __align__(16) unsigned char qr_smem[];
