@@ -179,29 +179,30 @@ __device__ __forceinline__ void qr_load(const DevLayer& L, float* sY, int pitch,
 // Diagonal block kb (8 x 8) of the factorisation by one warp, every lane on the whole block in registers: the chain is
 // then four times (rsqrt, multiply, multiply-add) with no exchange between lanes.  D = R_kk^-1 goes to the block of M
 // (zero below the diagonal): lane j takes row j, which goes through the elimination with the block instead of a back
-// substitution after it.
+// substitution after it.  kLive: the columns that can be live, four where no rank of the launch is larger (one 256 x 256 layer, r = 4: step 52 -> 49 us; as a
+// branch between the pivots it cost r = 8 1 % of a step of small layers).
 // A pivot with R_kk <= kRankTol * ||y_k|| (what is left of column k after the columns before it are projected out,
 // against the column's own length) marks a dependent column, which becomes zero.  The test is scale-free per column: the
 // columns of Y = H (H^T Q) carry squared singular values, so a short column is normal and says nothing about dependence.
-template <int NT>
+template <int NT, int kLive = kBlk>
 __device__ __forceinline__ void qr_factor_block(const double* A, double* M, const double* own, int kb, int r, DevStatus* status,
                                                 bool report) {
   constexpr int ap = QrCfg<NT>::ap, mp = QrCfg<NT>::mp;
   const int lane = threadIdx.x & 31, j = lane & 7;
   const int o = kb * kBlk;
-  double a[kBlk][kBlk];                      // the upper triangle is used
-  double b[kBlk];                            // e_j under the same elimination: column j of R^-T, which is row j of D
+  double a[kLive][kLive];                     // the upper triangle is used
+  double b[kLive];                           // e_j under the same elimination: column j of R^-T, which is row j of D
 #pragma unroll
-  for (int i = 0; i < kBlk; ++i)
+  for (int i = 0; i < kLive; ++i)
 #pragma unroll
-    for (int c = i; c < kBlk; ++c) a[i][c] = A[(o + i) * ap + o + c];
+    for (int c = i; c < kLive; ++c) a[i][c] = A[(o + i) * ap + o + c];
 #pragma unroll
-  for (int i = 0; i < kBlk; ++i) b[i] = i == j ? 1.0 : 0.0;
+  for (int i = 0; i < kLive; ++i) b[i] = i == j ? 1.0 : 0.0;
   bool any_bad = false;
   // two pivots at a time: with d1 = a_kk and det = d1 a_22 - a_12^2 both reciprocal roots start together
   // (1 / R_22 = sqrt(d1) / sqrt(det)); what a subtraction loses in det it loses in a_22 - R_12^2 as well
 #pragma unroll
-  for (int k = 0; k < kBlk; k += 2) {
+  for (int k = 0; k < kLive; k += 2) {
     const double d1 = a[k][k], a12 = a[k][k + 1], a22 = a[k + 1][k + 1];
     const double det = fma(d1, a22, -(a12 * a12));
     const double r1 = rsqrt(d1), rd = rsqrt(det);
@@ -215,22 +216,22 @@ __device__ __forceinline__ void qr_factor_block(const double* A, double* M, cons
     if (!live2 || bad2) i2 = 0.0;
     any_bad = any_bad || (live1 && bad1) || (live2 && bad2);
 #pragma unroll
-    for (int c = k + 1; c < kBlk; ++c) a[k][c] *= i1;
+    for (int c = k + 1; c < kLive; ++c) a[k][c] *= i1;
 #pragma unroll
-    for (int c = k + 2; c < kBlk; ++c) a[k + 1][c] = (a[k + 1][c] - a[k][k + 1] * a[k][c]) * i2;
+    for (int c = k + 2; c < kLive; ++c) a[k + 1][c] = (a[k + 1][c] - a[k][k + 1] * a[k][c]) * i2;
     b[k] *= i1;
     b[k + 1] = (b[k + 1] - a[k][k + 1] * b[k]) * i2;
 #pragma unroll
-    for (int i = k + 2; i < kBlk; ++i) {
+    for (int i = k + 2; i < kLive; ++i) {
 #pragma unroll
-      for (int c = i; c < kBlk; ++c) a[i][c] = (a[i][c] - a[k][i] * a[k][c]) - a[k + 1][i] * a[k + 1][c];
+      for (int c = i; c < kLive; ++c) a[i][c] = (a[i][c] - a[k][i] * a[k][c]) - a[k + 1][i] * a[k + 1][c];
       b[i] = (b[i] - a[k][i] * b[k]) - a[k + 1][i] * b[k + 1];
     }
   }
   if (any_bad && report && lane == 0) atomicExch(&status->rank_deficient, 1);
   if (lane < kBlk) {
 #pragma unroll
-    for (int i = 0; i < kBlk; ++i) M[(o + j) * mp + o + i] = b[i];
+    for (int i = 0; i < kBlk; ++i) M[(o + j) * mp + o + i] = i < kLive ? b[i < kLive ? i : 0] : 0.0;
   }
 }
 
@@ -265,7 +266,7 @@ __device__ __forceinline__ void qr_inverse_block(double* A, double* M, int i, in
 // the block row, the trailing update and the off-diagonal blocks of M are tiles on the FP64 tensor cores.  Column kb - 1
 // of M is made by the other warps while warp 0 factors block kb.  Up to 16 columns one warp does it all.  (One thread
 // arrangement over the whole matrix with a barrier per pivot, the form before this one, took 63 us at r = 64; this 15.)
-template <int NT>
+template <int NT, int kLive = kBlk>
 __device__ __forceinline__ void qr_factor(double* A, double* M, const double* own, int r, DevStatus* status, bool report) {
   constexpr int ap = QrCfg<NT>::ap, mp = QrCfg<NT>::mp;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, fr = lane >> 2, fc = lane & 3;
@@ -276,7 +277,7 @@ __device__ __forceinline__ void qr_factor(double* A, double* M, const double* ow
   auto sync = [&]() { if (kOneWarp) __syncwarp(); else __syncthreads(); };
   for (int kb = 0; kb < nb; ++kb) {
     const int o = kb * kBlk;
-    if (warp == 0) qr_factor_block<NT>(A, M, own, kb, r, status, report);
+    if (warp == 0) qr_factor_block<NT, kLive>(A, M, own, kb, r, status, report);
     if (!kOneWarp && warp > 0)
       for (int i = warp - 1; i < kb - 1; i += kQrWarps - 1) qr_inverse_block<NT>(A, M, i, kb - 1);
     sync();
@@ -382,7 +383,7 @@ __device__ __forceinline__ void qr_store(const DevLayer& L, const float* sY, int
 
 // kResident: the CTA's whole slice stays in shared memory from load to apply; otherwise it is staged 128 columns at
 // a time and read a second time (from L.Y, through L2) for the apply.
-template <int NT, bool kResident>
+template <int NT, bool kResident, int kLive = kBlk>
 __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer* __restrict__ layers, int l0, int C, int pitch,
                                                                  int y_reduced, int after_fused, int last, DevStatus* status) {
   static_assert(NT <= 4, "larger ranks take the three launches");
@@ -454,7 +455,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
   }
   __syncthreads();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // done with the peers' shares
-  qr_factor<NT>(A, M, own, r, status, rank == 0);
+  qr_factor<NT, kLive>(A, M, own, r, status, rank == 0);
 
   const bool to_v = last || !L.Qb, to_qb = !last && L.Qb;
   if (kResident) {
@@ -632,7 +633,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_apply_kernel(const DevLay
 template <int NT>
 size_t qr_smem(int slice) { return QrCfg<NT>::fixed + (size_t)QrCfg<NT>::r8 * qr_pitch(slice) * sizeof(float); }
 
-template <int NT>
+template <int NT, int kLive = kBlk>
 cudaError_t launch_qr(const ExtractWave& w, bool last, DevStatus* d_status, cudaStream_t s) {
   const int nl = w.l1 - w.l0;
   auto slice_of = [&](int c) { return (w.max_gchunks + c - 1) / c * kQrChunk; };
@@ -641,8 +642,8 @@ cudaError_t launch_qr(const ExtractWave& w, bool last, DevStatus* d_status, cuda
   if (C > w.max_gchunks) C = w.max_gchunks;
   const bool resident = qr_smem<NT>(slice_of(C)) <= kQrResidentSmem;
   const int slice = resident ? slice_of(C) : kQrChunk;
-  return launch_chained(resident ? panel_qr_kernel<NT, true> : panel_qr_kernel<NT, false>, dim3((unsigned)(C * nl)), kQrThreads,
-                        qr_smem<NT>(slice), C, s, w.d_layers, w.l0, C, qr_pitch(slice), w.y_reduced, w.after_fused, last ? 1 : 0,
+  return launch_chained(resident ? panel_qr_kernel<NT, true, kLive> : panel_qr_kernel<NT, false, kLive>, dim3((unsigned)(C * nl)),
+                        kQrThreads, qr_smem<NT>(slice), C, s, w.d_layers, w.l0, C, qr_pitch(slice), w.y_reduced, w.after_fused, last ? 1 : 0,
                         d_status);
 }
 
@@ -686,14 +687,17 @@ bool allow_wide(K* kernel) {
 }  // namespace
 
 cudaError_t panel_qr_init(bool* wide) {
-  cudaError_t e = allow_smem(panel_qr_kernel<1, true>, kQrResidentSmem);
+  cudaError_t e = allow_smem(panel_qr_kernel<1, true, 4>, kQrResidentSmem);
+  if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<1, false, 4>, kQrResidentSmem);
+  if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<1, true>, kQrResidentSmem);
   if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<1, false>, kQrResidentSmem);
   if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<2, true>, kQrResidentSmem);
   if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<2, false>, kQrResidentSmem);
   if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<4, true>, kQrResidentSmem);
   if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<4, false>, kQrResidentSmem);
-  *wide = allow_wide(panel_qr_kernel<1, true>) && allow_wide(panel_qr_kernel<1, false>) && allow_wide(panel_qr_kernel<2, true>) &&
-              allow_wide(panel_qr_kernel<2, false>) && allow_wide(panel_qr_kernel<4, true>) && allow_wide(panel_qr_kernel<4, false>);
+  *wide = allow_wide(panel_qr_kernel<1, true, 4>) && allow_wide(panel_qr_kernel<1, false, 4>) && allow_wide(panel_qr_kernel<1, true>) &&
+          allow_wide(panel_qr_kernel<1, false>) && allow_wide(panel_qr_kernel<2, true>) &&
+          allow_wide(panel_qr_kernel<2, false>) && allow_wide(panel_qr_kernel<4, true>) && allow_wide(panel_qr_kernel<4, false>);
   cudaGetLastError();
   if (e == cudaSuccess) e = allow_smem(panel_factor_kernel, kFactorSmem);
   if (e == cudaSuccess) e = allow_smem(panel_apply_kernel, kApplySmem);
@@ -709,6 +713,7 @@ size_t panel_gram_bytes(int d_in, int r) {
 }
 
 cudaError_t launch_panel_qr(const ExtractWave& w, bool last, DevStatus* d_status, cudaStream_t s) {
+  if (w.max_r <= 4) return launch_qr<1, 4>(w, last, d_status, s);
   if (w.max_r <= 8) return launch_qr<1>(w, last, d_status, s);
   if (w.max_r <= 16) return launch_qr<2>(w, last, d_status, s);
   if (w.max_r <= 32) return launch_qr<4>(w, last, d_status, s);

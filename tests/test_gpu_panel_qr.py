@@ -45,3 +45,22 @@ def test_slices_in_and_out_of_shared_memory(r, dims):
 @pytest.mark.parametrize("n_layers", [40, 41, 80, 81])
 def test_layers_per_launch(n_layers):
     check(256, [1032, 128, 3080], 12, 1, bf16=True, n_layers=n_layers)
+
+
+@pytest.mark.parametrize("r", [3, 4, 8, 13, 24, 40, 64])
+@pytest.mark.parametrize("power", [-12, -5, 7, 12])
+def test_scaled_inputs_give_the_same_basis(r, power):
+    # every step scales exactly by powers of two (S by 4^n, its roots by 2^n, with two exponents of each parity), so V is
+    # the same bit for bit; the roots see mantissas over the whole of [1, 4)
+    X = WL.planted_activations(300, 264, 16, seed=r, bf16=True)
+    got = []
+    for scale in (1.0, 2.0 ** power):
+        Xd = to_dev(X * np.float32(scale), True)[0]
+        V = torch.zeros(r, 264, device=DEV)
+        layers = [B.make_layer(X=Xd, V=V, r=r, layer_id=2)]
+        with Ctx(layers) as ctx:
+            B.agzo_extract_subspace(ctx, layers, 5, 1)
+            assert B.agzo_poll(ctx) == B.AGZO_OK
+        got.append(V)
+    assert torch.equal(got[0], got[1])
+    assert projector_distance(to_host(got[0]), O.extract_subspace(X, r, 1, 5, 2)) <= 1e-3
