@@ -67,14 +67,15 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
   return v;
 }
 
-// Eight ranks k0 .. k0 + 7 of token t of T out, as bf16 hi and lo parts (Tt is [NB][m_pad], tokens contiguous)
-__device__ __forceinline__ void put_t8(const DevLayer& L, int k0, int t, const float (&v)[8]) {
+// Eight ranks of a token of T out, as bf16 hi and lo parts (Tt is [NB][m_pad], tokens contiguous): `hi` is where the first
+// rank's hi part goes, its lo part follows `lo_off` elements after
+__device__ __forceinline__ void put_t8(__nv_bfloat16* hi, long long lo_off, long long m_pad, const float (&v)[8]) {
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     __nv_bfloat16 h, l;
     split_bf16(v[j], &h, &l);
-    L.Tb[(long long)(k0 + j) * L.m_pad + t] = h;
-    L.Tb[(long long)(L.NP + k0 + j) * L.m_pad + t] = l;
+    hi[j * m_pad] = h;
+    hi[j * m_pad + lo_off] = l;
   }
 }
 
@@ -134,6 +135,7 @@ __global__ void __launch_bounds__(tc_threads(MB)) tc_x_q_kernel(const DevLayer* 
     }
   }
   chain_wait();
+  const long long m_pad = L.m_pad, lo_off = NP * m_pad;
   const bool early = short_launch();
   if (early) chain_next();
 
@@ -203,6 +205,7 @@ __global__ void __launch_bounds__(tc_threads(MB)) tc_x_q_kernel(const DevLayer* 
     if (!early) chain_next();
     if (!ok) sh.failed = 1;
     const int row = q * 32 + lane, t = t0 + 128 * blk + row;
+    __nv_bfloat16* out = L.Tb + t;
     if (ok && blk < nblk) {
       for (int k0 = 0; k0 < NP; k0 += 8) {
         float hi[8], lo[8];
@@ -216,7 +219,7 @@ __global__ void __launch_bounds__(tc_threads(MB)) tc_x_q_kernel(const DevLayer* 
           p[0] = make_float4(hi[0], hi[1], hi[2], hi[3]);
           p[1] = make_float4(hi[4], hi[5], hi[6], hi[7]);
         } else if (t < L.m) {
-          put_t8(L, k0, t, hi);
+          put_t8(out + k0 * m_pad, lo_off, m_pad, hi);
         }
       }
     }
@@ -235,7 +238,7 @@ __global__ void __launch_bounds__(tc_threads(MB)) tc_x_q_kernel(const DevLayer* 
           v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
           v[4] += y.x; v[5] += y.y; v[6] += y.z; v[7] += y.w;
         }
-        put_t8(L, 8 * g, t, v);
+        put_t8(L.Tb + t + 8 * g * m_pad, lo_off, m_pad, v);
       }
     }
     __syncwarp();
