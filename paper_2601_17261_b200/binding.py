@@ -6,6 +6,7 @@ kernels.  There is no fallback: if the shared library is missing, loading raises
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 from typing import List, Optional, Sequence
 
@@ -139,12 +140,13 @@ def _dtype_code(t: torch.Tensor) -> int:
 # the current stream's handle without building a Stream object (a few hundred nanoseconds instead of microseconds: the
 # smallest calls are host-bound); torch versions without it take the public way
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
 
 
 def _stream_ptr(stream) -> int:
     if stream is None:
         if _raw_stream is not None:
-            return _raw_stream(torch.cuda.current_device())
+            return _raw_stream(_current_device())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
@@ -408,14 +410,36 @@ def torch_allreduce(group=None):
     return fn
 
 
+_dense_call = None
+
+
+def _perturb_dense():
+    """The library's agzo_perturb_dense: through _agzo_calls.so (4.5 -> 3.3 us of host time a call), through ctypes for an
+    interpreter that it was not built for."""
+    global _dense_call
+    if _dense_call is None:
+        fn = lib().agzo_perturb_dense
+        try:
+            spec = importlib.util.spec_from_file_location("_agzo_calls", os.path.join(os.path.dirname(LIB_PATH), "_agzo_calls.so"))
+            calls = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(calls)
+            calls.bind(C.cast(fn, C.c_void_p).value)
+            fn = calls.perturb_dense
+        except ImportError:
+            pass
+        _dense_call = fn
+    return _dense_call
+
+
 def agzo_perturb_dense(ctx: Context, w: torch.Tensor, seed: int, layer_id: int, scale: float,
                        d_scale: Optional[torch.Tensor] = None, stream=None) -> None:
     if not w.is_contiguous():
         raise ValueError("w must be contiguous")
-    _check(lib().agzo_perturb_dense(ctx.handle, w.data_ptr(), w.numel(), _dtype_code(w), seed,
-                                    layer_id, scale,
-                                    d_scale.data_ptr() if d_scale is not None else None,
-                                    _stream_ptr(stream)), "agzo_perturb_dense")
+    h = ctx.handle
+    status = _perturb_dense()(h.value or 0 if h is not None else 0, w.data_ptr(), w.numel(), _dtype_code(w), seed, layer_id, scale,
+                              d_scale.data_ptr() if d_scale is not None else 0, _stream_ptr(stream))
+    if status != AGZO_OK:
+        raise AgzoError(status, "agzo_perturb_dense")
 
 
 def agzo_debug_wait_timeout(ctx: Context, stream=None) -> None:

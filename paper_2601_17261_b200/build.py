@@ -1,10 +1,12 @@
-"""Builds libagzo.so (sm_100a) in-tree with nvcc.  `python -m paper_2601_17261_b200.build`."""
+"""Builds libagzo.so (sm_100a) in-tree with nvcc, and _agzo_calls.so, the Python entry to its shortest call, with the C
+compiler.  `python -m paper_2601_17261_b200.build`."""
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -12,6 +14,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libagzo.so")
+CALLS = os.path.join(HERE, "_agzo_calls.so")
 SOURCES = ["agzo_api.cu", "agzo_rmw.cu", "agzo_rmw_tc.cu", "agzo_extract.cu", "agzo_panel_qr.cu", "agzo_extract_tc.cu", "agzo_extract_fused.cu", "agzo_static.cu"]
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
@@ -49,7 +52,7 @@ def build(verbose: bool = False, force: bool = False) -> str:
     def run(cmd):
         p = subprocess.run(cmd, capture_output=True, text=True)
         if p.returncode != 0:
-            raise RuntimeError("nvcc failed: %s\n%s\n%s" % (" ".join(cmd), p.stdout, p.stderr))
+            raise RuntimeError("compiler failed: %s\n%s\n%s" % (" ".join(cmd), p.stdout, p.stderr))
         return p.stderr
 
     with ThreadPoolExecutor(max_workers=4) as ex:
@@ -59,6 +62,10 @@ def build(verbose: bool = False, force: bool = False) -> str:
     if jobs or force or _stale(LIB, objs):
         run([nvcc, "-shared", "-o", LIB] + objs + ["-gencode", "arch=compute_100a,code=sm_100a",
                                                   "-lcudart"])
+    calls = os.path.join(CSRC, "py_calls.c")
+    include = sysconfig.get_paths()["include"]
+    if os.path.exists(os.path.join(include, "Python.h")) and (force or _stale(CALLS, [calls])):
+        run([shutil.which("gcc") or "cc", "-shared", "-fPIC", "-O2", "-I", include, calls, "-o", CALLS])
     return LIB
 
 
