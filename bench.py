@@ -34,11 +34,11 @@ K_POWER = 3
 # DRAM bytes moved per algorithmic byte, from the ncu capture of each kernel on a 4-block
 # slice of the 8B-shaped layer set (summaries under profiles/); traffic grows in proportion
 # to the activation bytes a launch sweeps.  Reset an entry to None when its kernel changes.
-TRAFFIC_PER_ALGORITHMIC_BYTE = {"tc_xt_t_kernel": (4.865880 + 0.011429) / 4.831838,
-                                "fused_power_step_kernel": (3.272938 + 0.009340) / 3.221225}
+TRAFFIC_PER_ALGORITHMIC_BYTE = {"tc_xt_t_kernel": (4.865345 + 0.011024) / 4.831838,
+                                "fused_power_step_kernel": (3.271826 + 0.005665) / 3.221225}
 # Thread-level instructions per weight of the dense-direction kernel (one Philox + Box-Muller normal per weight):
 # ncu smsp__thread_inst_executed.sum / weights on a 4096 x 4096 bf16 layer (profiles/dense_vec_kernel_*.md).
-DENSE_INST_PER_WEIGHT = 933126144 / (4096 * 4096)
+DENSE_INST_PER_WEIGHT = 697737216 / (4096 * 4096)
 EPS = 1e-3
 LR = 1e-6
 METRIC = "agzo_step_overhead_ms"
