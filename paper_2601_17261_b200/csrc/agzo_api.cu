@@ -18,7 +18,6 @@ namespace {
 constexpr uint32_t kMagic = 0xA620B200u;
 constexpr size_t kAlign = 256;
 constexpr size_t kHeaderBytes = 256;          // DevStatus + scalar slots
-constexpr size_t kCoefOffset = 64;            // float coefficient slot inside the header
 constexpr int64_t kDefaultWaveBytes = 8ll << 30;
 constexpr int64_t kL2ResidentWaveBytes = 64ll << 20;   // a wave's X up to this size is still in L2 at its next sweep
 
@@ -535,7 +534,6 @@ int* dev_tiles(agzo_ctx* c, int n) {
 }
 int* dev_items(agzo_ctx* c, int n) { return dev_tiles(c, n) + (n + 1); }
 DevStatus* dev_status(agzo_ctx* c) { return reinterpret_cast<DevStatus*>(c->ws); }
-float* dev_coef(agzo_ctx* c) { return reinterpret_cast<float*>(c->ws + kCoefOffset); }
 
 // Tables of up to 30 KiB (36 layers) travel as the parameters of a kernel that writes them to the workspace: the launch
 // takes its copy, so the host neither waits for an earlier upload nor keeps a buffer, and the stream stays a chain of
@@ -636,8 +634,8 @@ agzo_status check_ctx(agzo_ctx* c) {
   return AGZO_OK;
 }
 
-agzo_status rmw_pass(agzo_ctx* c, const agzo_layer* L, int n, uint64_t seed, float coef,
-                     const float* d_coef, bool pair_update, cudaStream_t s) {
+agzo_status rmw_pass(agzo_ctx* c, const agzo_layer* L, int n, uint64_t seed, PassCoef coef,
+                     bool pair_update, cudaStream_t s) {
   agzo_status st = validate(L, n, NEED_RMW);
   if (st != AGZO_OK) return st;
   if (n == 0) return AGZO_OK;
@@ -650,14 +648,13 @@ agzo_status rmw_pass(agzo_ctx* c, const agzo_layer* L, int n, uint64_t seed, flo
     Timed t(c, AGZO_KC_RMW_TC, s, fill ? 2 : 1);
     CU(c, launch_rmw_tc(dev_layers(c), dev_items(c, n), n, c->plan.total_items, c->plan.max_rp, c->plan.max_r,
                         c->plan.max_b_bytes, c->plan.max_row_tiles, c->plan.staged_r, fill, c->rmw_tc_slots,
-                        c->rmw_tc_inflight, seed, coef, d_coef, dev_status(c), c->sm_count, s));
+                        c->rmw_tc_inflight, seed, coef, dev_status(c), c->sm_count, s));
     if (c->plan.staged_r) { c->rimg_valid = true; c->rimg_seed = seed; c->rimg_stream = s; }
   }
   if (c->plan.total_tiles > 0) {
     Timed t(c, AGZO_KC_RMW, s);
     CU(c, launch_rmw(dev_layers(c), dev_tiles(c, n), n, c->plan.total_tiles, c->plan.tile_rows, c->plan.cc_max_r,
-                     c->plan.fast_mode_mask, c->plan.any_slow, seed, coef, d_coef, pair_update,
-                     c->sm_count, s));
+                     c->plan.fast_mode_mask, c->plan.any_slow, seed, coef, pair_update, c->sm_count, s));
   }
   return AGZO_OK;
 }
@@ -1040,7 +1037,7 @@ agzo_status agzo_perturb(agzo_ctx* ctx, const agzo_layer* h_layers, int n, uint6
                          float scale, void* stream) {
   agzo_status st = check_ctx(ctx);
   if (st != AGZO_OK) return st;
-  return rmw_pass(ctx, h_layers, n, seed, scale, nullptr, false, static_cast<cudaStream_t>(stream));
+  return rmw_pass(ctx, h_layers, n, seed, pass_coef(scale), false, static_cast<cudaStream_t>(stream));
 }
 
 agzo_status agzo_restore(agzo_ctx* ctx, const agzo_layer* h_layers, int n, uint64_t seed,
@@ -1052,7 +1049,7 @@ agzo_status agzo_restore(agzo_ctx* ctx, const agzo_layer* h_layers, int n, uint6
   for (int i = 0; h_layers && i < n; ++i) (h_layers[i].W16 ? any_pair : any_plain) = true;
   if (any_pair && any_plain) return AGZO_ERR_UNSUPPORTED;
   const float c = any_pair ? 0.0f : -scale;
-  return rmw_pass(ctx, h_layers, n, seed, c, nullptr, false, static_cast<cudaStream_t>(stream));
+  return rmw_pass(ctx, h_layers, n, seed, pass_coef(c), false, static_cast<cudaStream_t>(stream));
 }
 
 agzo_status agzo_update(agzo_ctx* ctx, const agzo_layer* h_layers, int n, uint64_t seed, float lr,
@@ -1064,9 +1061,7 @@ agzo_status agzo_update(agzo_ctx* ctx, const agzo_layer* h_layers, int n, uint64
   st = validate(h_layers, n, NEED_RMW);
   if (st != AGZO_OK) return st;
   if (n == 0) return AGZO_OK;
-  ctx->launches += 1;
-  CU(ctx, launch_coef(d_ghat, 0.f, lr, 2, dev_coef(ctx), s));
-  return rmw_pass(ctx, h_layers, n, seed, 0.f, dev_coef(ctx), true, s);
+  return rmw_pass(ctx, h_layers, n, seed, pass_coef(d_ghat, 0.f, lr, 2), true, s);
 }
 
 agzo_status agzo_ghat(agzo_ctx* ctx, const double* d_f_plus, const double* d_f_other, float eps,
@@ -1093,9 +1088,7 @@ agzo_status agzo_restore_update(agzo_ctx* ctx, const agzo_layer* h_layers, int n
   for (int i = 0; i < n; ++i) (h_layers[i].W16 ? any_pair : any_plain) = true;
   if (any_pair && any_plain) return AGZO_ERR_UNSUPPORTED;
   // a pair's master was never perturbed: only the update term applies to it
-  ctx->launches += 1;
-  CU(ctx, launch_coef(d_ghat, eps, lr, any_pair ? 2 : mode, dev_coef(ctx), s));
-  return rmw_pass(ctx, h_layers, n, seed, 0.f, dev_coef(ctx), true, s);
+  return rmw_pass(ctx, h_layers, n, seed, pass_coef(d_ghat, eps, lr, any_pair ? 2 : mode), true, s);
 }
 
 agzo_status agzo_step(agzo_ctx* ctx, const agzo_layer* h_layers, int n, const agzo_params* p,

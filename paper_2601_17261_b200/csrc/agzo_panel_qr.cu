@@ -393,7 +393,8 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
   __shared__ __align__(16) unsigned char record[sizeof(DevLayer)];
   static_assert(sizeof(DevLayer) % 8 == 0, "copied in words of eight bytes");
   for (int i = threadIdx.x; i < (int)(sizeof(DevLayer) / 8); i += kQrThreads)
-    reinterpret_cast<uint64_t*>(record)[i] = reinterpret_cast<const uint64_t*>(layers + l0 + (int)blockIdx.x / C)[i];
+    reinterpret_cast<unsigned long long*>(record)[i] =
+        __ldcg(reinterpret_cast<const unsigned long long*>(layers + l0 + (int)blockIdx.x / C) + i);
   __syncthreads();
   const DevLayer& L = *reinterpret_cast<const DevLayer*>(record);
   const int rank = (int)cluster_ctarank();

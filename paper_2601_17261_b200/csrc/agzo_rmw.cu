@@ -270,14 +270,14 @@ __device__ __forceinline__ int effective_mode(const DevLayer& L, int pair_update
 template <int RC, int MODE>
 __global__ void __launch_bounds__(kRmwThreads, (RC <= 8 ? 2 : 1))
 rmw_reg_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ tile_start,
-               int n_layers, int total_tiles, int tile_rows, uint64_t seed, float coef_imm,
-               const float* __restrict__ d_coef, int pair_update) {
+               int n_layers, int total_tiles, int tile_rows, uint64_t seed, PassCoef coef_of,
+               int pair_update) {
   extern __shared__ __align__(16) float smem[];
   __shared__ DevLayer sL;
   float* sG = smem;
   chain_wait();
   if (total_tiles <= (int)gridDim.x) chain_next();
-  const float coef = d_coef ? __ldcg(d_coef) : coef_imm;
+  const float coef = coef_of.value();
   for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
     const int li = find_layer(tile_start, n_layers, tile);
     __syncthreads();   // previous tile is done with sG and sL
@@ -300,15 +300,15 @@ rmw_reg_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ tile
 template <int MODE>
 __global__ void __launch_bounds__(kRmwThreads, 1)
 rmw_smem_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ tile_start,
-                int n_layers, int total_tiles, int tile_rows, int max_rs, uint64_t seed, float coef_imm,
-                const float* __restrict__ d_coef, int pair_update) {
+                int n_layers, int total_tiles, int tile_rows, int max_rs, uint64_t seed, PassCoef coef_of,
+                int pair_update) {
   extern __shared__ __align__(16) float smem[];
   __shared__ DevLayer sL;
   float* sG = smem;                              // [kTileRows][RS]
   float* sV = smem + kTileRows * max_rs;         // [RS][kTileCols]
   chain_wait();
   if (total_tiles <= (int)gridDim.x) chain_next();
-  const float coef = d_coef ? __ldcg(d_coef) : coef_imm;
+  const float coef = coef_of.value();
   for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
     const int li = find_layer(tile_start, n_layers, tile);
     __syncthreads();
@@ -335,13 +335,13 @@ rmw_smem_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ til
 // the layers the vector kernels cannot take.
 __global__ void __launch_bounds__(kRmwThreads)
 rmw_generic_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ tile_start,
-                   int n_layers, int total_tiles, int tile_rows, uint64_t seed, float coef_imm,
-                   const float* __restrict__ d_coef, int pair_update) {
+                   int n_layers, int total_tiles, int tile_rows, uint64_t seed, PassCoef coef_of,
+                   int pair_update) {
   __shared__ float sG[32 * AGZO_MAX_RANK];
   __shared__ DevLayer sL;
   chain_wait();
   if (total_tiles <= (int)gridDim.x) chain_next();
-  const float coef = d_coef ? __ldcg(d_coef) : coef_imm;
+  const float coef = coef_of.value();
   for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
     const int li = find_layer(tile_start, n_layers, tile);
     __syncthreads();
@@ -383,7 +383,7 @@ rmw_generic_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ 
 
 struct RmwArgs {
   const DevLayer* d_layers; const int* d_tile_start; int n_layers, total_tiles, tile_rows;
-  uint64_t seed; float coef; const float* d_coef; int pair_update; int sm_count;
+  uint64_t seed; PassCoef coef; int pair_update; int sm_count;
 };
 
 // A pass of one tile per CTA may start beside its predecessor.  A longer one may not: CTAs that take their places one by
@@ -397,7 +397,7 @@ static cudaError_t launch_reg(const RmwArgs& a, cudaStream_t s) {
   const int grid = a.total_tiles < a.sm_count * per_sm ? a.total_tiles : a.sm_count * per_sm;
   const size_t smem = (size_t)a.tile_rows * RC * 2 * sizeof(float);
   return launch_kernel(rmw_reg_kernel<RC, MODE>, dim3(grid), kRmwThreads, smem, 0, starts_early(a.total_tiles, grid), s, a.d_layers, a.d_tile_start, a.n_layers,
-                        a.total_tiles, a.tile_rows, a.seed, a.coef, a.d_coef, a.pair_update);
+                        a.total_tiles, a.tile_rows, a.seed, a.coef, a.pair_update);
 }
 
 template <int MODE>
@@ -411,15 +411,14 @@ static cudaError_t launch_mode(const RmwArgs& a, int max_r, cudaStream_t s) {
   const size_t smem = ((size_t)kTileRows * max_rs + (size_t)max_rs * kTileCols) * sizeof(float);
   const int grid = a.total_tiles < a.sm_count ? a.total_tiles : a.sm_count;
   return launch_kernel(rmw_smem_kernel<MODE>, dim3(grid), kRmwThreads, smem, 0, starts_early(a.total_tiles, grid), s, a.d_layers, a.d_tile_start, a.n_layers,
-                        a.total_tiles, a.tile_rows, max_rs, a.seed, a.coef, a.d_coef, a.pair_update);
+                        a.total_tiles, a.tile_rows, max_rs, a.seed, a.coef, a.pair_update);
 }
 
 cudaError_t launch_rmw(const DevLayer* d_layers, const int* d_tile_start, int n_layers,
                        int total_tiles, int tile_rows, int max_r, int fast_mode_mask, bool any_slow,
-                       uint64_t seed, float coef, const float* d_coef, bool pair_update,
-                       int sm_count, cudaStream_t s) {
+                       uint64_t seed, PassCoef coef, bool pair_update, int sm_count, cudaStream_t s) {
   if (total_tiles <= 0) return cudaSuccess;
-  RmwArgs a{d_layers, d_tile_start, n_layers, total_tiles, tile_rows, seed, coef, d_coef, pair_update ? 1 : 0, sm_count};
+  RmwArgs a{d_layers, d_tile_start, n_layers, total_tiles, tile_rows, seed, coef, pair_update ? 1 : 0, sm_count};
   cudaError_t e = cudaSuccess;
   if (pair_update && (fast_mode_mask & (1 << RMW_PAIR_COMPUTE)))
     fast_mode_mask = (fast_mode_mask & ~(1 << RMW_PAIR_COMPUTE)) | (1 << RMW_PAIR_UPDATE);
@@ -430,7 +429,7 @@ cudaError_t launch_rmw(const DevLayer* d_layers, const int* d_tile_start, int n_
   if (e == cudaSuccess && any_slow) {
     const int grid = total_tiles < sm_count * 4 ? total_tiles : sm_count * 4;
     e = launch_kernel(rmw_generic_kernel, dim3(grid), kRmwThreads, 0, 0, starts_early(total_tiles, grid), s, d_layers, d_tile_start, n_layers, total_tiles,
-                       tile_rows, seed, coef, d_coef, pair_update ? 1 : 0);
+                       tile_rows, seed, coef, pair_update ? 1 : 0);
   }
   return e;
 }
@@ -579,16 +578,6 @@ cudaError_t launch_ghat(const double* fp, const double* fo, float eps, int mode,
 }
 
 // kind 0: eps - lr*g   kind 1: -(eps + lr*g)   kind 2: -lr*g
-__global__ void coef_kernel(const float* g, float eps, float lr, int kind, float* out) {
-  chain_wait();
-  chain_next();
-  const double lg = (double)lr * (double)*g;
-  *out = (float)(kind == 0 ? (double)eps - lg : kind == 1 ? -((double)eps + lg) : -lg);
-}
-cudaError_t launch_coef(const float* g, float eps, float lr, int kind, float* d_coef, cudaStream_t s) {
-  return launch_chained(coef_kernel, dim3(1), 1, 0, 0, s, g, eps, lr, kind, d_coef);
-}
-
 // ------------------------------------------------------------------ test exports
 __global__ void debug_philox_kernel(uint64_t seed, uint32_t layer, uint32_t tag, uint64_t first,
                                     uint64_t n, uint32_t* out) {

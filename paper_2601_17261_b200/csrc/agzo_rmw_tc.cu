@@ -173,8 +173,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
 rmw_tc_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ item_start, int n_layers,
               int total_items, int a_bufs, int a_buf_bytes, int b_area_bytes, int slots, int inflight, int staged,
               uint64_t seed,
-              float coef_imm,
-              const float* __restrict__ d_coef, DevStatus* status) {
+              PassCoef coef_of, DevStatus* status) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* sA = base;                                   // a_bufs x a_buf_bytes
@@ -423,7 +422,7 @@ rmw_tc_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ item_
     const int q = warp & 3;            // TMEM lanes 32q .. 32q+31 belong to this warp
     const int h = e >> 2;              // which half of a box's 64 columns
     const int i = q * 32 + lane;       // row inside the tile
-    const float coef = d_coef ? __ldcg(d_coef) : coef_imm;
+    const float coef = coef_of.value();
     uint32_t off[4];                   // this thread's four 16-byte chunks inside any box
 #pragma unroll
     for (int c = 0; c < 4; ++c) off[c] = swz(i, h * 4 + c);
@@ -562,7 +561,7 @@ cudaError_t launch_rmw_tc(const DevLayer* d_layers, const int* d_item_start, int
                           int max_rp, int max_r, int max_b_bytes, int max_row_tiles, bool staged, bool fill,
                           int slots_wanted, int inflight,
                           uint64_t seed,
-                          float coef, const float* d_coef, DevStatus* d_status, int sm_count, cudaStream_t s) {
+                          PassCoef coef, DevStatus* d_status, int sm_count, cudaStream_t s) {
   if (total_items <= 0) return cudaSuccess;
   if (staged && fill) {
     cudaError_t e = launch_chained(rmw_tc_fill_r_kernel, dim3((unsigned)max_row_tiles, (unsigned)n_layers), 256, 0, 0, s, d_layers, seed);
@@ -585,7 +584,7 @@ cudaError_t launch_rmw_tc(const DevLayer* d_layers, const int* d_item_start, int
   if (inflight < 1) inflight = 4;
   if (inflight > slots) inflight = slots;
   return launch_chained(rmw_tc_kernel, dim3(grid), threads, smem, 0, s, d_layers, d_item_start, n_layers, total_items, a_bufs,
-                        a_buf_bytes, max_b_bytes, slots, inflight, staged ? 1 : 0, seed, coef, d_coef, d_status);
+                        a_buf_bytes, max_b_bytes, slots, inflight, staged ? 1 : 0, seed, coef, d_status);
 }
 
 }  // namespace agzo

@@ -54,7 +54,7 @@ int rmw_tc_b_bytes(const DevLayer& D);
 cudaError_t launch_rmw_tc(const DevLayer* d_layers, const int* d_item_start, int n_layers, int total_items,
                           int max_rp, int max_r, int max_b_bytes, int max_row_tiles, bool staged, bool fill,
                           int slots_wanted, int inflight,
-                          uint64_t seed, float coef, const float* d_coef, DevStatus* d_status, int sm_count, cudaStream_t s);
+                          uint64_t seed, PassCoef coef, DevStatus* d_status, int sm_count, cudaStream_t s);
 
 cudaError_t tc_fill_omega(const TcState& st, const ExtractWave& w, const DevLayer* h_dev,
                           uint64_t seed, cudaStream_t s);
