@@ -577,7 +577,6 @@ cudaError_t launch_ghat(const double* fp, const double* fo, float eps, int mode,
   return launch_chained(ghat_kernel, dim3(1), 1, 0, 0, s, fp, fo, eps, mode, g);
 }
 
-// kind 0: eps - lr*g   kind 1: -(eps + lr*g)   kind 2: -lr*g
 // ------------------------------------------------------------------ test exports
 __global__ void debug_philox_kernel(uint64_t seed, uint32_t layer, uint32_t tag, uint64_t first,
                                     uint64_t n, uint32_t* out) {
