@@ -116,6 +116,7 @@ struct agzo_ctx {
   std::vector<cudaEvent_t> events;   // pairs: start, stop
   size_t events_used;
   int64_t launches;
+  unsigned power_steps;    // fused power steps issued so far: the number that tells one from the one before it
 };
 
 namespace {
@@ -749,6 +750,7 @@ agzo_status agzo_create(agzo_ctx** out, int device, void* workspace, size_t work
   c->debug_fail_step_call = 0;
   c->events_used = 0;
   c->launches = 0;
+  c->power_steps = 0;
   cudaError_t e = cudaSetDevice(device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->stage_ev, cudaEventDisableTiming);
@@ -943,6 +945,7 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
       w.omega_row0 = ctx->allreduce ? ctx->token_offset : 0;
       w.y_reduced = ctx->allreduce ? 1 : 0;
       w.qr_wide = ctx->tc.qr_wide ? 1 : 0;
+      w.region = P.wave_region[wv] == 1 ? 1 : 0;
       bool all_tc = ctx->extract_path != 1;
       for (int i = l0; i < l1; ++i) {
         const DevLayer& D = P.dev[i];
@@ -992,12 +995,13 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
       auto power_fused = [&]() -> cudaError_t {              // Y <- H (H^T Q) in one pass
         // a launch per cluster size, the largest clusters first; they touch different layers and run into one another
         unsigned left = fz_classes;
+        const unsigned step = ++ctx->power_steps;
         for (int C = 16; C >= 1; --C) {
           if (!(left & (1u << C))) continue;
           left &= ~(1u << C);
           Timed t(ctx, AGZO_KC_FUSED_POWER, ws);
           const bool follows = (fz_classes >> (C + 1)) != 0;
-          cudaError_t e = launch_fused_power_step(ctx->tc.fused, w, P.dev.data(), C, follows, left != 0, dst, ws);
+          cudaError_t e = launch_fused_power_step(ctx->tc.fused, w, P.dev.data(), C, follows, left != 0, step, dst, ws);
           if (e != cudaSuccess) return e;
         }
         return cudaSuccess;

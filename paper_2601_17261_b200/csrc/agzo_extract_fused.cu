@@ -143,11 +143,14 @@ __device__ __forceinline__ uint32_t swz(int i, int j) {
 // follows / followed: a power step with several cluster sizes is several launches over different layers.  A followed one
 // lets the next start as soon as what it waits for itself is there, so the next one's clusters take over every SM that
 // falls free, and the next (follows) waits for it only before it ends (196 0.6B-shaped layers, 8192 tokens, r = 8, three
-// sizes: step 4710 -> 4570 us; two waves of 8B or 1.7B shapes with two sizes each: 0 to -1 %).
+// sizes: step 4710 -> 4570 us; two waves of 8B or 1.7B shapes with two sizes each: 0 to -1 %).  A follower therefore reads the
+// operand panel Q before any wait of its own.  The first launch, which has waited for the panel QR, publishes the step's number
+// (release) and a follower loads Q only after it has seen that number (acquire, then the proxy fence that its TMA loads need).
+// The number is there by then in practice: a follower starts when every CTA of the first launch has been past its wait.
 template <bool kWide, bool kSmall>
 __global__ void __launch_bounds__(kFzThreads, 1)
 fused_power_step_kernel(const DevLayer* __restrict__ layers, int l0, int l1, int C, int share_base, int share_rem,
-                        int follows, int followed, DevStatus* status) {
+                        int follows, int followed, unsigned* ready, unsigned step, DevStatus* status) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   __shared__ FzShared sh;
@@ -187,7 +190,10 @@ fused_power_step_kernel(const DevLayer* __restrict__ layers, int l0, int l1, int
   cluster_sync_all();          // every CTA's barriers exist before anyone arrives on them remotely
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
-  if (!follows) chain_wait();
+  if (!follows) {
+    chain_wait();
+    if (followed && blockIdx.x == 0 && threadIdx.x == 0) st_release_gpu(ready, step);
+  }
   if (followed) chain_next();
 
   if (warp == 0) {
@@ -195,7 +201,7 @@ fused_power_step_kernel(const DevLayer* __restrict__ layers, int l0, int l1, int
       // ------------------------------------------------ TMA producer, ring A: the first read of X (and the Q slice)
       const uint64_t keep = l2_policy_evict_last();
       int ns = 0, ic = 0;
-      bool ok = true;
+      bool ok = !follows || wait_published(ready, step);
       FzItem it;
       for (FzWalk walk(l0, cluster, share_base, share_rem); ok && walk.next(layers, l1, C, cluster, &it); ++ic) {
         const DevLayer& L = *it.L;
@@ -515,7 +521,7 @@ fused_power_step_kernel(const DevLayer* __restrict__ layers, int l0, int l1, int
   if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem, tmem_cols); }
 }
 
-using FzKernel = void (*)(const DevLayer*, int, int, int, int, int, int, int, DevStatus*);
+using FzKernel = void (*)(const DevLayer*, int, int, int, int, int, int, int, unsigned*, unsigned, DevStatus*);
 FzKernel fz_kernel(bool wide, bool small) {
   return wide ? (small ? fused_power_step_kernel<true, true> : fused_power_step_kernel<true, false>)
               : (small ? fused_power_step_kernel<false, true> : fused_power_step_kernel<false, false>);
@@ -661,9 +667,10 @@ void fused_plan_shares(const FusedCaps& caps, DevLayer* dev, int l0, int l1, int
   }
 }
 
-// One fused power step for the layers of the wave whose cluster size is C.
+// One fused power step for the layers of the wave whose cluster size is C.  step: a number that no other power step of this
+// scratch region had just before.
 cudaError_t launch_fused_power_step(const FusedCaps& caps, const ExtractWave& w, const DevLayer* h_dev, int C,
-                                    bool follows, bool followed, DevStatus* d_status, cudaStream_t s) {
+                                    bool follows, bool followed, unsigned step, DevStatus* d_status, cudaStream_t s) {
   int total = 0;
   bool wide = C > 8, small = true;
   for (int i = w.l0; i < w.l1; ++i)
@@ -678,7 +685,7 @@ cudaError_t launch_fused_power_step(const FusedCaps& caps, const ExtractWave& w,
   const int nclusters = total < caps.clusters[wide][C] ? total : caps.clusters[wide][C];
   return launch_chained(fz_kernel(wide, small), dim3((unsigned)(nclusters * C)), kFzThreads, fz_smem_bytes(wide, small), C, s,
                         w.d_layers, w.l0, w.l1, C, total / nclusters, total % nclusters, follows ? 1 : 0, followed ? 1 : 0,
-                        d_status);
+                        d_status->panel_ready + w.region, step, d_status);
 }
 
 }  // namespace agzo

@@ -385,7 +385,8 @@ __device__ __forceinline__ void qr_store(const DevLayer& L, const float* sY, int
 // a time and read a second time (from L.Y, through L2) for the apply.
 template <int NT, bool kResident, int kLive = kBlk>
 __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer* __restrict__ layers, int l0, int C, int pitch,
-                                                                 int y_reduced, int after_fused, int last, DevStatus* status) {
+                                                                 int y_reduced, int after_fused, int last, unsigned* published,
+                                                                 DevStatus* status) {
   static_assert(NT <= 4, "larger ranks take the three launches");
   using Cfg = QrCfg<NT>;
   // the layer's record comes into shared memory before the wait: read in place, each of its lines would cost the chain a
@@ -413,6 +414,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
 
   chain_wait();
   if (short_launch()) chain_next();
+  if (published && blockIdx.x == 0 && tid == 0) *published = 0u;
   double acc[Cfg::my_tiles][2];
 #pragma unroll
   for (int t = 0; t < Cfg::my_tiles; ++t) acc[t][0] = acc[t][1] = 0.0;
@@ -590,12 +592,14 @@ __global__ void __launch_bounds__(kQrThreads) panel_factor_kernel(const DevLayer
 }
 
 // Q = Y M on 128 columns of a layer
-__global__ void __launch_bounds__(kQrThreads, 2) panel_apply_kernel(const DevLayer* __restrict__ layers, int l0, int last) {
+__global__ void __launch_bounds__(kQrThreads, 2) panel_apply_kernel(const DevLayer* __restrict__ layers, int l0, int last,
+                                                                    unsigned* published) {
   using Cfg = QrCfg<8>;
   const DevLayer& L = layers[l0 + blockIdx.y];
   const int d0 = blockIdx.x * kQrChunk;
   chain_wait();
   if (short_launch()) chain_next();
+  if (published && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *published = 0u;
   if (d0 >= L.d_in) return;
   extern __shared__ __align__(16) unsigned char qr_smem[];
   double* M = reinterpret_cast<double*>(qr_smem);
@@ -626,6 +630,10 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_apply_kernel(const DevLay
   qr_store(L, sY, pitch, d0, kQrChunk, last || !L.Qb, !last && L.Qb);
 }
 
+// The extraction's last round takes back the number of its last power step (DevStatus::panel_ready): a replayed graph gives the
+// same numbers again and must not find its own there from the replay before.
+unsigned* published_at(const ExtractWave& w, bool last, DevStatus* d_status) { return last ? d_status->panel_ready + w.region : nullptr; }
+
 // CTAs per layer: eight, for up to eight layers sixteen, while the launch is a chain of latencies (two 8B-shaped blocks from
 // hooks, one group per launch: 3000 -> 2848 us per iteration with sixteen); with so many layers that eight each would queue for
 // the SMs (two CTAs each), four or two, since every CTA repeats the factorisation (r = 8, d_in = 2048, 196 layers: 44.5 /
@@ -645,7 +653,7 @@ cudaError_t launch_qr(const ExtractWave& w, bool last, DevStatus* d_status, cuda
   const int slice = resident ? slice_of(C) : kQrChunk;
   return launch_chained(resident ? panel_qr_kernel<NT, true, kLive> : panel_qr_kernel<NT, false, kLive>, dim3((unsigned)(C * nl)),
                         kQrThreads, qr_smem<NT>(slice), C, s, w.d_layers, w.l0, C, qr_pitch(slice), w.y_reduced, w.after_fused, last ? 1 : 0,
-                        d_status);
+                        published_at(w, last, d_status), d_status);
 }
 
 constexpr size_t kGramSmem = (size_t)64 * (kQrChunk + 12) * sizeof(float);
@@ -659,7 +667,7 @@ cudaError_t launch_qr_large(const ExtractWave& w, bool last, DevStatus* d_status
   if (e == cudaSuccess) e = launch_chained(panel_factor_kernel, dim3(nl), kQrThreads, kFactorSmem, 0, s, w.d_layers, w.l0, d_status);
   if (e == cudaSuccess)
     e = launch_chained(panel_apply_kernel, dim3((unsigned)w.max_gchunks, nl), kQrThreads, kApplySmem, 0, s, w.d_layers, w.l0,
-                       last ? 1 : 0);
+                       last ? 1 : 0, published_at(w, last, d_status));
   return e;
 }
 

@@ -85,6 +85,22 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
     if (global_ns() - t0 > kWaitCapNs) return false;
   }
 }
+// What the storing thread has observed of earlier kernels' writes is observed by a thread that sees the value (at gpu scope)
+__device__ __forceinline__ void st_release_gpu(unsigned* p, unsigned v) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// Bounded wait for *p == v, then for TMA loads of what was published: false when two seconds have passed
+__device__ __forceinline__ bool wait_published(const unsigned* p, unsigned v) {
+  const unsigned long long t0 = global_ns();
+  for (;;) {
+    unsigned got;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(got) : "l"(p) : "memory");
+    if (got == v) break;
+    if (global_ns() - t0 > kWaitCapNs) return false;
+  }
+  asm volatile("fence.proxy.async.global;" ::: "memory");   // written with ordinary stores, read by the async proxy
+  return true;
+}
 __device__ __forceinline__ void tma_load_2d(void* dst, const void* tmap, int c0, int c1, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"

@@ -78,6 +78,6 @@ int fused_split(const int* tiles, int n, int clusters, int* tile0, int* first, i
 int fused_share_begin(int k, int base, int rem);
 cudaError_t fused_init(int sm_count, FusedCaps* caps);   // asks the current device which cluster sizes fit
 cudaError_t launch_fused_power_step(const FusedCaps& caps, const ExtractWave& w, const DevLayer* h_dev, int C,
-                                    bool follows, bool followed, DevStatus* d_status, cudaStream_t s);
+                                    bool follows, bool followed, unsigned step, DevStatus* d_status, cudaStream_t s);
 
 }  // namespace agzo
