@@ -11,7 +11,7 @@ namespace agzo {
 // ------------------------------------------------------------------ Omega -> T
 // Local token t is row row0 + t of the test matrix of the whole batch: element e of the stream is
 // (row0 + t) * r + k, so the Philox blocks that cover the local rows are walked, whatever row0 is.
-__global__ void fill_omega_kernel(const DevLayer* __restrict__ layers, int l0, uint64_t seed, long long row0) {
+__global__ void fill_omega_kernel(const DevLayer* layers, int l0, uint64_t seed, long long row0) {
   chain_wait();
   if (short_launch()) chain_next();
   const DevLayer& L = layers[l0 + blockIdx.y];

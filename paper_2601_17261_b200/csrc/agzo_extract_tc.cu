@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(tc_threads(MB)) tc_xt_t_kernel(const DevLayer*
 // per unit: 196 layers, 8192 tokens, r = 8 49 -> 37 us, 50 layers, 16384 tokens, r = 16 43 -> 32;
 // one where two would leave SMs without work.
 template <int kTok>
-__global__ void __launch_bounds__(256) tc_fill_omega_kernel(const DevLayer* __restrict__ layers, int l0, uint64_t seed,
+__global__ void __launch_bounds__(256) tc_fill_omega_kernel(const DevLayer* layers, int l0, uint64_t seed,
                                                             long long row0) {
   chain_wait();
   if (short_launch()) chain_next();

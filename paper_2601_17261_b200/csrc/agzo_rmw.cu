@@ -245,7 +245,7 @@ __device__ __forceinline__ int find_layer(const int* tile_start, int n_layers, i
   while (n > 1) {
     const int step = (n + 31) >> 5;
     const int at = lo + lane * step;
-    const unsigned le = __ballot_sync(0xffffffffu, lane * step < n && __ldg(tile_start + at) <= tile);
+    const unsigned le = __ballot_sync(0xffffffffu, lane * step < n && tile_start[at] <= tile);
     const int last = 31 - __clz(le);           // entry `lo` always qualifies
     n = min(step, n - last * step);
     lo += last * step;
@@ -269,7 +269,7 @@ __device__ __forceinline__ int effective_mode(const DevLayer& L, int pair_update
 // skipped (another instance, or the generic kernel, takes them).
 template <int RC, int MODE>
 __global__ void __launch_bounds__(kRmwThreads, (RC <= 8 ? 2 : 1))
-rmw_reg_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ tile_start,
+rmw_reg_kernel(const DevLayer* layers, const int* tile_start,
                int n_layers, int total_tiles, int tile_rows, uint64_t seed, PassCoef coef_of,
                int pair_update) {
   extern __shared__ __align__(16) float smem[];
@@ -299,7 +299,7 @@ rmw_reg_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ tile
 
 template <int MODE>
 __global__ void __launch_bounds__(kRmwThreads, 1)
-rmw_smem_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ tile_start,
+rmw_smem_kernel(const DevLayer* layers, const int* tile_start,
                 int n_layers, int total_tiles, int tile_rows, int max_rs, uint64_t seed, PassCoef coef_of,
                 int pair_update) {
   extern __shared__ __align__(16) float smem[];
@@ -334,7 +334,7 @@ rmw_smem_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ til
 // Any pitch, alignment, storage mode and rank; one block per tile, scalar accesses.  Serves
 // the layers the vector kernels cannot take.
 __global__ void __launch_bounds__(kRmwThreads)
-rmw_generic_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ tile_start,
+rmw_generic_kernel(const DevLayer* layers, const int* tile_start,
                    int n_layers, int total_tiles, int tile_rows, uint64_t seed, PassCoef coef_of,
                    int pair_update) {
   __shared__ float sG[32 * AGZO_MAX_RANK];
@@ -537,7 +537,7 @@ cudaError_t launch_dense(void* w, long long n, int dtype, uint64_t seed, uint32_
 }
 
 // ------------------------------------------------------------------ Gaussian right factor (LOZO comparison)
-__global__ void fill_basis_kernel(const DevLayer* __restrict__ layers, uint64_t seed) {
+__global__ void fill_basis_kernel(const DevLayer* layers, uint64_t seed) {
   chain_wait();
   chain_next();
   const DevLayer& L = layers[blockIdx.y];

@@ -85,7 +85,7 @@ __device__ __forceinline__ int find_layer_of_item(const int* start, int n_layers
   int lo = 0, hi = n_layers - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (__ldg(start + mid) <= item) lo = mid; else hi = mid - 1;
+    if (start[mid] <= item) lo = mid; else hi = mid - 1;
   }
   return lo;
 }
@@ -170,7 +170,7 @@ __device__ __forceinline__ void gen_r_group(const DevLayer& L, long long row, in
 }
 
 __global__ void __launch_bounds__(kMaxThreads, 1)
-rmw_tc_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ item_start, int n_layers,
+rmw_tc_kernel(const DevLayer* layers, const int* item_start, int n_layers,
               int total_items, int a_bufs, int a_buf_bytes, int b_area_bytes, int slots, int inflight, int staged,
               uint64_t seed,
               PassCoef coef_of, DevStatus* status) {
@@ -483,7 +483,7 @@ rmw_tc_kernel(const DevLayer* __restrict__ layers, const int* __restrict__ item_
 // Staged R: CTA = (row tile, layer); writes the tile's split A operand [Rh | Rl] to
 // scratch exactly as rmw_tc_kernel lays it out in shared memory (K atoms of [128 rows][128 bytes],
 // 128-byte swizzle), so the pass can bulk-copy it.
-__global__ void __launch_bounds__(256) rmw_tc_fill_r_kernel(const DevLayer* __restrict__ layers, uint64_t seed) {
+__global__ void __launch_bounds__(256) rmw_tc_fill_r_kernel(const DevLayer* layers, uint64_t seed) {
   chain_wait();
   if (short_launch()) chain_next();
   const DevLayer& L = layers[blockIdx.y];

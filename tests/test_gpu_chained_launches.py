@@ -100,6 +100,45 @@ def test_layer_lists_alternate_without_waiting():
         assert torch.equal(x, y)
 
 
+@pytest.mark.parametrize("fused", [1, 2])
+@pytest.mark.parametrize("r", [5, 8, 24])              # 5: the group of three runs fused as one layer of 15 ranks
+def test_layer_lists_with_descriptors_alternate_without_waiting(r, fused):
+    # lists of equal and of different length whose activations, weights and shapes all differ, on the tensor-core kernels: every
+    # call finds new TMA descriptors and records at the addresses of the previous call's, which its kernels fetch first of all
+    lists = [[(1024, 300)], [(512, 136), (512, 264)], [(1160, 200)], [(264, 128)] * 3, [(2048, 96), (640, 520)], [(768, 1000)]]
+    got = []
+    for sync in (True, False):
+        made, layers = [], []
+        for k, shapes in enumerate(lists):
+            m = 300 + 64 * k
+            Xs = {d: to_dev(WL.planted_activations(m, d, 16, seed=k, bf16=True), True)[0] for d, _ in shapes}     # equal widths share
+            one = []
+            for d_in, d_out in shapes:
+                W, _ = to_dev(WL.gaussian_weights(d_out, d_in, 0.02, seed=len(made), bf16=True), True)
+                V = torch.zeros(r, d_in, device=DEV)
+                one.append(B.make_layer(X=Xs[d_in], W=W, V=V, r=r, layer_id=len(made)))
+                made.append((W, V, Xs[d_in]))
+            layers.append(one)
+        ctx = B.Context(0, max(B.agzo_workspace_bytes(one) for one in layers))
+        B.agzo_set_option(ctx, "extract_path", 2)
+        B.agzo_set_option(ctx, "extract_fused", fused)
+        torch.cuda.synchronize()
+        for seed in range(4):
+            for one in layers:
+                B.agzo_extract_subspace(ctx, one, seed, 1)
+                if sync:
+                    torch.cuda.synchronize()
+            for one in layers:                       # the first kernel of each call is the pass itself
+                B.agzo_perturb(ctx, one, seed, 1e-2)
+                if sync:
+                    torch.cuda.synchronize()
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+        B.agzo_destroy(ctx)
+        got.append([t for W, V, _ in made for t in (W, V)])
+    for x, y in zip(*got):
+        assert torch.equal(x, y)
+
+
 @pytest.mark.parametrize("r,bf16", [(4, False), (5, True), (8, True), (40, True)])
 @pytest.mark.parametrize("m,d_in", [(256, 128), (300, 200), (513, 520), (600, 1160), (2100, 264)])
 def test_activations_written_just_before_the_call(m, d_in, r, bf16):
