@@ -27,6 +27,10 @@
  *     Two pieces of state the library itself carries from call to call are made safe across a
  *     change of stream: the new stream waits for the last upload of the layer tables, and
  *     staged R operand images written on another stream are rewritten instead of reused.
+ *     The last kernel of a call, and the one before a callback, lets nothing start beside it:
+ *     a kernel of the caller that is launched with programmatic stream serialisation starts
+ *     when that one's blocks are done.  Such a kernel executes its grid-dependency wait before
+ *     it relies on what the call wrote, as it would behind any other kernel.
  *   - Every function returns an agzo_status; nothing throws, traps or aborts.  Argument
  *     errors are detected on the host before anything is launched.  Conditions that only
  *     the device can see (a rank-deficient panel, a wait that ran out) are written to a
@@ -343,6 +347,12 @@ agzo_status agzo_debug_philox(agzo_ctx* ctx, uint64_t seed, uint32_t layer_id, u
                               uint64_t first, uint64_t n, uint32_t* d_words, void* stream);
 agzo_status agzo_debug_gaussian(agzo_ctx* ctx, uint64_t seed, uint32_t layer_id, uint32_t tag,
                                 uint64_t first, uint64_t n, float* d_vals, void* stream);
+
+/* Launches, the way a caller's kernel with programmatic stream serialisation would be, a kernel
+ * that copies `bytes` (a multiple of 16, both pointers 16-byte aligned, device memory) from src
+ * to dst BEFORE it waits for the kernel in front of it.                                    */
+agzo_status agzo_debug_early_copy(agzo_ctx* ctx, const void* src, void* dst, uint64_t bytes,
+                                  void* stream);
 
 /* Test export, host only (no context, no device): the fused power step's work split.  Layer i has
  * h_tiles[i] token tiles; the tiles of the n layers form one list that is cut into

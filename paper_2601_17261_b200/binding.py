@@ -34,6 +34,7 @@ EXPORTS = [
     "agzo_perturb_dense", "agzo_debug_philox", "agzo_debug_gaussian", "agzo_read_counters",
     "agzo_extract_subspace_static", "agzo_fill_gaussian_basis", "agzo_set_allreduce",
     "agzo_debug_wait_timeout", "agzo_query_fused", "agzo_query_cluster_capacity", "agzo_debug_fused_split",
+    "agzo_debug_early_copy",
 ]
 KC_RMW, KC_XT_T, KC_X_Q, KC_PANEL_QR, KC_TC_XT_T, KC_TC_X_Q, KC_OMEGA, KC_RMW_TC, KC_FUSED_POWER = 1, 2, 3, 4, 5, 6, 7, 8, 9
 
@@ -98,6 +99,7 @@ def lib() -> C.CDLL:
         "agzo_step": (i32, [vp, LP, i32, C.POINTER(agzo_params), LOSS_FN, vp, vp, vp, vp]),
         "agzo_perturb_dense": (i32, [vp, vp, i64, i32, u64, u32, f32, vp, vp]),
         "agzo_debug_philox": (i32, [vp, u64, u32, u32, u64, u64, vp, vp]),
+        "agzo_debug_early_copy": (i32, [vp, vp, vp, u64, vp]),
         "agzo_debug_gaussian": (i32, [vp, u64, u32, u32, u64, u64, vp, vp]),
         "agzo_read_counters": (i32, [vp, C.POINTER(C.c_double), C.POINTER(i64), C.POINTER(i64)]),
         "agzo_set_allreduce": (i32, [vp, ALLREDUCE_FN, vp, i64]),
@@ -452,6 +454,14 @@ def agzo_debug_philox(ctx: Context, seed: int, layer_id: int, tag: int, first: i
     _check(lib().agzo_debug_philox(ctx.handle, seed, layer_id, tag, first, n, out.data_ptr(),
                                    _stream_ptr(stream)), "agzo_debug_philox")
     return out[:n]
+
+
+def agzo_debug_early_copy(ctx: Context, src: torch.Tensor, dst: torch.Tensor, stream=None) -> None:
+    """src's bytes to dst by a kernel that may start beside the one in front of it and copies before it waits for it."""
+    if not src.is_contiguous() or not dst.is_contiguous() or src.nbytes != dst.nbytes:
+        raise ValueError("src and dst must be contiguous and of one size")
+    _check(lib().agzo_debug_early_copy(ctx.handle, src.data_ptr(), dst.data_ptr(), src.nbytes, _stream_ptr(stream)),
+           "agzo_debug_early_copy")
 
 
 def agzo_debug_gaussian(ctx: Context, seed: int, layer_id: int, tag: int, first: int, n: int,

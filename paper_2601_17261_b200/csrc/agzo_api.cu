@@ -1196,6 +1196,15 @@ agzo_status agzo_debug_gaussian(agzo_ctx* ctx, uint64_t seed, uint32_t layer_id,
   return AGZO_OK;
 }
 
+agzo_status agzo_debug_early_copy(agzo_ctx* ctx, const void* src, void* dst, uint64_t bytes, void* stream) {
+  agzo_status st = check_ctx(ctx);
+  if (st != AGZO_OK) return st;
+  if (bytes > 0 && (!src || !dst)) return AGZO_ERR_INVALID_ARG;
+  if ((bytes & 15u) || !aligned16(src) || !aligned16(dst)) return AGZO_ERR_INVALID_ARG;
+  CU(ctx, launch_debug_early_copy(src, dst, bytes / 16, ctx->sm_count, static_cast<cudaStream_t>(stream)));
+  return AGZO_OK;
+}
+
 agzo_status agzo_debug_fused_split(const int32_t* h_tiles, int n, int clusters, int32_t* h_tile0, int32_t* h_first,
                                    int32_t* h_parts, int32_t* h_share_begin, int32_t* h_shares) {
   if (n < 0 || clusters < 1 || (n > 0 && (!h_tiles || !h_tile0 || !h_first || !h_parts)) || !h_share_begin || !h_shares)

@@ -369,8 +369,7 @@ cudaError_t launch_x_q(const ExtractWave& w, cudaStream_t s) {
 // the ranks before the panel QR reads it
 __global__ void __launch_bounds__(256) sum_slabs_kernel(const DevLayer* __restrict__ layers, int l0, int after_fused) {
   const DevLayer& L = layers[l0 + blockIdx.y];
-  chain_wait();
-  if (short_launch()) chain_next();
+  chain_wait();                          // releases nobody: the caller's all-reduce follows
   const int nparts = y_parts(L, after_fused);
   const long long n = (long long)L.r * L.d_in;
   for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {

@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
   const int d0 = ch0 * kQrChunk;
 
   chain_wait();
-  if (short_launch()) chain_next();
+  if (!last && short_launch()) chain_next();
   if (published && blockIdx.x == 0 && tid == 0) *published = 0u;
   double acc[Cfg::my_tiles][2];
 #pragma unroll
@@ -598,7 +598,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_apply_kernel(const DevLay
   const DevLayer& L = layers[l0 + blockIdx.y];
   const int d0 = blockIdx.x * kQrChunk;
   chain_wait();
-  if (short_launch()) chain_next();
+  if (!last && short_launch()) chain_next();
   if (published && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *published = 0u;
   if (d0 >= L.d_in) return;
   extern __shared__ __align__(16) unsigned char qr_smem[];

@@ -276,7 +276,6 @@ rmw_reg_kernel(const DevLayer* layers, const int* tile_start,
   __shared__ DevLayer sL;
   float* sG = smem;
   chain_wait();
-  if (total_tiles <= (int)gridDim.x) chain_next();
   const float coef = coef_of.value();
   for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
     const int li = find_layer(tile_start, n_layers, tile);
@@ -307,7 +306,6 @@ rmw_smem_kernel(const DevLayer* layers, const int* tile_start,
   float* sG = smem;                              // [kTileRows][RS]
   float* sV = smem + kTileRows * max_rs;         // [RS][kTileCols]
   chain_wait();
-  if (total_tiles <= (int)gridDim.x) chain_next();
   const float coef = coef_of.value();
   for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
     const int li = find_layer(tile_start, n_layers, tile);
@@ -340,7 +338,6 @@ rmw_generic_kernel(const DevLayer* layers, const int* tile_start,
   __shared__ float sG[32 * AGZO_MAX_RANK];
   __shared__ DevLayer sL;
   chain_wait();
-  if (total_tiles <= (int)gridDim.x) chain_next();
   const float coef = coef_of.value();
   for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
     const int li = find_layer(tile_start, n_layers, tile);
@@ -450,7 +447,6 @@ template <typename T>
 __global__ void dense_kernel(T* w, long long n, long long b_first, uint64_t seed, uint32_t layer_id, float scale,
                              const float* d_scale) {
   chain_wait();
-  if (short_launch()) chain_next();
   const float c = d_scale ? scale * __ldcg(d_scale) : scale;
   const long long nb = (n + 3) >> 2;
   for (long long b = b_first + blockIdx.x * (long long)blockDim.x + threadIdx.x; b < nb;
@@ -469,11 +465,10 @@ __global__ void dense_kernel(T* w, long long n, long long b_first, uint64_t seed
 // blocks) per step, one 16-byte load and store for bf16, two for fp32.  A long vector is bound by the
 // arithmetic of one Philox + Box-Muller normal per weight, not by HBM (67 M weights: 142 us with logf, sqrtf and sincospif,
 // 117 now; HBM would allow 41); a short one by its launch, so the first normals are made before the kernel waits for its
-// predecessor, and the next kernel may be there already.
+// predecessor.
 template <typename T>
 __global__ void __launch_bounds__(256) dense_vec_kernel(T* w, long long n8, uint64_t seed, uint32_t layer_id, float scale,
                                                         const float* d_scale) {
-  if (short_launch()) chain_next();
   const long long stride = (long long)gridDim.x * blockDim.x;
   long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   float4 ga = gaussian_block((uint64_t)(2 * g), layer_id, kTagDense, seed);
@@ -506,7 +501,6 @@ __global__ void __launch_bounds__(256) dense_vec_kernel(T* w, long long n8, uint
     ga = gaussian_block((uint64_t)(2 * g), layer_id, kTagDense, seed);
     gb = gaussian_block((uint64_t)(2 * g + 1), layer_id, kTagDense, seed);
   }
-  if (!short_launch()) chain_next();
 }
 
 template <typename T>
@@ -539,7 +533,6 @@ cudaError_t launch_dense(void* w, long long n, int dtype, uint64_t seed, uint32_
 // ------------------------------------------------------------------ Gaussian right factor (LOZO comparison)
 __global__ void fill_basis_kernel(const DevLayer* layers, uint64_t seed) {
   chain_wait();
-  chain_next();
   const DevLayer& L = layers[blockIdx.y];
   const long long n = (long long)L.r * L.d_in;
   const long long nb = (n + 3) >> 2;
@@ -569,7 +562,6 @@ cudaError_t launch_fill_basis(const DevLayer* d_layers, int n_layers, int max_el
 // ------------------------------------------------------------------ scalars (Algorithm 2, step 3)
 __global__ void ghat_kernel(const double* fp, const double* fo, float eps, int mode, float* g) {
   chain_wait();
-  chain_next();
   const double d = *fp - *fo;
   *g = (float)(mode == 0 ? d / (2.0 * (double)eps) : d / (double)eps);
 }
@@ -578,6 +570,16 @@ cudaError_t launch_ghat(const double* fp, const double* fo, float eps, int mode,
 }
 
 // ------------------------------------------------------------------ test exports
+__global__ void debug_early_copy_kernel(const uint4* src, uint4* dst, uint64_t n16) {
+  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n16; i += (uint64_t)gridDim.x * blockDim.x) dst[i] = __ldcg(src + i);
+  chain_wait();
+}
+cudaError_t launch_debug_early_copy(const void* src, void* dst, uint64_t n16, int sm_count, cudaStream_t s) {
+  if (n16 == 0) return cudaSuccess;
+  const uint64_t cap = (uint64_t)sm_count;
+  const unsigned grid = (unsigned)((n16 + 255) / 256 < cap ? (n16 + 255) / 256 : cap);
+  return launch_chained(debug_early_copy_kernel, dim3(grid), 256, 0, 0, s, static_cast<const uint4*>(src), static_cast<uint4*>(dst), n16);
+}
 __global__ void debug_philox_kernel(uint64_t seed, uint32_t layer, uint32_t tag, uint64_t first,
                                     uint64_t n, uint32_t* out) {
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;

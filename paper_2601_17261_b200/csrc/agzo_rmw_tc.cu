@@ -233,7 +233,6 @@ rmw_tc_kernel(const DevLayer* layers, const int* item_start, int n_layers,
           }
         }
       }
-      chain_next();             // the last weights are on their way
       if (!ok) sh.failed = 1;
       if (!ok || sh.failed) {   // leaving early: the copies in flight must land before the CTA goes away
         for (int k = n > slots ? n - slots : 0; k < n; ++k) mbar_wait(&sh.full_w[k % slots], (k / slots) & 1);
