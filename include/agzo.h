@@ -328,7 +328,7 @@ agzo_status agzo_fill_gaussian_basis(agzo_ctx* ctx, const agzo_layer* h_layers, 
  *   (each term rounded up to 256 bytes; slabs = ceil(m / max(256, ceil32(ceil(m/32)))));
  *   for example m = 4096, d_in = 2048, r = 16 fits, m = 16384, d_in = 4096, r = 16 does not.
  *   Larger problems are refused with AGZO_ERR_WORKSPACE and nothing is launched.
- * Uses the CURRENT CUDA device.  The first call on each device looks up the array's device
+ * Uses the CURRENT CUDA device.  The first call in a CUDA context looks up the array's device
  * address (cudaGetSymbolAddress); make that first call before starting any stream capture.
  * All calls on a device share the one array, which keeps the previous call's contents (the
  * call clears what must start clean).  Two calls whose GPU work can overlap -- different

@@ -1,9 +1,10 @@
 // C ABI of the AGZO library: context, host-side validation, workspace planning and the
 // sequencing of Algorithm 1 / Algorithm 2 over the grouped kernels.
+#include <cuda.h>
+
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
-#include <map>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -121,21 +122,23 @@ struct agzo_ctx {
 
 namespace {
 
-// What is asked of a device and set for its kernels is the same for every context: done once per device.
+// What is asked of a device and set for its kernels is the same for every agzo_ctx: done once per CUDA context, since the
+// kernels' limits end with the context (cudaDeviceReset).
 cudaError_t device_init(int device, TcState* tc) {
+  struct Known { unsigned long long id; TcState st; };
   static std::mutex mu;
-  static std::map<int, TcState> known;
+  static Known known[kMaxDevices];
+  const unsigned long long id = current_context_id(device);
   std::lock_guard<std::mutex> lock(mu);
-  auto it = known.find(device);
-  if (it == known.end()) {
-    TcState st;
-    cudaError_t e = panel_qr_init(&st.qr_wide);
-    if (e == cudaSuccess) e = rmw_init();
-    if (e == cudaSuccess) e = tc_init(&st, device);
-    if (e != cudaSuccess) return e;
-    it = known.emplace(device, st).first;
-  }
-  *tc = it->second;
+  Known* k = device < kMaxDevices ? known + device : nullptr;
+  if (k && id != 0 && k->id == id) { *tc = k->st; return cudaSuccess; }
+  TcState st;
+  cudaError_t e = panel_qr_init(&st.qr_wide);
+  if (e == cudaSuccess) e = rmw_init();
+  if (e == cudaSuccess) e = tc_init(&st, device);
+  if (e != cudaSuccess) return e;
+  if (k) { k->id = id; k->st = st; }
+  *tc = st;
   return cudaSuccess;
 }
 
@@ -661,6 +664,29 @@ agzo_status rmw_pass(agzo_ctx* c, const agzo_layer* L, int n, uint64_t seed, Pas
 }
 
 }  // namespace
+
+namespace agzo {
+
+unsigned long long current_context_id(int device) {
+  typedef CUresult (*GetIdFn)(CUcontext, unsigned long long*);
+  static const GetIdFn get_id = [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuCtxGetId", &fn, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      fn = nullptr;
+    }
+    return reinterpret_cast<GetIdFn>(fn);
+  }();
+  unsigned long long id = 0;
+  if (!get_id) return 0;
+  if (get_id(nullptr, &id) == CUDA_SUCCESS) return id;
+  // no context on this thread yet (or one that a reset has ended): the device's primary one
+  if (cudaSetDevice(device) != cudaSuccess || get_id(nullptr, &id) != CUDA_SUCCESS) return 0;
+  return id;
+}
+
+}  // namespace agzo
 
 // =================================================================== C ABI
 extern "C" {

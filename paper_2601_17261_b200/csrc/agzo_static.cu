@@ -14,31 +14,36 @@
 namespace {
 
 constexpr size_t kStaticScratchBytes = 4u << 20;   // 4 MiB, held by every GPU that loads the library
-constexpr int kMaxDevices = 64;
 
 // The name below is a host-side handle for the symbol, not a device address: kernels must be
 // given the address that cudaGetSymbolAddress returns for the current device.
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
 
+// Looked up once per CUDA context: the address and the kernels' limits end with it (cudaDeviceReset).
+struct Scratch {
+  unsigned long long context;
+  void* addr;
+  bool qr_wide;
+};
 std::mutex g_mu;
-void* g_scratch_addr[kMaxDevices] = {};
-bool g_qr_wide[kMaxDevices] = {};
+Scratch g_scratch[agzo::kMaxDevices] = {};
 
-cudaError_t scratch_of_current_device(int* dev_out, unsigned char** out) {
+cudaError_t scratch_of_current_device(Scratch* out) {
   int dev = -1;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  if (dev < 0 || dev >= agzo::kMaxDevices) return cudaErrorInvalidDevice;
+  const unsigned long long id = agzo::current_context_id(dev);
   std::lock_guard<std::mutex> lock(g_mu);
-  if (!g_scratch_addr[dev]) {
-    void* p = nullptr;
-    e = cudaGetSymbolAddress(&p, g_static_scratch);   // once per device, with that device current
-    if (e == cudaSuccess) e = agzo::panel_qr_init(&g_qr_wide[dev]);
+  Scratch& known = g_scratch[dev];
+  if (!known.addr || id == 0 || known.context != id) {
+    Scratch fresh{id, nullptr, false};
+    e = cudaGetSymbolAddress(&fresh.addr, g_static_scratch);   // with that device current
+    if (e == cudaSuccess) e = agzo::panel_qr_init(&fresh.qr_wide);
     if (e != cudaSuccess) return e;
-    g_scratch_addr[dev] = p;
+    known = fresh;
   }
-  *dev_out = dev;
-  *out = static_cast<unsigned char*>(g_scratch_addr[dev]);
+  *out = known;
   return cudaSuccess;
 }
 
@@ -94,11 +99,10 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
     if (need - up256((size_t)slabs * R * D * 4) + up256(n * R * D * 4) <= kStaticScratchBytes) { slab_rows = rows; slabs = (int)n; break; }
   }
 
-  int dev = -1;
-  unsigned char* base = nullptr;
-  if (scratch_of_current_device(&dev, &base) != cudaSuccess) return AGZO_ERR_CUDA;
+  Scratch scratch;
+  if (scratch_of_current_device(&scratch) != cudaSuccess) return AGZO_ERR_CUDA;
 
-  unsigned char* p = base;
+  unsigned char* p = static_cast<unsigned char*>(scratch.addr);
   DevLayer* d_rec = reinterpret_cast<DevLayer*>(p);
   DevStatus* d_status = reinterpret_cast<DevStatus*>(p + 384);
   p += 512;
@@ -119,7 +123,7 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
   ExtractWave w{};
   w.d_layers = d_rec;
   w.l0 = 0; w.l1 = 1;
-  w.qr_wide = g_qr_wide[dev] ? 1 : 0;
+  w.qr_wide = scratch.qr_wide ? 1 : 0;
   w.max_m = m; w.max_din = d_in; w.max_r = r; w.max_slabs = slabs; w.max_gchunks = (int)gch;
   if (launch_fill_omega(w, seed, s) != cudaSuccess) return AGZO_ERR_CUDA;     // Omega
   if (launch_xt_t(w, s) != cudaSuccess) return AGZO_ERR_CUDA;                 // Y <- H Omega
