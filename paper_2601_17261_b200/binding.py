@@ -8,6 +8,7 @@ from __future__ import annotations
 import ctypes as C
 import importlib.util
 import os
+import sysconfig
 from typing import List, Optional, Sequence
 
 import torch
@@ -416,13 +417,14 @@ _dense_call = None
 
 
 def _perturb_dense():
-    """The library's agzo_perturb_dense: through _agzo_calls.so (4.5 -> 3.3 us of host time a call), through ctypes for an
-    interpreter that it was not built for."""
+    """The library's agzo_perturb_dense: through the extension module _agzo_calls (4.5 -> 3.3 us of host time a call), through ctypes
+    for an interpreter that it was not built for (the file's name carries the interpreter's ABI)."""
     global _dense_call
     if _dense_call is None:
         fn = lib().agzo_perturb_dense
         try:
-            spec = importlib.util.spec_from_file_location("_agzo_calls", os.path.join(os.path.dirname(LIB_PATH), "_agzo_calls.so"))
+            path = os.path.join(os.path.dirname(LIB_PATH), "_agzo_calls" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
+            spec = importlib.util.spec_from_file_location("_agzo_calls", path)
             calls = importlib.util.module_from_spec(spec)
             spec.loader.exec_module(calls)
             calls.bind(C.cast(fn, C.c_void_p).value)

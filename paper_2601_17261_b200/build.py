@@ -1,5 +1,5 @@
-"""Builds libagzo.so (sm_100a) in-tree with nvcc, and _agzo_calls.so, the Python entry to its shortest call, with the C
-compiler.  `python -m paper_2601_17261_b200.build`."""
+"""Builds libagzo.so (sm_100a) in-tree with nvcc, and the extension module _agzo_calls, the Python entry to its shortest call,
+with the C compiler for the interpreter that runs this.  `python -m paper_2601_17261_b200.build`."""
 from __future__ import annotations
 
 import os
@@ -14,7 +14,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libagzo.so")
-CALLS = os.path.join(HERE, "_agzo_calls.so")
+CALLS = os.path.join(HERE, "_agzo_calls" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 SOURCES = ["agzo_api.cu", "agzo_rmw.cu", "agzo_rmw_tc.cu", "agzo_extract.cu", "agzo_panel_qr.cu", "agzo_extract_tc.cu", "agzo_extract_fused.cu", "agzo_static.cu"]
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
@@ -64,8 +64,9 @@ def build(verbose: bool = False, force: bool = False) -> str:
                                                   "-lcudart"])
     calls = os.path.join(CSRC, "py_calls.c")
     include = sysconfig.get_paths()["include"]
-    if os.path.exists(os.path.join(include, "Python.h")) and (force or _stale(CALLS, [calls])):
-        run([shutil.which("gcc") or "cc", "-shared", "-fPIC", "-O2", "-I", include, calls, "-o", CALLS])
+    header = os.path.join(ROOT, "include", "agzo.h")
+    if os.path.exists(os.path.join(include, "Python.h")) and (force or _stale(CALLS, [calls, header])):
+        run([shutil.which("gcc") or "cc", "-shared", "-fPIC", "-O2", "-I", include, "-I", os.path.dirname(header), calls, "-o", CALLS])
     return LIB
 
 

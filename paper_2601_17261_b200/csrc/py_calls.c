@@ -7,15 +7,15 @@
 #include <Python.h>
 #include <stdint.h>
 
-typedef int (*perturb_dense_fn)(void* ctx, void* w, int64_t n_elems, int dtype, uint64_t seed, uint32_t layer_id, float scale,
-                                const float* d_scale, void* stream);
-static perturb_dense_fn perturb_dense_at;
+#include "agzo.h"
+
+static __typeof__(&agzo_perturb_dense) perturb_dense_at;      /* the header's signature; the symbol itself is not linked */
 
 static PyObject* bind(PyObject* self, PyObject* address) {
   (void)self;
   void* p = PyLong_AsVoidPtr(address);
   if (p == NULL && PyErr_Occurred()) return NULL;
-  perturb_dense_at = (perturb_dense_fn)p;
+  perturb_dense_at = (__typeof__(perturb_dense_at))p;
   Py_RETURN_NONE;
 }
 
@@ -25,7 +25,7 @@ static PyObject* perturb_dense(PyObject* self, PyObject* const* a, Py_ssize_t n)
     PyErr_SetString(PyExc_TypeError, "perturb_dense takes nine arguments, after bind()");
     return NULL;
   }
-  void* ctx = PyLong_AsVoidPtr(a[0]);
+  agzo_ctx* ctx = (agzo_ctx*)PyLong_AsVoidPtr(a[0]);
   void* w = PyLong_AsVoidPtr(a[1]);
   const int64_t elems = PyLong_AsLongLong(a[2]);
   const int dtype = (int)PyLong_AsLong(a[3]);

@@ -1,5 +1,6 @@
 """agzo_perturb_dense by the compiled entry and by ctypes: the same arguments reach the library."""
 import ctypes as C
+import sysconfig
 
 import pytest
 import torch
@@ -18,6 +19,14 @@ def test_arguments_are_checked_as_before():
         fn(0, 0, 4, 0, 1, 2, 0.5, 0)
     with pytest.raises(ValueError):
         B.agzo_perturb_dense(None, torch.zeros(4, 4).t()[:2], 1, 2, 0.5)
+
+
+def test_only_the_interpreter_it_was_built_for_loads_the_entry(monkeypatch):
+    loaded = B._perturb_dense()
+    assert loaded.__self__.__file__.endswith("_agzo_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
+    monkeypatch.setattr(B, "_dense_call", None)
+    monkeypatch.setattr(sysconfig, "get_config_var", lambda name: ".cpython-399-x86_64-linux-gnu.so")
+    assert B._perturb_dense() is B.lib().agzo_perturb_dense
 
 
 @pytest.mark.gpu
