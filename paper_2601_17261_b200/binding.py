@@ -440,8 +440,11 @@ def agzo_perturb_dense(ctx: Context, w: torch.Tensor, seed: int, layer_id: int, 
     if not w.is_contiguous():
         raise ValueError("w must be contiguous")
     h = ctx.handle
-    status = _perturb_dense()(h.value or 0 if h is not None else 0, w.data_ptr(), w.numel(), _dtype_code(w), seed, layer_id, scale,
-                              d_scale.data_ptr() if d_scale is not None else 0, _stream_ptr(stream))
+    code, g, st = _dtype_code(w), d_scale.data_ptr() if d_scale is not None else 0, _stream_ptr(stream)
+    try:
+        status = _perturb_dense()(h.value or 0 if h is not None else 0, w.data_ptr(), w.numel(), code, seed, layer_id, scale, g, st)
+    except TypeError:          # ctypes objects, and what only ctypes knows how to refuse
+        status = lib().agzo_perturb_dense(h, w.data_ptr(), w.numel(), code, seed, layer_id, scale, g, st)
     if status != AGZO_OK:
         raise AgzoError(status, "agzo_perturb_dense")
 

@@ -1,7 +1,9 @@
 """agzo_perturb_dense by the compiled entry and by ctypes: the same arguments reach the library."""
 import ctypes as C
 import sysconfig
+import types
 
+import numpy as np
 import pytest
 import torch
 
@@ -19,6 +21,20 @@ def test_arguments_are_checked_as_before():
         fn(0, 0, 4, 0, 1, 2, 0.5, 0)
     with pytest.raises(ValueError):
         B.agzo_perturb_dense(None, torch.zeros(4, 4).t()[:2], 1, 2, 0.5)
+
+
+def test_what_ctypes_takes_and_refuses(monkeypatch):
+    ctx, w = types.SimpleNamespace(handle=None), torch.zeros(8)
+    monkeypatch.setattr(B, "_raw_stream", lambda device: 0)
+    monkeypatch.setattr(B, "_current_device", lambda: 0)
+    for seed, layer, scale in ((C.c_uint64(5), C.c_uint32(1), C.c_float(0.5)), (True, 1, np.float32(0.5)), (1 << 70, -1, 1),
+                               (np.int64(5), np.int32(1), 0.5)):
+        with pytest.raises(B.AgzoError) as e:            # they reach the library, which has no context here
+            B.agzo_perturb_dense(ctx, w, seed, layer, scale)
+        assert e.value.status == B.AGZO_ERR_STATE
+    for seed, layer, scale in ((1.5, 1, 0.5), (1, 1.0, 0.5), (1, 1, "x"), (None, 1, 0.5)):
+        with pytest.raises(C.ArgumentError):
+            B.agzo_perturb_dense(ctx, w, seed, layer, scale)
 
 
 def test_only_the_interpreter_it_was_built_for_loads_the_entry(monkeypatch):
