@@ -348,6 +348,12 @@ agzo_status agzo_debug_philox(agzo_ctx* ctx, uint64_t seed, uint32_t layer_id, u
 agzo_status agzo_debug_gaussian(agzo_ctx* ctx, uint64_t seed, uint32_t layer_id, uint32_t tag,
                                 uint64_t first, uint64_t n, float* d_vals, void* stream);
 
+/* The functions that make a normal, for the 24-bit numbers k = first .. first+n-1 <= 2^24 - 1: four
+ * floats each, y = -2 ln((k + 1) 2^-24), sqrt(y), sin(2 pi k 2^-24), cos(2 pi k 2^-24), written to
+ * device memory (d_parts 16-byte aligned).                                                 */
+agzo_status agzo_debug_normal_parts(agzo_ctx* ctx, uint32_t first, uint32_t n, float* d_parts,
+                                    void* stream);
+
 /* Launches, the way a caller's kernel with programmatic stream serialisation would be, a kernel
  * that copies `bytes` (a multiple of 16, both pointers 16-byte aligned, device memory) from src
  * to dst BEFORE it waits for the kernel in front of it.                                    */

@@ -35,7 +35,7 @@ EXPORTS = [
     "agzo_perturb_dense", "agzo_debug_philox", "agzo_debug_gaussian", "agzo_read_counters",
     "agzo_extract_subspace_static", "agzo_fill_gaussian_basis", "agzo_set_allreduce",
     "agzo_debug_wait_timeout", "agzo_query_fused", "agzo_query_cluster_capacity", "agzo_debug_fused_split",
-    "agzo_debug_early_copy",
+    "agzo_debug_early_copy", "agzo_debug_normal_parts",
 ]
 KC_RMW, KC_XT_T, KC_X_Q, KC_PANEL_QR, KC_TC_XT_T, KC_TC_X_Q, KC_OMEGA, KC_RMW_TC, KC_FUSED_POWER = 1, 2, 3, 4, 5, 6, 7, 8, 9
 
@@ -100,6 +100,7 @@ def lib() -> C.CDLL:
         "agzo_step": (i32, [vp, LP, i32, C.POINTER(agzo_params), LOSS_FN, vp, vp, vp, vp]),
         "agzo_perturb_dense": (i32, [vp, vp, i64, i32, u64, u32, f32, vp, vp]),
         "agzo_debug_philox": (i32, [vp, u64, u32, u32, u64, u64, vp, vp]),
+        "agzo_debug_normal_parts": (i32, [vp, u32, u32, vp, vp]),
         "agzo_debug_early_copy": (i32, [vp, vp, vp, u64, vp]),
         "agzo_debug_gaussian": (i32, [vp, u64, u32, u32, u64, u64, vp, vp]),
         "agzo_read_counters": (i32, [vp, C.POINTER(C.c_double), C.POINTER(i64), C.POINTER(i64)]),
@@ -458,6 +459,13 @@ def agzo_debug_philox(ctx: Context, seed: int, layer_id: int, tag: int, first: i
     out = torch.empty(max(n, 1), dtype=torch.int32, device=f"cuda:{ctx.device}")
     _check(lib().agzo_debug_philox(ctx.handle, seed, layer_id, tag, first, n, out.data_ptr(),
                                    _stream_ptr(stream)), "agzo_debug_philox")
+    return out[:n]
+
+
+def agzo_debug_normal_parts(ctx: Context, first: int, n: int, stream=None) -> torch.Tensor:
+    """[n][4]: -2 ln((k + 1) 2^-24), its root, sin and cos of 2 pi k 2^-24 for k = first .. first + n - 1."""
+    out = torch.empty(max(n, 1), 4, dtype=torch.float32, device=f"cuda:{ctx.device}")
+    _check(lib().agzo_debug_normal_parts(ctx.handle, first, n, out.data_ptr(), _stream_ptr(stream)), "agzo_debug_normal_parts")
     return out[:n]
 
 

@@ -1222,6 +1222,15 @@ agzo_status agzo_debug_gaussian(agzo_ctx* ctx, uint64_t seed, uint32_t layer_id,
   return AGZO_OK;
 }
 
+agzo_status agzo_debug_normal_parts(agzo_ctx* ctx, uint32_t first, uint32_t n, float* d_parts, void* stream) {
+  agzo_status st = check_ctx(ctx);
+  if (st != AGZO_OK) return st;
+  if ((n > 0 && !d_parts) || !aligned16(d_parts)) return AGZO_ERR_INVALID_ARG;
+  if (first > (1u << 24) || n > (1u << 24) - first) return AGZO_ERR_INVALID_ARG;
+  CU(ctx, launch_debug_normal_parts(first, n, d_parts, ctx->sm_count, static_cast<cudaStream_t>(stream)));
+  return AGZO_OK;
+}
+
 agzo_status agzo_debug_early_copy(agzo_ctx* ctx, const void* src, void* dst, uint64_t bytes, void* stream) {
   agzo_status st = check_ctx(ctx);
   if (st != AGZO_OK) return st;

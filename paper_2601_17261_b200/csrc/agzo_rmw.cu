@@ -600,6 +600,15 @@ __global__ void debug_gauss_kernel(uint64_t seed, uint32_t layer, uint32_t tag, 
     out[i] = gv[e & 3];
   }
 }
+__global__ void debug_normal_parts_kernel(uint32_t first, uint32_t n, float4* out) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) out[i] = normal_parts(first + i);
+}
+cudaError_t launch_debug_normal_parts(uint32_t first, uint32_t n, float* out, int sm_count, cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
+  const uint32_t cap = (uint32_t)sm_count * 8, want = (n + 255) / 256;
+  debug_normal_parts_kernel<<<want < cap ? want : cap, 256, 0, s>>>(first, n, reinterpret_cast<float4*>(out));
+  return cudaGetLastError();
+}
 cudaError_t launch_debug_philox(uint64_t seed, uint32_t layer, uint32_t tag, uint64_t first,
                                 uint64_t n, uint32_t* out, int sm_count, cudaStream_t s) {
   if (n == 0) return cudaSuccess;

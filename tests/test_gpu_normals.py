@@ -29,6 +29,30 @@ def test_normals(seed, layer):
     B.agzo_destroy(ctx)
 
 
+def test_parts_of_a_normal():
+    """Every argument that the generator can get, against float64: the logarithm within 1.4 x 2^-24 relative, the root of what the
+    logarithm gave within 1.01 x 2^-24 relative (one rounding and the step's own error), sine and cosine within 2^-24."""
+    ctx, chunk, ulp = B.Context(0, 4096), 1 << 22, 2.0 ** -24
+    for first in range(0, 1 << 24, chunk):
+        y, s, sn, cs = B.agzo_debug_normal_parts(ctx, first, chunk).cpu().numpy().T
+        k = np.arange(first, first + chunk, dtype=np.float64)
+        want = -2.0 * np.log1p((k + 1.0 - 2.0 ** 24) * ulp)              # exact argument, accurate next to 1
+        assert (np.abs(y - want) <= 1.4 * ulp * want).all()
+        last = k == (1 << 24) - 1                                        # u = 1: y = 0, and a root that is no more than 1e-10
+        assert (np.abs(s - np.sqrt(y.astype(np.float64))) <= np.where(last, 1e-10, 1.01 * ulp * s)).all()
+        # quarter turns are exact: reduce by them in integers before the float64 functions
+        turn, rest = np.divmod(np.arange(first, first + chunk) + (1 << 21), 1 << 22)
+        x = 2.0 * np.pi * ulp * (rest - (1 << 21))
+        quads = np.stack([np.sin(x), np.cos(x), -np.sin(x), -np.cos(x)])
+        i = np.arange(chunk)
+        assert (np.abs(sn - quads[turn % 4, i]) <= ulp).all()
+        assert (np.abs(cs - quads[(turn + 1) % 4, i]) <= ulp).all()
+    for first, n in ((0, (1 << 24) + 1), (1 << 24, 1), ((1 << 24) + 1, 0)):
+        with pytest.raises(B.AgzoError):
+            B.agzo_debug_normal_parts(ctx, first, n)
+    B.agzo_destroy(ctx)
+
+
 @pytest.mark.parametrize("m", [301, 75777])
 @pytest.mark.parametrize("r", [3, 61, 64])
 def test_first_product_with_the_test_matrix(m, r):
