@@ -221,14 +221,14 @@ bool same_input(const agzo_layer& a, const agzo_layer& b) {
 // panel QR), and the CTAs' pipelines start and drain less often.
 constexpr int kLongSlabColumnBlocks = 1024;   // 128-column blocks over all layers from which slabs are long
 // cc_blocks: 128-column blocks over the call's layers on the CUDA-core path; 0 = the most slabs the layer can get (sizing).
-void slab_shape(const agzo_layer& a, bool tc, bool long_slabs, long long cc_blocks, int* slabs, int* slab_rows) {
+void slab_shape(const agzo_layer& a, bool tc, bool long_slabs, long long cc_blocks, int sm_count, int* slabs, int* slab_rows) {
   int rows;
   if (tc) {
     rows = a.m >= 8192 ? (long_slabs ? (a.m < 16384 ? a.m : 16384) : 2048) : (a.m + 3) / 4;
     rows = (rows + 127) / 128 * 128;      // whole tiles of every tensor-core kernel (64 or 128 tokens)
     if (rows < 256) rows = 256;
   } else if (cc_blocks > 0) {
-    rows = cc_slab_rows(a.m, cc_blocks);
+    rows = cc_slab_rows(a.m, cc_blocks, sm_count);
   } else {
     const int most = (a.m + kCcMinSlabRows - 1) / kCcMinSlabRows;
     *slabs = most < kCcMaxSlabs ? most : kCcMaxSlabs;
@@ -392,7 +392,7 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
   // partial sums of Y that a unit's last product can leave: slabs, or shares of a fused launch
   auto parts_of = [&](const agzo_layer& a, bool tc, bool fused, int ranks) {
     int slabs, slab_rows;
-    slab_shape(a, tc, long_slabs_any, ws ? cc_blocks : 0, &slabs, &slab_rows);
+    slab_shape(a, tc, long_slabs_any, ws ? cc_blocks : 0, opts.sm_count, &slabs, &slab_rows);
     if (!fused) return slabs;
     const int C = ws ? fused_cluster_size(opts.fused_caps, with_ranks(a, ranks), opts.extract_fused == 2) : fused_min_cluster(a);
     return std::max(slabs, fused_parts_bound(a, C));
@@ -463,7 +463,7 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
         for (int g = 0; g < glen; ++g) {
           DevLayer& D = plan->dev[j + g];
           const agzo_layer& a = L[j + g];
-          slab_shape(a, tc, long_slabs_any, cc_blocks, &D.slabs, &D.slab_rows);
+          slab_shape(a, tc, long_slabs_any, cc_blocks, opts.sm_count, &D.slabs, &D.slab_rows);
           D.gchunks = (a.d_in + 127) / 128;
           D.Ypart = ypart + (size_t)off * a.d_in;
           D.ypart_stride = (long long)ranks * a.d_in;
@@ -971,6 +971,7 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
       w.omega_row0 = ctx->allreduce ? ctx->token_offset : 0;
       w.y_reduced = ctx->allreduce ? 1 : 0;
       w.qr_wide = ctx->tc.qr_wide ? 1 : 0;
+      w.sm_count = ctx->sm_count;
       w.region = P.wave_region[wv] == 1 ? 1 : 0;
       bool all_tc = ctx->extract_path != 1;
       for (int i = l0; i < l1; ++i) {

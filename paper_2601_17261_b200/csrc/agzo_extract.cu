@@ -361,7 +361,7 @@ cudaError_t launch_x_q_split(const ExtractWave& w, cudaStream_t s) {
   return launch_chained(kernel, grid, kXThreads, 0, 0, s, w.d_layers, w.l0);
 }
 cudaError_t launch_x_q(const ExtractWave& w, cudaStream_t s) {
-  const bool few = (long long)w.max_m * (w.l1 - w.l0) <= 148ll * kXWarps * kXqTokens;
+  const bool few = (long long)w.max_m * (w.l1 - w.l0) <= (long long)w.sm_count * kXWarps * kXqTokens;
   return few ? launch_x_q_split<2>(w, s) : launch_x_q_split<1>(w, s);
 }
 

@@ -586,7 +586,7 @@ bool tc_encode_maps(const TcState& st, const DevLayer& D, void* host_maps) {
 
 cudaError_t tc_fill_omega(const TcState&, const ExtractWave& w, const DevLayer*, uint64_t seed, cudaStream_t s) {
   const unsigned nl = (unsigned)(w.l1 - w.l0), groups = (unsigned)((w.max_r + 14) >> 3);   // padding rows of a panel included
-  const bool pairs = (long long)w.max_m * groups * nl >= 2ll * 148 * 2048;
+  const bool pairs = (long long)w.max_m * groups * nl >= 2ll * w.sm_count * 2048;
   const unsigned per = pairs ? 512 : 256;
   return launch_chained(pairs ? tc_fill_omega_kernel<2> : tc_fill_omega_kernel<1>, dim3(((unsigned)w.max_m + per - 1) / per, nl, groups),
                         256, 0, 0, s, w.d_layers, w.l0, seed, w.omega_row0);
@@ -595,7 +595,7 @@ cudaError_t tc_fill_omega(const TcState&, const ExtractWave& w, const DevLayer*,
 cudaError_t tc_xt_t(const TcState&, const ExtractWave& w, const DevLayer* h_dev, DevStatus* d_status,
                     bool skip_fused, cudaStream_t s) {
   const ProductShape p = product_shape(w, h_dev, skip_fused, [](const DevLayer& D) { return (long long)D.gchunks * D.slabs; });
-  const int mb = p.max_nb >= kTwoBlockRows && p.tiles >= 2 * 148 * 2 ? 2 : 1;
+  const int mb = p.max_nb >= kTwoBlockRows && p.tiles >= 4 * w.sm_count ? 2 : 1;
   const int stages = stages_for(p.max_nb, mb);
   const dim3 grid((w.max_din + 128 * mb - 1) / (128 * mb), w.max_slabs, w.l1 - w.l0);
   return launch_chained(mb == 1 ? tc_xt_t_kernel<1> : tc_xt_t_kernel<2>, grid, tc_threads(mb), smem_for(p.max_nb, mb, stages), 0, s,
@@ -605,9 +605,9 @@ cudaError_t tc_xt_t(const TcState&, const ExtractWave& w, const DevLayer* h_dev,
 cudaError_t tc_x_q(const TcState&, const ExtractWave& w, const DevLayer* h_dev, DevStatus* d_status,
                    bool skip_fused, cudaStream_t s) {
   const ProductShape p = product_shape(w, h_dev, skip_fused, [](const DevLayer& D) { return (long long)(D.m + 127) / 128; });
-  const int mb = p.max_nb >= kTwoBlockRows && p.tiles >= 2 * 148 * 2 ? 2 : 1;
+  const int mb = p.max_nb >= kTwoBlockRows && p.tiles >= 4 * w.sm_count ? 2 : 1;
   int ck = 1;       // CTAs per token tile: up to two per SM, and at least two k-steps each
-  while (mb == 1 && ck < 8 && p.tiles * ck * 2 <= 296 && p.min_nk >= 4 * ck) ck *= 2;
+  while (mb == 1 && ck < 8 && p.tiles * ck <= w.sm_count && p.min_nk >= 4 * ck) ck *= 2;
   const int stages = stages_for(p.max_nb, mb);
   const dim3 grid((w.max_m + 128 * mb - 1) / (128 * mb) * ck, w.l1 - w.l0);
   return launch_chained(mb == 1 ? tc_x_q_kernel<1> : tc_x_q_kernel<2>, grid, tc_threads(mb), smem_for(p.max_nb, mb, stages),

@@ -24,6 +24,7 @@ struct Scratch {
   unsigned long long context;
   void* addr;
   bool qr_wide;
+  int sm_count;
 };
 std::mutex g_mu;
 Scratch g_scratch[agzo::kMaxDevices] = {};
@@ -37,9 +38,10 @@ cudaError_t scratch_of_current_device(Scratch* out) {
   std::lock_guard<std::mutex> lock(g_mu);
   Scratch& known = g_scratch[dev];
   if (!known.addr || id == 0 || known.context != id) {
-    Scratch fresh{id, nullptr, false};
+    Scratch fresh{id, nullptr, false, 0};
     e = cudaGetSymbolAddress(&fresh.addr, g_static_scratch);   // with that device current
     if (e == cudaSuccess) e = agzo::panel_qr_init(&fresh.qr_wide);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&fresh.sm_count, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     known = fresh;
   }
@@ -94,13 +96,12 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
   const size_t need = 512 + up256(M * R * 4) + up256((size_t)slabs * R * D * 4) + up256(R * D * 4) +
                       up256(gch * R * R * 8) + up256(R * R * 8);
   if (need > kStaticScratchBytes) return AGZO_ERR_WORKSPACE;   // problem too large for the fixed array
-  for (int rows = cc_slab_rows(m, (long long)gch);; rows += 32) {      // ends at 256 tokens per slab at the latest
+  Scratch scratch;
+  if (scratch_of_current_device(&scratch) != cudaSuccess) return AGZO_ERR_CUDA;
+  for (int rows = cc_slab_rows(m, (long long)gch, scratch.sm_count);; rows += 32) {      // ends at 256 tokens per slab at the latest
     const size_t n = ((size_t)m + rows - 1) / rows;
     if (need - up256((size_t)slabs * R * D * 4) + up256(n * R * D * 4) <= kStaticScratchBytes) { slab_rows = rows; slabs = (int)n; break; }
   }
-
-  Scratch scratch;
-  if (scratch_of_current_device(&scratch) != cudaSuccess) return AGZO_ERR_CUDA;
 
   unsigned char* p = static_cast<unsigned char*>(scratch.addr);
   DevLayer* d_rec = reinterpret_cast<DevLayer*>(p);
@@ -123,6 +124,7 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
   ExtractWave w{};
   w.d_layers = d_rec;
   w.l0 = 0; w.l1 = 1;
+  w.sm_count = scratch.sm_count;
   w.qr_wide = scratch.qr_wide ? 1 : 0;
   w.max_m = m; w.max_din = d_in; w.max_r = r; w.max_slabs = slabs; w.max_gchunks = (int)gch;
   if (launch_fill_omega(w, seed, s) != cudaSuccess) return AGZO_ERR_CUDA;     // Omega
