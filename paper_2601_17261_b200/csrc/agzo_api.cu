@@ -389,10 +389,27 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     if (has_x(L[k]))
       (on_tc(L[k]) ? column_blocks : cc_blocks) += (L[k].d_in + 127) / 128;
   const bool long_slabs_any = column_blocks >= kLongSlabColumnBlocks;
+  int extract_max_r = 0;
+  for (int k = 0; k < n; ++k)
+    if (has_x(L[k])) extract_max_r = std::max(extract_max_r, L[k].r);
+  // scratch of a layer that does not depend on its slabs: T, Y and, where the call has a rank whose panel QR uses them, the Gram shares
+  auto layer_need = [&](const agzo_layer& a, bool tc) {
+    return (tc ? 0 : align_up((size_t)a.m * a.r * 4)) + align_up((size_t)a.r * a.d_in * 4) + align_up(panel_gram_bytes(a.d_in, a.r, extract_max_r));
+  };
+  auto ypart_bytes = [&](int parts, int ranks, int d_in) { return align_up((size_t)parts * ranks * (size_t)d_in * 4); };
+  auto slabs_of = [&](const agzo_layer& a, bool tc, int* slabs, int* slab_rows) {
+    slab_shape(a, tc, long_slabs_any, ws ? cc_blocks : 0, opts.sm_count, slabs, slab_rows);
+    // a workspace of less than agzo_workspace_bytes takes fewer slabs on the CUDA-core path, as long as one is left
+    for (int want = *slabs; ws && !tc && want > 1 && ypart_bytes(*slabs, a.r, a.d_in) + layer_need(a, tc) > scratch_cap;) {
+      --want;
+      *slab_rows = ((a.m + want - 1) / want + 31) / 32 * 32;
+      *slabs = (a.m + *slab_rows - 1) / *slab_rows;
+    }
+  };
   // partial sums of Y that a unit's last product can leave: slabs, or shares of a fused launch
   auto parts_of = [&](const agzo_layer& a, bool tc, bool fused, int ranks) {
     int slabs, slab_rows;
-    slab_shape(a, tc, long_slabs_any, ws ? cc_blocks : 0, opts.sm_count, &slabs, &slab_rows);
+    slabs_of(a, tc, &slabs, &slab_rows);
     if (!fused) return slabs;
     const int C = ws ? fused_cluster_size(opts.fused_caps, with_ranks(a, ranks), opts.extract_fused == 2) : fused_min_cluster(a);
     return std::max(slabs, fused_parts_bound(a, C));
@@ -432,13 +449,8 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
         }
       }
       auto unit_need = [&]() {
-        size_t b = align_up((size_t)parts_of(L[j], tc, fused, ranks) * ranks * (size_t)L[j].d_in * 4);      // Ypart
-        for (int g = 0; g < glen; ++g) {
-          const agzo_layer& a = L[j + g];
-          if (!tc) b += align_up((size_t)a.m * a.r * 4);        // T
-          b += align_up((size_t)a.r * a.d_in * 4);              // Y
-          b += align_up(panel_gram_bytes(a.d_in, a.r));         // Gpart
-        }
+        size_t b = ypart_bytes(parts_of(L[j], tc, fused, ranks), ranks, L[j].d_in);
+        for (int g = 0; g < glen; ++g) b += layer_need(L[j + g], tc);
         if (tc) b += tc_panel_bytes(L[j], ranks);
         return b;
       };
@@ -458,18 +470,18 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
       if (ws) {
         char* p = ws + base + (size_t)region * scratch_cap + (used - used_y);
         float* ypart = reinterpret_cast<float*>(p);
-        p += align_up((size_t)parts_of(L[j], tc, fused, ranks) * ranks * (size_t)L[j].d_in * 4);
+        p += ypart_bytes(parts_of(L[j], tc, fused, ranks), ranks, L[j].d_in);
         int off = 0;
         for (int g = 0; g < glen; ++g) {
           DevLayer& D = plan->dev[j + g];
           const agzo_layer& a = L[j + g];
-          slab_shape(a, tc, long_slabs_any, cc_blocks, opts.sm_count, &D.slabs, &D.slab_rows);
+          slabs_of(a, tc, &D.slabs, &D.slab_rows);
           D.gchunks = (a.d_in + 127) / 128;
           D.Ypart = ypart + (size_t)off * a.d_in;
           D.ypart_stride = (long long)ranks * a.d_in;
           off += a.r;
           if (!tc) { D.T = reinterpret_cast<float*>(p); p += align_up((size_t)a.m * a.r * 4); }
-          D.Gpart = reinterpret_cast<double*>(p); p += align_up(panel_gram_bytes(a.d_in, a.r));
+          D.Gpart = reinterpret_cast<double*>(p); p += align_up(panel_gram_bytes(a.d_in, a.r, extract_max_r));
         }
         off = 0;
         for (int g = 0; tc && g < glen; ++g) {

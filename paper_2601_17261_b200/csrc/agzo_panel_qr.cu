@@ -716,7 +716,8 @@ cudaError_t panel_qr_init(bool* wide) {
 int panel_qr_launches(int max_r) { return max_r > 32 ? 3 : 1; }
 
 // Scratch of a layer for the three-launch form, which a wave with a larger rank takes for all its layers
-size_t panel_gram_bytes(int d_in, int r) {
+size_t panel_gram_bytes(int d_in, int r, int max_r) {
+  if (panel_qr_launches(max_r) == 1) return 0;
   const size_t groups = (size_t)((d_in + kGramGroup * kQrChunk - 1) / (kGramGroup * kQrChunk));
   return groups * qr_share_elems(r) * sizeof(double);
 }

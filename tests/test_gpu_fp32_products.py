@@ -33,3 +33,26 @@ def test_cuda_core_extraction(r, m, d_in, bf16, extra):
     for Vg in (to_host(V), to_host(V2)):
         assert np.abs(Vg.astype(np.float64) @ Vg.T - np.eye(r)).max() <= 1e-5
         assert projector_distance(Vg, Vo) <= 1e-4
+
+
+@pytest.mark.parametrize("m,d_in,r,bf16", [(528, 1376, 16, False), (194, 1568, 24, True), (447, 4538, 32, True), (1020, 2720, 5, False),
+                                           (2016, 1500, 40, False), (243, 6272, 2, True)])
+def test_a_workspace_with_room_for_slabs_of_256_tokens_is_enough(m, d_in, r, bf16):
+    # more and shorter slabs are taken where the workspace has room for them; what must fit is slabs of at least 256 tokens
+    up = lambda x: (x + 255) // 256 * 256
+    slabs = -(-m // max(256, -(-(-(-m // 32)) // 32) * 32))
+    need = up(4 * m * r) + up(4 * slabs * r * d_in) + up(4 * r * d_in) + up(8 * -(-d_in // 128) * r * r) + up(8 * r * r)
+    X = WL.planted_activations(m, d_in, 16, seed=m, bf16=bf16)
+    Xd = to_dev(X, bf16)[0]
+    V = torch.zeros(r, d_in, device=DEV)
+    layers = [B.make_layer(X=Xd, V=V, r=r, layer_id=1)]
+    tables = 2048                                          # header, record, prefixes and descriptors of one layer, alignment
+    assert tables + need < B.agzo_workspace_bytes(layers)
+    ctx = B.Context(0, tables + need)
+    B.agzo_set_option(ctx, "extract_path", 1)
+    B.agzo_extract_subspace(ctx, layers, 7, 2)
+    assert B.agzo_poll(ctx) == B.AGZO_OK
+    B.agzo_destroy(ctx)
+    Vg = to_host(V)
+    assert np.abs(Vg.astype(np.float64) @ Vg.T - np.eye(r)).max() <= 1e-5
+    assert projector_distance(Vg, O.extract_subspace(X, r, 2, 7, 1)) <= 1e-3
