@@ -132,9 +132,10 @@ agzo_status agzo_destroy(agzo_ctx* ctx);
  * tensor-core kernels (UNSUPPORTED at call time if a layer cannot use them), 3 = as 2 but
  * without the fused power-step kernel (T = X Q and Y = X^T T as two sweeps over X);
  * "rmw_path" selects the kernel of the in-place passes: 0 = automatic (bf16 weights with
- * 16-byte aligned rows and r >= "rmw_tc_min_rank", default 5, take the tensor-core kernel, and so do
- * those of rank 3 on whose d_in or V rules out 16-byte accesses; everything else the CUDA-core kernels), 1 = CUDA-core kernels only, 2 = tensor-core kernel
- * for every layer that allows it; tuning knobs of that kernel, 0 = chosen by rank:
+ * 16-byte aligned rows and r >= "rmw_tc_min_rank", default 5, take the tensor-core kernel, and so
+ * from rank 3 on do those whose d_in or V rules out 16-byte accesses; everything else the CUDA-core
+ * kernels), 1 = CUDA-core kernels only, 2 = tensor-core kernel for every layer that allows it;
+ * tuning knobs of that kernel, 0 = chosen by rank:
  * "rmw_tc_slots" (shared-memory ring slots), "rmw_tc_inflight" (loads in flight per CTA),
  * "rmw_tc_panels" (column panels per work item, 1 or 2); "rmw_stage_r" 0 = when some layer's rank
  * exceeds 16 the split R operand of every 128-row tile is written once per pass to the scratch
@@ -143,8 +144,8 @@ agzo_status agzo_destroy(agzo_ctx* ctx);
  * flip and the restore/update of the same step, find it there and skip the writing), 1 = never,
  * 2 = always;
  * "share_inputs" 1 (default) = consecutive layers whose X is the same buffer (same pointer, pitch,
- * m, d_in: q/k/v or gate/up of a transformer block) are served by one sweep over X per product,
- * with identical results; 0 = every layer sweeps its X itself;
+ * m, d_in: q/k/v or gate/up of a transformer block) are served by one sweep over X per product;
+ * results agree to fp32 rounding (a layer may take another kernel than it would alone); 0 = every layer sweeps its X itself;
  * "extract_fused" 1 = layers with r <= 16 and d_in <= 12288 on the tensor-core path run each
  * power step in the fused kernel in which X crosses HBM once (thread-block clusters of
  * ceil(d_in / 512) CTAs, or ceil(d_in / 768)), where that cluster size keeps at least 70 % of
@@ -214,8 +215,10 @@ agzo_status agzo_read_counters(agzo_ctx* ctx, double* h_ms, int64_t* h_timed_lau
  * the next call with the same array; its tables are uploaded on `stream`) and writes, per layer,
  * the thread-block cluster size with which its power steps run in the fused kernel, 0 for a
  * layer served by the two-sweep kernels (no X, the "extract_fused" / "extract_path" options,
- * its shape, an X shared by layers of more than 16 ranks, or a launch wave small enough for L2).  h_cluster: host, n entries.  Launches
- * no kernel.                                                                               */
+ * its shape, an X shared by layers of more than 16 ranks, or a launch wave small enough for L2).
+ * h_cluster: host, n entries.  Launches nothing that computes: tables of up to 30 KiB are uploaded
+ * by a small kernel, here and in every call that finds a changed array, and agzo_read_counters
+ * counts it.                                                                               */
 agzo_status agzo_query_fused(agzo_ctx* ctx, const agzo_layer* h_layers, int n, int32_t* h_cluster,
                              void* stream);
 

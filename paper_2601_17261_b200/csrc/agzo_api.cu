@@ -18,7 +18,7 @@ namespace {
 
 constexpr uint32_t kMagic = 0xA620B200u;
 constexpr size_t kAlign = 256;
-constexpr size_t kHeaderBytes = 256;          // DevStatus + scalar slots
+constexpr size_t kHeaderBytes = 256;          // DevStatus
 constexpr int64_t kDefaultWaveBytes = 8ll << 30;
 constexpr int64_t kL2ResidentWaveBytes = 64ll << 20;   // a wave's X up to this size is still in L2 at its next sweep
 
@@ -29,7 +29,6 @@ struct Plan {
   std::vector<int> tile_start;     // n + 1
   std::vector<int> wave_end;       // exclusive end index of each extraction wave
   std::vector<int> wave_region;    // scratch region (= helper stream) of each wave, -1 = nothing to do
-  std::vector<int64_t> wave_xbytes;   // activation bytes of each wave (a shared X counted once)
   // the Y panels of a wave's layers lie one after another at the end of the wave's scratch, so that a
   // token-sharded run can sum all of them over the ranks in one call
   std::vector<float*> wave_y;
@@ -215,8 +214,8 @@ bool same_input(const agzo_layer& a, const agzo_layer& b) {
   return a.X == b.X && a.ldx == b.ldx && a.m == b.m && a.d_in == b.d_in && a.x_dtype == b.x_dtype;
 }
 
-// Token slabs of the X^T T product.  CUDA-core kernels: cc_slab_rows.  Tensor-core kernels: slabs of 2048 tokens (32 pipeline steps per CTA) when the layer has that many.  When
-// the call's layers fill the grid by their column blocks alone (long_slabs), a slab is up to
+// Token slabs of the X^T T product.  CUDA-core kernels: cc_slab_rows.  Tensor-core kernels: slabs of 2048 tokens (32 pipeline
+// steps per CTA) when the layer has that many.  When the call's layers fill the grid by their column blocks alone (long_slabs), a slab is up to
 // 16384 tokens: every slab costs a partial Y (r x d_in floats written, and read again by the
 // panel QR), and the CTAs' pipelines start and drain less often.
 constexpr int kLongSlabColumnBlocks = 1024;   // 128-column blocks over all layers from which slabs are long
@@ -257,7 +256,6 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
   plan->tile_start.assign(n + 1, 0);
   plan->wave_end.clear();
   plan->wave_region.clear();
-  plan->wave_xbytes.clear();
   plan->wave_y.clear();
   plan->wave_y_count.clear();
   const int regions = opts.extract_regions == 2 ? 2 : 1;
@@ -418,7 +416,7 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
   while (i < n) {
     if (!has_x(L[i])) {
       ++i;
-      plan->wave_end.push_back(i); plan->wave_region.push_back(-1); plan->wave_xbytes.push_back(0);
+      plan->wave_end.push_back(i); plan->wave_region.push_back(-1);
       plan->wave_y.push_back(nullptr); plan->wave_y_count.push_back(0);
       continue;
     }
@@ -529,7 +527,6 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     }
     plan->wave_end.push_back(j);
     plan->wave_region.push_back(region);
-    plan->wave_xbytes.push_back(xbytes);
     i = j;
   }
   if (scratch_needed) {

@@ -115,7 +115,7 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
   rec.ypart_stride = (long long)r * d_in;
   rec.Ypart = reinterpret_cast<float*>(p);  p += up256((size_t)slabs * R * D * 4);
   rec.Y = reinterpret_cast<float*>(p);      p += up256(R * D * 4);
-  rec.Gpart = reinterpret_cast<double*>(p);     // never more than the two terms in r^2 of the limit above
+  rec.Gpart = reinterpret_cast<double*>(p);     // used above rank 32 only; never more than the two terms in r^2 of the limit there
   static_assert(sizeof(DevLayer) <= 384, "layer record must fit its slot");
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);

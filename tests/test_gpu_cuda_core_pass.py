@@ -66,7 +66,12 @@ def test_tall_tiles():
     want = W0
     for seed in range(2):
         want = O.apply_direction(want, Vh, seed, 0, np.float32(1e-3), "bf16")
-    # two passes: one bf16 step each
-    got = to_host(Wd)[rows]
-    assert np.abs(got - want[rows]).max() <= 2 * 2.0 ** -7 * np.abs(W0).max()
-    assert (got != want[rows]).mean() <= 2e-3
+    # Two passes, one bf16 step each (a step is at most 2^-7 of the larger of what went in and what came out), at most 1e-3 of
+    # the elements differing in each: 1.04 of a row's 520 on average, and 10 or more in some row of 900 once in 10^4 runs.  A
+    # row that one pass left out differs in a sixth of its elements or more.
+    got, want, before = to_host(Wd)[rows], want[rows], W0[rows]
+    assert (np.abs(got - want) <= 2 * 2.0 ** -7 * np.maximum(np.abs(before), np.abs(want)) + 1e-9).all()
+    off = got != want
+    assert off.mean() <= 2e-3
+    assert off.sum(axis=1).max() < 10
+    assert off[:, 512:].mean() <= 4e-3
