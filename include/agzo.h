@@ -31,6 +31,10 @@
  *     a kernel of the caller that is launched with programmatic stream serialisation starts
  *     when that one's blocks are done.  Such a kernel executes its grid-dependency wait before
  *     it relies on what the call wrote, as it would behind any other kernel.
+ *     Calls may be captured into a CUDA graph once their layer list has been used outside a
+ *     capture (its tables are in place then).  Above rank 16 a graph holds an extraction together
+ *     with the passes that follow it: the passes of a seed share R images in the workspace, and
+ *     what a capture would stage counts as staged for the calls after it.
  *   - Every function returns an agzo_status; nothing throws, traps or aborts.  Argument
  *     errors are detected on the host before anything is launched.  Conditions that only
  *     the device can see (a rank-deficient panel, a wait that ran out) are written to a
@@ -119,7 +123,9 @@ typedef int (*agzo_loss_fn)(void* user, void* stream, int phase, double* d_loss)
 
 /* Bytes of workspace that every call on these layers needs (host only, no CUDA call).
  * A workspace sized for one layer list is also valid for any list whose per-field maxima
- * and layer count are not larger.  Error: INVALID_ARG for a bad descriptor.              */
+ * and layer count are not larger, unless its layers qualify for the tensor-core kernels of
+ * extraction where the first list's did not (bf16 X with 16-byte aligned rows, d_in a multiple
+ * of 8 and at least 128, m >= 256).  Error: INVALID_ARG for a bad descriptor.             */
 agzo_status agzo_workspace_bytes(const agzo_layer* h_layers, int n, size_t* h_bytes);
 
 /* Creates a context bound to CUDA device `device` that will use `workspace`
