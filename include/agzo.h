@@ -161,6 +161,10 @@ agzo_status agzo_destroy(agzo_ctx* ctx);
  * that share their X run fused as one layer where their ranks add up to at most 16; beyond that they
  * stay with the sweeps that serve the whole group (with 2: fused one by one);
  * 0 = off: two sweeps over X per power step.  Default 1;
+ * "extract_resident" 1 (default) = a call whose activations all fit the device's shared memory (ranks of at most 16, at most
+ * 24 over layers that share an X, at most 12 different X) is extracted by one kernel that keeps them there; it takes the place of
+ * all others unless an option above asks for one of those ("extract_path", "extract_fused" other than 1, "wave_bytes") or an
+ * all-reduce is set.  0 = never;
  * "wave_bytes" = activation bytes grouped into one launch wave of extraction;
  * "extract_streams" 2 (default) = alternate waves use two scratch regions and two helper
  * streams forked from and joined to the caller's stream, so that one wave's short kernels
@@ -322,7 +326,8 @@ agzo_status agzo_fill_gaussian_basis(agzo_ctx* ctx, const agzo_layer* h_layers, 
 /* (No counterpart in the paper: this entry point exists for callers, not for the method.)
  * Algorithm 1 for ONE layer without a context or a workspace: the same kernels as
  * agzo_extract_subspace's CUDA-core path, with their scratch in a fixed 4 MiB array that is
- * part of the library image on every GPU that loads it.  It is meant for callers that cannot
+ * part of the library image on every GPU that loads it, or the one kernel of "extract_resident" where that takes
+ * the layer (with a scratch of 5 MiB of its own and operands of 24 bits, as precise as fp32).  It is meant for callers that cannot
  * allocate device memory where they need a subspace -- a forward hook that runs while
  * another framework owns (or has frozen) the allocator, a callback in which an allocation
  * would synchronise the device, a job whose memory is fixed up front.  X and V are still

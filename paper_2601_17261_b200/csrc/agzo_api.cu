@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "agzo_common.cuh"
+#include "agzo_resident.cuh"
 #include "agzo_tc.cuh"
 
 using namespace agzo;
@@ -18,7 +19,9 @@ namespace {
 
 constexpr uint32_t kMagic = 0xA620B200u;
 constexpr size_t kAlign = 256;
-constexpr size_t kHeaderBytes = 256;          // DevStatus
+constexpr size_t kHeaderBytes = 256;          // DevStatus, and from kCountersAt on the counters of the resident extraction
+constexpr size_t kCountersAt = 128;
+static_assert(sizeof(DevStatus) <= kCountersAt && kCountersAt + 2 * kResMaxUnits * sizeof(unsigned) <= kHeaderBytes, "header");
 constexpr int64_t kDefaultWaveBytes = 8ll << 30;
 constexpr int64_t kL2ResidentWaveBytes = 64ll << 20;   // a wave's X up to this size is still in L2 at its next sweep
 
@@ -88,6 +91,11 @@ struct agzo_ctx {
   int extract_streams;     // 1 or 2 (see PlanOpts::extract_regions)
   int extract_fused;       // 0 off, 1 fused power-step kernel where it pays, 2 wherever a layer's shape allows it
   int share_inputs;        // 1: consecutive layers with the same X share the sweeps over it
+  int extract_resident;    // 1: inputs that fit the chip's shared memory are extracted by one kernel; 0: never
+  // the layer list that extraction last looked at for that kernel, and what came of it
+  std::vector<agzo_layer> resident_cached;
+  bool resident_known, resident_ok;
+  ResidentLaunch resident;
   // staged R images in scratch: valid for this seed until the plan changes or extraction uses the scratch
   bool rimg_valid;
   uint64_t rimg_seed;
@@ -110,6 +118,7 @@ struct agzo_ctx {
   bool stage_pending;
   cudaStream_t stage_stream;  // stream of the last table upload: a call on another stream waits for stage_ev
   TcState tc;
+  ResidentCaps resident_caps;
   // measurement aid: event pairs around the launches of one kernel class
   int debug_fail_step_call;   // test option: the n-th internal call of agzo_step fails on the host, 0 = off
   int time_class;
@@ -123,21 +132,24 @@ namespace {
 
 // What is asked of a device and set for its kernels is the same for every agzo_ctx: done once per CUDA context, since the
 // kernels' limits end with the context (cudaDeviceReset).
-cudaError_t device_init(int device, TcState* tc) {
-  struct Known { unsigned long long id; TcState st; };
+cudaError_t device_init(int device, TcState* tc, ResidentCaps* resident) {
+  struct Known { unsigned long long id; TcState st; ResidentCaps resident; };
   static std::mutex mu;
   static Known known[kMaxDevices];
   const unsigned long long id = current_context_id(device);
   std::lock_guard<std::mutex> lock(mu);
   Known* k = device < kMaxDevices ? known + device : nullptr;
-  if (k && id != 0 && k->id == id) { *tc = k->st; return cudaSuccess; }
+  if (k && id != 0 && k->id == id) { *tc = k->st; *resident = k->resident; return cudaSuccess; }
   TcState st;
+  ResidentCaps rc;
   cudaError_t e = panel_qr_init(&st.qr_wide);
   if (e == cudaSuccess) e = rmw_init();
   if (e == cudaSuccess) e = tc_init(&st, device);
+  if (e == cudaSuccess && st.available) e = resident_init(st.fused.sm_count, &rc);
   if (e != cudaSuccess) return e;
-  if (k) { k->id = id; k->st = st; }
+  if (k) { k->id = id; k->st = st; k->resident = rc; }
   *tc = st;
+  *resident = rc;
   return cudaSuccess;
 }
 
@@ -574,6 +586,11 @@ cudaError_t upload_as_parameters(const std::vector<char>& t, char* dst, cudaStre
   return launch_table<(int)kTableParamBytes>(t, dst, s);
 }
 
+PlanOpts plan_opts(const agzo_ctx* c, int regions) {
+  return PlanOpts{c->wave_bytes, c->extract_path, c->rmw_path, c->rmw_tc_min_rank, c->rmw_tc_panels, c->rmw_stage_r,
+                  c->tc.available, c->extract_fused, c->share_inputs != 0, regions, c->sm_count, &c->tc.fused};
+}
+
 // Makes the device tables describe `L`; uploads only when the descriptors changed.
 agzo_status prepare(agzo_ctx* c, const agzo_layer* L, int n, cudaStream_t s) {
   if (same_layers(c, L, n)) {
@@ -584,10 +601,7 @@ agzo_status prepare(agzo_ctx* c, const agzo_layer* L, int n, cudaStream_t s) {
   c->rimg_valid = false;
   if (kHeaderBytes + table_bytes(n) > c->ws_bytes) return AGZO_ERR_WORKSPACE;
   Plan plan;
-  PlanOpts opts{c->wave_bytes, c->extract_path, c->rmw_path, c->rmw_tc_min_rank, c->rmw_tc_panels, c->rmw_stage_r,
-                c->tc.available, c->extract_fused, c->share_inputs != 0,
-                c->allreduce ? 1 : c->extract_streams,    // the ranks' sums run in wave order on the caller's stream
-                c->sm_count, &c->tc.fused};
+  PlanOpts opts = plan_opts(c, c->allreduce ? 1 : c->extract_streams);    // the ranks' sums run in wave order on the caller's stream
   agzo_status st = build_plan(L, n, c->ws, c->ws_bytes, opts, &plan, nullptr);
   if (st == AGZO_ERR_WORKSPACE && opts.extract_regions == 2) {   // a workspace sized for one region
     opts.extract_regions = 1;
@@ -636,6 +650,32 @@ agzo_status prepare(agzo_ctx* c, const agzo_layer* L, int n, cudaStream_t s) {
   c->cached.assign(L, L + n);
   c->cached_valid = true;
   return AGZO_OK;
+}
+
+// Whether the resident kernel extracts this list: c->resident is its launch then.  It takes part of the scratch area, at its
+// end, and leaves the tables of the list that was prepared last alone.
+bool plan_resident(agzo_ctx* c, const agzo_layer* L, int n) {
+  // an option that asks for one of the other paths, or cuts the list into waves, is meant for those
+  if (!c->extract_resident || c->allreduce || c->extract_path != 0 || c->extract_fused != 1 || c->wave_bytes != kDefaultWaveBytes) return false;
+  if (!c->resident_known || c->resident_cached.size() != (size_t)n ||
+      std::memcmp(c->resident_cached.data(), L, (size_t)n * sizeof(agzo_layer)) != 0) {
+    bool two_parts = c->tc.available;
+    for (int i = 0; i < n && two_parts; ++i) two_parts = tc_eligible(L[i]);
+    c->resident_ok = resident_plan(c->resident_caps, L, n, c->share_inputs != 0, two_parts, &c->resident);
+    // a workspace that the other kernels would refuse is refused by all
+    Plan others;
+    if (c->resident_ok)
+      c->resident_ok = kHeaderBytes + table_bytes(n) <= c->ws_bytes &&
+                       build_plan(L, n, c->ws, c->ws_bytes, plan_opts(c, 1), &others, nullptr) == AGZO_OK;
+    c->resident_cached.assign(L, L + n);
+    c->resident_known = true;
+  }
+  if (!c->resident_ok) return false;
+  const size_t tables = kHeaderBytes + (c->cached_valid ? table_bytes((int)c->cached.size()) : 0);
+  const size_t end = c->ws_bytes & ~(kAlign - 1), need = align_up(c->resident.scratch);
+  if (end < tables || end - tables < need) return false;
+  resident_bind(&c->resident, c->ws + end - need);
+  return true;
 }
 
 agzo_status check_ctx(agzo_ctx* c) {
@@ -773,6 +813,8 @@ agzo_status agzo_create(agzo_ctx** out, int device, void* workspace, size_t work
   c->allreduce_user = nullptr;
   c->token_offset = 0;
   c->share_inputs = 1;
+  c->extract_resident = 1;
+  c->resident_known = c->resident_ok = false;
   c->aux[0] = c->aux[1] = nullptr;
   c->fork_ev = c->join_ev[0] = c->join_ev[1] = nullptr;
   c->cached_valid = false;
@@ -796,7 +838,7 @@ agzo_status agzo_create(agzo_ctx** out, int device, void* workspace, size_t work
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMemset(c->ws, 0, kHeaderBytes);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
-  if (e == cudaSuccess) e = device_init(device, &c->tc);
+  if (e == cudaSuccess) e = device_init(device, &c->tc, &c->resident_caps);
   if (e != cudaSuccess) {
     if (c->stage_ev) cudaEventDestroy(c->stage_ev);
     if (c->fork_ev) cudaEventDestroy(c->fork_ev);
@@ -857,6 +899,10 @@ agzo_status agzo_set_option(agzo_ctx* ctx, const char* name, int64_t value) {
   } else if (std::strcmp(name, "share_inputs") == 0) {
     if (value < 0 || value > 1) return AGZO_ERR_INVALID_ARG;
     ctx->share_inputs = (int)value;
+  } else if (std::strcmp(name, "extract_resident") == 0) {
+    if (value < 0 || value > 1) return AGZO_ERR_INVALID_ARG;
+    ctx->extract_resident = (int)value;
+    return AGZO_OK;
   } else if (std::strcmp(name, "extract_fused") == 0) {
     if (value < 0 || value > 2) return AGZO_ERR_INVALID_ARG;
     ctx->extract_fused = (int)value;
@@ -877,7 +923,7 @@ agzo_status agzo_set_option(agzo_ctx* ctx, const char* name, int64_t value) {
   } else {
     return AGZO_ERR_INVALID_ARG;
   }
-  ctx->cached_valid = false;   // the plan depends on the options
+  ctx->cached_valid = ctx->resident_known = false;   // the plans depend on the options
   return AGZO_OK;
 }
 
@@ -955,8 +1001,23 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
   if (ctx->extract_path >= 2)
     for (int i = 0; i < n; ++i)
       if (!ctx->tc.available || !tc_eligible(h_layers[i])) return AGZO_ERR_UNSUPPORTED;
-  st = prepare(ctx, h_layers, n, s);
-  if (st != AGZO_OK) return st;
+  bool tables = false;       // a list with weights gets its tables here, whichever kernels extract it: the passes read them
+  for (int i = 0; i < n; ++i) tables = tables || h_layers[i].W;
+  if (tables && (st = prepare(ctx, h_layers, n, s)) != AGZO_OK) return st;
+  if (plan_resident(ctx, h_layers, n)) {
+    if (ctx->stage_pending && s != ctx->stage_stream) CU(ctx, cudaStreamWaitEvent(s, ctx->stage_ev, 0));
+    ctx->rimg_valid = false;
+    ResidentParams& p = ctx->resident.p;
+    p.K = K;
+    p.seed = seed;
+    p.status = dev_status(ctx);
+    p.flag = nullptr;
+    p.counters = reinterpret_cast<unsigned*>(ctx->ws + kCountersAt);
+    ctx->launches += 1;
+    CU(ctx, launch_resident(ctx->resident, s));
+    return AGZO_OK;
+  }
+  if (!tables && (st = prepare(ctx, h_layers, n, s)) != AGZO_OK) return st;
   ctx->rimg_valid = false;   // extraction takes the scratch area
 
   const Plan& P = ctx->plan;

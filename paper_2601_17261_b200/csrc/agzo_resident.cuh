@@ -1,0 +1,71 @@
+// Algorithm 1 for small inputs in one launch, X resident in shared memory: host interface.
+#pragma once
+
+#include "agzo_common.cuh"
+
+namespace agzo {
+
+constexpr int kResMaxUnits = 12;        // units (runs of layers on one X) of a launch
+constexpr int kResMaxLayers = 4;        // layers of a unit
+constexpr int kResMaxRank = 16;         // rank of a layer
+// Ranks of a unit.  Beyond, the sweeps over X are what takes the time and their chain has more SMs for them: two layers of rank 16 on
+// 2000 x 1024, 82 us here and 74 there; three of rank 8 on 613 x 1024 51 and 54.
+constexpr int kResMaxPanel = 24;
+
+struct ResidentLayer {
+  float* V;
+  long long ldv;
+  unsigned layer_id;
+  int r;
+  int off;               // first rank in the unit's panel
+  int row;               // first row of the staged Y (layers start at multiples of 8)
+};
+// Layers that read one X.  The X of a unit is cut into blocks of 128 tokens x 128 columns; a CTA keeps tb x cb of them.  The
+// cj CTAs side by side cover the columns, ni such rows the tokens; a cluster holds whole rows.
+struct ResidentUnit {
+  const void* X;
+  long long ldx;
+  int x_dtype, x_vec, m, d;
+  int n_layers, ranks, NP, NB;          // ranks of the panel, rounded up to 8; operand rows (parts x NP, rounded up to 16)
+  int rows;                             // rows of the staged Y
+  int cb, tb, cj, ni;
+  int gram_split;                       // warps per layer of the Gram products
+  int cluster0, clusters;               // clusters of the launch that work on this unit
+  int sub;                              // columns of Y that a CTA adds up for the unit, 0: all of its cb blocks for itself
+  int counter;                          // index of the unit's pair of counters
+  float* ypart;                         // [ni][ranks][cj cb 128] partial sums of Y; twice, by turns, where sub = 0
+  float* y;                             // [ranks][cj cb 128], where sub > 0
+  double* gshare;                       // [clusters][layers][192], where sub > 0
+  ResidentLayer layer[kResMaxLayers];
+};
+struct ResidentParams {
+  int n_units, cs, K, pad;
+  unsigned long long seed;
+  DevStatus* status;                    // may be null
+  int* flag;                            // may be null: set to whether a column was dependent
+  unsigned* counters;                   // two per unit, zero between launches
+  ResidentUnit unit[kResMaxUnits];
+};
+
+struct ResidentCaps {
+  int sm_count = 0;
+  int clusters[9] = {};                 // resident clusters of 1, 2, 4 and 8 CTAs, by size; 0: not usable
+};
+struct ResidentLaunch {
+  ResidentParams p;
+  int planes, parts;                    // bf16 planes of X (1: bf16, 3: fp32), parts of the operands Q and T
+  int n_clusters;
+  bool grid_wide;                       // some unit has several clusters, which wait for one another
+  size_t smem;
+  size_t scratch;                       // bytes behind ypart, y and gshare
+};
+
+cudaError_t resident_init(int sm_count, ResidentCaps* caps);      // once per device
+// Plans one launch for the layers; false where the resident kernel does not take them.  two_parts: the products of every layer
+// would run on the tensor-core path, whose operands are two bf16 parts; else they are three (24 bits, as the CUDA-core path's fp32).
+bool resident_plan(const ResidentCaps& caps, const agzo_layer* layers, int n, bool share_inputs, bool two_parts, ResidentLaunch* out);
+// points the plan at its scratch (256-byte aligned, out->scratch bytes)
+void resident_bind(ResidentLaunch* plan, char* scratch);
+cudaError_t launch_resident(const ResidentLaunch& plan, cudaStream_t s);
+
+}  // namespace agzo

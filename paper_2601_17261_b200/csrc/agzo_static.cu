@@ -10,6 +10,7 @@
 #include <mutex>
 
 #include "agzo_common.cuh"
+#include "agzo_resident.cuh"
 
 namespace {
 
@@ -18,6 +19,11 @@ constexpr size_t kStaticScratchBytes = 4u << 20;   // 4 MiB, held by every GPU t
 // The name below is a host-side handle for the symbol, not a device address: kernels must be
 // given the address that cudaGetSymbolAddress returns for the current device.
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
+// What the resident kernel needs where the problem fits the limit above (a partial sum of Y per row of CTAs), and its counters,
+// which are zero between launches.
+constexpr size_t kResidentScratchBytes = 5u << 20;
+static __device__ __align__(256) unsigned char g_resident_scratch[kResidentScratchBytes];
+static __device__ unsigned g_resident_counters[2];
 
 // Looked up once per CUDA context: the address and the kernels' limits end with it (cudaDeviceReset).
 struct Scratch {
@@ -25,6 +31,9 @@ struct Scratch {
   void* addr;
   bool qr_wide;
   int sm_count;
+  agzo::ResidentCaps resident;
+  void* resident_addr;
+  void* resident_counters;
 };
 std::mutex g_mu;
 Scratch g_scratch[agzo::kMaxDevices] = {};
@@ -38,10 +47,14 @@ cudaError_t scratch_of_current_device(Scratch* out) {
   std::lock_guard<std::mutex> lock(g_mu);
   Scratch& known = g_scratch[dev];
   if (!known.addr || id == 0 || known.context != id) {
-    Scratch fresh{id, nullptr, false, 0};
+    Scratch fresh{};
+    fresh.context = id;
     e = cudaGetSymbolAddress(&fresh.addr, g_static_scratch);   // with that device current
+    if (e == cudaSuccess) e = cudaGetSymbolAddress(&fresh.resident_addr, g_resident_scratch);
+    if (e == cudaSuccess) e = cudaGetSymbolAddress(&fresh.resident_counters, g_resident_counters);
     if (e == cudaSuccess) e = agzo::panel_qr_init(&fresh.qr_wide);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&fresh.sm_count, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = agzo::resident_init(fresh.sm_count, &fresh.resident);
     if (e != cudaSuccess) return e;
     known = fresh;
   }
@@ -98,6 +111,21 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
   if (need > kStaticScratchBytes) return AGZO_ERR_WORKSPACE;   // problem too large for the fixed array
   Scratch scratch;
   if (scratch_of_current_device(&scratch) != cudaSuccess) return AGZO_ERR_CUDA;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  {
+    agzo_layer a{};
+    a.X = X; a.ldx = ldx; a.x_dtype = x_dtype; a.m = m; a.d_in = d_in; a.r = r; a.layer_id = layer_id;
+    a.V = V; a.ldv = ldv;
+    ResidentLaunch plan;
+    if (resident_plan(scratch.resident, &a, 1, false, false, &plan) && plan.scratch <= kResidentScratchBytes) {
+      resident_bind(&plan, static_cast<char*>(scratch.resident_addr));
+      plan.p.K = K;
+      plan.p.seed = seed;
+      plan.p.flag = d_rank_deficient;
+      plan.p.counters = static_cast<unsigned*>(scratch.resident_counters);
+      return launch_resident(plan, s) == cudaSuccess ? AGZO_OK : AGZO_ERR_CUDA;
+    }
+  }
   for (int rows = cc_slab_rows(m, (long long)gch, scratch.sm_count);; rows += 32) {      // ends at 256 tokens per slab at the latest
     const size_t n = ((size_t)m + rows - 1) / rows;
     if (need - up256((size_t)slabs * R * D * 4) + up256(n * R * D * 4) <= kStaticScratchBytes) { slab_rows = rows; slabs = (int)n; break; }
@@ -118,7 +146,6 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
   rec.Gpart = reinterpret_cast<double*>(p);     // used above rank 32 only; never more than the two terms in r^2 of the limit there
   static_assert(sizeof(DevLayer) <= 384, "layer record must fit its slot");
 
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (launch_chained(static_begin_kernel, dim3(1), 1, 0, 0, s, rec, d_rec, d_status) != cudaSuccess) return AGZO_ERR_CUDA;
 
   ExtractWave w{};

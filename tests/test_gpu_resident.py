@@ -1,0 +1,141 @@
+"""Extraction by one kernel that keeps X in shared memory: blocks of 128 x 128 full, ragged and nearly empty, units on one CTA, one cluster
+and several, columns of Y summed whole and in pieces, groups on one X, the forms of X that are read element by element, and the
+launches in a row that share its counters.
+
+Against the oracle at the suite's tolerances for extraction (1e-5 orthonormality, 1e-3 projector distance), and against the kernels
+of the other paths on the same inputs: operands in three bf16 parts carry 24 bits, as fp32 does, so that both sides are within a
+few 2^-24 sqrt(K + 1) of the exact basis times the spread of the spectrum (at most 5 in these inputs): 1e-5; operands in two
+parts leave 2^-17 of a product: 1e-3 as the suite."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import agzo_oracle as O
+from paper_2601_17261_b200 import binding as B
+from paper_2601_17261_b200 import workloads as WL
+
+from gpu_helpers import DEV, Ctx, projector_distance, to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+
+def launches(ctx, layers, seed, K):
+    B.agzo_read_counters(ctx)
+    B.agzo_extract_subspace(ctx, layers, seed, K)
+    return B.agzo_read_counters(ctx)[2]
+
+
+def check(units, K, seed=6, served=True):
+    """units: (m, d_in, ranks of the layers on that X, bf16, pitch)"""
+    Xs, Vs, layers, held = [], [], [], []
+    for n, (m, d, ranks, bf16, pitch) in enumerate(units):
+        X = WL.planted_activations(m, d, min(16, d, m), seed=m + n, bf16=bf16)
+        Xd = to_dev(X, bf16, pitch=pitch)[0]
+        held.append(Xd)
+        for r in ranks:
+            Vb = torch.full((r + 2, d + 5), 7.0, device=DEV)
+            Xs.append((X, r))
+            Vs.append((Vb, Vb[1:1 + r, :d]))
+            layers.append(B.make_layer(X=Xd, V=Vs[-1][1], r=r, layer_id=len(layers)))
+    three = any(not b or d % 8 or d < 128 or m < 256 or (p or 0) % 8 for m, d, _, b, p in units)
+    with Ctx(layers) as ctx:
+        n = launches(ctx, layers, seed, K)
+        assert (n == 1) == served, n
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+        first = [V.clone() for _, V in Vs]
+        launches(ctx, layers, seed + 1, K)
+        launches(ctx, layers, seed, K)
+        assert all(torch.equal(a, V) for a, (_, V) in zip(first, Vs))
+        B.agzo_set_option(ctx, "extract_resident", 0)
+        assert launches(ctx, layers, seed, K) > 1
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+    for i, ((X, r), a, (Vb, V)) in enumerate(zip(Xs, first, Vs)):
+        got = to_host(a)
+        assert np.abs(got.astype(np.float64) @ got.T - np.eye(r)).max() <= 1e-5, i
+        assert projector_distance(got, O.extract_subspace(X, r, K, seed, i)) <= 1e-3, i
+        assert float((a - V).norm() / V.norm()) <= (1e-5 if three else 1e-3), i
+        edge = Vb.clone()
+        edge[1:1 + r, :X.shape[1]] = 7.0
+        assert bool((edge == 7.0).all()), i
+
+
+@pytest.mark.parametrize("K", [0, 2])
+@pytest.mark.parametrize("m,d_in,r,bf16,pitch", [
+    (16, 16, 16, False, None), (64, 64, 4, True, None), (128, 128, 1, False, None), (129, 130, 3, False, 131), (127, 257, 8, True, 259),
+    (300, 520, 16, True, 528), (512, 256, 4, False, None), (613, 1024, 8, True, None), (1000, 1000, 5, True, None), (1111, 515, 9, False, 516),
+    (4096, 256, 16, False, None), (2100, 2048, 16, True, None), (4096, 2048, 16, True, None), (700, 4096, 12, True, None)])
+def test_one_layer(m, d_in, r, bf16, pitch, K):
+    check([(m, d_in, (r,), bf16, pitch)], K)
+
+
+@pytest.mark.parametrize("ranks", [(8, 8, 8), (1, 1), (4, 4, 4), (5, 11), (16, 9), (3, 2, 11, 7), (1, 1, 1, 1, 1)])
+@pytest.mark.parametrize("m,d_in,bf16", [(300, 264, True), (613, 1024, True), (257, 130, False)])
+def test_layers_on_one_x(ranks, m, d_in, bf16):
+    check([(m, d_in, ranks, bf16, None)], 2, served=sum(ranks) <= 24 and len(ranks) <= 4)
+
+
+@pytest.mark.parametrize("units", [
+    [(300, 256, (8, 8), True, None), (300, 512, (4,), True, None), (300, 264, (16, 2, 1), True, None)],
+    [(512, 200 + 40 * i, (4,), False, None) for i in range(8)],
+    [(613, 1024, (8, 8, 8), True, None), (613, 2048, (8,), True, None), (130, 128, (2,), True, None)]])
+def test_units_side_by_side(units):
+    check(units, 2)
+
+
+def test_static_entry_and_what_it_reports():
+    for m, d_in, r, bf16 in [(700, 256, 4, False), (300, 130, 16, True), (1500, 520, 8, True)]:
+        X = WL.planted_activations(m, d_in, 16, seed=m, bf16=bf16)
+        Xd = to_dev(X, bf16)[0]
+        V, flag = torch.zeros(r, d_in, device=DEV), torch.full((1,), -1, dtype=torch.int32, device=DEV)
+        B.agzo_extract_subspace_static(Xd, V, r, 2, 3, 7, flag)
+        assert flag.item() == 0
+        assert projector_distance(to_host(V), O.extract_subspace(X, r, 2, 3, 7)) <= 1e-3
+        Xd[:, 2:] = 0                                          # rank two
+        B.agzo_extract_subspace_static(Xd, V, r, 2, 3, 7, flag)
+        assert flag.item() == 1 and int((V.norm(dim=1) == 0).sum()) == r - 2
+
+
+def test_dependent_columns_and_a_small_workspace():
+    m, d_in, r = 400, 384, 8
+    X = torch.zeros(m, d_in, dtype=torch.bfloat16, device=DEV)
+    X[:, :3] = torch.randn(m, 3, device=DEV)
+    V = torch.zeros(r, d_in, device=DEV)
+    layers = [B.make_layer(X=X, V=V, r=r, layer_id=0)]
+    with Ctx(layers) as ctx:
+        assert launches(ctx, layers, 1, 2) == 1
+        assert B.agzo_poll(ctx) == B.AGZO_WARN_RANK_DEFICIENT
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+        assert int((V.norm(dim=1) == 0).sum()) == r - 3
+    # a workspace without room for it: the other kernels, or their refusal
+    Y = torch.randn(2048, 256, device=DEV)
+    W = torch.zeros(4, 256, device=DEV)
+    layers = [B.make_layer(X=Y, V=W, r=4, layer_id=0)]
+    small = B.Context(0, 4096 + 2048 * 16 + 3 * 4096)
+    B.agzo_extract_subspace(small, layers, 1, 1)
+    a = W.clone()
+    with Ctx(layers) as ctx:
+        assert launches(ctx, layers, 1, 1) == 1
+    assert float((a - W).norm() / W.norm()) <= 1e-5
+    B.agzo_destroy(small)
+
+
+def test_a_graph_of_it_replays():
+    X = to_dev(WL.planted_activations(900, 640, 16, seed=1, bf16=True), True)[0]
+    V = torch.zeros(8, 640, device=DEV)
+    layers = [B.make_layer(X=X, V=V, r=8, layer_id=0)]
+    s = torch.cuda.Stream()
+    with Ctx(layers) as ctx:
+        with torch.cuda.stream(s):
+            assert launches(ctx, layers, 5, 2) == 1
+        torch.cuda.synchronize()
+        want = V.clone()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            B.agzo_extract_subspace(ctx, layers, 5, 2)
+        for _ in range(3):
+            V.zero_()
+            graph.replay()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(V, want)
+        del graph
