@@ -226,6 +226,7 @@ agzo_status agzo_read_counters(agzo_ctx* ctx, double* h_ms, int64_t* h_timed_lau
  * the thread-block cluster size with which its power steps run in the fused kernel, 0 for a
  * layer served by the two-sweep kernels (no X, the "extract_fused" / "extract_path" options,
  * its shape, an X shared by layers of more than 16 ranks, or a launch wave small enough for L2).
+ * A call that "extract_resident" serves runs none of these kernels.
  * h_cluster: host, n entries.  Launches nothing that computes: tables of up to 30 KiB are uploaded
  * by a small kernel, here and in every call that finds a changed array, and agzo_read_counters
  * counts it.                                                                               */

@@ -1013,9 +1013,10 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
     p.status = dev_status(ctx);
     p.flag = nullptr;
     p.counters = reinterpret_cast<unsigned*>(ctx->ws + kCountersAt);
-    ctx->launches += 1;
-    CU(ctx, launch_resident(ctx->resident, s));
-    return AGZO_OK;
+    const cudaError_t e = launch_resident(ctx->resident, s);
+    if (e == cudaSuccess) { ctx->launches += 1; return AGZO_OK; }
+    ctx->resident_ok = false;
+    if (!resident_refused(e)) { ctx->last_cuda = (int)e; return AGZO_ERR_CUDA; }
   }
   if (!tables && (st = prepare(ctx, h_layers, n, s)) != AGZO_OK) return st;
   ctx->rimg_valid = false;   // extraction takes the scratch area

@@ -15,8 +15,10 @@
 // three (24 bits) where the CUDA-core products would run, X in fp32 as three planes with the six products down to 2^-24.
 // Accumulation is fp32, over at most 128 tb tokens or 128 cb columns before the sums leave TMEM.
 //
-// What bounds it is the chain of synchronisations: a cluster barrier 0.4 us, a unit-wide one 1.2, the exchange of T 1.2, the
-// factor 1 to 2.
+// What bounds it is the chain of synchronisations of a round: a cluster barrier 0.2 us, all CTAs of a unit at a counter 1.3, the
+// partial sums of Y from L2 1.2, the exchange of T 2.3, the Gram matrix and its exchange 2, the factor 0.5 to 2.4.  Against the
+// chain of launches, K = 3: without workspace 4096 x 2048, r = 16 158 -> 85 us; 8192 x 256 bf16, r = 8 85 -> 47; 1500 x 515 fp32,
+// r = 5 97 -> 51; 613 x 1024 bf16, three layers of r = 8 53 -> 51.
 #include "agzo_qr.cuh"
 #include "agzo_resident.cuh"
 
@@ -956,6 +958,12 @@ cudaError_t launch_resident(const ResidentLaunch& plan, cudaStream_t s) {
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, res_kernel(plan.planes, plan.parts), plan.p);
+}
+
+bool resident_refused(cudaError_t e) {
+  if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorLaunchOutOfResources && e != cudaErrorNotSupported) return false;
+  cudaGetLastError();
+  return true;
 }
 
 }  // namespace agzo

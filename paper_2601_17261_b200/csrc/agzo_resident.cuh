@@ -67,5 +67,8 @@ bool resident_plan(const ResidentCaps& caps, const agzo_layer* layers, int n, bo
 // points the plan at its scratch (256-byte aligned, out->scratch bytes)
 void resident_bind(ResidentLaunch* plan, char* scratch);
 cudaError_t launch_resident(const ResidentLaunch& plan, cudaStream_t s);
+// The launch was refused for want of SMs (a context that has been given a part of the device): the other kernels serve the call.
+// Clears the runtime's last error then.
+bool resident_refused(cudaError_t e);
 
 }  // namespace agzo

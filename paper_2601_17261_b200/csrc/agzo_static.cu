@@ -123,7 +123,9 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
       plan.p.seed = seed;
       plan.p.flag = d_rank_deficient;
       plan.p.counters = static_cast<unsigned*>(scratch.resident_counters);
-      return launch_resident(plan, s) == cudaSuccess ? AGZO_OK : AGZO_ERR_CUDA;
+      const cudaError_t e = launch_resident(plan, s);
+      if (e == cudaSuccess) return AGZO_OK;
+      if (!resident_refused(e)) return AGZO_ERR_CUDA;
     }
   }
   for (int rows = cc_slab_rows(m, (long long)gch, scratch.sm_count);; rows += 32) {      // ends at 256 tokens per slab at the latest
