@@ -163,8 +163,8 @@ agzo_status agzo_destroy(agzo_ctx* ctx);
  * 0 = off: two sweeps over X per power step.  Default 1;
  * "extract_resident" 1 (default) = a call whose activations all fit the device's shared memory (ranks of at most 16, at most
  * 24 over layers that share an X, at most 12 different X) is extracted by one kernel that keeps them there; it takes the place of
- * all others unless an option above asks for one of those ("extract_path", "extract_fused" other than 1, "wave_bytes") or an
- * all-reduce is set.  0 = never;
+ * all others where it is estimated to be faster, unless an option asks for one of those ("extract_path", "extract_fused" other
+ * than 1, "wave_bytes") or an all-reduce is set.  2 = wherever it can run, 0 = never;
  * "wave_bytes" = activation bytes grouped into one launch wave of extraction;
  * "extract_streams" 2 (default) = alternate waves use two scratch regions and two helper
  * streams forked from and joined to the caller's stream, so that one wave's short kernels

@@ -91,7 +91,7 @@ struct agzo_ctx {
   int extract_streams;     // 1 or 2 (see PlanOpts::extract_regions)
   int extract_fused;       // 0 off, 1 fused power-step kernel where it pays, 2 wherever a layer's shape allows it
   int share_inputs;        // 1: consecutive layers with the same X share the sweeps over it
-  int extract_resident;    // 1: inputs that fit the chip's shared memory are extracted by one kernel; 0: never
+  int extract_resident;    // 1: inputs that fit the chip's shared memory are extracted by one kernel where that is faster; 2: always; 0: never
   // the layer list that extraction last looked at for that kernel, and what came of it
   std::vector<agzo_layer> resident_cached;
   bool resident_known, resident_ok;
@@ -900,7 +900,7 @@ agzo_status agzo_set_option(agzo_ctx* ctx, const char* name, int64_t value) {
     if (value < 0 || value > 1) return AGZO_ERR_INVALID_ARG;
     ctx->share_inputs = (int)value;
   } else if (std::strcmp(name, "extract_resident") == 0) {
-    if (value < 0 || value > 1) return AGZO_ERR_INVALID_ARG;
+    if (value < 0 || value > 2) return AGZO_ERR_INVALID_ARG;
     ctx->extract_resident = (int)value;
     return AGZO_OK;
   } else if (std::strcmp(name, "extract_fused") == 0) {
@@ -1004,7 +1004,7 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
   bool tables = false;       // a list with weights gets its tables here, whichever kernels extract it: the passes read them
   for (int i = 0; i < n; ++i) tables = tables || h_layers[i].W;
   if (tables && (st = prepare(ctx, h_layers, n, s)) != AGZO_OK) return st;
-  if (plan_resident(ctx, h_layers, n)) {
+  if (plan_resident(ctx, h_layers, n) && (ctx->extract_resident == 2 || resident_pays(ctx->resident, K))) {
     if (ctx->stage_pending && s != ctx->stage_stream) CU(ctx, cudaStreamWaitEvent(s, ctx->stage_ev, 0));
     ctx->rimg_valid = false;
     ResidentParams& p = ctx->resident.p;

@@ -771,23 +771,53 @@ struct Shape {
   double cost;
 };
 
+// The estimate: least squares over 196 layouts (256 to 4096 columns, 300 to 4000 tokens, one to three layers of ranks 1 to 16, K = 1 and
+// 3), 6 % rms; a unit of several clusters pays most for meeting.
 Shape shape_of(const ResidentUnit& u, int planes, int cs, int cj, int cb, int tb) {
   Shape s{cj, cb, tb, 0, 0, 0, 0.0};
   const int blocks_m = (u.m + kBlock - 1) / kBlock, per = cs / cj;
   s.ni = (blocks_m + tb - 1) / tb;
   s.clusters = (s.ni + per - 1) / per;
-  // measured at 1.9 GHz: a product instruction of N rows 32 + N / 4 cycles, a barrier, the exchange of T, 60 KB of partial sums a us
-  double cycles = 0.0;
+  double cycles = 0.0;                 // of a product's instructions for 16 of the contracted dimension, all planes of X
   for (int p = 0; p < planes; ++p) cycles += 32.0 + (double)(p == 0 ? u.NB : (3 - p) * u.NP) / 4.0;
-  const double meet = s.clusters > 1 ? 1.2 : 0.4, kb = (double)u.ranks * cb * kBlock * 4.0 / 60e3;
-  s.cost = 2.0 * tb * cb * 8 * cycles / 1900.0 + (cj > 1 ? 1.2 + 0.1 * tb : 0.3) + 0.05 * (cb + tb) * (u.NP / 8) + 0.06 * cb * u.NP / 8;
+  int groups = 0, rank = 0;
+  for (int l = 0; l < u.n_layers; ++l) { groups += (u.layer[l].r + 7) / 8; rank = std::max(rank, u.layer[l].r); }
+  s.cost = 1.3 + 2.6 * (2.0 * tb * cb * 8 * cycles / 1900.0) + (cj > 1 ? 1.1 : 0.0) + 0.54 * cb * groups + 0.41 * (cb + tb) * (u.NP / 8) +
+           (rank > 4 ? 0.2 : 0.0) + (rank > 8 ? 1.4 : 0.0);
   if (s.ni > 1) {
-    const double all = meet + s.ni * kb, part = 2.0 * meet + 2.0 * kb + 0.02 * s.clusters * u.n_layers;
+    const double kb = (double)u.ranks * cb * kBlock * 4.0 / 60e3;      // a partial sum of the CTA's columns
+    // all of the columns: five partial sums a trip to L2, a trip per 128 columns
+    const double all = 0.45 * cb * ((s.ni + 4) / 5) + 0.1 * s.ni * kb, part = (s.clusters > 1 ? 3.2 : 1.2) + kb;
+    s.cost += s.clusters > 1 ? 3.4 : 1.2;
     if (part < all) s.sub = ((cb * kBlock + s.ni - 1) / s.ni + 3) & ~3;
-    s.cost += part < all ? part : all;
+    s.cost += std::min(part, all);
   }
-  if (cs > 1) s.cost += 0.5;
   return s;
+}
+
+// What a round of the other kernels takes (us): a chain of three launches whose time hardly depends on the size while all is in L2.
+// Fitted to the same lists; the products element by element take long enough not to be looked at.
+double round_of_others(const std::vector<ResidentUnit>& units, int planes, bool two_parts) {
+  double most = 0.0, all = 0.0, round = 0.0;
+  int layers = 0;
+  for (const ResidentUnit& u : units) {
+    if (!u.x_vec) return 1e9;
+    int rank = 0;
+    for (int l = 0; l < u.n_layers; ++l) rank = std::max(rank, u.layer[l].r);
+    const double md = 1e-6 * u.m * (double)u.d, m = 1e-3 * u.m, d = 1e-3 * u.d;
+    double t;
+    if (two_parts) t = 10.8 + (rank > 8 ? 2.5 : 0.0) + 1.24 * md + 0.23 * d + 0.8 * u.ranks / 8;
+    else if (planes == 1) return 1e9;                       // bf16 by the fp32 kernels
+    else if (rank <= 4) t = 7.7 + 1.15 * m + 1.6 * d + 0.6 * md;
+    else if (rank <= 8) t = 9.0 + 1.4 * m + 1.9 * d + 0.7 * md;
+    else t = 12.0 + 2.2 * m + 5.5 * d + 0.8 * md;
+    if (!two_parts) t += 2.3 * md * (u.n_layers - 1);       // they read X once per layer
+    round = std::max(round, t);
+    most = std::max(most, md);
+    all += md;
+    layers += u.n_layers;
+  }
+  return round + (two_parts ? 0.55 : 2.3) * (all - most) + 0.15 * std::min(layers - 1, 8);
 }
 
 // Shapes for all units on clusters of cs CTAs within the device's clusters: from the fewest clusters on, the slowest unit gets more.
@@ -902,6 +932,8 @@ bool resident_plan(const ResidentCaps& caps, const agzo_layer* L, int n, bool sh
       cs = c; least = slowest; best = shapes;
     }
   if (cs == 0) return false;
+  out->round_us = least;
+  out->others_us = round_of_others(units, planes, parts == 2);
   ResidentParams& p = out->p;
   p = ResidentParams{};
   p.n_units = (int)units.size();
@@ -920,6 +952,11 @@ bool resident_plan(const ResidentCaps& caps, const agzo_layer* L, int n, bool sh
   }
   resident_bind(out, nullptr);
   return true;
+}
+
+// One launch costs 4.8 us beside its K + 1 rounds, a cooperative one 5.5
+bool resident_pays(const ResidentLaunch& plan, int K) {
+  return (plan.grid_wide ? 5.5 : 4.8) + (K + 1) * plan.round_us < 0.95 * (K + 1) * plan.others_us;
 }
 
 void resident_bind(ResidentLaunch* plan, char* scratch) {

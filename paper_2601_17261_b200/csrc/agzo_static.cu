@@ -117,7 +117,7 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
     a.X = X; a.ldx = ldx; a.x_dtype = x_dtype; a.m = m; a.d_in = d_in; a.r = r; a.layer_id = layer_id;
     a.V = V; a.ldv = ldv;
     ResidentLaunch plan;
-    if (resident_plan(scratch.resident, &a, 1, false, false, &plan) && plan.scratch <= kResidentScratchBytes) {
+    if (resident_plan(scratch.resident, &a, 1, false, false, &plan) && plan.scratch <= kResidentScratchBytes && resident_pays(plan, K)) {
       resident_bind(&plan, static_cast<char*>(scratch.resident_addr));
       plan.p.K = K;
       plan.p.seed = seed;

@@ -39,6 +39,7 @@ def check(units, K, seed=6, served=True):
             layers.append(B.make_layer(X=Xd, V=Vs[-1][1], r=r, layer_id=len(layers)))
     three = any(not b or d % 8 or d < 128 or m < 256 or (p or 0) % 8 for m, d, _, b, p in units)
     with Ctx(layers) as ctx:
+        B.agzo_set_option(ctx, "extract_resident", 2)
         n = launches(ctx, layers, seed, K)
         assert (n == 1) == served, n
         assert B.agzo_poll(ctx) == B.AGZO_OK
@@ -102,6 +103,7 @@ def test_dependent_columns_and_a_small_workspace():
     V = torch.zeros(r, d_in, device=DEV)
     layers = [B.make_layer(X=X, V=V, r=r, layer_id=0)]
     with Ctx(layers) as ctx:
+        B.agzo_set_option(ctx, "extract_resident", 2)
         assert launches(ctx, layers, 1, 2) == 1
         assert B.agzo_poll(ctx) == B.AGZO_WARN_RANK_DEFICIENT
         assert B.agzo_poll(ctx) == B.AGZO_OK
@@ -111,9 +113,11 @@ def test_dependent_columns_and_a_small_workspace():
     W = torch.zeros(4, 256, device=DEV)
     layers = [B.make_layer(X=Y, V=W, r=4, layer_id=0)]
     small = B.Context(0, 4096 + 2048 * 16 + 3 * 4096)
+    B.agzo_set_option(small, "extract_resident", 2)
     B.agzo_extract_subspace(small, layers, 1, 1)
     a = W.clone()
     with Ctx(layers) as ctx:
+        B.agzo_set_option(ctx, "extract_resident", 2)
         assert launches(ctx, layers, 1, 1) == 1
     assert float((a - W).norm() / W.norm()) <= 1e-5
     B.agzo_destroy(small)
@@ -125,6 +129,7 @@ def test_a_graph_of_it_replays():
     layers = [B.make_layer(X=X, V=V, r=8, layer_id=0)]
     s = torch.cuda.Stream()
     with Ctx(layers) as ctx:
+        B.agzo_set_option(ctx, "extract_resident", 2)
         with torch.cuda.stream(s):
             assert launches(ctx, layers, 5, 2) == 1
         torch.cuda.synchronize()
