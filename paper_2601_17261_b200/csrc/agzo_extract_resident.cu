@@ -476,34 +476,39 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
     if (!direct) {
       unit_barrier(counter, clusters, cs, &met, &sh);
       const long long part = (long long)ranks * cols_pad;
-      if (U.sub == 0) {              // a warp per rank, ranks warp, warp + 8 ... three at a time
+      if (U.sub == 0) {              // a warp per rank and 128 columns, three of them and five partial sums in flight
         constexpr int kE = 3, kP = 5;
+        const int n_items = ranks * cb;
 #pragma unroll 1
-        for (int c = 4 * lane; c < ncols; c += 128)
+        for (int i0 = warp; i0 < n_items; i0 += kE * kWarps) {
+          const float* src[kE];
+          float* dst[kE];
+          float4 sum[kE];
+#pragma unroll
+          for (int e = 0; e < kE; ++e) {
+            const int it = min(i0 + e * kWarps, n_items - 1), k = it / cb, c = (it - k * cb) * kBlock + 4 * lane;
+            src[e] = ypart + (long long)k * cols_pad + col0 + c;
+            dst[e] = sY + sh.row_of[k] * pitch + c;
+            sum[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+          }
 #pragma unroll 1
-          for (int k0 = warp; k0 < ranks; k0 += kE * kWarps) {
-            float4 sum[kE];
-#pragma unroll
-            for (int e = 0; e < kE; ++e) sum[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
-            for (int s0 = 0; s0 < ni; s0 += kP) {
-              float4 t[kE][kP];
-#pragma unroll
-              for (int e = 0; e < kE; ++e)
-#pragma unroll
-                for (int x = 0; x < kP; ++x)
-                  t[e][x] = k0 + e * kWarps < ranks && s0 + x < ni
-                                ? __ldcg(reinterpret_cast<const float4*>(ypart + (s0 + x) * part + (long long)(k0 + e * kWarps) * cols_pad + col0 + c))
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-              for (int e = 0; e < kE; ++e)
-#pragma unroll
-                for (int x = 0; x < kP; ++x) { sum[e].x += t[e][x].x; sum[e].y += t[e][x].y; sum[e].z += t[e][x].z; sum[e].w += t[e][x].w; }
-            }
+          for (int s0 = 0; s0 < ni; s0 += kP) {
+            float4 t[kE][kP];
 #pragma unroll
             for (int e = 0; e < kE; ++e)
-              if (k0 + e * kWarps < ranks) *reinterpret_cast<float4*>(sY + sh.row_of[k0 + e * kWarps] * pitch + c) = sum[e];
+#pragma unroll
+              for (int x = 0; x < kP; ++x)
+                t[e][x] = i0 + e * kWarps < n_items && s0 + x < ni ? __ldcg(reinterpret_cast<const float4*>(src[e] + (s0 + x) * part))
+                                                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int e = 0; e < kE; ++e)
+#pragma unroll
+              for (int x = 0; x < kP; ++x) { sum[e].x += t[e][x].x; sum[e].y += t[e][x].y; sum[e].z += t[e][x].z; sum[e].w += t[e][x].w; }
           }
+#pragma unroll
+          for (int e = 0; e < kE; ++e)
+            if (i0 + e * kWarps < n_items) *reinterpret_cast<float4*>(dst[e]) = sum[e];
+        }
       } else {                       // few columns, many partial sums: four neighbouring lanes share a sum
         const int v4 = width / 4;
 #pragma unroll 1
@@ -786,8 +791,8 @@ Shape shape_of(const ResidentUnit& u, int planes, int cs, int cj, int cb, int tb
            (rank > 4 ? 0.2 : 0.0) + (rank > 8 ? 1.4 : 0.0);
   if (s.ni > 1) {
     const double kb = (double)u.ranks * cb * kBlock * 4.0 / 60e3;      // a partial sum of the CTA's columns
-    // all of the columns: five partial sums a trip to L2, a trip per 128 columns
-    const double all = 0.45 * cb * ((s.ni + 4) / 5) + 0.1 * s.ni * kb, part = (s.clusters > 1 ? 3.2 : 1.2) + kb;
+    // all of the columns: five partial sums of 24 rows of 128 columns a trip to L2
+    const double all = 0.45 * ((u.ranks * cb + 23) / 24) * ((s.ni + 4) / 5) + 0.1 * s.ni * kb, part = (s.clusters > 1 ? 3.2 : 1.2) + kb;
     s.cost += s.clusters > 1 ? 3.4 : 1.2;
     if (part < all) s.sub = ((cb * kBlock + s.ni - 1) / s.ni + 3) & ~3;
     s.cost += std::min(part, all);
