@@ -811,7 +811,7 @@ double round_of_others(const std::vector<ResidentUnit>& units, int planes, bool 
     for (int l = 0; l < u.n_layers; ++l) rank = std::max(rank, u.layer[l].r);
     const double md = 1e-6 * u.m * (double)u.d, m = 1e-3 * u.m, d = 1e-3 * u.d;
     double t;
-    if (two_parts) t = 10.8 + (rank > 8 ? 2.5 : 0.0) + 1.24 * md + 0.23 * d + 0.8 * u.ranks / 8;
+    if (two_parts) t = 10.2 + (rank > 8 ? 2.2 : 0.0) + 1.1 * m + d + 0.22 * md + 0.08 * (u.ranks - rank);
     else if (planes == 1) return 1e9;                       // bf16 by the fp32 kernels
     else if (rank <= 4) t = 7.7 + 1.15 * m + 1.6 * d + 0.6 * md;
     else if (rank <= 8) t = 9.0 + 1.4 * m + 1.9 * d + 0.7 * md;
@@ -961,7 +961,7 @@ bool resident_plan(const ResidentCaps& caps, const agzo_layer* L, int n, bool sh
 
 // One launch costs 4.8 us beside its K + 1 rounds, a cooperative one 5.5
 bool resident_pays(const ResidentLaunch& plan, int K) {
-  return (plan.grid_wide ? 5.5 : 4.8) + (K + 1) * plan.round_us < 0.95 * (K + 1) * plan.others_us;
+  return (plan.grid_wide ? 5.5 : 4.8) + (K + 1) * plan.round_us < 0.97 * (K + 1) * plan.others_us;
 }
 
 void resident_bind(ResidentLaunch* plan, char* scratch) {
