@@ -32,7 +32,7 @@
  *     when that one's blocks are done.  Such a kernel executes its grid-dependency wait before
  *     it relies on what the call wrote, as it would behind any other kernel.
  *     Calls may be captured into a CUDA graph once their layer list has been used outside a
- *     capture (its tables are in place then).  Above rank 16 a graph holds an extraction together
+ *     capture (its tables are in place then, or nothing needs them).  Above rank 16 a graph holds an extraction together
  *     with the passes that follow it: the passes of a seed share R images in the workspace, and
  *     what a capture would stage counts as staged for the calls after it.
  *   - Every function returns an agzo_status; nothing throws, traps or aborts.  Argument

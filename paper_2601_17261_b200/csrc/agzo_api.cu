@@ -117,6 +117,8 @@ struct agzo_ctx {
   cudaEvent_t stage_ev;
   bool stage_pending;
   cudaStream_t stage_stream;  // stream of the last table upload: a call on another stream waits for stage_ev
+  unsigned long long tables_capture;   // the capture that holds that upload, 0: it was made outside of any
+  bool tables_captured;    // a captured call reads the tables of a list without weights (see prepare)
   TcState tc;
   ResidentCaps resident_caps;
   // measurement aid: event pairs around the launches of one kernel class
@@ -573,17 +575,29 @@ __global__ void __launch_bounds__(kTableThreads) table_kernel(const __grid_const
   for (int i = blockIdx.x * kTableThreads + threadIdx.x; i < n16; i += gridDim.x * kTableThreads) dst[i] = blob.d[i];
 }
 template <int BYTES>
-cudaError_t launch_table(const std::vector<char>& t, char* dst, cudaStream_t s) {
+cudaError_t launch_table(const char* t, size_t bytes, char* dst, cudaStream_t s) {
   TableBlob<BYTES> blob;
-  std::memcpy(&blob, t.data(), t.size());
-  const int n16 = (int)(t.size() / 16), ctas = std::min(kTableCtas, (n16 + kTableThreads - 1) / kTableThreads);
+  std::memcpy(&blob, t, bytes);
+  const int n16 = (int)(bytes / 16), ctas = std::min(kTableCtas, (n16 + kTableThreads - 1) / kTableThreads);
   return launch_chained(table_kernel<BYTES>, dim3((unsigned)ctas), kTableThreads, 0, 0, s, blob, reinterpret_cast<uint4*>(dst), n16);
 }
 constexpr size_t kTableParamBytes = 30 * 1024;
 cudaError_t upload_as_parameters(const std::vector<char>& t, char* dst, cudaStream_t s) {
-  if (t.size() <= 3 * 1024) return launch_table<3 * 1024>(t, dst, s);
-  if (t.size() <= 10 * 1024) return launch_table<10 * 1024>(t, dst, s);
-  return launch_table<(int)kTableParamBytes>(t, dst, s);
+  if (t.size() <= 3 * 1024) return launch_table<3 * 1024>(t.data(), t.size(), dst, s);
+  if (t.size() <= 10 * 1024) return launch_table<10 * 1024>(t.data(), t.size(), dst, s);
+  for (size_t at = 0; at < t.size(); at += kTableParamBytes) {
+    const cudaError_t e = launch_table<(int)kTableParamBytes>(t.data() + at, std::min(kTableParamBytes, t.size() - at), dst + at, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+// A number of the capture that the stream takes part in, 0 outside of any
+unsigned long long capture_of(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(s, &st, &id) != cudaSuccess) { cudaGetLastError(); return 0; }
+  return st == cudaStreamCaptureStatusActive ? id : 0;
 }
 
 PlanOpts plan_opts(const agzo_ctx* c, int regions) {
@@ -591,9 +605,17 @@ PlanOpts plan_opts(const agzo_ctx* c, int regions) {
                   c->tc.available, c->extract_fused, c->share_inputs != 0, regions, c->sm_count, &c->tc.fused};
 }
 
-// Makes the device tables describe `L`; uploads only when the descriptors changed.
+bool any_weights(const agzo_layer* L, int n) {
+  for (int i = 0; i < n; ++i)
+    if (L[i].W) return true;
+  return false;
+}
+
+// Makes the device tables describe `L`; uploads only when the descriptors changed.  An upload that is captured is a node of the
+// graph: the tables are in place for the rest of that capture and for nobody else.
 agzo_status prepare(agzo_ctx* c, const agzo_layer* L, int n, cudaStream_t s) {
-  if (same_layers(c, L, n)) {
+  if (!c->tables_captured && !any_weights(L, n)) c->tables_captured = capture_of(s) != 0;
+  if (same_layers(c, L, n) && (c->tables_capture == 0 || c->tables_capture == capture_of(s))) {
     // the tables were uploaded on another stream: this one must not read them before they have landed
     if (c->stage_pending && s != c->stage_stream) CU(c, cudaStreamWaitEvent(s, c->stage_ev, 0));
     return AGZO_OK;
@@ -625,8 +647,9 @@ agzo_status prepare(agzo_ctx* c, const agzo_layer* L, int n, cudaStream_t s) {
         return AGZO_ERR_UNSUPPORTED;
     }
     c->cached_valid = false;             // until the upload is on its way
-    if (lb + tb <= kTableParamBytes) {
-      c->launches += 1;
+    const unsigned long long capture = capture_of(s);
+    if (lb + tb <= kTableParamBytes || capture != 0) {       // a copy that is captured would find the pinned buffer rewritten
+      c->launches += (int64_t)((lb + tb + kTableParamBytes - 1) / kTableParamBytes);
       CU(c, upload_as_parameters(c->h_tables, c->ws + kHeaderBytes, s));
     } else {
       if (c->h_stage_busy) CU(c, cudaEventSynchronize(c->stage_ev));
@@ -642,8 +665,9 @@ agzo_status prepare(agzo_ctx* c, const agzo_layer* L, int n, cudaStream_t s) {
       CU(c, cudaMemcpyAsync(c->ws + kHeaderBytes, c->h_stage, lb + tb, cudaMemcpyHostToDevice, s));
       c->h_stage_busy = true;
     }
-    CU(c, cudaEventRecord(c->stage_ev, s));
-    c->stage_pending = true;
+    c->tables_capture = capture;
+    c->stage_pending = capture == 0;     // inside a capture the graph's edges order it
+    if (c->stage_pending) CU(c, cudaEventRecord(c->stage_ev, s));
     c->stage_stream = s;
   }
   c->plan = std::move(plan);
@@ -818,6 +842,8 @@ agzo_status agzo_create(agzo_ctx** out, int device, void* workspace, size_t work
   c->aux[0] = c->aux[1] = nullptr;
   c->fork_ev = c->join_ev[0] = c->join_ev[1] = nullptr;
   c->cached_valid = false;
+  c->tables_capture = 0;
+  c->tables_captured = false;
   c->h_stage = nullptr;
   c->h_stage_bytes = 0;
   c->h_stage_busy = false;
@@ -1001,8 +1027,10 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
   if (ctx->extract_path >= 2)
     for (int i = 0; i < n; ++i)
       if (!ctx->tc.available || !tc_eligible(h_layers[i])) return AGZO_ERR_UNSUPPORTED;
-  bool tables = false;       // a list with weights gets its tables here, whichever kernels extract it: the passes read them
-  for (int i = 0; i < n; ++i) tables = tables || h_layers[i].W;
+  // A list with weights gets its tables here, whichever kernels extract it: the passes read them.  One without gets them where it
+  // takes the other kernels; but once calls that read such a list's tables have been captured, every use of the list outside the
+  // capture leaves them in place for the graph.
+  const bool tables = any_weights(h_layers, n) || (ctx->tables_captured && capture_of(s) == 0);
   if (tables && (st = prepare(ctx, h_layers, n, s)) != AGZO_OK) return st;
   if (plan_resident(ctx, h_layers, n) && (ctx->extract_resident == 2 || resident_pays(ctx->resident, K))) {
     if (ctx->stage_pending && s != ctx->stage_stream) CU(ctx, cudaStreamWaitEvent(s, ctx->stage_ev, 0));

@@ -67,3 +67,72 @@ def test_replays(r, bf16, wave_bytes, K):
         assert all(torch.equal(a, b) for a, b in zip(Vs, want[len(Ws):]))
         assert B.agzo_poll(ctx) == B.AGZO_OK
         del graph
+
+
+def two_lists(m=300, r=8):
+    Xs = [to_dev(WL.planted_activations(m, d, 16, seed=d, bf16=True), True)[0] for d in (512, 264)]
+    Vs = [torch.zeros(r, X.shape[1], device=DEV) for X in Xs]
+    return Xs, Vs, [[B.make_layer(X=X, V=V, r=r, layer_id=i)] for i, (X, V) in enumerate(zip(Xs, Vs))]
+
+
+def test_tables_uploaded_inside_a_capture_are_not_in_place_outside():
+    # a list without weights that only the resident kernel has served has no tables: captured on the other kernels, its upload is a
+    # node of the graph, so a call before the first replay brings its own
+    _, Vs, (one, _) = two_lists()
+    s = torch.cuda.Stream()
+    with Ctx(one) as ctx:
+        B.agzo_set_option(ctx, "extract_resident", 0)
+        with torch.cuda.stream(s):
+            B.agzo_extract_subspace(ctx, one, 5, 2)
+        torch.cuda.synchronize()
+        want = Vs[0].clone()
+    with Ctx(one) as ctx:
+        B.agzo_set_option(ctx, "extract_resident", 2)
+        with torch.cuda.stream(s):
+            B.agzo_extract_subspace(ctx, one, 5, 1)
+        B.agzo_set_option(ctx, "extract_resident", 0)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            B.agzo_extract_subspace(ctx, one, 5, 2)
+        B.agzo_read_counters(ctx)
+        for replay in (False, True, True):
+            Vs[0].zero_()
+            if replay:
+                graph.replay()
+            else:
+                B.agzo_extract_subspace(ctx, one, 5, 2)
+                n = B.agzo_read_counters(ctx)[2]
+            torch.cuda.synchronize()
+            assert torch.equal(Vs[0], want)
+        B.agzo_extract_subspace(ctx, one, 5, 2)                  # now they are: a launch less
+        assert B.agzo_read_counters(ctx)[2] == n - 1
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+        del graph
+
+
+def test_a_list_used_again_is_in_place_for_its_graph():
+    # another list's tables took the place of the captured one's; using that one again, by whichever kernels, brings them back
+    _, Vs, (one, other) = two_lists()
+    s = torch.cuda.Stream()
+    ctx = B.Context(0, max(B.agzo_workspace_bytes(L) for L in (one, other)))
+    B.agzo_set_option(ctx, "extract_resident", 0)
+    with torch.cuda.stream(s):
+        B.agzo_extract_subspace(ctx, one, 5, 2)
+    torch.cuda.synchronize()
+    want = Vs[0].clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        B.agzo_extract_subspace(ctx, one, 5, 2)
+    with torch.cuda.stream(s):
+        B.agzo_extract_subspace(ctx, other, 5, 2)
+        B.agzo_set_option(ctx, "extract_resident", 2)
+        B.agzo_extract_subspace(ctx, one, 5, 1)
+    torch.cuda.synchronize()
+    for V in Vs:
+        V.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(Vs[0], want) and not Vs[1].any()
+    assert B.agzo_poll(ctx) == B.AGZO_OK
+    del graph
+    B.agzo_destroy(ctx)
