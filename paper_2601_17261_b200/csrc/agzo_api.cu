@@ -1033,7 +1033,7 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
   const bool tables = any_weights(h_layers, n) || (ctx->tables_captured && capture_of(s) == 0);
   if (tables && (st = prepare(ctx, h_layers, n, s)) != AGZO_OK) return st;
   if (plan_resident(ctx, h_layers, n) && (ctx->extract_resident == 2 || resident_pays(ctx->resident, K))) {
-    if (ctx->stage_pending && s != ctx->stage_stream) CU(ctx, cudaStreamWaitEvent(s, ctx->stage_ev, 0));
+    // it reads no tables, so an upload that another stream has under way is not waited for (a capturing stream could not)
     ctx->rimg_valid = false;
     ResidentParams& p = ctx->resident.p;
     p.K = K;

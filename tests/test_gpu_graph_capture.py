@@ -136,3 +136,28 @@ def test_a_list_used_again_is_in_place_for_its_graph():
     assert B.agzo_poll(ctx) == B.AGZO_OK
     del graph
     B.agzo_destroy(ctx)
+
+
+def test_a_list_without_tables_is_captured_beside_an_upload_on_another_stream():
+    _, Vs, (one, other) = two_lists()
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    ctx = B.Context(0, max(B.agzo_workspace_bytes(L) for L in (one, other)))
+    B.agzo_set_option(ctx, "extract_resident", 0)
+    with torch.cuda.stream(a):
+        B.agzo_extract_subspace(ctx, other, 5, 2)                # uploads its tables on this stream
+    torch.cuda.synchronize()
+    B.agzo_set_option(ctx, "extract_resident", 2)
+    with torch.cuda.stream(b):
+        B.agzo_extract_subspace(ctx, one, 5, 2)
+    torch.cuda.synchronize()
+    want = Vs[0].clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=b):
+        B.agzo_extract_subspace(ctx, one, 5, 2)
+    Vs[0].zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(Vs[0], want)
+    assert B.agzo_poll(ctx) == B.AGZO_OK
+    del graph
+    B.agzo_destroy(ctx)
