@@ -387,6 +387,10 @@ agzo_status agzo_debug_fused_split(const int32_t* h_tiles, int n, int clusters, 
                                    int32_t* h_first, int32_t* h_parts, int32_t* h_share_begin,
                                    int32_t* h_shares);
 
+/* Test export, host only: what the arrivals of n blocks at a meeting of the resident extraction add to its counter, the
+ * first block's and every other one's.                                                     */
+agzo_status agzo_debug_meeting_increments(int32_t n, uint32_t* h_first, uint32_t* h_other);
+
 /* Exercises the bounded device-side wait that every pipeline of the tensor-core kernels uses:
  * launches one small block that waits, with the library's own wait routine, on a barrier that
  * nothing ever completes.  The wait gives up after its time limit (two seconds), the block

@@ -35,7 +35,7 @@ EXPORTS = [
     "agzo_perturb_dense", "agzo_debug_philox", "agzo_debug_gaussian", "agzo_read_counters",
     "agzo_extract_subspace_static", "agzo_fill_gaussian_basis", "agzo_set_allreduce",
     "agzo_debug_wait_timeout", "agzo_query_fused", "agzo_query_cluster_capacity", "agzo_debug_fused_split",
-    "agzo_debug_early_copy", "agzo_debug_normal_parts",
+    "agzo_debug_early_copy", "agzo_debug_normal_parts", "agzo_debug_meeting_increments",
 ]
 KC_RMW, KC_XT_T, KC_X_Q, KC_PANEL_QR, KC_TC_XT_T, KC_TC_X_Q, KC_OMEGA, KC_RMW_TC, KC_FUSED_POWER = 1, 2, 3, 4, 5, 6, 7, 8, 9
 
@@ -106,6 +106,7 @@ def lib() -> C.CDLL:
         "agzo_read_counters": (i32, [vp, C.POINTER(C.c_double), C.POINTER(i64), C.POINTER(i64)]),
         "agzo_set_allreduce": (i32, [vp, ALLREDUCE_FN, vp, i64]),
         "agzo_debug_wait_timeout": (i32, [vp, vp]),
+        "agzo_debug_meeting_increments": (i32, [i32, C.POINTER(u32), C.POINTER(u32)]),
         "agzo_query_fused": (i32, [vp, LP, i32, C.POINTER(C.c_int32), vp]),
         "agzo_query_cluster_capacity": (i32, [vp, C.POINTER(C.c_int32)]),
         "agzo_debug_fused_split": (i32, [C.POINTER(C.c_int32), i32, i32, C.POINTER(C.c_int32), C.POINTER(C.c_int32),

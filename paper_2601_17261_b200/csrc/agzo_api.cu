@@ -21,7 +21,7 @@ constexpr uint32_t kMagic = 0xA620B200u;
 constexpr size_t kAlign = 256;
 constexpr size_t kHeaderBytes = 256;          // DevStatus, and from kCountersAt on the counters of the resident extraction
 constexpr size_t kCountersAt = 128;
-static_assert(sizeof(DevStatus) <= kCountersAt && kCountersAt + 2 * kResMaxUnits * sizeof(unsigned) <= kHeaderBytes, "header");
+static_assert(sizeof(DevStatus) <= kCountersAt && kCountersAt + kResMaxUnits * sizeof(unsigned) <= kHeaderBytes, "header");
 constexpr int64_t kDefaultWaveBytes = 8ll << 30;
 constexpr int64_t kL2ResidentWaveBytes = 64ll << 20;   // a wave's X up to this size is still in L2 at its next sweep
 
@@ -1354,6 +1354,13 @@ agzo_status agzo_debug_fused_split(const int32_t* h_tiles, int n, int clusters, 
   const int G = fused_split(h_tiles, n, clusters, h_tile0, h_first, h_parts, &base, &rem);
   for (int k = 0; k <= G; ++k) h_share_begin[k] = fused_share_begin(k, base, rem);
   *h_shares = G;
+  return AGZO_OK;
+}
+
+agzo_status agzo_debug_meeting_increments(int32_t n, uint32_t* h_first, uint32_t* h_other) {
+  if (n < 1 || !h_first || !h_other) return AGZO_ERR_INVALID_ARG;
+  *h_first = meeting_increment(n, true);
+  *h_other = meeting_increment(n, false);
   return AGZO_OK;
 }
 

@@ -224,8 +224,8 @@ __device__ __forceinline__ void tmem_sum8(uint32_t at, int NP, int NB, int chunk
 }
 
 // All CTAs of a unit meet, and what they wrote to global memory before is visible after.  Where the unit is one cluster, the
-// cluster's barrier; else a counter that the last CTA to leave the kernel sets back.
-__device__ __forceinline__ void unit_barrier(unsigned* counter, int clusters, int cs, unsigned* met, ResShared* sh) {
+// cluster's barrier; else a counter that a meeting advances by 2^31 (meeting_increment): who waits does so for the high bit to turn.
+__device__ __forceinline__ void unit_barrier(unsigned* counter, int clusters, int cs, bool first, unsigned* phase, ResShared* sh) {
   if (clusters == 1) {
     __syncwarp();
     if (cs > 1) cluster_sync_all(); else __syncthreads();
@@ -233,15 +233,15 @@ __device__ __forceinline__ void unit_barrier(unsigned* counter, int clusters, in
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(counter), "r"(1u) : "memory");
-    *met += (unsigned)(clusters * cs);
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(counter), "r"(meeting_increment(clusters * cs, first)) : "memory");
+    *phase ^= 0x80000000u;
     if (!sh->failed) {
       const unsigned long long t_start = global_ns();
 #pragma unroll 1
       for (;;) {
         unsigned got;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(got) : "l"(counter) : "memory");
-        if (got >= *met) break;
+        if (((got ^ *phase) & 0x80000000u) == 0u) break;
         if (global_ns() - t_start > kWaitCapNs) { sh->failed = 1; break; }
       }
     }
@@ -375,8 +375,8 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
   const int cj = U.cj, j = rank % cj, row0 = rank - j, ni = U.ni, i = (cluster - U.cluster0) * (cs / cj) + rank / cj;
   const int cb = U.cb, tb = U.tb, NB = U.NB, NP = U.NP, ranks = U.ranks, nl = U.n_layers, clusters = U.clusters;
   const int ncols = cb * kBlock, col0 = j * ncols, cols_pad = cj * ncols, t0 = i * tb * kBlock, pitch = qr_pitch(ncols);
-  unsigned* counter = P.counters + 2 * U.counter;
-  unsigned met = 0;
+  unsigned* counter = P.counters + U.counter;
+  unsigned phase = 0;             // of the counter, thread 0
 
   const int plane = tb * cb * 2 * kSlotBytes;
   uint8_t* sX = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -415,6 +415,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
   __syncthreads();
   if (!(PLANES == 1 && U.x_vec)) fill_omega<PARTS>(U, sT, t0, tb, P.seed);      // needs nothing from before the launch
   chain_wait();
+  if (clusters > 1 && tid == 0) phase = __ldcg(counter) & 0x80000000u;      // nobody turns it before this CTA has arrived
   load_x<PLANES>(U, sX, plane, t0, col0, tb, cb);
   if (PLANES == 1 && U.x_vec) fill_omega<PARTS>(U, sT, t0, tb, P.seed);         // while X arrives
   asm volatile("cp.async.wait_all;" ::: "memory");
@@ -474,7 +475,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
       for (int k = tid; k < pad * (pitch / 4); k += kThreads) y[k] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     if (!direct) {
-      unit_barrier(counter, clusters, cs, &met, &sh);
+      unit_barrier(counter, clusters, cs, i == 0 && j == 0, &phase, &sh);
       const long long part = (long long)ranks * cols_pad;
       if (U.sub == 0) {              // a warp per rank and 128 columns, three of them and five partial sums in flight
         constexpr int kE = 3, kP = 5;
@@ -599,7 +600,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
           if (wide) U.gshare[(cluster - U.cluster0) * n_share + e] = sum; else place(e, sum);
         }
       if (wide) {
-        unit_barrier(counter, clusters, cs, &met, &sh);
+        unit_barrier(counter, clusters, cs, i == 0 && j == 0, &phase, &sh);
 #pragma unroll 1
         for (int e = tid; e < n_share; e += kThreads) {
           double sum = 0.0;
@@ -744,10 +745,6 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
     if (i == 0 && j == 0) {
       if (P.status && sh.st.rank_deficient) atomicExch(&P.status->rank_deficient, 1);
       if (P.flag) *P.flag = sh.st.rank_deficient;
-    }
-    if (clusters > 1 && atomicAdd(counter + 1, 1u) == (unsigned)(clusters * cs) - 1u) {      // nobody waits any more
-      counter[0] = 0u;
-      counter[1] = 0u;
     }
   }
   if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem, ncol); }

@@ -32,7 +32,7 @@ struct ResidentUnit {
   int gram_split;                       // warps per layer of the Gram products
   int cluster0, clusters;               // clusters of the launch that work on this unit
   int sub;                              // columns of Y that a CTA adds up for the unit, 0: all of its cb blocks for itself
-  int counter;                          // index of the unit's pair of counters
+  int counter;                          // index of the unit's counter
   float* ypart;                         // [ni][ranks][cj cb 128] partial sums of Y; twice, by turns, where sub = 0
   float* y;                             // [ranks][cj cb 128], where sub > 0
   double* gshare;                       // [clusters][layers][192], where sub > 0
@@ -43,9 +43,14 @@ struct ResidentParams {
   unsigned long long seed;
   DevStatus* status;                    // may be null
   int* flag;                            // may be null: set to whether a column was dependent
-  unsigned* counters;                   // two per unit, zero between launches
+  unsigned* counters;                   // one per unit
   ResidentUnit unit[kResMaxUnits];
 };
+
+// What an arrival adds to a unit's counter: each of n CTAs once, 2^31 in all, the high bit turning with the last one whatever the
+// order.  So a meeting leaves the low bits as it found them, and nothing has to be set back: launches that overlap against the rules
+// (two streams without an order) spoil one another's results, but when they are over the counter serves the next one again.
+__host__ __device__ constexpr unsigned meeting_increment(int n, bool first) { return first ? 0x80000000u - (unsigned)(n - 1) : 1u; }
 
 struct ResidentCaps {
   int sm_count = 0;

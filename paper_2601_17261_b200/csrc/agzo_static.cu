@@ -19,11 +19,11 @@ constexpr size_t kStaticScratchBytes = 4u << 20;   // 4 MiB, held by every GPU t
 // The name below is a host-side handle for the symbol, not a device address: kernels must be
 // given the address that cudaGetSymbolAddress returns for the current device.
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
-// What the resident kernel needs where the problem fits the limit above (a partial sum of Y per row of CTAs), and its counters,
-// which are zero between launches.
+// What the resident kernel needs where the problem fits the limit above (a partial sum of Y per row of CTAs), and its counter, which
+// a launch leaves as good as it found it.
 constexpr size_t kResidentScratchBytes = 5u << 20;
 static __device__ __align__(256) unsigned char g_resident_scratch[kResidentScratchBytes];
-static __device__ unsigned g_resident_counters[2];
+static __device__ unsigned g_resident_counter;
 
 // Looked up once per CUDA context: the address and the kernels' limits end with it (cudaDeviceReset).
 struct Scratch {
@@ -33,7 +33,7 @@ struct Scratch {
   int sm_count;
   agzo::ResidentCaps resident;
   void* resident_addr;
-  void* resident_counters;
+  void* resident_counter;
 };
 std::mutex g_mu;
 Scratch g_scratch[agzo::kMaxDevices] = {};
@@ -51,7 +51,7 @@ cudaError_t scratch_of_current_device(Scratch* out) {
     fresh.context = id;
     e = cudaGetSymbolAddress(&fresh.addr, g_static_scratch);   // with that device current
     if (e == cudaSuccess) e = cudaGetSymbolAddress(&fresh.resident_addr, g_resident_scratch);
-    if (e == cudaSuccess) e = cudaGetSymbolAddress(&fresh.resident_counters, g_resident_counters);
+    if (e == cudaSuccess) e = cudaGetSymbolAddress(&fresh.resident_counter, g_resident_counter);
     if (e == cudaSuccess) e = agzo::panel_qr_init(&fresh.qr_wide);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&fresh.sm_count, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = agzo::resident_init(fresh.sm_count, &fresh.resident);
@@ -122,7 +122,7 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
       plan.p.K = K;
       plan.p.seed = seed;
       plan.p.flag = d_rank_deficient;
-      plan.p.counters = static_cast<unsigned*>(scratch.resident_counters);
+      plan.p.counters = static_cast<unsigned*>(scratch.resident_counter);
       const cudaError_t e = launch_resident(plan, s);
       if (e == cudaSuccess) return AGZO_OK;
       if (!resident_refused(e)) return AGZO_ERR_CUDA;

@@ -134,6 +134,32 @@ def test_fused_work_split_covers_every_tile_once(lib):
     assert lib.agzo_debug_fused_split(bad, 1, 0, out, out, out, out, C.byref(n)) == B.AGZO_ERR_INVALID_ARG
 
 
+def test_meetings_leave_the_counter_as_they_found_it(lib):
+    # the resident extraction's counter: its high bit turns with the last arrival of a meeting, in whatever order they come, and
+    # launches whose arrivals mix (which the rules forbid) leave the low bits at zero, so that later meetings are whole again
+    import random
+    rng = random.Random(5)
+    first, other = C.c_uint32(), C.c_uint32()
+
+    def arrivals(n):
+        assert lib.agzo_debug_meeting_increments(n, C.byref(first), C.byref(other)) == B.AGZO_OK
+        return [first.value] + [other.value] * (n - 1)
+
+    for n in (1, 2, 8, 40, 128, 148, 1024):
+        for high in (0, 1 << 31):
+            a, at = arrivals(n), high
+            rng.shuffle(a)
+            for k, x in enumerate(a):
+                at = (at + x) % 2 ** 32
+                assert ((at ^ high) >> 31 == 1) == (k == n - 1), (n, k)
+            assert at == high ^ 1 << 31
+    for _ in range(20):
+        mixed = [x for n in rng.choices(range(1, 149), k=6) for x in arrivals(n)]
+        rng.shuffle(mixed)
+        assert sum(mixed) % 2 ** 31 == 0
+    assert lib.agzo_debug_meeting_increments(0, C.byref(first), C.byref(other)) == B.AGZO_ERR_INVALID_ARG
+
+
 def test_missing_library_fails_loudly(monkeypatch):
     monkeypatch.setattr(B, "_lib", None)
     monkeypatch.setattr(B, "LIB_PATH", "/nonexistent/libagzo.so")
