@@ -337,7 +337,9 @@ agzo_status agzo_fill_gaussian_basis(agzo_ctx* ctx, const agzo_layer* h_layers, 
  * library's kernels, for which the driver may set device memory aside; from the second call
  * on a device the free device memory is the same before and after a call.)
  *   X [m][ldx] (x_dtype), V [r][ldv] fp32 out, d_rank_deficient: optional device int32 that
- *   receives 1 when a panel column was zeroed (see AGZO_WARN_RANK_DEFICIENT), else 0.
+ *   receives 1 when a panel column was zeroed (see AGZO_WARN_RANK_DEFICIENT), else 0; 2 when a
+ *   bounded wait of the kernel ran out (its blocks waited two seconds for one another, for which
+ *   the device must have been kept from running them): V is zero then.
  * Limit: the scratch of the problem must fit the array,
  *   512 + 4 m r + 4 slabs r d_in + 4 r d_in + 8 ceil(d_in/128) r^2 + 8 r^2  <=  4 MiB
  *   (each term rounded up to 256 bytes; slabs = ceil(m / max(256, ceil32(ceil(m/32)))));
@@ -387,9 +389,19 @@ agzo_status agzo_debug_fused_split(const int32_t* h_tiles, int n, int clusters, 
                                    int32_t* h_first, int32_t* h_parts, int32_t* h_share_begin,
                                    int32_t* h_shares);
 
-/* Test export, host only: what the arrivals of n blocks at a meeting of the resident extraction add to its counter, the
- * first block's and every other one's.                                                     */
-agzo_status agzo_debug_meeting_increments(int32_t n, uint32_t* h_first, uint32_t* h_other);
+/* Test export: agzo_extract_subspace_static by the kernels that `route` names, 0 = the faster ones, 1 = the chain of CUDA-core
+ * kernels, 2 = the resident kernel (UNSUPPORTED where it does not take the layer), whose waits for other blocks end after
+ * wait_ns nanoseconds (at most the two seconds that they otherwise do; where it is less, one block comes to every meeting of
+ * several clusters 0.1 ms later than that).                                                */
+agzo_status agzo_debug_extract_static(const void* X, int64_t ldx, int32_t x_dtype, int32_t m, int32_t d_in, int32_t r, int32_t K,
+                                      uint64_t seed, uint32_t layer_id, float* V, int64_t ldv,
+                                      int32_t* d_rank_deficient, int32_t route, int64_t wait_ns, void* stream);
+
+/* Test export, host only: the counter at which the n blocks of a resident extraction meet.  What the first block's arrival
+ * (first != 0) or another one's adds to it while it shows `phase`, and the phase and the number of waits that ran out which
+ * `value` shows.                                                                           */
+agzo_status agzo_debug_meeting(int32_t n, int32_t first, uint32_t phase, uint64_t value, uint64_t* h_increment, uint32_t* h_phase,
+                               uint32_t* h_failures);
 
 /* Exercises the bounded device-side wait that every pipeline of the tensor-core kernels uses:
  * launches one small block that waits, with the library's own wait routine, on a barrier that

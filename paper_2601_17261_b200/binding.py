@@ -35,7 +35,8 @@ EXPORTS = [
     "agzo_perturb_dense", "agzo_debug_philox", "agzo_debug_gaussian", "agzo_read_counters",
     "agzo_extract_subspace_static", "agzo_fill_gaussian_basis", "agzo_set_allreduce",
     "agzo_debug_wait_timeout", "agzo_query_fused", "agzo_query_cluster_capacity", "agzo_debug_fused_split",
-    "agzo_debug_early_copy", "agzo_debug_normal_parts", "agzo_debug_meeting_increments",
+    "agzo_debug_early_copy", "agzo_debug_normal_parts", "agzo_debug_meeting",
+    "agzo_debug_extract_static",
 ]
 KC_RMW, KC_XT_T, KC_X_Q, KC_PANEL_QR, KC_TC_XT_T, KC_TC_X_Q, KC_OMEGA, KC_RMW_TC, KC_FUSED_POWER = 1, 2, 3, 4, 5, 6, 7, 8, 9
 
@@ -106,7 +107,9 @@ def lib() -> C.CDLL:
         "agzo_read_counters": (i32, [vp, C.POINTER(C.c_double), C.POINTER(i64), C.POINTER(i64)]),
         "agzo_set_allreduce": (i32, [vp, ALLREDUCE_FN, vp, i64]),
         "agzo_debug_wait_timeout": (i32, [vp, vp]),
-        "agzo_debug_meeting_increments": (i32, [i32, C.POINTER(u32), C.POINTER(u32)]),
+        "agzo_debug_extract_static": (i32, [vp, i64, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int32, u64, u32, vp, i64, vp,
+                                            C.c_int32, i64, vp]),
+        "agzo_debug_meeting": (i32, [i32, i32, u32, u64, C.POINTER(u64), C.POINTER(u32), C.POINTER(u32)]),
         "agzo_query_fused": (i32, [vp, LP, i32, C.POINTER(C.c_int32), vp]),
         "agzo_query_cluster_capacity": (i32, [vp, C.POINTER(C.c_int32)]),
         "agzo_debug_fused_split": (i32, [C.POINTER(C.c_int32), i32, i32, C.POINTER(C.c_int32), C.POINTER(C.c_int32),
@@ -293,6 +296,18 @@ def agzo_extract_subspace_static(X: torch.Tensor, V: torch.Tensor, r: int, K: in
                                               X.shape[1], r, K, seed, layer_id, V.data_ptr(),
                                               V.stride(0), flag, _stream_ptr(stream)),
            "agzo_extract_subspace_static")
+
+
+STATIC_CHAIN, STATIC_RESIDENT = 1, 2
+
+
+def agzo_debug_extract_static(X: torch.Tensor, V: torch.Tensor, r: int, K: int, seed: int, layer_id: int, route: int,
+                              d_rank_deficient: Optional[torch.Tensor] = None, wait_ns: int = 2_000_000_000, stream=None) -> None:
+    """agzo_extract_subspace_static by the kernels that `route` names (see include/agzo.h)."""
+    flag = d_rank_deficient.data_ptr() if d_rank_deficient is not None else None
+    _check(lib().agzo_debug_extract_static(X.data_ptr(), X.stride(0), _dtype_code(X), X.shape[0], X.shape[1], r, K, seed, layer_id,
+                                           V.data_ptr(), V.stride(0), flag, route, wait_ns, _stream_ptr(stream)),
+           "agzo_debug_extract_static")
 
 
 def agzo_fill_gaussian_basis(ctx: Context, layers, seed: int, stream=None, arr=None) -> None:

@@ -21,7 +21,7 @@ constexpr uint32_t kMagic = 0xA620B200u;
 constexpr size_t kAlign = 256;
 constexpr size_t kHeaderBytes = 256;          // DevStatus, and from kCountersAt on the counters of the resident extraction
 constexpr size_t kCountersAt = 128;
-static_assert(sizeof(DevStatus) <= kCountersAt && kCountersAt + kResMaxUnits * sizeof(unsigned) <= kHeaderBytes, "header");
+static_assert(sizeof(DevStatus) <= kCountersAt && kCountersAt + kResMaxUnits * sizeof(unsigned long long) <= kHeaderBytes, "header");
 constexpr int64_t kDefaultWaveBytes = 8ll << 30;
 constexpr int64_t kL2ResidentWaveBytes = 64ll << 20;   // a wave's X up to this size is still in L2 at its next sweep
 
@@ -1040,7 +1040,7 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
     p.seed = seed;
     p.status = dev_status(ctx);
     p.flag = nullptr;
-    p.counters = reinterpret_cast<unsigned*>(ctx->ws + kCountersAt);
+    p.counters = reinterpret_cast<unsigned long long*>(ctx->ws + kCountersAt);
     const cudaError_t e = launch_resident(ctx->resident, s);
     if (e == cudaSuccess) { ctx->launches += 1; return AGZO_OK; }
     ctx->resident_ok = false;
@@ -1357,10 +1357,12 @@ agzo_status agzo_debug_fused_split(const int32_t* h_tiles, int n, int clusters, 
   return AGZO_OK;
 }
 
-agzo_status agzo_debug_meeting_increments(int32_t n, uint32_t* h_first, uint32_t* h_other) {
-  if (n < 1 || !h_first || !h_other) return AGZO_ERR_INVALID_ARG;
-  *h_first = meeting_increment(n, true);
-  *h_other = meeting_increment(n, false);
+agzo_status agzo_debug_meeting(int32_t n, int32_t first, uint32_t phase, uint64_t value, uint64_t* h_increment, uint32_t* h_phase,
+                               uint32_t* h_failures) {
+  if (n < 1 || phase > 1 || !h_increment || !h_phase || !h_failures) return AGZO_ERR_INVALID_ARG;
+  *h_increment = meeting_increment(n, first != 0, phase);
+  *h_phase = meeting_phase(value);
+  *h_failures = meeting_failures(value);
   return AGZO_OK;
 }
 

@@ -89,6 +89,9 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
   asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
   return v;
 }
+__device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
 __device__ __forceinline__ void st_cluster_u4(uint32_t addr, uint4 v) {
   asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
@@ -224,8 +227,16 @@ __device__ __forceinline__ void tmem_sum8(uint32_t at, int NP, int NB, int chunk
 }
 
 // All CTAs of a unit meet, and what they wrote to global memory before is visible after.  Where the unit is one cluster, the
-// cluster's barrier; else a counter that a meeting advances by 2^31 (meeting_increment): who waits does so for the high bit to turn.
-__device__ __forceinline__ void unit_barrier(unsigned* counter, int clusters, int cs, bool first, unsigned* phase, ResShared* sh) {
+// cluster's barrier; else a counter (Meeting).  A CTA that has given up waiting says so in the counter while the meeting still lacks
+// somebody, so that whoever completes it or finds it complete sees that too: all of them have sh->failed set from there on.  (One that
+// starts only then takes what it finds for the count of earlier launches; the others say so again at the next meeting.)
+struct Meeting {
+  unsigned long long* counter;
+  int n;                          // CTAs
+  bool first;
+  unsigned phase, failures;       // what it showed before the launch (thread 0)
+};
+__device__ __forceinline__ void unit_barrier(Meeting& m, int clusters, int cs, const ResidentParams& P, ResShared* sh) {
   if (clusters == 1) {
     __syncwarp();
     if (cs > 1) cluster_sync_all(); else __syncthreads();
@@ -233,16 +244,24 @@ __device__ __forceinline__ void unit_barrier(unsigned* counter, int clusters, in
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(counter), "r"(meeting_increment(clusters * cs, first)) : "memory");
-    *phase ^= 0x80000000u;
+    if (m.first && P.late_ns) {
+      const unsigned long long t_late = global_ns() + P.late_ns;
+      while (global_ns() < t_late) {}
+    }
+    const unsigned long long add = meeting_increment(m.n, m.first, m.phase) + (sh->failed ? kMeetingFailure : 0ull);
+    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(m.counter), "l"(add) : "memory");
+    m.phase ^= 1u;
     if (!sh->failed) {
       const unsigned long long t_start = global_ns();
 #pragma unroll 1
       for (;;) {
-        unsigned got;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(got) : "l"(counter) : "memory");
-        if (((got ^ *phase) & 0x80000000u) == 0u) break;
-        if (global_ns() - t_start > kWaitCapNs) { sh->failed = 1; break; }
+        unsigned long long got;
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(got) : "l"(m.counter) : "memory");
+        if (meeting_phase(got) == m.phase) {
+          if (meeting_failures(got) != m.failures) sh->failed = 1;
+          break;
+        }
+        if (global_ns() - t_start > P.wait_ns && atomicCAS(m.counter, got, got + kMeetingFailure) == got) { sh->failed = 1; break; }
       }
     }
   }
@@ -375,8 +394,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
   const int cj = U.cj, j = rank % cj, row0 = rank - j, ni = U.ni, i = (cluster - U.cluster0) * (cs / cj) + rank / cj;
   const int cb = U.cb, tb = U.tb, NB = U.NB, NP = U.NP, ranks = U.ranks, nl = U.n_layers, clusters = U.clusters;
   const int ncols = cb * kBlock, col0 = j * ncols, cols_pad = cj * ncols, t0 = i * tb * kBlock, pitch = qr_pitch(ncols);
-  unsigned* counter = P.counters + U.counter;
-  unsigned phase = 0;             // of the counter, thread 0
+  Meeting meeting{P.counters + U.counter, clusters * cs, i == 0 && j == 0, 0u, 0u};
 
   const int plane = tb * cb * 2 * kSlotBytes;
   uint8_t* sX = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -415,7 +433,11 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
   __syncthreads();
   if (!(PLANES == 1 && U.x_vec)) fill_omega<PARTS>(U, sT, t0, tb, P.seed);      // needs nothing from before the launch
   chain_wait();
-  if (clusters > 1 && tid == 0) phase = __ldcg(counter) & 0x80000000u;      // nobody turns it before this CTA has arrived
+  if (clusters > 1 && tid == 0) {         // no meeting of this launch is complete before this CTA has arrived
+    const unsigned long long now = __ldcg(meeting.counter);
+    meeting.phase = meeting_phase(now);
+    meeting.failures = meeting_failures(now);
+  }
   load_x<PLANES>(U, sX, plane, t0, col0, tb, cb);
   if (PLANES == 1 && U.x_vec) fill_omega<PARTS>(U, sT, t0, tb, P.seed);         // while X arrives
   asm volatile("cp.async.wait_all;" ::: "memory");
@@ -475,7 +497,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
       for (int k = tid; k < pad * (pitch / 4); k += kThreads) y[k] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     if (!direct) {
-      unit_barrier(counter, clusters, cs, i == 0 && j == 0, &phase, &sh);
+      unit_barrier(meeting, clusters, cs, P, &sh);
       const long long part = (long long)ranks * cols_pad;
       if (U.sub == 0) {              // a warp per rank and 128 columns, three of them and five partial sums in flight
         constexpr int kE = 3, kP = 5;
@@ -578,6 +600,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
       for (int w = 0; w < kWarps; ++w) sum += v[w];
       sG[e] = sum;
     }
+    if (sh.failed && tid < cs && cs > 1) st_cluster_u32(mapa_shared(smem_u32(&sh.failed), (uint32_t)tid), 1u);      // all of the cluster know
     __syncwarp();
     if (cs > 1) cluster_sync_all(); else __syncthreads();
     {
@@ -600,7 +623,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
           if (wide) U.gshare[(cluster - U.cluster0) * n_share + e] = sum; else place(e, sum);
         }
       if (wide) {
-        unit_barrier(counter, clusters, cs, i == 0 && j == 0, &phase, &sh);
+        unit_barrier(meeting, clusters, cs, P, &sh);
 #pragma unroll 1
         for (int e = tid; e < n_share; e += kThreads) {
           double sum = 0.0;
@@ -644,6 +667,11 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
       }
     }
     __syncthreads();
+    if (last && sh.failed) {             // a wait has run out and the sums are not whole: V = 0, with which a pass changes nothing
+      for (int k = tid; k < nl * kAmBytes / 4; k += kThreads) reinterpret_cast<uint32_t*>(sAM)[k] = 0u;
+      for (int k = tid; k < U.rows * pitch; k += kThreads) sY[k] = 0.f;
+      __syncthreads();
+    }
     // ---------------------------------------------------------------- Q = Y M: the operand, or V (whose strips the rows of CTAs share)
 #pragma unroll 1
     for (int l = 0; l < nl; ++l) {
@@ -744,7 +772,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
     if (sh.failed && P.status) { atomicExch(&P.status->timeout, 1); atomicExch(&P.status->where, 5); }
     if (i == 0 && j == 0) {
       if (P.status && sh.st.rank_deficient) atomicExch(&P.status->rank_deficient, 1);
-      if (P.flag) *P.flag = sh.st.rank_deficient;
+      if (P.flag) *P.flag = sh.failed ? 2 : sh.st.rank_deficient;
     }
   }
   if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem, ncol); }
@@ -939,6 +967,7 @@ bool resident_plan(const ResidentCaps& caps, const agzo_layer* L, int n, bool sh
   ResidentParams& p = out->p;
   p = ResidentParams{};
   p.n_units = (int)units.size();
+  p.wait_ns = ptx::kWaitCapNs;
   p.cs = cs;
   out->planes = planes; out->parts = parts;
   out->n_clusters = 0; out->grid_wide = false; out->smem = 0;

@@ -39,18 +39,26 @@ struct ResidentUnit {
   ResidentLayer layer[kResMaxLayers];
 };
 struct ResidentParams {
-  int n_units, cs, K, pad;
+  int n_units, cs, K;
+  unsigned long long wait_ns;           // limit of a wait for the other CTAs of a unit
+  unsigned long long late_ns;           // a test's: how late the unit's first CTA comes to a meeting
   unsigned long long seed;
   DevStatus* status;                    // may be null
-  int* flag;                            // may be null: set to whether a column was dependent
-  unsigned* counters;                   // one per unit
+  int* flag;                            // may be null: set to whether a column was dependent, to 2 where a wait ran out
+  unsigned long long* counters;         // one per unit
   ResidentUnit unit[kResMaxUnits];
 };
 
-// What an arrival adds to a unit's counter: each of n CTAs once, 2^31 in all, the high bit turning with the last one whatever the
-// order.  So a meeting leaves the low bits as it found them, and nothing has to be set back: launches that overlap against the rules
-// (two streams without an order) spoil one another's results, but when they are over the counter serves the next one again.
-__host__ __device__ constexpr unsigned meeting_increment(int n, bool first) { return first ? 0x80000000u - (unsigned)(n - 1) : 1u; }
+// The counter at which n CTAs meet: bit 31 turns with the last arrival whatever the order, and the low bits are as they were then,
+// so nothing has to be set back.  Launches that overlap against the rules (two streams without an order) spoil one another's
+// results, but when they are over the counter serves the next one again.  The upper half counts waits that ran out; a meeting that
+// turns the bit back to zero borrows one from it until it is complete (bits 31 and 30 are both set then, and only then).
+__host__ __device__ constexpr unsigned long long meeting_increment(int n, bool first, unsigned phase) {
+  return first ? (phase ? 0ull - (1ull << 31) : 1ull << 31) - (unsigned long long)(n - 1) : 1ull;
+}
+constexpr unsigned long long kMeetingFailure = 1ull << 32;
+__host__ __device__ constexpr unsigned meeting_phase(unsigned long long v) { return (unsigned)(v >> 31) & 1u; }
+__host__ __device__ constexpr unsigned meeting_failures(unsigned long long v) { return (unsigned)(v >> 32) + (((unsigned)v >> 30) == 3u ? 1u : 0u); }
 
 struct ResidentCaps {
   int sm_count = 0;

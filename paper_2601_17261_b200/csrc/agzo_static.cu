@@ -10,6 +10,7 @@
 #include <mutex>
 
 #include "agzo_common.cuh"
+#include "agzo_ptx.cuh"
 #include "agzo_resident.cuh"
 
 namespace {
@@ -23,7 +24,7 @@ static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBy
 // a launch leaves as good as it found it.
 constexpr size_t kResidentScratchBytes = 5u << 20;
 static __device__ __align__(256) unsigned char g_resident_scratch[kResidentScratchBytes];
-static __device__ unsigned g_resident_counter;
+static __device__ unsigned long long g_resident_counter;
 
 // Looked up once per CUDA context: the address and the kernels' limits end with it (cudaDeviceReset).
 struct Scratch {
@@ -84,11 +85,12 @@ __global__ void static_end_kernel(const agzo::DevStatus* st, int32_t* flag) {
 
 }  // namespace
 
-extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, int32_t x_dtype,
-                                                    int32_t m, int32_t d_in, int32_t r, int32_t K,
-                                                    uint64_t seed, uint32_t layer_id, float* V,
-                                                    int64_t ldv, int32_t* d_rank_deficient,
-                                                    void* stream) {
+namespace {
+
+// route: 0 = the faster kernels, 1 = the chain, 2 = the resident kernel, whose waits for other blocks end after wait_ns
+agzo_status extract_static(const void* X, int64_t ldx, int32_t x_dtype, int32_t m, int32_t d_in, int32_t r, int32_t K, uint64_t seed,
+                           uint32_t layer_id, float* V, int64_t ldv, int32_t* d_rank_deficient, int route, unsigned long long wait_ns,
+                           void* stream) {
   using namespace agzo;
   if (!X || !V || m < 1 || d_in < 1 || r < 1 || r > AGZO_MAX_RANK || r > d_in || r > m ||
       ldx < d_in || ldv < d_in || K < 0 || K > 16)
@@ -112,21 +114,25 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
   Scratch scratch;
   if (scratch_of_current_device(&scratch) != cudaSuccess) return AGZO_ERR_CUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  {
+  if (route != 1) {
     agzo_layer a{};
     a.X = X; a.ldx = ldx; a.x_dtype = x_dtype; a.m = m; a.d_in = d_in; a.r = r; a.layer_id = layer_id;
     a.V = V; a.ldv = ldv;
-    ResidentLaunch plan;
-    if (resident_plan(scratch.resident, &a, 1, false, false, &plan) && plan.scratch <= kResidentScratchBytes && resident_pays(plan, K)) {
+    ResidentLaunch plan;      // K = 0: a block that comes too late to the only meeting would not see that others have given up
+    if (resident_plan(scratch.resident, &a, 1, false, false, &plan) && plan.scratch <= kResidentScratchBytes &&
+        !(plan.grid_wide && K == 0) && (route == 2 || resident_pays(plan, K))) {
       resident_bind(&plan, static_cast<char*>(scratch.resident_addr));
       plan.p.K = K;
+      plan.p.wait_ns = wait_ns;
+      plan.p.late_ns = wait_ns < ptx::kWaitCapNs ? wait_ns + 100000 : 0;
       plan.p.seed = seed;
       plan.p.flag = d_rank_deficient;
-      plan.p.counters = static_cast<unsigned*>(scratch.resident_counter);
+      plan.p.counters = static_cast<unsigned long long*>(scratch.resident_counter);
       const cudaError_t e = launch_resident(plan, s);
       if (e == cudaSuccess) return AGZO_OK;
       if (!resident_refused(e)) return AGZO_ERR_CUDA;
     }
+    if (route == 2) return AGZO_ERR_UNSUPPORTED;
   }
   for (int rows = cc_slab_rows(m, (long long)gch, scratch.sm_count);; rows += 32) {      // ends at 256 tokens per slab at the latest
     const size_t n = ((size_t)m + rows - 1) / rows;
@@ -168,4 +174,21 @@ extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, 
     if (launch_chained(static_end_kernel, dim3(1), 1, 0, 0, s, d_status, d_rank_deficient) != cudaSuccess) return AGZO_ERR_CUDA;
   }
   return AGZO_OK;
+}
+
+}  // namespace
+
+extern "C" agzo_status agzo_extract_subspace_static(const void* X, int64_t ldx, int32_t x_dtype,
+                                                    int32_t m, int32_t d_in, int32_t r, int32_t K,
+                                                    uint64_t seed, uint32_t layer_id, float* V,
+                                                    int64_t ldv, int32_t* d_rank_deficient,
+                                                    void* stream) {
+  return extract_static(X, ldx, x_dtype, m, d_in, r, K, seed, layer_id, V, ldv, d_rank_deficient, 0, agzo::ptx::kWaitCapNs, stream);
+}
+
+extern "C" agzo_status agzo_debug_extract_static(const void* X, int64_t ldx, int32_t x_dtype, int32_t m, int32_t d_in, int32_t r,
+                                                 int32_t K, uint64_t seed, uint32_t layer_id, float* V, int64_t ldv,
+                                                 int32_t* d_rank_deficient, int32_t route, int64_t wait_ns, void* stream) {
+  if (route < 0 || route > 2 || wait_ns < 0 || (unsigned long long)wait_ns > agzo::ptx::kWaitCapNs) return AGZO_ERR_INVALID_ARG;
+  return extract_static(X, ldx, x_dtype, m, d_in, r, K, seed, layer_id, V, ldv, d_rank_deficient, route, (unsigned long long)wait_ns, stream);
 }

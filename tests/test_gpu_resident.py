@@ -144,3 +144,18 @@ def test_a_graph_of_it_replays():
             torch.cuda.synchronize()
             assert torch.equal(V, want)
         del graph
+
+
+def test_static_entry_reports_a_wait_that_ran_out():
+    # 128 blocks that meet eight times, one of which comes 0.1 ms later than the others wait
+    X = to_dev(WL.planted_activations(4096, 2048, 16, seed=3, bf16=True), True)[0]
+    want, V = torch.zeros(16, 2048, device=DEV), torch.zeros(16, 2048, device=DEV)
+    flag = torch.full((1,), -1, dtype=torch.int32, device=DEV)
+    B.agzo_debug_extract_static(X, want, 16, 3, 5, 1, B.STATIC_RESIDENT, flag)
+    assert flag.item() == 0 and want.any()
+    for _ in range(3):
+        V.fill_(7.0)
+        B.agzo_debug_extract_static(X, V, 16, 3, 5, 1, B.STATIC_RESIDENT, flag, wait_ns=0)
+        assert flag.item() == 2 and not V.any()
+        B.agzo_extract_subspace_static(X, V, 16, 3, 5, 1, flag)         # the next call is whole again
+        assert flag.item() == 0 and torch.equal(V, want)

@@ -135,29 +135,48 @@ def test_fused_work_split_covers_every_tile_once(lib):
 
 
 def test_meetings_leave_the_counter_as_they_found_it(lib):
-    # the resident extraction's counter: its high bit turns with the last arrival of a meeting, in whatever order they come, and
-    # launches whose arrivals mix (which the rules forbid) leave the low bits at zero, so that later meetings are whole again
+    # the resident extraction's counter: its phase turns with the last arrival of a meeting, in whatever order they come and whoever
+    # of the next meeting is there already, and everyone who sees it turned sees the waits that ran out before; launches whose
+    # arrivals mix (which the rules forbid) leave the low bits at zero, so that later meetings are whole again
     import random
     rng = random.Random(5)
-    first, other = C.c_uint32(), C.c_uint32()
+    inc, ph, fails = C.c_uint64(), C.c_uint32(), C.c_uint32()
 
-    def arrivals(n):
-        assert lib.agzo_debug_meeting_increments(n, C.byref(first), C.byref(other)) == B.AGZO_OK
-        return [first.value] + [other.value] * (n - 1)
+    def read(v):
+        assert lib.agzo_debug_meeting(1, 0, 0, v % 2 ** 64, C.byref(inc), C.byref(ph), C.byref(fails)) == B.AGZO_OK
+        return ph.value, fails.value
 
-    for n in (1, 2, 8, 40, 128, 148, 1024):
-        for high in (0, 1 << 31):
-            a, at = arrivals(n), high
-            rng.shuffle(a)
-            for k, x in enumerate(a):
-                at = (at + x) % 2 ** 32
-                assert ((at ^ high) >> 31 == 1) == (k == n - 1), (n, k)
-            assert at == high ^ 1 << 31
+    def arrivals(n, phase):
+        out = []
+        for k in range(n):
+            assert lib.agzo_debug_meeting(n, k == 0, phase, 0, C.byref(inc), C.byref(ph), C.byref(fails)) == B.AGZO_OK
+            out.append(inc.value)
+        return out
+
+    for n in (2, 8, 40, 128, 148, 1024):
+        for start in (0, 5, 2 ** 32 - 1):                        # waits that ran out in earlier launches
+            at, failed = start << 32, start
+            for meeting in range(6):
+                a = arrivals(n, meeting & 1)
+                rng.shuffle(a)
+                for k, x in enumerate(a):
+                    assert read(at) == (meeting & 1, failed), (n, meeting, k)      # what a late reader of the one before finds, too
+                    if rng.random() < 0.3 / n ** 0.5:
+                        at, failed = (at + 2 ** 32) % 2 ** 64, (failed + 1) % 2 ** 32
+                        assert read(at) == (meeting & 1, failed)
+                    at = (at + x) % 2 ** 64
+                assert read(at) == (1 - (meeting & 1), failed) and at % 2 ** 31 == 0
     for _ in range(20):
-        mixed = [x for n in rng.choices(range(1, 149), k=6) for x in arrivals(n)]
+        mixed = [x for n in rng.choices(range(2, 149), k=6) for x in arrivals(n, rng.randint(0, 1))]
         rng.shuffle(mixed)
         assert sum(mixed) % 2 ** 31 == 0
-    assert lib.agzo_debug_meeting_increments(0, C.byref(first), C.byref(other)) == B.AGZO_ERR_INVALID_ARG
+    assert lib.agzo_debug_meeting(0, 0, 0, 0, C.byref(inc), C.byref(ph), C.byref(fails)) == B.AGZO_ERR_INVALID_ARG
+
+
+def test_static_routes_are_checked(lib):
+    bad = [(-1, 0), (3, 0), (2, -1), (2, 2_000_000_001)]
+    for route, wait in bad:
+        assert lib.agzo_debug_extract_static(64, 64, 0, 64, 64, 4, 1, 0, 0, 64, 64, None, route, wait, None) == B.AGZO_ERR_INVALID_ARG
 
 
 def test_missing_library_fails_loudly(monkeypatch):
