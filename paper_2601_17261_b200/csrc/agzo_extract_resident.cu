@@ -987,6 +987,9 @@ bool resident_plan(const ResidentCaps& caps, const agzo_layer* L, int n, bool sh
 
 // One launch costs 4.8 us beside its K + 1 rounds, a cooperative one 5.5
 bool resident_pays(const ResidentLaunch& plan, int K) {
+  // Below 2^-109 an fp32 value's third part is no bf16 number any more.  With a power step such inputs underflow whatever the kernel,
+  // without one the fp32 products keep them (2^-118 of N(0, 1): 5e-9 against 64 bits, the parts 9e-6): they stay there.
+  if (K == 0 && plan.planes == 3) return false;
   return (plan.grid_wide ? 5.5 : 4.8) + (K + 1) * plan.round_us < 0.97 * (K + 1) * plan.others_us;
 }
 

@@ -159,3 +159,22 @@ def test_static_entry_reports_a_wait_that_ran_out():
         assert flag.item() == 2 and not V.any()
         B.agzo_extract_subspace_static(X, V, 16, 3, 5, 1, flag)         # the next call is whole again
         assert flag.item() == 0 and torch.equal(V, want)
+
+
+@pytest.mark.parametrize("d_in", [128, 130])
+def test_tiny_fp32_inputs_keep_their_bits(d_in):
+    # scaled by a power of two that leaves every element a normal fp32 number: without a power step nothing underflows, so V is that of
+    # the unscaled inputs to fp32 rounding of sums of 300 terms (300 x 2^-24 = 2e-5 at worst, 1e-6 with rounding errors of random sign)
+    X = to_dev(WL.planted_activations(300, d_in, 16, seed=2, bf16=False), False)[0]
+    X = torch.where(X.abs() < 2.0 ** -6, torch.zeros_like(X), X)
+    tiny = X * 2.0 ** -118
+    assert torch.equal(tiny * 2.0 ** 118, X)
+    V, T = torch.zeros(8, d_in, device=DEV), torch.zeros(8, d_in, device=DEV)
+    one, two = [[B.make_layer(X=A, V=A2, r=8, layer_id=1)] for A, A2 in ((X, V), (tiny, T))]
+    with Ctx(one) as ctx:
+        B.agzo_extract_subspace(ctx, one, 5, 0)
+        B.agzo_extract_subspace(ctx, two, 5, 0)
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+    assert float((T - V).norm() / V.norm()) <= 1e-6
+    B.agzo_extract_subspace_static(tiny, T, 8, 0, 5, 1)
+    assert float((T - V).norm() / V.norm()) <= 1e-6
