@@ -164,7 +164,7 @@ agzo_status agzo_destroy(agzo_ctx* ctx);
  * "extract_resident" 1 (default) = a call whose activations all fit the device's shared memory (ranks of at most 16, at most
  * 24 over layers that share an X, at most 12 different X) is extracted by one kernel that keeps them there; it takes the place of
  * all others where it is estimated to be faster, unless an option asks for one of those ("extract_path", "extract_fused" other
- * than 1, "wave_bytes") or an all-reduce is set.  2 = wherever it can run, 0 = never;
+ * than 1, "wave_bytes"; "time_kernel_class" with a class of theirs) or an all-reduce is set.  2 = wherever it can run, 0 = never;
  * "wave_bytes" = activation bytes grouped into one launch wave of extraction;
  * "extract_streams" 2 (default) = alternate waves use two scratch regions and two helper
  * streams forked from and joined to the caller's stream, so that one wave's short kernels
@@ -211,7 +211,8 @@ typedef enum agzo_kernel_class {
   AGZO_KC_TC_X_Q = 6,     /* T = X Q, tensor-core kernel                                   */
   AGZO_KC_OMEGA = 7,      /* Gaussian test matrix fill                                     */
   AGZO_KC_RMW_TC = 8,     /* the in-place low-rank pass, tensor-core kernel                */
-  AGZO_KC_FUSED_POWER = 9 /* Y = X^T (X Q) in one pass over X, tensor-core cluster kernel  */
+  AGZO_KC_FUSED_POWER = 9,/* Y = X^T (X Q) in one pass over X, tensor-core cluster kernel  */
+  AGZO_KC_RESIDENT = 10   /* all of Algorithm 1 on inputs that the SMs hold                */
 } agzo_kernel_class;
 
 /* Measurement aid.  Waits for the timed launches recorded since the last read, then returns

@@ -38,7 +38,7 @@ EXPORTS = [
     "agzo_debug_early_copy", "agzo_debug_normal_parts", "agzo_debug_meeting",
     "agzo_debug_extract_static",
 ]
-KC_RMW, KC_XT_T, KC_X_Q, KC_PANEL_QR, KC_TC_XT_T, KC_TC_X_Q, KC_OMEGA, KC_RMW_TC, KC_FUSED_POWER = 1, 2, 3, 4, 5, 6, 7, 8, 9
+KC_RMW, KC_XT_T, KC_X_Q, KC_PANEL_QR, KC_TC_XT_T, KC_TC_X_Q, KC_OMEGA, KC_RMW_TC, KC_FUSED_POWER, KC_RESIDENT = 1, 2, 3, 4, 5, 6, 7, 8, 9, 10
 
 
 class agzo_layer(C.Structure):

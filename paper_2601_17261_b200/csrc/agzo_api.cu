@@ -679,8 +679,10 @@ agzo_status prepare(agzo_ctx* c, const agzo_layer* L, int n, cudaStream_t s) {
 // Whether the resident kernel extracts this list: c->resident is its launch then.  It takes part of the scratch area, at its
 // end, and leaves the tables of the list that was prepared last alone.
 bool plan_resident(agzo_ctx* c, const agzo_layer* L, int n) {
-  // an option that asks for one of the other paths, or cuts the list into waves, is meant for those
-  if (!c->extract_resident || c->allreduce || c->extract_path != 0 || c->extract_fused != 1 || c->wave_bytes != kDefaultWaveBytes) return false;
+  // an option that asks for one of the other paths, cuts the list into waves or times their kernels is meant for those
+  const bool times_others = c->time_class != AGZO_KC_NONE && c->time_class != AGZO_KC_RMW && c->time_class != AGZO_KC_RMW_TC &&
+                            c->time_class != AGZO_KC_RESIDENT;
+  if (times_others || !c->extract_resident || c->allreduce || c->extract_path != 0 || c->extract_fused != 1 || c->wave_bytes != kDefaultWaveBytes) return false;
   if (!c->resident_known || c->resident_cached.size() != (size_t)n ||
       std::memcmp(c->resident_cached.data(), L, (size_t)n * sizeof(agzo_layer)) != 0) {
     bool two_parts = c->tc.available;
@@ -943,7 +945,7 @@ agzo_status agzo_set_option(agzo_ctx* ctx, const char* name, int64_t value) {
     ctx->debug_fail_step_call = (int)value;
     return AGZO_OK;
   } else if (std::strcmp(name, "time_kernel_class") == 0) {
-    if (value < 0 || value > 9) return AGZO_ERR_INVALID_ARG;
+    if (value < 0 || value > AGZO_KC_RESIDENT) return AGZO_ERR_INVALID_ARG;
     ctx->time_class = (int)value;
     return AGZO_OK;
   } else {
@@ -1041,8 +1043,14 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
     p.status = dev_status(ctx);
     p.flag = nullptr;
     p.counters = reinterpret_cast<unsigned long long*>(ctx->ws + kCountersAt);
-    const cudaError_t e = launch_resident(ctx->resident, s);
-    if (e == cudaSuccess) { ctx->launches += 1; return AGZO_OK; }
+    cudaError_t e;
+    {
+      Timed t(ctx, AGZO_KC_RESIDENT, s);
+      e = launch_resident(ctx->resident, s);
+    }
+    if (e == cudaSuccess) return AGZO_OK;
+    ctx->launches -= 1;      // refused: not a launch, and no time of one
+    if (ctx->time_class == AGZO_KC_RESIDENT && ctx->events_used >= 2) ctx->events_used -= 2;
     ctx->resident_ok = false;
     if (!resident_refused(e)) { ctx->last_cuda = (int)e; return AGZO_ERR_CUDA; }
   }

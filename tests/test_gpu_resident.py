@@ -178,3 +178,19 @@ def test_tiny_fp32_inputs_keep_their_bits(d_in):
     assert float((T - V).norm() / V.norm()) <= 1e-6
     B.agzo_extract_subspace_static(tiny, T, 8, 0, 5, 1)
     assert float((T - V).norm() / V.norm()) <= 1e-6
+
+
+def test_kernel_classes_are_timed():
+    # asking for the time of a kernel of the chain has the chain run, asking for the resident kernel's or for a pass's does not
+    X = to_dev(WL.planted_activations(300, 256, 16, seed=1, bf16=True), True)[0]
+    V = torch.zeros(4, 256, device=DEV)
+    layers = [B.make_layer(X=X, V=V, r=4, layer_id=0)]
+    with Ctx(layers) as ctx:
+        B.agzo_extract_subspace(ctx, layers, 5, 2)
+        B.agzo_read_counters(ctx)
+        for kind, timed, all_of_them in ((B.KC_RESIDENT, 1, 1), (B.KC_RMW, 0, 1), (B.KC_PANEL_QR, 3, None), (B.KC_TC_XT_T, 3, None), (0, 0, 1)):
+            B.agzo_set_option(ctx, "time_kernel_class", kind)
+            B.agzo_extract_subspace(ctx, layers, 5, 2)
+            ms, n, total = B.agzo_read_counters(ctx)
+            assert n == timed and (ms > 0) == (timed > 0), kind
+            assert total == 1 if all_of_them else total > 3, kind
