@@ -95,6 +95,7 @@ struct agzo_ctx {
   // the layer list that extraction last looked at for that kernel, and what came of it
   std::vector<agzo_layer> resident_cached;
   bool resident_known, resident_ok;
+  int resident_admitted;   // whether the other kernels would take the list in this workspace: 1, 0, -1 not looked at yet
   ResidentLaunch resident;
   // staged R images in scratch: valid for this seed until the plan changes or extraction uses the scratch
   bool rimg_valid;
@@ -677,8 +678,10 @@ agzo_status prepare(agzo_ctx* c, const agzo_layer* L, int n, cudaStream_t s) {
 }
 
 // Whether the resident kernel extracts this list: c->resident is its launch then.  It takes part of the scratch area, at its
-// end, and leaves the tables of the list that was prepared last alone.
-bool plan_resident(agzo_ctx* c, const agzo_layer* L, int n) {
+// end, and leaves the tables of the list that was prepared last alone.  prepared: the tables are this list's.  What a list that goes to
+// the other kernels pays for the question is the layouts (1 us on the host); whether those would take the list, half a microsecond more
+// that their own planning repeats, is asked last.
+bool plan_resident(agzo_ctx* c, const agzo_layer* L, int n, int K, bool prepared) {
   // an option that asks for one of the other paths, cuts the list into waves or times their kernels is meant for those
   const bool times_others = c->time_class != AGZO_KC_NONE && c->time_class != AGZO_KC_RMW && c->time_class != AGZO_KC_RMW_TC &&
                             c->time_class != AGZO_KC_RESIDENT;
@@ -688,15 +691,18 @@ bool plan_resident(agzo_ctx* c, const agzo_layer* L, int n) {
     bool two_parts = c->tc.available;
     for (int i = 0; i < n && two_parts; ++i) two_parts = tc_eligible(L[i]);
     c->resident_ok = resident_plan(c->resident_caps, L, n, c->share_inputs != 0, two_parts, &c->resident);
-    // a workspace that the other kernels would refuse is refused by all
-    Plan others;
-    if (c->resident_ok)
-      c->resident_ok = kHeaderBytes + table_bytes(n) <= c->ws_bytes &&
-                       build_plan(L, n, c->ws, c->ws_bytes, plan_opts(c, 1), &others, nullptr) == AGZO_OK;
+    c->resident_admitted = -1;
     c->resident_cached.assign(L, L + n);
     c->resident_known = true;
   }
-  if (!c->resident_ok) return false;
+  if (!c->resident_ok || (c->extract_resident != 2 && !resident_pays(c->resident, K))) return false;
+  // a workspace that the other kernels would refuse is refused by all
+  if (c->resident_admitted < 0) {
+    Plan others;
+    c->resident_admitted = prepared || (kHeaderBytes + table_bytes(n) <= c->ws_bytes &&
+                                        build_plan(L, n, c->ws, c->ws_bytes, plan_opts(c, 1), &others, nullptr) == AGZO_OK);
+  }
+  if (!c->resident_admitted) return false;
   const size_t tables = kHeaderBytes + (c->cached_valid ? table_bytes((int)c->cached.size()) : 0);
   const size_t end = c->ws_bytes & ~(kAlign - 1), need = align_up(c->resident.scratch);
   if (end < tables || end - tables < need) return false;
@@ -841,6 +847,7 @@ agzo_status agzo_create(agzo_ctx** out, int device, void* workspace, size_t work
   c->share_inputs = 1;
   c->extract_resident = 1;
   c->resident_known = c->resident_ok = false;
+  c->resident_admitted = -1;
   c->aux[0] = c->aux[1] = nullptr;
   c->fork_ev = c->join_ev[0] = c->join_ev[1] = nullptr;
   c->cached_valid = false;
@@ -1034,7 +1041,7 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
   // capture leaves them in place for the graph.
   const bool tables = any_weights(h_layers, n) || (ctx->tables_captured && capture_of(s) == 0);
   if (tables && (st = prepare(ctx, h_layers, n, s)) != AGZO_OK) return st;
-  if (plan_resident(ctx, h_layers, n) && (ctx->extract_resident == 2 || resident_pays(ctx->resident, K))) {
+  if (plan_resident(ctx, h_layers, n, K, tables)) {
     // it reads no tables, so an upload that another stream has under way is not waited for (a capturing stream could not)
     ctx->rimg_valid = false;
     ResidentParams& p = ctx->resident.p;

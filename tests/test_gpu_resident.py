@@ -194,3 +194,18 @@ def test_kernel_classes_are_timed():
             ms, n, total = B.agzo_read_counters(ctx)
             assert n == timed and (ms > 0) == (timed > 0), kind
             assert total == 1 if all_of_them else total > 3, kind
+
+
+@pytest.mark.parametrize("resident", [0, 1, 2])
+def test_a_workspace_that_the_other_kernels_refuse_is_refused(resident):
+    X, V = torch.randn(2048, 256, device=DEV), torch.full((4, 256), 7.0, device=DEV)
+    layers = [B.make_layer(X=X, V=V, r=4, layer_id=0)]
+    ctx = B.Context(0, 16384)                                    # tables fit, T does not
+    B.agzo_set_option(ctx, "extract_resident", resident)
+    for _ in range(2):
+        with pytest.raises(B.AgzoError) as e:
+            B.agzo_extract_subspace(ctx, layers, 1, 3)
+        assert e.value.status == B.AGZO_ERR_WORKSPACE
+    torch.cuda.synchronize()
+    assert bool((V == 7.0).all())
+    B.agzo_destroy(ctx)
