@@ -695,7 +695,7 @@ bool plan_resident(agzo_ctx* c, const agzo_layer* L, int n, int K, bool prepared
     c->resident_cached.assign(L, L + n);
     c->resident_known = true;
   }
-  if (!c->resident_ok || (c->extract_resident != 2 && !resident_pays(c->resident, K))) return false;
+  if (!c->resident_ok || (c->extract_resident != 2 && !resident_pays(c->resident, K, !any_weights(L, n)))) return false;
   // a workspace that the other kernels would refuse is refused by all
   if (c->resident_admitted < 0) {
     Plan others;

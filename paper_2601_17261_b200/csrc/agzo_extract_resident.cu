@@ -801,8 +801,8 @@ struct Shape {
   double cost;
 };
 
-// The estimate: least squares over 196 layouts (256 to 4096 columns, 300 to 4000 tokens, one to three layers of ranks 1 to 16, K = 1 and
-// 3), 6 % rms; a unit of several clusters pays most for meeting.
+// The estimate that puts layouts in order: what it picks takes 0.6 % longer than the best of the layouts that were measured beside it
+// (geometric mean over 1236 units; a unit of several clusters pays most for meeting).
 Shape shape_of(const ResidentUnit& u, int planes, int cs, int cj, int cb, int tb) {
   Shape s{cj, cb, tb, 0, 0, 0, 0.0};
   const int blocks_m = (u.m + kBlock - 1) / kBlock, per = cs / cj;
@@ -823,31 +823,6 @@ Shape shape_of(const ResidentUnit& u, int planes, int cs, int cj, int cb, int tb
     s.cost += std::min(part, all);
   }
   return s;
-}
-
-// What a round of the other kernels takes (us): a chain of three launches whose time hardly depends on the size while all is in L2.
-// Fitted to the same lists; the products element by element take long enough not to be looked at.
-double round_of_others(const std::vector<ResidentUnit>& units, int planes, bool two_parts) {
-  double most = 0.0, all = 0.0, round = 0.0;
-  int layers = 0;
-  for (const ResidentUnit& u : units) {
-    if (!u.x_vec) return 1e9;
-    int rank = 0;
-    for (int l = 0; l < u.n_layers; ++l) rank = std::max(rank, u.layer[l].r);
-    const double md = 1e-6 * u.m * (double)u.d, m = 1e-3 * u.m, d = 1e-3 * u.d;
-    double t;
-    if (two_parts) t = 10.2 + (rank > 8 ? 2.2 : 0.0) + 1.1 * m + d + 0.22 * md + 0.08 * (u.ranks - rank);
-    else if (planes == 1) return 1e9;                       // bf16 by the fp32 kernels
-    else if (rank <= 4) t = 7.7 + 1.15 * m + 1.6 * d + 0.6 * md;
-    else if (rank <= 8) t = 9.0 + 1.4 * m + 1.9 * d + 0.7 * md;
-    else t = 12.0 + 2.2 * m + 5.5 * d + 0.8 * md;
-    if (!two_parts) t += 2.3 * md * (u.n_layers - 1);       // they read X once per layer
-    round = std::max(round, t);
-    most = std::max(most, md);
-    all += md;
-    layers += u.n_layers;
-  }
-  return round + (two_parts ? 0.55 : 2.3) * (all - most) + 0.15 * std::min(layers - 1, 8);
 }
 
 // Shapes for all units on clusters of cs CTAs within the device's clusters: from the fewest clusters on, the slowest unit gets more.
@@ -962,8 +937,6 @@ bool resident_plan(const ResidentCaps& caps, const agzo_layer* L, int n, bool sh
       cs = c; least = slowest; best = shapes;
     }
   if (cs == 0) return false;
-  out->round_us = least;
-  out->others_us = round_of_others(units, planes, parts == 2);
   ResidentParams& p = out->p;
   p = ResidentParams{};
   p.n_units = (int)units.size();
@@ -985,12 +958,88 @@ bool resident_plan(const ResidentCaps& caps, const agzo_layer* L, int n, bool sh
   return true;
 }
 
-// One launch costs 4.8 us beside its K + 1 rounds, a cooperative one 5.5
-bool resident_pays(const ResidentLaunch& plan, int K) {
+// ------------------------------------------------------------------ which kernels are the faster ones
+// Both sides as K + 1 times what every round has, K times what only those with T = X Q have, and the rest.  Weighted least squares over
+// 1800 units of one X and 230 lists of several, 32 to 8192 tokens, 32 to 4096 columns, one to four layers of ranks 1 to 16, K = 0, 1
+// and 3, all types and alignments.  The resident kernel is estimated to 4.6 % rms, the others to 4 to 6 % (8 % element by element).
+struct Rounds { double once, every, power; };
+
+Rounds resident_rounds(const ResidentUnit& u, int planes, int parts) {
+  int groups = 0, rank = 0;
+  for (int l = 0; l < u.n_layers; ++l) { groups += (u.layer[l].r + 7) / 8; rank = std::max(rank, u.layer[l].r); }
+  double cycles = 0.0;                 // of a product's instructions for 16 of the contracted dimension, all planes of X
+  for (int p = 0; p < planes; ++p) cycles += 32.0 + (double)(p == 0 ? u.NB : (3 - p) * u.NP) / 4.0;
+  const double blocks = u.tb * u.cb, panel = 0.01 * u.ranks * u.cb;
+  Rounds t;
+  t.once = (0.41 * planes + (u.x_vec ? 0.0 : 1.89)) * blocks;                    // X
+  t.every = 1.2 + 3.1 * (8.0 * blocks * cycles / 1900.0) + 0.56 * u.cb * groups + (rank > 4 ? 0.84 : 0.0) + (rank > 8 ? 2.0 : 0.0) +
+            0.53 * (u.n_layers - 1);
+  if (u.ni > 1) t.every += 0.73;
+  if (u.clusters > 1) t.every += 0.49;
+  if (u.sub) t.every += (u.clusters > 1 ? 2.92 : 1.43) + 1.08 * panel;
+  else if (u.ni > 1) t.every += 0.48 * ((u.ranks * u.cb + 23) / 24) * ((u.ni + 4) / 5) + 0.26 * u.ni * panel;
+  t.power = 0.71 + (u.cj > 1 ? 2.35 : 0.0) + 0.39 * u.tb * (u.NP / 8) * (parts == 3 ? 1.5 * u.cb : 1.0);
+  return t;
+}
+// The chain of launches, for the unit alone.  By kernels: tensor-core products, fp32 products on bf16 and on fp32 in 16- or 8-byte
+// pieces, element by element.  m, d in thousands, md in millions; r4, r8: ranks above 4, 8; more: md per further layer on the X, which
+// the fp32 products read once per layer.
+struct ChainFit {
+  double once;
+  double every, every_r4, every_r8, every_m, every_d, every_md, every_r8_d, every_r8_md, every_more;
+  double power, power_m, power_d, power_md, power_r4_d, power_r8_d, power_r8_md, power_more;
+};
+constexpr ChainFit kChain[3] = {
+    {3.66, 4.37, 1.35, 3.82, 0.83, 0.39, 0.39, 0.0, 0.86, 0.54, 3.49, 0.45, 1.74, 0.0, 0.91, 4.58, 0.93, 0.50},
+    {4.15, 4.19, 1.44, 3.46, 0.84, 0.36, 0.62, 0.0, 1.15, 0.93, 4.08, 0.33, 1.10, 0.0, 0.29, 2.68, 3.96, 0.66},
+    {4.54, 8.34, 2.90, 6.87, 2.38, 0.98, 0.71, 0.39, 0.96, 1.49, 3.80, 0.79, 5.78, 0.22, 7.01, 10.14, 1.62, 2.26}};
+
+Rounds other_rounds(const ResidentUnit& u, int planes, bool two_parts) {
+  int rank = 0;
+  for (int l = 0; l < u.n_layers; ++l) rank = std::max(rank, u.layer[l].r);
+  const double m = 1e-3 * u.m, d = 1e-3 * u.d, md = m * d, r4 = rank > 4, r8 = rank > 8;
+  if (two_parts) {
+    const double group = u.n_layers > 1 ? md : 0.0;
+    return Rounds{4.14, 4.55 + 0.66 * r4 + (2.12 + 0.41 * d) * r8 + 1.17 * m + 0.37 * d + 0.024 * u.ranks + 0.07 * group,
+                  4.94 + 0.67 * d + 0.37 * md + 0.019 * u.ranks + 0.32 * group};
+  }
+  const bool in_pieces = u.d % 4 == 0 && u.ldx % 4 == 0 && (reinterpret_cast<uintptr_t>(u.X) & (planes == 3 ? 15u : 7u)) == 0;
+  const ChainFit& f = kChain[!in_pieces ? 2 : planes == 3 ? 1 : 0];
+  const double more = md * (u.n_layers - 1);
+  return Rounds{f.once,
+                f.every + f.every_r4 * r4 + f.every_r8 * r8 + f.every_m * m + f.every_d * d + f.every_md * md + (f.every_r8_d * d + f.every_r8_md * md) * r8 +
+                    f.every_more * more,
+                f.power + f.power_m * m + f.power_d * d + f.power_md * md + f.power_r4_d * d * r4 + (f.power_r8_d * d + f.power_r8_md * md) * r8 +
+                    f.power_more * more};
+}
+
+// Over those lists the rule takes the slower kernels by more than 2 % for 1.6, 1.3 and 0.5 % of them (K = 0, 1, 3; at most 25, 8 and 6 %
+// slower) and leaves 1 to 12 % of the logarithm of what the faster kernel each time would gain.  An estimate without the rounds apart,
+// fitted before the partial sums of several column blocks were read together and without bf16 on the fp32 kernels: 23, 11 and 4.7 %.
+bool resident_pays(const ResidentLaunch& plan, int K, bool fresh) {
   // Below 2^-109 an fp32 value's third part is no bf16 number any more.  With a power step such inputs underflow whatever the kernel,
   // without one the fp32 products keep them (2^-118 of N(0, 1): 5e-9 against 64 bits, the parts 9e-6): they stay there.
   if (K == 0 && plan.planes == 3) return false;
-  return (plan.grid_wide ? 5.5 : 4.8) + (K + 1) * plan.round_us < 0.97 * (K + 1) * plan.others_us;
+  double here = 0.0, there = 0.0, most = 0.0, all = 0.0;
+  int layers = 0;
+  for (int k = 0; k < plan.p.n_units; ++k) {
+    const ResidentUnit& u = plan.p.unit[k];
+    const Rounds a = resident_rounds(u, plan.planes, plan.parts), b = other_rounds(u, plan.planes, plan.parts == 2);
+    const double md = 1e-6 * u.m * (double)u.d;
+    here = std::max(here, a.once + (K + 1) * a.every + K * a.power);
+    there = std::max(there, b.once + (K + 1) * b.every + K * b.power);
+    most = std::max(most, md);
+    all += md;
+    layers += u.n_layers;
+  }
+  here += plan.grid_wide ? 8.43 : 5.65;
+  if (plan.p.n_units > 1) {            // their launches serve all units, which share the SMs
+    const bool two_parts = plan.parts == 2;
+    const int more = std::min(layers - 1, 8);
+    there += (two_parts ? 0.19 : plan.planes == 3 ? 0.74 : 0.59) * (2 * K + 1) * (all - most) + (two_parts ? 0.13 : plan.planes == 3 ? 0.09 : 0.18) * (K + 1) * more;
+  }
+  if (fresh) there += 1.3;
+  return here < 0.97 * there;
 }
 
 void resident_bind(ResidentLaunch* plan, char* scratch) {

@@ -71,14 +71,14 @@ struct ResidentLaunch {
   bool grid_wide;                       // some unit has several clusters, which wait for one another
   size_t smem;
   size_t scratch;                       // bytes behind ypart, y and gshare
-  double round_us, others_us;           // estimates of a round here and by the other kernels
 };
 
 cudaError_t resident_init(int sm_count, ResidentCaps* caps);      // once per device
 // Plans one launch for the layers; false where the resident kernel does not take them.  two_parts: the products of every layer
 // would run on the tensor-core path, whose operands are two bf16 parts; else they are three (24 bits, as the CUDA-core path's fp32).
 bool resident_plan(const ResidentCaps& caps, const agzo_layer* layers, int n, bool share_inputs, bool two_parts, ResidentLaunch* out);
-bool resident_pays(const ResidentLaunch& plan, int K);            // it is estimated to be the faster one
+// It is estimated to be the faster one.  fresh: the others would have the list's tables or records to write first.
+bool resident_pays(const ResidentLaunch& plan, int K, bool fresh);
 // points the plan at its scratch (256-byte aligned, out->scratch bytes)
 void resident_bind(ResidentLaunch* plan, char* scratch);
 cudaError_t launch_resident(const ResidentLaunch& plan, cudaStream_t s);

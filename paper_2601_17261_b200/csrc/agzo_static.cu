@@ -120,7 +120,7 @@ agzo_status extract_static(const void* X, int64_t ldx, int32_t x_dtype, int32_t 
     a.V = V; a.ldv = ldv;
     ResidentLaunch plan;      // K = 0: a block that comes too late to the only meeting would not see that others have given up
     if (resident_plan(scratch.resident, &a, 1, false, false, &plan) && plan.scratch <= kResidentScratchBytes &&
-        !(plan.grid_wide && K == 0) && (route == 2 || resident_pays(plan, K))) {
+        !(plan.grid_wide && K == 0) && (route == 2 || resident_pays(plan, K, true))) {
       resident_bind(&plan, static_cast<char*>(scratch.resident_addr));
       plan.p.K = K;
       plan.p.wait_ns = wait_ns;
