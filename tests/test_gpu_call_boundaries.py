@@ -87,11 +87,13 @@ def test_scalar_and_basis():
 
 @pytest.mark.parametrize("r,m,d_in,bf16", [(4, 512, 256, False), (8, 613, 1024, True), (16, 2048, 4096, True), (24, 613, 1024, True),
                                            (64, 1024, 4096, True)])
-def test_basis_behind_an_extraction(r, m, d_in, bf16):
+@pytest.mark.parametrize("resident", [0, 2])
+def test_basis_behind_an_extraction(r, m, d_in, bf16, resident):
     X, _ = to_dev(WL.planted_activations(m, d_in, 16, seed=m, bf16=bf16), bf16)
     V = torch.zeros(r, d_in, device=DEV)
     layers = [B.make_layer(X=X, V=V, r=r, layer_id=0)]
     with Ctx(layers) as ctx:
+        B.agzo_set_option(ctx, "extract_resident", resident)
         look = early(ctx, V)
         torch.cuda.synchronize()
         for seed in range(ROUNDS):
@@ -99,10 +101,11 @@ def test_basis_behind_an_extraction(r, m, d_in, bf16):
             B.agzo_extract_subspace(ctx, layers, seed, 1)
             compare(look(), V)
         if d_in <= 1024 and r <= 8:
+            route = B.STATIC_RESIDENT if resident else B.STATIC_CHAIN
             for flag in (None, torch.zeros(1, dtype=torch.int32, device=DEV)):
                 for seed in range(ROUNDS):
                     busy()
-                    B.agzo_extract_subspace_static(X, V, r, 1, seed, 1, flag)
+                    B.agzo_debug_extract_static(X, V, r, 1, seed, 1, route, flag)
                     compare(look(), V)
 
 

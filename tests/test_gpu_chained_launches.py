@@ -23,8 +23,10 @@ def build(shapes, m, r, bf16):
     return out
 
 
-def iterate(sets, sync, streams=(None,)):
+def iterate(sets, sync, resident, streams=(None,)):
     ctxs = [B.agzo_create([t[3] for t in s], 0) for s in sets]
+    for ctx in ctxs:
+        B.agzo_set_option(ctx, "extract_resident", resident)
     losses = torch.tensor([1.0, 0.999], dtype=torch.float64, device=DEV)
     ghats = [torch.zeros(1, device=DEV) for _ in sets]
     torch.cuda.synchronize()
@@ -47,23 +49,24 @@ def iterate(sets, sync, streams=(None,)):
 
 
 @pytest.mark.parametrize("n_streams", [1, 2])
-@pytest.mark.parametrize("r,bf16", [(3, False), (4, True), (8, True), (24, True), (40, True)])
-def test_back_to_back_equals_one_by_one(r, bf16, n_streams):
+@pytest.mark.parametrize("r,bf16,resident", [(3, False, 0), (4, True, 0), (8, True, 0), (24, True, 0), (40, True, 0), (3, False, 2), (8, True, 2)])
+def test_back_to_back_equals_one_by_one(r, bf16, resident, n_streams):
     shapes = [[(256, 64)], [(1024, 300), (512, 96)], [(1160, 40)] * 3]
     streams = [torch.cuda.Stream() for _ in range(n_streams)]
-    a = iterate([build(s, 600, r, bf16) for s in shapes], sync=True)
-    b = iterate([build(s, 600, r, bf16) for s in shapes], sync=False, streams=streams)
+    a = iterate([build(s, 600, r, bf16) for s in shapes], sync=True, resident=resident)
+    b = iterate([build(s, 600, r, bf16) for s in shapes], sync=False, resident=resident, streams=streams)
     for x, y in zip(a, b):
         assert torch.equal(x, y)
 
 
-def test_workspace_free_calls_back_to_back():
+@pytest.mark.parametrize("route", [B.STATIC_CHAIN, B.STATIC_RESIDENT])
+def test_workspace_free_calls_back_to_back(route):
     Xs = [to_dev(WL.planted_activations(m, d, 8, seed=m, bf16=False), False)[0] for m, d in ((300, 200), (1000, 512), (64, 128))]
     got = []
     for sync in (True, False):
         Vs = [torch.zeros(8, X.shape[1], device=DEV) for X in Xs for _ in range(2)]
         for i, V in enumerate(Vs):
-            B.agzo_extract_subspace_static(Xs[i // 2], V, 8, 2, i, i)
+            B.agzo_debug_extract_static(Xs[i // 2], V, 8, 2, i, i, route)
             if sync:
                 torch.cuda.synchronize()
         torch.cuda.synchronize()
@@ -82,6 +85,7 @@ def test_layer_lists_alternate_without_waiting():
         Vs = [torch.zeros(4, 64, device=DEV) for _ in Ws]
         layers = [B.make_layer(X=X, W=W, V=V, r=4, layer_id=i) for i, (W, V) in enumerate(zip(Ws, Vs))]
         ctx = B.agzo_create(layers, 0)
+        B.agzo_set_option(ctx, "extract_resident", 0)            # the kernels that read the tables
         torch.cuda.synchronize()
         for seed in range(3):
             at = 0

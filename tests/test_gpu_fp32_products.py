@@ -22,15 +22,16 @@ pytestmark = pytest.mark.gpu
 def test_cuda_core_extraction(r, m, d_in, bf16, extra):
     X = WL.planted_activations(m, d_in, min(16, d_in // 2), seed=m + d_in, bf16=bf16)
     Xd, _ = to_dev(X, bf16, pitch=d_in + extra if extra else None)
-    V, V2 = torch.zeros(r, d_in, device=DEV), torch.zeros(r, d_in, device=DEV)
+    V, V2, V3 = (torch.zeros(r, d_in, device=DEV) for _ in range(3))
     layers = [B.make_layer(X=Xd, V=V, r=r, layer_id=3)]
     with Ctx(layers) as ctx:
         B.agzo_set_option(ctx, "extract_path", 1)
         B.agzo_extract_subspace(ctx, layers, 9, 2)
         assert B.agzo_poll(ctx) == B.AGZO_OK
     Vo = O.extract_subspace(X, r, 2, 9, 3)
-    B.agzo_extract_subspace_static(Xd, V2, r, 2, 9, 3)
-    for Vg in (to_host(V), to_host(V2)):
+    B.agzo_debug_extract_static(Xd, V2, r, 2, 9, 3, B.STATIC_CHAIN)
+    B.agzo_extract_subspace_static(Xd, V3, r, 2, 9, 3)           # by the faster kernels, these or the resident one
+    for Vg in (to_host(V), to_host(V2), to_host(V3)):
         assert np.abs(Vg.astype(np.float64) @ Vg.T - np.eye(r)).max() <= 1e-5
         assert projector_distance(Vg, Vo) <= 1e-4
 

@@ -23,6 +23,7 @@ def check(m, dims, r, K, bf16, n_layers=1):
     Vs = [torch.full((r, dims[p]), 7.0, device=DEV) for p in pick]
     layers = [B.make_layer(X=devs[p], V=V, r=r, layer_id=i) for i, (p, V) in enumerate(zip(pick, Vs))]
     with Ctx(layers) as ctx:
+        B.agzo_set_option(ctx, "extract_resident", 0)            # the kernel of this file, whatever would be faster
         B.agzo_extract_subspace(ctx, layers, 5, K)
         assert B.agzo_poll(ctx) == B.AGZO_OK
     for i in sorted({0, n_layers // 2, n_layers - 1}):
@@ -49,7 +50,8 @@ def test_layers_per_launch(n_layers):
 
 @pytest.mark.parametrize("r", [3, 4, 8, 13, 24, 40, 64])
 @pytest.mark.parametrize("power", [-12, -5, 7, 12])
-def test_scaled_inputs_give_the_same_basis(r, power):
+@pytest.mark.parametrize("resident", [0, 2])                     # whose factorisation is the same code
+def test_scaled_inputs_give_the_same_basis(r, power, resident):
     # every step scales exactly by powers of two (S by 4^n, its roots by 2^n, with two exponents of each parity), so V is
     # the same bit for bit; the roots see mantissas over the whole of [1, 4)
     X = WL.planted_activations(300, 264, 16, seed=r, bf16=True)
@@ -59,6 +61,7 @@ def test_scaled_inputs_give_the_same_basis(r, power):
         V = torch.zeros(r, 264, device=DEV)
         layers = [B.make_layer(X=Xd, V=V, r=r, layer_id=2)]
         with Ctx(layers) as ctx:
+            B.agzo_set_option(ctx, "extract_resident", resident)
             B.agzo_extract_subspace(ctx, layers, 5, 1)
             assert B.agzo_poll(ctx) == B.AGZO_OK
         got.append(V)

@@ -24,7 +24,7 @@ def _regular(Xd, r, K, seed, layer_id):
     V = torch.zeros(r, Xd.shape[1], device=DEV)
     layers = [B.make_layer(X=Xd, V=V, r=r, layer_id=layer_id)]
     with Ctx(layers) as ctx:
-        B.agzo_set_option(ctx, "extract_path", 1)      # the kernels the static variant uses
+        B.agzo_set_option(ctx, "extract_path", 1)      # the kernels of the static variant's chain
         B.agzo_extract_subspace(ctx, layers, seed, K)
         assert B.agzo_poll(ctx) == B.AGZO_OK
     return to_host(V)
@@ -40,7 +40,10 @@ def _warm_up_the_static_entry_point():
     torch.cuda.synchronize()
 
 
-def test_static_scratch_variant_matches_the_regular_entry_point_twice_in_a_row():
+# the entry itself, and the chain of kernels that it shares with the regular one, whichever it would take
+@pytest.mark.parametrize("extract", [B.agzo_extract_subspace_static, lambda *a, **k: B.agzo_debug_extract_static(*a, B.STATIC_CHAIN, **k)],
+                         ids=["entry", "chain"])
+def test_static_scratch_variant_matches_the_regular_entry_point_twice_in_a_row(extract):
     _warm_up_the_static_entry_point()
     cases = [(1500, 520, 8, 3, 21, 4, True, 528),      # ragged sizes, padded pitch, bf16
              (700, 256, 4, 2, 22, 9, False, None)]     # a smaller fp32 problem right after
@@ -58,14 +61,14 @@ def test_static_scratch_variant_matches_the_regular_entry_point_twice_in_a_row()
         # the meantime cannot move it, a new allocation would).
         free_before = torch.cuda.mem_get_info()[0]
         before = torch.cuda.memory_stats()["allocation.all.allocated"]
-        B.agzo_extract_subspace_static(Xd, V, r, K, seed, layer_id, d_rank_deficient=flag)
+        extract(Xd, V, r, K, seed, layer_id, d_rank_deficient=flag)
         torch.cuda.synchronize()
         assert torch.cuda.mem_get_info()[0] == free_before
         assert torch.cuda.memory_stats()["allocation.all.allocated"] == before
         got = to_host(V)
         assert int(flag) == 0
         assert np.abs(got.astype(np.float64) @ got.T - np.eye(r)).max() <= 1e-5
-        # against the existing entry point (same kernels, workspace scratch) ...
+        # against the existing entry point (the chain's kernels, workspace scratch) ...
         assert projector_distance(got, want) <= 1e-3
         assert np.abs(got - want).max() <= 1e-3
         # ... and against the oracle itself
