@@ -162,7 +162,7 @@ agzo_status agzo_destroy(agzo_ctx* ctx);
  * stay with the sweeps that serve the whole group (with 2: fused one by one);
  * 0 = off: two sweeps over X per power step.  Default 1;
  * "extract_resident" 1 (default) = a call whose activations all fit the device's shared memory (ranks of at most 16, at most
- * 24 over layers that share an X, at most 12 different X) is extracted by one kernel that keeps them there; it takes the place of
+ * 4 layers and 24 ranks on one X, at most 12 different X) is extracted by one kernel that keeps them there; it takes the place of
  * all others where it is estimated to be faster, unless an option asks for one of those ("extract_path", "extract_fused" other
  * than 1, "wave_bytes"; "time_kernel_class" with a class of theirs) or an all-reduce is set.  2 = wherever it can run, 0 = never;
  * "wave_bytes" = activation bytes grouped into one launch wave of extraction;
@@ -173,7 +173,9 @@ agzo_status agzo_destroy(agzo_ctx* ctx);
  * caller's stream (0 = none), read back by agzo_read_counters;
  * "debug_fail_step_call" = n (test aid, 0 = off): the n-th internal call of agzo_step
  * (extract, perturb, [flip,] ghat, restore_update) returns AGZO_ERR_CUDA on the host before
- * launching anything, so that the step's error path can be exercised without a fault.    */
+ * launching anything, so that the step's error path can be exercised without a fault;
+ * "debug_refuse_resident" 1 (test aid, 0 = off): launches of the resident kernel end on the host as
+ * if the device had refused them for want of SMs, so that the other kernels serve the call. */
 agzo_status agzo_set_option(agzo_ctx* ctx, const char* name, int64_t value);
 
 /* Token-sharded extraction over data-parallel ranks.  Algorithm 1 touches the activations only
@@ -233,6 +235,13 @@ agzo_status agzo_read_counters(agzo_ctx* ctx, double* h_ms, int64_t* h_timed_lau
  * counts it.                                                                               */
 agzo_status agzo_query_fused(agzo_ctx* ctx, const agzo_layer* h_layers, int n, int32_t* h_cluster,
                              void* stream);
+
+/* Inspection aid, host only: whether agzo_extract_subspace would extract the list by the resident kernel ("extract_resident"), as
+ * the options are and for this K, and how.  *h_count: units (runs of layers on one X) of its launch, 0 where the other kernels
+ * serve the call.  h_units: 8 entries per unit, 96 in all: blocks per cluster; then of the unit, whose X is cut into blocks of 128
+ * tokens x 128 columns, the thread blocks side by side over the columns, blocks of columns and of tokens per thread block, rows of
+ * thread blocks over the tokens, clusters, columns of Y that one adds up for all (0: each its own), bf16 parts of an operand. */
+agzo_status agzo_query_resident(agzo_ctx* ctx, const agzo_layer* h_layers, int n, int K, int32_t* h_units, int32_t* h_count);
 
 /* Inspection aid.  h_clusters[C], C = 1..16 (17 host entries, entry 0 is 0): how many thread-block
  * clusters of C CTAs of the fused power-step kernel the context's device holds at once (a cluster

@@ -36,7 +36,7 @@ EXPORTS = [
     "agzo_extract_subspace_static", "agzo_fill_gaussian_basis", "agzo_set_allreduce",
     "agzo_debug_wait_timeout", "agzo_query_fused", "agzo_query_cluster_capacity", "agzo_debug_fused_split",
     "agzo_debug_early_copy", "agzo_debug_normal_parts", "agzo_debug_meeting",
-    "agzo_debug_extract_static",
+    "agzo_debug_extract_static", "agzo_query_resident",
 ]
 KC_RMW, KC_XT_T, KC_X_Q, KC_PANEL_QR, KC_TC_XT_T, KC_TC_X_Q, KC_OMEGA, KC_RMW_TC, KC_FUSED_POWER, KC_RESIDENT = 1, 2, 3, 4, 5, 6, 7, 8, 9, 10
 
@@ -111,6 +111,7 @@ def lib() -> C.CDLL:
                                             C.c_int32, i64, vp]),
         "agzo_debug_meeting": (i32, [i32, i32, u32, u64, C.POINTER(u64), C.POINTER(u32), C.POINTER(u32)]),
         "agzo_query_fused": (i32, [vp, LP, i32, C.POINTER(C.c_int32), vp]),
+        "agzo_query_resident": (i32, [vp, LP, i32, i32, C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
         "agzo_query_cluster_capacity": (i32, [vp, C.POINTER(C.c_int32)]),
         "agzo_debug_fused_split": (i32, [C.POINTER(C.c_int32), i32, i32, C.POINTER(C.c_int32), C.POINTER(C.c_int32),
                                          C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
@@ -252,6 +253,16 @@ def agzo_query_fused(ctx: Context, layers, stream=None, arr=None):
     out = (C.c_int32 * len(layers))()
     _check(lib().agzo_query_fused(ctx.handle, arr, len(layers), out, _stream_ptr(stream)), "agzo_query_fused")
     return list(out)
+
+
+RESIDENT_UNIT = ("cs", "cj", "cb", "tb", "ni", "clusters", "sub", "parts")
+
+
+def agzo_query_resident(ctx: Context, layers, K: int):
+    """How the resident kernel would extract the list (a dict per unit), [] where the other kernels serve it."""
+    units, n = (C.c_int32 * 96)(), C.c_int32(0)
+    _check(lib().agzo_query_resident(ctx.handle, layer_array(layers), len(layers), K, units, C.byref(n)), "agzo_query_resident")
+    return [dict(zip(RESIDENT_UNIT, units[8 * k:8 * k + 8])) for k in range(n.value)]
 
 
 def agzo_debug_fused_split(tiles, clusters: int):

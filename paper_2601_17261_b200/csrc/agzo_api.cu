@@ -124,6 +124,7 @@ struct agzo_ctx {
   ResidentCaps resident_caps;
   // measurement aid: event pairs around the launches of one kernel class
   int debug_fail_step_call;   // test option: the n-th internal call of agzo_step fails on the host, 0 = off
+  int debug_refuse_resident;  // test option: launches of the resident kernel end as if the device had refused them
   int time_class;
   std::vector<cudaEvent_t> events;   // pairs: start, stop
   size_t events_used;
@@ -860,6 +861,7 @@ agzo_status agzo_create(agzo_ctx** out, int device, void* workspace, size_t work
   c->stage_ev = nullptr;
   c->time_class = 0;
   c->debug_fail_step_call = 0;
+  c->debug_refuse_resident = 0;
   c->events_used = 0;
   c->launches = 0;
   c->power_steps = 0;
@@ -951,6 +953,10 @@ agzo_status agzo_set_option(agzo_ctx* ctx, const char* name, int64_t value) {
     if (value < 0 || value > 16) return AGZO_ERR_INVALID_ARG;
     ctx->debug_fail_step_call = (int)value;
     return AGZO_OK;
+  } else if (std::strcmp(name, "debug_refuse_resident") == 0) {
+    if (value < 0 || value > 1) return AGZO_ERR_INVALID_ARG;
+    ctx->debug_refuse_resident = (int)value;
+    return AGZO_OK;
   } else if (std::strcmp(name, "time_kernel_class") == 0) {
     if (value < 0 || value > AGZO_KC_RESIDENT) return AGZO_ERR_INVALID_ARG;
     ctx->time_class = (int)value;
@@ -1011,6 +1017,24 @@ agzo_status agzo_query_fused(agzo_ctx* ctx, const agzo_layer* h_layers, int n, i
   return AGZO_OK;
 }
 
+agzo_status agzo_query_resident(agzo_ctx* ctx, const agzo_layer* h_layers, int n, int K, int32_t* h_units, int32_t* h_count) {
+  agzo_status st = check_ctx(ctx);
+  if (st != AGZO_OK) return st;
+  if (!h_units || !h_count || K < 0 || K > 16) return AGZO_ERR_INVALID_ARG;
+  st = validate(h_layers, n, NEED_EXTRACT);
+  if (st != AGZO_OK) return st;
+  *h_count = 0;
+  if (n == 0 || !plan_resident(ctx, h_layers, n, K, false)) return AGZO_OK;
+  const ResidentLaunch& r = ctx->resident;
+  for (int k = 0; k < r.p.n_units; ++k) {
+    const ResidentUnit& u = r.p.unit[k];
+    const int32_t v[8] = {r.p.cs, u.cj, u.cb, u.tb, u.ni, u.clusters, u.sub, r.parts};
+    std::memcpy(h_units + 8 * k, v, sizeof(v));
+  }
+  *h_count = r.p.n_units;
+  return AGZO_OK;
+}
+
 agzo_status agzo_poll(agzo_ctx* ctx, void* stream) {
   agzo_status st = check_ctx(ctx);
   if (st != AGZO_OK) return st;
@@ -1053,7 +1077,7 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
     cudaError_t e;
     {
       Timed t(ctx, AGZO_KC_RESIDENT, s);
-      e = launch_resident(ctx->resident, s);
+      e = ctx->debug_refuse_resident ? cudaErrorCooperativeLaunchTooLarge : launch_resident(ctx->resident, s);
     }
     if (e == cudaSuccess) return AGZO_OK;
     ctx->launches -= 1;      // refused: not a launch, and no time of one

@@ -5,7 +5,10 @@ launches in a row that share its counters.
 Against the oracle at the suite's tolerances for extraction (1e-5 orthonormality, 1e-3 projector distance), and against the kernels
 of the other paths on the same inputs: operands in three bf16 parts carry 24 bits, as fp32 does, so that both sides are within a
 few 2^-24 sqrt(K + 1) of the exact basis times the spread of the spectrum (at most 5 in these inputs): 1e-5; operands in two
-parts leave 2^-17 of a product: 1e-3 as the suite."""
+parts leave up to 2^-17 of an element, 2^-17 / sqrt(3) rms and of either sign, in each of 2 K + 1 products on both sides: times the
+spread 7e-5 for K = 2, and 1e-4 (a product without one of its parts leaves 2^-9)."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
@@ -25,8 +28,8 @@ def launches(ctx, layers, seed, K):
     return B.agzo_read_counters(ctx)[2]
 
 
-def check(units, K, seed=6, served=True):
-    """units: (m, d_in, ranks of the layers on that X, bf16, pitch)"""
+def check(units, K, seed=6, served=True, pieces=None):
+    """units: (m, d_in, ranks of the layers on that X, bf16, pitch); pieces: which of them add Y up in pieces of its columns"""
     Xs, Vs, layers, held = [], [], [], []
     for n, (m, d, ranks, bf16, pitch) in enumerate(units):
         X = WL.planted_activations(m, d, min(16, d, m), seed=m + n, bf16=bf16)
@@ -40,6 +43,8 @@ def check(units, K, seed=6, served=True):
     three = any(not b or d % 8 or d < 128 or m < 256 or (p or 0) % 8 for m, d, _, b, p in units)
     with Ctx(layers) as ctx:
         B.agzo_set_option(ctx, "extract_resident", 2)
+        how = B.agzo_query_resident(ctx, layers, K)
+        assert (len(how) == len(units)) == served and (pieces is None or [u["sub"] > 0 for u in how] == pieces), how
         n = launches(ctx, layers, seed, K)
         assert (n == 1) == served, n
         assert B.agzo_poll(ctx) == B.AGZO_OK
@@ -54,7 +59,7 @@ def check(units, K, seed=6, served=True):
         got = to_host(a)
         assert np.abs(got.astype(np.float64) @ got.T - np.eye(r)).max() <= 1e-5, i
         assert projector_distance(got, O.extract_subspace(X, r, K, seed, i)) <= 1e-3, i
-        assert float((a - V).norm() / V.norm()) <= (1e-5 if three else 1e-3), i
+        assert float((a - V).norm() / V.norm()) <= (1e-5 if three else 1e-4), i
         edge = Vb.clone()
         edge[1:1 + r, :X.shape[1]] = 7.0
         assert bool((edge == 7.0).all()), i
@@ -83,16 +88,48 @@ def test_units_side_by_side(units):
     check(units, 2)
 
 
+# columns of Y added up in pieces that meet once more: groups of layers on one X with rows of padding between them, the last piece
+# ragged or empty, element by element and in three parts, beside a unit that adds up whole columns
+@pytest.mark.parametrize("units,pieces", [
+    ([(8000, 1024, (12, 12), True, None)], [True]), ([(8000, 1000, (3, 5, 9), True, None)], [True]), ([(4000, 500, (5, 6, 8), False, None)], [True]),
+    ([(8000, 250, (4, 4, 4), False, None)], [True]), ([(8000, 253, (2, 7), True, None)], [True]), ([(4096, 256, (8, 8), False, None)], [True]),
+    ([(2000, 2048, (8, 8, 8), True, None)], None), ([(4000, 512, (9, 12), True, None), (300, 256, (4,), True, None)], None)])      # by the device's clusters
+def test_columns_in_pieces(units, pieces):
+    check(units, 2, pieces=pieces)
+
+
+def test_a_refused_launch_leaves_the_call_to_the_other_kernels():
+    X = to_dev(WL.planted_activations(300, 256, 16, seed=1, bf16=True), True)[0]
+    V = torch.zeros(4, 256, device=DEV)
+    layers = [B.make_layer(X=X, V=V, r=4, layer_id=0)]
+    with Ctx(layers) as ctx:
+        B.agzo_set_option(ctx, "extract_resident", 0)
+        n = launches(ctx, layers, 5, 2)
+        want = V.clone()
+        B.agzo_set_option(ctx, "extract_resident", 2)
+        assert launches(ctx, layers, 5, 2) == 1
+        B.agzo_set_option(ctx, "debug_refuse_resident", 1)
+        V.zero_()
+        assert launches(ctx, layers, 5, 2) == n - 1              # the same kernels; the tables are in place
+        assert torch.equal(V, want)
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+
+
 def test_static_entry_and_what_it_reports():
     for m, d_in, r, bf16 in [(700, 256, 4, False), (300, 130, 16, True), (1500, 520, 8, True)]:
         X = WL.planted_activations(m, d_in, 16, seed=m, bf16=bf16)
         Xd = to_dev(X, bf16)[0]
         V, flag = torch.zeros(r, d_in, device=DEV), torch.full((1,), -1, dtype=torch.int32, device=DEV)
-        B.agzo_extract_subspace_static(Xd, V, r, 2, 3, 7, flag)
+        B.agzo_debug_extract_static(Xd, V, r, 2, 3, 7, B.STATIC_RESIDENT, flag)
         assert flag.item() == 0
+        other, both = torch.zeros_like(V), torch.zeros_like(V)
+        B.agzo_extract_subspace_static(Xd, both, r, 2, 3, 7)     # one of the two, bit for bit
+        B.agzo_debug_extract_static(Xd, other, r, 2, 3, 7, B.STATIC_CHAIN)
+        assert not torch.equal(V, other) and (torch.equal(both, V) or torch.equal(both, other))
+        assert float((V - other).norm() / V.norm()) <= 1e-5
         assert projector_distance(to_host(V), O.extract_subspace(X, r, 2, 3, 7)) <= 1e-3
         Xd[:, 2:] = 0                                          # rank two
-        B.agzo_extract_subspace_static(Xd, V, r, 2, 3, 7, flag)
+        B.agzo_debug_extract_static(Xd, V, r, 2, 3, 7, B.STATIC_RESIDENT, flag)
         assert flag.item() == 1 and int((V.norm(dim=1) == 0).sum()) == r - 2
 
 
@@ -112,10 +149,16 @@ def test_dependent_columns_and_a_small_workspace():
     Y = torch.randn(2048, 256, device=DEV)
     W = torch.zeros(4, 256, device=DEV)
     layers = [B.make_layer(X=Y, V=W, r=4, layer_id=0)]
-    small = B.Context(0, 4096 + 2048 * 16 + 3 * 4096)
+    size = 4096 + 2048 * 16 + 3 * 4096
+    small = B.Context(0, size)
+    B.agzo_destroy(small)                                        # the same on the inside of a larger buffer
+    around = torch.full((size + 2 * (1 << 20),), 0x5a, dtype=torch.uint8, device=DEV)
+    small.handle = C.c_void_p()
+    assert B.lib().agzo_create(C.byref(small.handle), 0, around.data_ptr() + (1 << 20), size) == B.AGZO_OK
     B.agzo_set_option(small, "extract_resident", 2)
-    B.agzo_extract_subspace(small, layers, 1, 1)
+    assert launches(small, layers, 1, 1) > 1 and B.agzo_query_resident(small, layers, 1) == []
     a = W.clone()
+    assert bool((around[:1 << 20] == 0x5a).all()) and bool((around[-(1 << 20):] == 0x5a).all())
     with Ctx(layers) as ctx:
         B.agzo_set_option(ctx, "extract_resident", 2)
         assert launches(ctx, layers, 1, 1) == 1
