@@ -401,8 +401,8 @@ agzo_status agzo_debug_fused_split(const int32_t* h_tiles, int n, int clusters, 
 
 /* Test export: agzo_extract_subspace_static by the kernels that `route` names, 0 = the faster ones, 1 = the chain of CUDA-core
  * kernels, 2 = the resident kernel (UNSUPPORTED where it does not take the layer), whose waits for other blocks end after
- * wait_ns nanoseconds (at most the two seconds that they otherwise do; where it is less, one block comes to every meeting of
- * several clusters 0.1 ms later than that).                                                */
+ * wait_ns nanoseconds (at most the two seconds that they otherwise do; where it is less, one block comes to the first
+ * meeting of several clusters 0.1 ms later than that).                                     */
 agzo_status agzo_debug_extract_static(const void* X, int64_t ldx, int32_t x_dtype, int32_t m, int32_t d_in, int32_t r, int32_t K,
                                       uint64_t seed, uint32_t layer_id, float* V, int64_t ldv,
                                       int32_t* d_rank_deficient, int32_t route, int64_t wait_ns, void* stream);

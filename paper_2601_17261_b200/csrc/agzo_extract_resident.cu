@@ -230,12 +230,29 @@ __device__ __forceinline__ void tmem_sum8(uint32_t at, int NP, int NB, int chunk
 // cluster's barrier; else a counter (Meeting).  A CTA that has given up waiting says so in the counter while the meeting still lacks
 // somebody, so that whoever completes it or finds it complete sees that too: all of them have sh->failed set from there on.  (One that
 // starts only then takes what it finds for the count of earlier launches; the others say so again at the next meeting.)
+// What is done when a wait runs out, and the meeting itself, are out of line: a round's code is larger than the instruction cache as
+// it is, and every line of it costs (mean of 77 calls of 27 to 130 us 61.1 -> 62.2 us with this in the rounds, 61.0 out of line).
 struct Meeting {
   unsigned long long* counter;
   int n;                          // CTAs
   bool first;
   unsigned phase, failures;       // what it showed before the launch (thread 0)
 };
+// arrives and waits for the phase; whether a wait of this CTA's or another's has run out
+__device__ __noinline__ bool meet(unsigned long long* counter, unsigned long long add, unsigned phase, unsigned failures, bool failed,
+                                  unsigned long long wait_ns) {
+  if (failed) add += kMeetingFailure;
+  asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(counter), "l"(add) : "memory");
+  if (failed) return true;
+  const unsigned long long t_start = global_ns();
+#pragma unroll 1
+  for (;;) {
+    unsigned long long got;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(got) : "l"(counter) : "memory");
+    if (meeting_phase(got) == phase) return meeting_failures(got) != failures;
+    if (global_ns() - t_start > wait_ns && atomicCAS(counter, got, got + kMeetingFailure) == got) return true;
+  }
+}
 __device__ __forceinline__ void unit_barrier(Meeting& m, int clusters, int cs, const ResidentParams& P, ResShared* sh) {
   if (clusters == 1) {
     __syncwarp();
@@ -244,28 +261,26 @@ __device__ __forceinline__ void unit_barrier(Meeting& m, int clusters, int cs, c
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    if (m.first && P.late_ns) {
-      const unsigned long long t_late = global_ns() + P.late_ns;
-      while (global_ns() < t_late) {}
-    }
-    const unsigned long long add = meeting_increment(m.n, m.first, m.phase) + (sh->failed ? kMeetingFailure : 0ull);
-    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(m.counter), "l"(add) : "memory");
+    const unsigned long long add = meeting_increment(m.n, m.first, m.phase);
     m.phase ^= 1u;
-    if (!sh->failed) {
-      const unsigned long long t_start = global_ns();
-#pragma unroll 1
-      for (;;) {
-        unsigned long long got;
-        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(got) : "l"(m.counter) : "memory");
-        if (meeting_phase(got) == m.phase) {
-          if (meeting_failures(got) != m.failures) sh->failed = 1;
-          break;
-        }
-        if (global_ns() - t_start > P.wait_ns && atomicCAS(m.counter, got, got + kMeetingFailure) == got) { sh->failed = 1; break; }
-      }
-    }
+    if (meet(m.counter, add, m.phase, m.failures, sh->failed != 0, P.wait_ns)) sh->failed = 1;
   }
   __syncthreads();
+}
+// A product that did not come: known to the n CTAs of the cluster where that is all of the unit, else to the others by the next meeting
+__device__ __noinline__ void product_failed(ResShared* sh, int n) {
+  sh->failed = 1;
+  if ((int)threadIdx.x < n) st_cluster_u32(mapa_shared(smem_u32(&sh->failed), threadIdx.x), 1u);
+}
+// V = 0, with which a pass changes nothing: the strips of the CTA in row i whose first column is col0
+__device__ __noinline__ void zero_strips(const ResidentUnit& U, int i, int col0) {
+  const int lane = threadIdx.x & 31;
+  for (int l = 0; l < U.n_layers; ++l)
+    for (int s0 = threadIdx.x >> 5; s0 < U.cb * 8; s0 += kWarps) {
+      const int c = 16 * s0 + (lane & 15);
+      if (s0 % U.ni != i || c >= U.d - col0) continue;
+      for (int k = lane >> 4; k < U.layer[l].r; k += 2) U.layer[l].V[col0 + k * U.layer[l].ldv + c] = 0.f;
+    }
 }
 
 // Gram products of one layer's rows of the staged Y, by `split` warps of which this is number `me`
@@ -437,6 +452,10 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
     const unsigned long long now = __ldcg(meeting.counter);
     meeting.phase = meeting_phase(now);
     meeting.failures = meeting_failures(now);
+    if (meeting.first && P.late_ns) {
+      const unsigned long long t_late = global_ns() + P.late_ns;
+      while (global_ns() < t_late) {}
+    }
   }
   load_x<PLANES>(U, sX, plane, t0, col0, tb, cb);
   if (PLANES == 1 && U.x_vec) fill_omega<PARTS>(U, sT, t0, tb, P.seed);         // while X arrives
@@ -468,7 +487,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
                                    (uint32_t)(2 * cb * kSlotBytes), kSlotBytes, 128u, 1, NB, NP);
       mma_commit_if(go, &sh.mma);
     }
-    if (!mbar_wait(&sh.mma, mma_par)) sh.failed = 1;
+    if (!mbar_wait(&sh.mma, mma_par)) product_failed(&sh, clusters == 1 ? cs : 1);
     mma_par ^= 1u;
     tc_fence_after();
     if (i < ni)
@@ -600,7 +619,6 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
       for (int w = 0; w < kWarps; ++w) sum += v[w];
       sG[e] = sum;
     }
-    if (sh.failed && tid < cs && cs > 1) st_cluster_u32(mapa_shared(smem_u32(&sh.failed), (uint32_t)tid), 1u);      // all of the cluster know
     __syncwarp();
     if (cs > 1) cluster_sync_all(); else __syncthreads();
     {
@@ -667,11 +685,6 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
       }
     }
     __syncthreads();
-    if (last && sh.failed) {             // a wait has run out and the sums are not whole: V = 0, with which a pass changes nothing
-      for (int k = tid; k < nl * kAmBytes / 4; k += kThreads) reinterpret_cast<uint32_t*>(sAM)[k] = 0u;
-      for (int k = tid; k < U.rows * pitch; k += kThreads) sY[k] = 0.f;
-      __syncthreads();
-    }
     // ---------------------------------------------------------------- Q = Y M: the operand, or V (whose strips the rows of CTAs share)
 #pragma unroll 1
     for (int l = 0; l < nl; ++l) {
@@ -697,7 +710,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
                                    2 * kSlotBytes, 0u, 2u, 0, NB, NP);
       mma_commit_if(go, &sh.mma);
     }
-    if (!mbar_wait(&sh.mma, mma_par)) sh.failed = 1;
+    if (!mbar_wait(&sh.mma, mma_par)) product_failed(&sh, clusters == 1 ? cs : 1);
     mma_par ^= 1u;
     tc_fence_after();
 #pragma unroll 1
@@ -767,6 +780,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
 
   tc_fence_before();
   __syncthreads();
+  if (sh.failed) zero_strips(U, i, col0);                    // a wait has run out and the sums are not whole
   if (cs > 1) cluster_sync_all();                            // nobody leaves while a peer may read its share
   if (tid == 0) {
     if (sh.failed && P.status) { atomicExch(&P.status->timeout, 1); atomicExch(&P.status->where, 5); }

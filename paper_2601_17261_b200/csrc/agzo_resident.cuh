@@ -41,7 +41,7 @@ struct ResidentUnit {
 struct ResidentParams {
   int n_units, cs, K;
   unsigned long long wait_ns;           // limit of a wait for the other CTAs of a unit
-  unsigned long long late_ns;           // a test's: how late the unit's first CTA comes to a meeting
+  unsigned long long late_ns;           // a test's: how late the unit's first CTA comes to the first meeting
   unsigned long long seed;
   DevStatus* status;                    // may be null
   int* flag;                            // may be null: set to whether a column was dependent, to 2 where a wait ran out

@@ -190,7 +190,7 @@ def test_a_graph_of_it_replays():
 
 
 def test_static_entry_reports_a_wait_that_ran_out():
-    # 128 blocks that meet eight times, one of which comes 0.1 ms later than the others wait
+    # 128 blocks that meet eight times, one of which comes to the first meeting 0.1 ms later than the others wait
     X = to_dev(WL.planted_activations(4096, 2048, 16, seed=3, bf16=True), True)[0]
     want, V = torch.zeros(16, 2048, device=DEV), torch.zeros(16, 2048, device=DEV)
     flag = torch.full((1,), -1, dtype=torch.int32, device=DEV)
