@@ -17,7 +17,7 @@
 //
 // What bounds it is the chain of synchronisations of a round: a cluster barrier 0.2 us, all CTAs of a unit at a counter 1.3, the
 // partial sums of Y from L2 1.2, the exchange of T 2.3, the Gram matrix and its exchange 2, the factor 0.5 to 2.4.  Against the
-// chain of launches, K = 3: without workspace 4096 x 2048, r = 16 158 -> 85 us; 8192 x 256 bf16, r = 8 85 -> 47; 1500 x 515 fp32,
+// chain of launches, K = 3: without workspace 4096 x 2048, r = 16 158 -> 86 us; 8000 x 256 bf16, r = 8 83 -> 51; 1500 x 515 fp32,
 // r = 5 97 -> 51; 613 x 1024 bf16, three layers of r = 8 53 -> 51.
 #include "agzo_qr.cuh"
 #include "agzo_resident.cuh"
@@ -925,7 +925,7 @@ bool resident_plan(const ResidentCaps& caps, const agzo_layer* L, int n, bool sh
   for (int k = 0; k < n;) {
     const agzo_layer& a = L[k];
     ResidentUnit u{};
-    u.X = a.X; u.ldx = a.ldx; u.x_dtype = a.x_dtype; u.m = a.m; u.d = a.d_in;
+    u.X = a.X; u.ldx = a.ldx; u.m = a.m; u.d = a.d_in;
     const int per16 = a.x_dtype == AGZO_F32 ? 4 : 8;
     u.x_vec = (reinterpret_cast<uintptr_t>(a.X) & 15u) == 0 && a.ldx % per16 == 0 && a.d_in % per16 == 0;
     for (; k < n; ++k) {

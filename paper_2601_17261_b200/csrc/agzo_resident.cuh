@@ -9,7 +9,8 @@ constexpr int kResMaxUnits = 12;        // units (runs of layers on one X) of a 
 constexpr int kResMaxLayers = 4;        // layers of a unit
 constexpr int kResMaxRank = 16;         // rank of a layer
 // Ranks of a unit.  Beyond, the sweeps over X are what takes the time and their chain has more SMs for them: two layers of rank 16 on
-// 2000 x 1024, 82 us here and 74 there; three of rank 8 on 613 x 1024 51 and 54.
+// 2000 x 1024 80 us here and 73 there, on 613 x 2048 82 and 69, three on 2000 x 1024 96 and 82 (the other way about only where X is
+// tall and narrow: two on 8000 x 512 84 and 109); three of rank 8 on 613 x 1024 51 and 53.
 constexpr int kResMaxPanel = 24;
 
 struct ResidentLayer {
@@ -25,7 +26,7 @@ struct ResidentLayer {
 struct ResidentUnit {
   const void* X;
   long long ldx;
-  int x_dtype, x_vec, m, d;
+  int x_vec, m, d;                      // x_vec: rows of X in 16-byte pieces
   int n_layers, ranks, NP, NB;          // ranks of the panel, rounded up to 8; operand rows (parts x NP, rounded up to 16)
   int rows;                             // rows of the staged Y
   int cb, tb, cj, ni;
