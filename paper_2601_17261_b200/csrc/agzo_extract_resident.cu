@@ -17,7 +17,7 @@
 //
 // What bounds it is the chain of synchronisations of a round: a cluster barrier 0.2 us, all CTAs of a unit at a counter 1.3, the
 // partial sums of Y from L2 1.2, the exchange of T 2.3, the Gram matrix and its exchange 2, the factor 0.5 to 2.4.  Against the
-// chain of launches, K = 3: without workspace 4096 x 2048, r = 16 158 -> 86 us; 8000 x 256 bf16, r = 8 83 -> 51; 1500 x 515 fp32,
+// chain of launches, K = 3: without workspace 4096 x 2048, r = 16 158 -> 85 us; 8000 x 256 bf16, r = 8 83 -> 51; 1500 x 515 fp32,
 // r = 5 97 -> 51; 613 x 1024 bf16, three layers of r = 8 53 -> 51.
 #include "agzo_qr.cuh"
 #include "agzo_resident.cuh"
@@ -410,6 +410,10 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
   const int cb = U.cb, tb = U.tb, NB = U.NB, NP = U.NP, ranks = U.ranks, nl = U.n_layers, clusters = U.clusters;
   const int ncols = cb * kBlock, col0 = j * ncols, cols_pad = cj * ncols, t0 = i * tb * kBlock, pitch = qr_pitch(ncols);
   Meeting meeting{P.counters + U.counter, clusters * cs, i == 0 && j == 0, 0u, 0u};
+  // no meeting of this launch is complete before this CTA has arrived; asked for here, where nothing waits for it (a launch of several
+  // clusters per unit does not start before the kernel in front is done; beside the loads of X: twenty calls of the entry without
+  // workspace 53.8 -> 54.6 us on the mean)
+  const unsigned long long met = clusters > 1 && tid == 0 ? __ldcg(meeting.counter) : 0ull;
 
   const int plane = tb * cb * 2 * kSlotBytes;
   uint8_t* sX = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -448,18 +452,15 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
   __syncthreads();
   if (!(PLANES == 1 && U.x_vec)) fill_omega<PARTS>(U, sT, t0, tb, P.seed);      // needs nothing from before the launch
   chain_wait();
-  if (clusters > 1 && tid == 0) {         // no meeting of this launch is complete before this CTA has arrived
-    const unsigned long long now = __ldcg(meeting.counter);
-    meeting.phase = meeting_phase(now);
-    meeting.failures = meeting_failures(now);
-    if (meeting.first && P.late_ns) {
-      const unsigned long long t_late = global_ns() + P.late_ns;
-      while (global_ns() < t_late) {}
-    }
-  }
   load_x<PLANES>(U, sX, plane, t0, col0, tb, cb);
   if (PLANES == 1 && U.x_vec) fill_omega<PARTS>(U, sT, t0, tb, P.seed);         // while X arrives
   asm volatile("cp.async.wait_all;" ::: "memory");
+  meeting.phase = meeting_phase(met);
+  meeting.failures = meeting_failures(met);
+  if (clusters > 1 && tid == 0 && meeting.first && P.late_ns) {
+    const unsigned long long t_late = global_ns() + P.late_ns;
+    while (global_ns() < t_late) {}
+  }
 
   const uint32_t tmem = sh.tmem_base;
   const uint32_t go = elect_one();
