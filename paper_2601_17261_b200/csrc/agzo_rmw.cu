@@ -461,45 +461,42 @@ __global__ void dense_kernel(T* w, long long n, long long b_first, uint64_t seed
   }
 }
 
-// Vector form for 16-byte aligned vectors: a thread takes eight consecutive elements (two Philox
-// blocks) per step, one 16-byte load and store for bf16, two for fp32.  A long vector is bound by the
-// arithmetic of one Philox + Box-Muller normal per weight, not by HBM (67 M weights: 142 us with logf, sqrtf and sincospif,
-// 117 now; HBM would allow 41); a short one by its launch, so the first normals are made before the kernel waits for its
-// predecessor.
+// Vector form for 16-byte aligned vectors: a thread takes eight consecutive elements (two Philox blocks), one 16-byte load and
+// store for bf16, two for fp32.  A long vector is bound by the arithmetic of one Philox + Box-Muller normal per weight, not by HBM
+// (67 M weights: 142 us with logf, sqrtf and sincospif, 119 with one pair of normals after another and a grid that stays resident, 97 now; HBM would
+// allow 43); a short one by its launch, so the normals are made, and the weights asked for as far as L2, before the kernel waits
+// for its predecessor.  Every thread has one step: with a share of the vector per resident thread the scheduler runs some warps far ahead
+// of others, and the SM ends on few (121 -> 109 us for that alone, 105 with 32-bit block numbers).
+// hi: upper word of the block numbers, the same in the whole launch, so that what the first two rounds of Philox make of it is made once.
 template <typename T>
-__global__ void __launch_bounds__(256) dense_vec_kernel(T* w, long long n8, uint64_t seed, uint32_t layer_id, float scale,
+__global__ void __launch_bounds__(256) dense_vec_kernel(T* w, uint32_t n8, uint32_t hi, uint64_t seed, uint32_t layer_id, float scale,
                                                         const float* d_scale) {
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  float4 ga = gaussian_block((uint64_t)(2 * g), layer_id, kTagDense, seed);
-  float4 gb = gaussian_block((uint64_t)(2 * g + 1), layer_id, kTagDense, seed);
+  const uint32_t g = blockIdx.x * 256u + threadIdx.x;
+  if (g < n8) asm volatile("prefetch.global.L2 [%0];" ::"l"(w + 8 * (size_t)g));
+  const uint64_t b = (uint64_t)hi << 32 | 2u * g;
+  const float4 ga = gaussian_block(b, layer_id, kTagDense, seed), gb = gaussian_block(b | 1u, layer_id, kTagDense, seed);
   chain_wait();
+  if (g >= n8) return;
   const float c = d_scale ? scale * __ldcg(d_scale) : scale;
-  while (g < n8) {
-    const float u[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
-    if constexpr (sizeof(T) == 2) {
-      uint4* p = reinterpret_cast<uint4*>(w) + g;
-      const uint4 v = *p;
-      const uint32_t in[4] = {v.x, v.y, v.z, v.w};
-      uint32_t out[4];
+  const float u[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
+  if constexpr (sizeof(T) == 2) {
+    uint4* p = reinterpret_cast<uint4*>(w) + g;
+    const uint4 v = *p;
+    const uint32_t in[4] = {v.x, v.y, v.z, v.w};
+    uint32_t out[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float w0 = __uint_as_float(in[k] << 16), w1 = __uint_as_float(in[k] & 0xFFFF0000u);
-        __nv_bfloat162 r = __floats2bfloat162_rn(fmaf(c, u[2 * k], w0), fmaf(c, u[2 * k + 1], w1));
-        out[k] = *reinterpret_cast<uint32_t*>(&r);
-      }
-      *p = make_uint4(out[0], out[1], out[2], out[3]);
-    } else {
-      float4* p = reinterpret_cast<float4*>(w) + 2 * g;
-      float4 a = p[0], b = p[1];
-      a.x = fmaf(c, u[0], a.x); a.y = fmaf(c, u[1], a.y); a.z = fmaf(c, u[2], a.z); a.w = fmaf(c, u[3], a.w);
-      b.x = fmaf(c, u[4], b.x); b.y = fmaf(c, u[5], b.y); b.z = fmaf(c, u[6], b.z); b.w = fmaf(c, u[7], b.w);
-      p[0] = a; p[1] = b;
+    for (int k = 0; k < 4; ++k) {
+      const float w0 = __uint_as_float(in[k] << 16), w1 = __uint_as_float(in[k] & 0xFFFF0000u);
+      __nv_bfloat162 r = __floats2bfloat162_rn(fmaf(c, u[2 * k], w0), fmaf(c, u[2 * k + 1], w1));
+      out[k] = *reinterpret_cast<uint32_t*>(&r);
     }
-    g += stride;
-    if (g >= n8) break;
-    ga = gaussian_block((uint64_t)(2 * g), layer_id, kTagDense, seed);
-    gb = gaussian_block((uint64_t)(2 * g + 1), layer_id, kTagDense, seed);
+    *p = make_uint4(out[0], out[1], out[2], out[3]);
+  } else {
+    float4* p = reinterpret_cast<float4*>(w) + 2 * (size_t)g;
+    float4 a = p[0], b2 = p[1];
+    a.x = fmaf(c, u[0], a.x); a.y = fmaf(c, u[1], a.y); a.z = fmaf(c, u[2], a.z); a.w = fmaf(c, u[3], a.w);
+    b2.x = fmaf(c, u[4], b2.x); b2.y = fmaf(c, u[5], b2.y); b2.z = fmaf(c, u[6], b2.z); b2.w = fmaf(c, u[7], b2.w);
+    p[0] = a; p[1] = b2;
   }
 }
 
@@ -509,9 +506,11 @@ cudaError_t launch_dense_t(T* w, long long n, uint64_t seed, uint32_t layer_id, 
   const long long cap = (long long)sm_count * 8;      // eight resident blocks of 256 threads per SM
   long long n8 = 0;
   if ((reinterpret_cast<uintptr_t>(w) & 15u) == 0) n8 = n >> 3;
-  if (n8 > 0) {
-    const int grid = (int)((n8 + 255) / 256 < cap ? (n8 + 255) / 256 : cap);
-    cudaError_t e = launch_chained(dense_vec_kernel<T>, dim3(grid), 256, 0, 0, s, w, n8, seed, layer_id, scale, d_scale);
+  constexpr long long kLaunch8 = 1ll << 31;           // steps of a launch: 2^32 blocks, which share their upper word
+  for (long long at = 0; at < n8; at += kLaunch8) {
+    const uint32_t steps = (uint32_t)(n8 - at < kLaunch8 ? n8 - at : kLaunch8);
+    cudaError_t e = launch_chained(dense_vec_kernel<T>, dim3((steps + 255u) / 256u), 256, 0, 0, s, w + 8 * at, steps,
+                                   (uint32_t)(at / kLaunch8), seed, layer_id, scale, d_scale);
     if (e != cudaSuccess) return e;
   }
   if (8 * n8 < n) {                                    // the rest: blocks from 2 n8 on

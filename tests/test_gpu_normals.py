@@ -69,3 +69,20 @@ def test_first_product_with_the_test_matrix(m, r):
     Vg = to_host(V)
     assert np.abs(Vg.astype(np.float64) @ Vg.T - np.eye(r)).max() <= 1e-5
     assert projector_distance(Vg, O.extract_subspace(X, r, 0, 9, 4)) <= 1e-3
+
+
+def test_dense_direction_beyond_one_launch():
+    """A launch of the dense pass holds 2^34 elements; the ones after it belong to blocks whose numbers have another upper word."""
+    n = (1 << 34) + 4096 + 5
+    if torch.cuda.mem_get_info()[0] < 2 * n + (4 << 30):
+        pytest.skip("needs 36 GB")
+    w = torch.zeros(n, dtype=torch.bfloat16, device=DEV)
+    ctx = B.Context(0, 4096)
+    B.agzo_perturb_dense(ctx, w, 77, 3, 1.0)
+    for first in (0, (1 << 34) - 2048, 1 << 34):
+        k = min(4096 + 5, n - first)
+        want = B.agzo_debug_gaussian(ctx, 77, 3, 2, first, k).to(torch.bfloat16)
+        assert torch.equal(w[first:first + k], want)
+    B.agzo_destroy(ctx)
+    del w
+    torch.cuda.empty_cache()
