@@ -90,7 +90,7 @@ __device__ __forceinline__ void generate_G(float* sG, int RS, int r, long long r
   const int nb = (int)(((e_last - 1) >> 2) - b_first + 1);
   for (int i = threadIdx.x; i < nb; i += kRmwThreads) {
     const long long b = b_first + i;
-    const float4 g = gaussian_block((uint64_t)b, layer_id, kTagG, seed);
+    const float4 g = gaussian_block<false>((uint64_t)b, layer_id, kTagG, seed);
     const float gv[4] = {g.x, g.y, g.z, g.w};
 #pragma unroll
     for (int lane = 0; lane < 4; ++lane) {
