@@ -165,6 +165,10 @@ agzo_status agzo_destroy(agzo_ctx* ctx);
  * 4 layers and 24 ranks on one X, at most 12 different X) is extracted by one kernel that keeps them there; it takes the place of
  * all others where it is estimated to be faster, unless an option asks for one of those ("extract_path", "extract_fused" other
  * than 1, "wave_bytes"; "time_kernel_class" with a class of theirs) or an all-reduce is set.  2 = wherever it can run, 0 = never;
+ * "extract_split" 1 (default) = products of layers that the tensor-core kernels above do not take (fp32 activations, rows of bf16 that
+ * are not whole 16-byte pieces, fewer than 256 tokens) run on the tensor cores in bf16 parts of fp32 numbers, three of each factor,
+ * where that is estimated to be faster than the CUDA-core kernels, whose precision it has; 2 = wherever it can run, 0 = never.  fp32
+ * activations without a power step (K = 0), waves of both types and "extract_path" 1 stay with the CUDA cores;
  * "wave_bytes" = activation bytes grouped into one launch wave of extraction;
  * "extract_streams" 2 (default) = alternate waves use two scratch regions and two helper
  * streams forked from and joined to the caller's stream, so that one wave's short kernels
@@ -206,8 +210,8 @@ agzo_status agzo_set_allreduce(agzo_ctx* ctx, agzo_allreduce_fn fn, void* user, 
 typedef enum agzo_kernel_class {
   AGZO_KC_NONE = 0,
   AGZO_KC_RMW = 1,        /* the in-place low-rank pass                                    */
-  AGZO_KC_XT_T = 2,       /* Y = X^T T, CUDA-core kernel                                   */
-  AGZO_KC_X_Q = 3,        /* T = X Q, CUDA-core kernel                                     */
+  AGZO_KC_XT_T = 2,       /* Y = X^T T in fp32: CUDA-core kernel, or in parts              */
+  AGZO_KC_X_Q = 3,        /* T = X Q in fp32: CUDA-core kernel, or in parts                */
   AGZO_KC_PANEL_QR = 4,   /* qr(Y)                                                         */
   AGZO_KC_TC_XT_T = 5,    /* Y = X^T T, tensor-core kernel                                 */
   AGZO_KC_TC_X_Q = 6,     /* T = X Q, tensor-core kernel                                   */

@@ -11,6 +11,7 @@
 
 #include "agzo_common.cuh"
 #include "agzo_resident.cuh"
+#include "agzo_split.cuh"
 #include "agzo_tc.cuh"
 
 using namespace agzo;
@@ -44,6 +45,7 @@ struct Plan {
   int fast_mode_mask = 0;          // storage modes present among layers on the vector path
   bool any_slow = false;           // some layer needs the scalar kernel
   bool has_extract = false;
+  bool split = false;              // products in parts (agzo_split.cuh) for the waves that they can serve
   // tensor-core in-place pass: work items per layer (prefix, n + 1), zero-length for other layers
   std::vector<int> item_start;
   int total_items = 0;
@@ -67,6 +69,7 @@ struct PlanOpts {
   bool share_inputs;     // consecutive layers with the same X are served by one sweep
   int extract_regions;   // 1: waves run one after another; 2: alternate waves use two scratch regions
                          // and two helper streams, so one wave's small kernels overlap the other's sweeps
+  int split;             // the products that the TMA kernels do not take run in parts on the tensor cores: 0 never, 1 where that pays, 2 always
   int sm_count;          // of the device; when sizing without one, any number will do
   const FusedCaps* fused_caps;   // what the device holds of the fused kernel; null when sizing without a device
 };
@@ -91,6 +94,7 @@ struct agzo_ctx {
   int extract_streams;     // 1 or 2 (see PlanOpts::extract_regions)
   int extract_fused;       // 0 off, 1 fused power-step kernel where it pays, 2 wherever a layer's shape allows it
   int share_inputs;        // 1: consecutive layers with the same X share the sweeps over it
+  int extract_split;       // products that the TMA kernels do not take, in bf16 parts on the tensor cores: 1 where that is faster, 2 always, 0 never
   int extract_resident;    // 1: inputs that fit the chip's shared memory are extracted by one kernel where that is faster; 2: always; 0: never
   // the layer list that extraction last looked at for that kernel, and what came of it
   std::vector<agzo_layer> resident_cached;
@@ -236,14 +240,15 @@ bool same_input(const agzo_layer& a, const agzo_layer& b) {
 // panel QR), and the CTAs' pipelines start and drain less often.
 constexpr int kLongSlabColumnBlocks = 1024;   // 128-column blocks over all layers from which slabs are long
 // cc_blocks: 128-column blocks over the call's layers on the CUDA-core path; 0 = the most slabs the layer can get (sizing).
-void slab_shape(const agzo_layer& a, bool tc, bool long_slabs, long long cc_blocks, int sm_count, int* slabs, int* slab_rows) {
+// split: cc_blocks counts units of the products in parts.
+void slab_shape(const agzo_layer& a, bool tc, bool long_slabs, long long cc_blocks, bool split, int sm_count, int* slabs, int* slab_rows) {
   int rows;
   if (tc) {
     rows = a.m >= 8192 ? (long_slabs ? (a.m < 16384 ? a.m : 16384) : 2048) : (a.m + 3) / 4;
     rows = (rows + 127) / 128 * 128;      // whole tiles of every tensor-core kernel (64 or 128 tokens)
     if (rows < 256) rows = 256;
   } else if (cc_blocks > 0) {
-    rows = cc_slab_rows(a.m, cc_blocks, sm_count);
+    rows = split ? split_slab_rows(a.m, cc_blocks, sm_count) : cc_slab_rows(a.m, cc_blocks, sm_count);
   } else {
     const int most = (a.m + kCcMinSlabRows - 1) / kCcMinSlabRows;
     *slabs = most < kCcMaxSlabs ? most : kCcMaxSlabs;
@@ -402,6 +407,22 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
   for (int k = 0; k < n; ++k)
     if (has_x(L[k]))
       (on_tc(L[k]) ? column_blocks : cc_blocks) += (L[k].d_in + 127) / 128;
+  plan->split = false;
+  if (opts.split && cc_blocks > 0) {
+    std::vector<int> which;
+    for (int k = 0; k < n; ++k)
+      if (has_x(L[k]) && !on_tc(L[k])) which.push_back(k);
+    plan->split = opts.split == 2 || split_pays(L, which, opts.share_inputs, opts.sm_count);
+  }
+  if (plan->split) {                       // its units are panels of the layers on one X
+    cc_blocks = 0;
+    for (int k = 0; k < n;) {
+      int run = 1, all = L[k].r;
+      while (opts.share_inputs && has_x(L[k]) && k + run < n && has_x(L[k + run]) && same_input(L[k], L[k + run])) all += L[k + run++].r;
+      if (has_x(L[k]) && !on_tc(L[k])) cc_blocks += (long long)((L[k].d_in + 127) / 128) * ((all + kSplitMaxRanks - 1) / kSplitMaxRanks);
+      k += run;
+    }
+  }
   const bool long_slabs_any = column_blocks >= kLongSlabColumnBlocks;
   int extract_max_r = 0;
   for (int k = 0; k < n; ++k)
@@ -412,7 +433,7 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
   };
   auto ypart_bytes = [&](int parts, int ranks, int d_in) { return align_up((size_t)parts * ranks * (size_t)d_in * 4); };
   auto slabs_of = [&](const agzo_layer& a, bool tc, int* slabs, int* slab_rows) {
-    slab_shape(a, tc, long_slabs_any, ws ? cc_blocks : 0, opts.sm_count, slabs, slab_rows);
+    slab_shape(a, tc, long_slabs_any, ws ? cc_blocks : 0, plan->split, opts.sm_count, slabs, slab_rows);
     // a workspace of less than agzo_workspace_bytes takes fewer slabs on the CUDA-core path, as long as one is left
     for (int want = *slabs; ws && !tc && want > 1 && ypart_bytes(*slabs, a.r, a.d_in) + layer_need(a, tc) > scratch_cap;) {
       --want;
@@ -604,7 +625,7 @@ unsigned long long capture_of(cudaStream_t s) {
 
 PlanOpts plan_opts(const agzo_ctx* c, int regions) {
   return PlanOpts{c->wave_bytes, c->extract_path, c->rmw_path, c->rmw_tc_min_rank, c->rmw_tc_panels, c->rmw_stage_r,
-                  c->tc.available, c->extract_fused, c->share_inputs != 0, regions, c->sm_count, &c->tc.fused};
+                  c->tc.available, c->extract_fused, c->share_inputs != 0, regions, c->extract_path == 0 ? c->extract_split : 0, c->sm_count, &c->tc.fused};
 }
 
 bool any_weights(const agzo_layer* L, int n) {
@@ -798,13 +819,13 @@ agzo_status agzo_workspace_bytes(const agzo_layer* h_layers, int n, size_t* h_by
   // the CUDA-core kernels, whose slabs are shaped differently)
   Plan plan;
   size_t scratch = 0, scratch_cc = 0;
-  st = build_plan(h_layers, n, nullptr, 0, PlanOpts{kDefaultWaveBytes, 0, 0, 3, 0, 0, true, 0, false, 2, 148, nullptr}, &plan, &scratch);
+  st = build_plan(h_layers, n, nullptr, 0, PlanOpts{kDefaultWaveBytes, 0, 0, 3, 0, 0, true, 0, false, 2, 0, 148, nullptr}, &plan, &scratch);
   if (st != AGZO_OK) return st;
-  st = build_plan(h_layers, n, nullptr, 0, PlanOpts{kDefaultWaveBytes, 1, 1, 0, 1, 1, false, 0, false, 2, 148, nullptr}, &plan, &scratch_cc);
+  st = build_plan(h_layers, n, nullptr, 0, PlanOpts{kDefaultWaveBytes, 1, 1, 0, 1, 1, false, 0, false, 2, 0, 148, nullptr}, &plan, &scratch_cc);
   if (st != AGZO_OK) return st;
   if (scratch_cc > scratch) scratch = scratch_cc;
   // ... and for the fused power step, whose layers keep room for one partial sum of Y per share of a launch
-  st = build_plan(h_layers, n, nullptr, 0, PlanOpts{kDefaultWaveBytes, 0, 0, 3, 0, 0, true, 2, false, 2, 148, nullptr}, &plan, &scratch_cc);
+  st = build_plan(h_layers, n, nullptr, 0, PlanOpts{kDefaultWaveBytes, 0, 0, 3, 0, 0, true, 2, false, 2, 0, 148, nullptr}, &plan, &scratch_cc);
   if (st != AGZO_OK) return st;
   if (scratch_cc > scratch) scratch = scratch_cc;
   *h_bytes = kHeaderBytes + table_bytes(n) + scratch + kAlign;
@@ -847,6 +868,7 @@ agzo_status agzo_create(agzo_ctx** out, int device, void* workspace, size_t work
   c->token_offset = 0;
   c->share_inputs = 1;
   c->extract_resident = 1;
+  c->extract_split = 1;
   c->resident_known = c->resident_ok = false;
   c->resident_admitted = -1;
   c->aux[0] = c->aux[1] = nullptr;
@@ -940,6 +962,9 @@ agzo_status agzo_set_option(agzo_ctx* ctx, const char* name, int64_t value) {
     if (value < 0 || value > 2) return AGZO_ERR_INVALID_ARG;
     ctx->extract_resident = (int)value;
     return AGZO_OK;
+  } else if (std::strcmp(name, "extract_split") == 0) {
+    if (value < 0 || value > 2) return AGZO_ERR_INVALID_ARG;
+    ctx->extract_split = (int)value;
   } else if (std::strcmp(name, "extract_fused") == 0) {
     if (value < 0 || value > 2) return AGZO_ERR_INVALID_ARG;
     ctx->extract_fused = (int)value;
@@ -1139,6 +1164,8 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
         if (ctx->allreduce(ctx->allreduce_user, ws, P.wave_y[wv], P.wave_y_count[wv]) != 0) return AGZO_ERR_CALLBACK;
         return AGZO_OK;
       };
+      // products of this wave in parts: layers of one dtype, and for fp32 a power step (see split_takes)
+      const bool split = !all_tc && P.split && split_takes(w, P.dev.data(), K);
       auto omega = [&]() -> cudaError_t {
         Timed t(ctx, AGZO_KC_OMEGA, ws);
         return all_tc ? tc_fill_omega(ctx->tc, w, P.dev.data(), seed, ws) : launch_fill_omega(w, seed, ws);
@@ -1151,10 +1178,12 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
       }
       auto xt_t = [&](bool skip_fused) -> cudaError_t {       // Y <- H T
         Timed t(ctx, all_tc ? AGZO_KC_TC_XT_T : AGZO_KC_XT_T, ws);
+        if (split) return launch_split_xt_t(w, P.dev.data(), ctx->share_inputs != 0, dst, ws);
         return all_tc ? tc_xt_t(ctx->tc, w, P.dev.data(), dst, skip_fused, ws) : launch_xt_t(w, ws);
       };
       auto x_q = [&]() -> cudaError_t {        // T <- H^T Q
         Timed t(ctx, all_tc ? AGZO_KC_TC_X_Q : AGZO_KC_X_Q, ws);
+        if (split) return launch_split_x_q(w, P.dev.data(), ctx->share_inputs != 0, dst, ws);
         return all_tc ? tc_x_q(ctx->tc, w, P.dev.data(), dst, true, ws) : launch_x_q(w, ws);
       };
       auto power_fused = [&]() -> cudaError_t {              // Y <- H (H^T Q) in one pass

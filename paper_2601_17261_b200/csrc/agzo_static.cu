@@ -12,6 +12,7 @@
 #include "agzo_common.cuh"
 #include "agzo_ptx.cuh"
 #include "agzo_resident.cuh"
+#include "agzo_split.cuh"
 
 namespace {
 
@@ -78,9 +79,12 @@ __global__ void static_begin_kernel(agzo::DevLayer rec, agzo::DevLayer* dst, agz
   st->pad = 0;
 }
 
-__global__ void static_end_kernel(const agzo::DevStatus* st, int32_t* flag) {
+// a wait of the products that ran out: V = 0, and the flag says so with a 2
+__global__ void static_end_kernel(const agzo::DevStatus* st, int32_t* flag, float* V, long long ldv, int r, int d_in) {
   agzo::chain_wait();
-  *flag = st->rank_deficient;
+  if (flag && threadIdx.x == 0) *flag = st->timeout ? 2 : st->rank_deficient;
+  if (st->timeout)
+    for (long long i = threadIdx.x; i < (long long)r * d_in; i += blockDim.x) V[i / d_in * ldv + i % d_in] = 0.f;
 }
 
 }  // namespace
@@ -114,10 +118,10 @@ agzo_status extract_static(const void* X, int64_t ldx, int32_t x_dtype, int32_t 
   Scratch scratch;
   if (scratch_of_current_device(&scratch) != cudaSuccess) return AGZO_ERR_CUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  agzo_layer a{};
+  a.X = X; a.ldx = ldx; a.x_dtype = x_dtype; a.m = m; a.d_in = d_in; a.r = r; a.layer_id = layer_id;
+  a.V = V; a.ldv = ldv;
   if (route != 1) {
-    agzo_layer a{};
-    a.X = X; a.ldx = ldx; a.x_dtype = x_dtype; a.m = m; a.d_in = d_in; a.r = r; a.layer_id = layer_id;
-    a.V = V; a.ldv = ldv;
     ResidentLaunch plan;      // K = 0: a block that comes too late to the only meeting would not see that others have given up
     if (resident_plan(scratch.resident, &a, 1, false, false, &plan) && plan.scratch <= kResidentScratchBytes &&
         !(plan.grid_wide && K == 0) && (route == 2 || resident_pays(plan, K, true))) {
@@ -134,7 +138,9 @@ agzo_status extract_static(const void* X, int64_t ldx, int32_t x_dtype, int32_t 
     }
     if (route == 2) return AGZO_ERR_UNSUPPORTED;
   }
-  for (int rows = cc_slab_rows(m, (long long)gch, scratch.sm_count);; rows += 32) {      // ends at 256 tokens per slab at the latest
+  const bool split = (K > 0 || x_dtype == AGZO_BF16) && split_pays(&a, std::vector<int>{0}, true, scratch.sm_count);
+  const long long panels = (r + kSplitMaxRanks - 1) / kSplitMaxRanks;
+  for (int rows = split ? split_slab_rows(m, (long long)gch * panels, scratch.sm_count) : cc_slab_rows(m, (long long)gch, scratch.sm_count);; rows += 32) {      // ends at 256 tokens per slab at the latest
     const size_t n = ((size_t)m + rows - 1) / rows;
     if (need - up256((size_t)slabs * R * D * 4) + up256(n * R * D * 4) <= kStaticScratchBytes) { slab_rows = rows; slabs = (int)n; break; }
   }
@@ -163,15 +169,18 @@ agzo_status extract_static(const void* X, int64_t ldx, int32_t x_dtype, int32_t 
   w.qr_wide = scratch.qr_wide ? 1 : 0;
   w.max_m = m; w.max_din = d_in; w.max_r = r; w.max_slabs = slabs; w.max_gchunks = (int)gch;
   if (launch_fill_omega(w, seed, s) != cudaSuccess) return AGZO_ERR_CUDA;     // Omega
-  if (launch_xt_t(w, s) != cudaSuccess) return AGZO_ERR_CUDA;                 // Y <- H Omega
+  const auto xt_t = [&] { return split ? launch_split_xt_t(w, &rec, true, d_status, s) : launch_xt_t(w, s); };
+  const auto x_q = [&] { return split ? launch_split_x_q(w, &rec, true, d_status, s) : launch_x_q(w, s); };
+  if (xt_t() != cudaSuccess) return AGZO_ERR_CUDA;                            // Y <- H Omega
   for (int k = 0; k < K; ++k) {
     if (launch_panel_qr(w, false, d_status, s) != cudaSuccess) return AGZO_ERR_CUDA;  // Q <- qr(Y)
-    if (launch_x_q(w, s) != cudaSuccess) return AGZO_ERR_CUDA;
-    if (launch_xt_t(w, s) != cudaSuccess) return AGZO_ERR_CUDA;               // Y <- H (H^T Q)
+    if (x_q() != cudaSuccess) return AGZO_ERR_CUDA;
+    if (xt_t() != cudaSuccess) return AGZO_ERR_CUDA;                          // Y <- H (H^T Q)
   }
   if (launch_panel_qr(w, true, d_status, s) != cudaSuccess) return AGZO_ERR_CUDA;    // A <- qr(Y)
-  if (d_rank_deficient) {
-    if (launch_chained(static_end_kernel, dim3(1), 1, 0, 0, s, d_status, d_rank_deficient) != cudaSuccess) return AGZO_ERR_CUDA;
+  if (d_rank_deficient || split) {
+    if (launch_chained(static_end_kernel, dim3(1), split ? 256 : 1, 0, 0, s, d_status, d_rank_deficient, V, (long long)ldv, r, d_in) != cudaSuccess)
+      return AGZO_ERR_CUDA;
   }
   return AGZO_OK;
 }
