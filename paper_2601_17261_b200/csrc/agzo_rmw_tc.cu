@@ -138,7 +138,8 @@ __device__ __forceinline__ void put_group(uint8_t* base, int atom_bytes, int row
 
 // Rank indices 8g .. 8g+7 of row `row` of R (d_out x r, i.i.d. N(0,1) from the Philox stream
 // (seed, layer_id, tag 0), element e = row * r + k), as bf16 hi parts and bf16 lo parts; zero
-// beyond the matrix.
+// beyond the matrix.  kPacked: see box_muller4; in the pass, whose kernel is at the registers of its block, the pairs one by one.
+template <bool kPacked>
 __device__ __forceinline__ void gen_r_group(const DevLayer& L, long long row, int g, uint64_t seed, uint4* hi_out,
                                             uint4* lo_out) {
   const int r = L.r;
@@ -153,11 +154,11 @@ __device__ __forceinline__ void gen_r_group(const DevLayer& L, long long row, in
     const int off = (int)(e_first & 3);
     const int nblk = (off + nv + 3) >> 2;
     float x[12];
-    const float4 ga = gaussian_block((uint64_t)b0, L.layer_id, kTagG, seed);
+    const float4 ga = gaussian_block<kPacked>((uint64_t)b0, L.layer_id, kTagG, seed);
     x[0] = ga.x; x[1] = ga.y; x[2] = ga.z; x[3] = ga.w;
     float4 gb = make_float4(0.f, 0.f, 0.f, 0.f), gc = gb;
-    if (nblk > 1) gb = gaussian_block((uint64_t)(b0 + 1), L.layer_id, kTagG, seed);
-    if (nblk > 2) gc = gaussian_block((uint64_t)(b0 + 2), L.layer_id, kTagG, seed);
+    if (nblk > 1) gb = gaussian_block<kPacked>((uint64_t)(b0 + 1), L.layer_id, kTagG, seed);
+    if (nblk > 2) gc = gaussian_block<kPacked>((uint64_t)(b0 + 2), L.layer_id, kTagG, seed);
     x[4] = gb.x; x[5] = gb.y; x[6] = gb.z; x[7] = gb.w;
     x[8] = gc.x; x[9] = gc.y; x[10] = gc.z; x[11] = gc.w;
 #pragma unroll
@@ -404,7 +405,7 @@ rmw_tc_kernel(const DevLayer* layers, const int* item_start, int n_layers,
         for (int unit = gt; unit < kRows * g8; unit += gen_threads) {
           const int g = unit >> 7, i = unit & (kRows - 1);
           uint4 hi, lo;
-          gen_r_group(L, (long long)rb * kRows + i, g, seed, &hi, &lo);
+          gen_r_group<false>(L, (long long)rb * kRows + i, g, seed, &hi, &lo);
           put_group(a_base, kAtomBytesA, i, g, g8, hi, lo);
         }
         fence_proxy_async();
@@ -494,7 +495,7 @@ __global__ void __launch_bounds__(256) rmw_tc_fill_r_kernel(const DevLayer* laye
   for (int unit = threadIdx.x; unit < kRows * g8; unit += 256) {
     const int g = unit >> 7, i = unit & (kRows - 1);
     uint4 hi, lo;
-    gen_r_group(L, (long long)rb * kRows + i, g, seed, &hi, &lo);
+    gen_r_group<true>(L, (long long)rb * kRows + i, g, seed, &hi, &lo);
     put_group(img, kAtomBytesA, i, g, g8, hi, lo);
   }
 }
