@@ -75,3 +75,17 @@ def test_tall_tiles():
     assert off.mean() <= 2e-3
     assert off.sum(axis=1).max() < 10
     assert off[:, 512:].mean() <= 4e-3
+
+
+@pytest.mark.parametrize("kind", ["bf16", "f32", "pair"])
+@pytest.mark.parametrize("r", [1, 4, 15, 16, 17, 33, 64])
+@pytest.mark.parametrize("d_out,d_in", [(1, 67), (7, 511), (33, 513), (259, 301)])
+def test_element_by_element(kind, r, d_out, d_in):
+    # rows that are not whole 16-byte pieces: columns around a thread's two, rows around its eight and the 32 of a piece of R, ranks
+    # around the sixteen that it has in registers
+    W0, Vh, Wd, W16, (_, layer) = one(d_out, d_in, r, kind)
+    with Ctx([layer]) as ctx:
+        B.agzo_set_option(ctx, "rmw_path", 1)
+        B.agzo_perturb(ctx, [layer], 11, 1e-3)
+        torch.cuda.synchronize()
+    verify(W0, Vh, Wd, W16, kind, 1e-3, 11, 0)
