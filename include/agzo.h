@@ -138,7 +138,8 @@ agzo_status agzo_destroy(agzo_ctx* ctx);
  * tensor-core kernels (UNSUPPORTED at call time if a layer cannot use them), 3 = as 2 but
  * without the fused power-step kernel (T = X Q and Y = X^T T as two sweeps over X);
  * "rmw_path" selects the kernel of the in-place passes: 0 = automatic (bf16 weights with
- * 16-byte aligned rows and r >= "rmw_tc_min_rank", default 5, take the tensor-core kernel, and so
+ * 16-byte aligned rows and r >= "rmw_tc_min_rank", default 5 (which lists of few weights do not heed: up to
+ * 32 million at ranks up to 8, 3 million up to 16, stay with the CUDA cores), take the tensor-core kernel, and so
  * from rank 3 on do those whose d_in or V rules out 16-byte accesses; everything else the CUDA-core
  * kernels), 1 = CUDA-core kernels only, 2 = tensor-core kernel for every layer that allows it;
  * tuning knobs of that kernel, 0 = chosen by rank:

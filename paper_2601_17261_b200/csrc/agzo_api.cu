@@ -56,6 +56,8 @@ struct Plan {
   size_t image_bytes = 0;
 };
 
+constexpr int kRmwTcMinRank = 5;   // default of the option
+
 struct PlanOpts {
   int64_t wave_bytes;
   int extract_path;      // 0 auto, 1 CUDA-core only, 2 tensor-core required
@@ -259,6 +261,7 @@ void slab_shape(const agzo_layer& a, bool tc, bool long_slabs, long long cc_bloc
   *slabs = (a.m + rows - 1) / rows;
 }
 
+
 constexpr size_t kMapBytes = 512;   // four TMA descriptors per layer
 // device tables after the header: layer records | tile prefix and item prefix (n + 1 ints each) | TMA descriptors
 size_t prefix_bytes(int n) { return align_up((size_t)2 * (n + 1) * sizeof(int)); }
@@ -306,10 +309,25 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     if (a.W16) vec = vec && aligned16(a.W16) && (a.ldw16 * 2) % 16 == 0;
     return vec;
   };
+  // A list of few weights, which L2 holds between the passes, is a matter of set-up, of which the tensor-core pass has more: where it
+  // would take over at its own rank it does so from 32 M weights up to rank 8, from 3 M up to rank 16 (CUDA cores / tensor cores, us per pass:
+  // 0.8 M r = 8 4.8 / 8.6, r = 16 5.0 / 8.5; 8.4 M r = 8 9.5 / 10.9, r = 16 13.0 / 11.2; 31 M r = 5 23.4 / 27.2, r = 8 23.5 / 25.0; 50 M r = 5
+  // 41.3 / 40.7, r = 8 43.4 / 37.9).
+  bool few_weights = false;
+  if (opts.rmw_path == 0 && opts.rmw_tc_min_rank == kRmwTcMinRank) {
+    int64_t weights = 0;
+    int max_r = 0;
+    for (int i = 0; i < n; ++i)
+      if (rmw_tc_eligible(L[i])) {
+        weights += (int64_t)L[i].d_out * L[i].d_in;
+        max_r = std::max(max_r, L[i].r);
+      }
+    few_weights = weights <= (max_r <= 8 ? 32000000ll : max_r <= 16 ? 3000000ll : 0ll);
+  }
   auto takes_tc_rmw = [&](const agzo_layer& a) {
     // from rank 3 on the element-by-element kernel is no alternative where the vector kernels cannot run
     return tc_available && opts.rmw_path != 1 && rmw_tc_eligible(a) &&
-           (opts.rmw_path == 2 || a.r >= opts.rmw_tc_min_rank || (a.r >= 3 && !vector_rows(a)));
+           (opts.rmw_path == 2 || (a.r >= opts.rmw_tc_min_rank && !few_weights) || (a.r >= 3 && !vector_rows(a)));
   };
   {
     size_t img = 0;
@@ -326,12 +344,46 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     plan->max_row_tiles = max_tiles;
     plan->image_bytes = want ? img : 0;
   }
+  // Rows per tile of the CUDA-core pass.  The CTAs, all resident, take tiles in turn, so a pass lasts as many rounds as the one with most
+  // tiles has, each a tile's rows and what setting up a tile costs, twelve more (R, the slice of A^T, the record; with the slice in shared
+  // memory as many again as there are ranks); where there are several rounds, CTAs have drifted apart by half a tile at the end.
+  // Multiples of eight, the tallest of the cheapest.  Measured on 18 lists at 14 heights each; against the other rule two fp32 0.6B-shaped blocks,
+  // r = 8, 51 -> 45 us, eight 1024 x 1024 pairs 14.7 -> 9.7, a bf16 0.6B-shaped block, r = 3, 16.7 -> 10.3, twelve, r = 2, 125 -> 122.
+  // Lists of more than 640 MB are bound by HBM whatever the rounds: the tallest tiles of which each CTA gets sixteen, for rank 1, whose set-up
+  // is least, half as tall (sixty 2048 x 2048 fp32 layers, r = 4, at 64 rows 316 us, 336 by rounds; eight 8B-shaped blocks, r = 1, at 256 / 128 / 64
+  // rows 979 / 943 / 969, twenty, r = 4, at 256 / 128 2456 / 2502).
   {
-    long long strips = 0;
-    for (int i = 0; i < n; ++i)
-      if (L[i].W && !takes_tc_rmw(L[i]))
-        strips += (long long)((L[i].d_in + kRmwTileCols - 1) / kRmwTileCols) * ((L[i].d_out + kRmwMinTileRows - 1) / kRmwMinTileRows);
-    plan->tile_rows = rmw_tile_rows(strips, opts.sm_count);
+    struct Strip { int d_out, n; };
+    std::vector<Strip> strips;             // 512 columns wide, by height
+    int max_r = 0;
+    int64_t bytes = 0;
+    bool slow = false;
+    for (int i = 0; i < n; ++i) {
+      if (!L[i].W || takes_tc_rmw(L[i])) continue;
+      const int count = (L[i].d_in + kRmwTileCols - 1) / kRmwTileCols;
+      max_r = std::max(max_r, L[i].r);
+      bytes += (int64_t)L[i].d_out * L[i].d_in * ((L[i].w_dtype == AGZO_BF16 ? 2 : 4) + (L[i].W16 ? 2 : 0));
+      slow = slow || !vector_rows(L[i]);
+      auto same = std::find_if(strips.begin(), strips.end(), [&](const Strip& s) { return s.d_out == L[i].d_out; });
+      if (same != strips.end()) same->n += count; else strips.push_back(Strip{L[i].d_out, count});
+    }
+    const long long ctas = (slow ? 4ll : max_r <= 8 ? 2ll : 1ll) * opts.sm_count;       // element by element: four on an SM
+    long long least = -1;
+    auto tiles_of = [&](int rows) {
+      long long tiles = 0;
+      for (const Strip& s : strips) tiles += (long long)s.n * ((s.d_out + rows - 1) / rows);
+      return tiles;
+    };
+    if (bytes > (640ll << 20)) {
+      plan->tile_rows = slow ? 32 : max_r == 1 ? kRmwMaxTileRows / 2 : kRmwMaxTileRows;
+      while (plan->tile_rows > 32 && tiles_of(plan->tile_rows) < 32ll * opts.sm_count) plan->tile_rows /= 2;
+      strips.clear();
+    }
+    for (int rows = slow ? 32 : kRmwMaxTileRows; rows >= 8 && !strips.empty(); rows -= 8) {
+      const long long rounds = (tiles_of(rows) + ctas - 1) / ctas;
+      const long long cost = 2 * rounds * (rows + 12 + (max_r > 16 ? max_r : 0)) + (rounds > 1 ? rows : 0);
+      if (least < 0 || cost < least) { least = cost; plan->tile_rows = rows; }
+    }
   }
   // A list with fewer items than three quarters of the SMs gets shorter ones (one 4096 x 4096 layer, r = 64: 64 items of eight
   // row tiles 23.7 us, 128 of four 16.5, 256 of two 20.3; r = 8: 128 of four 14.5, 256 of two 16.7).
@@ -850,7 +902,7 @@ agzo_status agzo_create(agzo_ctx** out, int device, void* workspace, size_t work
   c->last_cuda = 0;
   c->extract_path = 0;
   c->rmw_path = 0;
-  c->rmw_tc_min_rank = 5;   // 8B shapes, six blocks, one pass, CUDA cores / tensor cores: r = 1 736 / 786 us, r = 4 732 / 783,
+  c->rmw_tc_min_rank = kRmwTcMinRank;   // 8B shapes, six blocks, one pass, CUDA cores / tensor cores: r = 1 736 / 786 us, r = 4 732 / 783,
                             // r = 6 822 / 780, r = 8 823 / 783, r = 16 1471 / 770; 0.6B shapes r = 4 282 / 302, r = 6 331 / 316
   c->rmw_tc_slots = 0;
   c->rmw_tc_inflight = 0;

@@ -89,3 +89,16 @@ def test_element_by_element(kind, r, d_out, d_in):
         B.agzo_perturb(ctx, [layer], 11, 1e-3)
         torch.cuda.synchronize()
     verify(W0, Vh, Wd, W16, kind, 1e-3, 11, 0)
+
+
+@pytest.mark.parametrize("r,d_out,n,tensor_cores", [(8, 4000, 8, False), (8, 4008, 8, True), (16, 1500, 2, False), (16, 1504, 2, True),
+                                                     (17, 64, 1, True), (4, 4008, 8, False)])
+def test_lists_of_few_weights_stay_with_the_cuda_cores(r, d_out, n, tensor_cores):
+    W = [torch.zeros(d_out, 1000, dtype=torch.bfloat16, device=DEV) for _ in range(n)]
+    V = torch.zeros(r, 1000, device=DEV)
+    layers = [B.make_layer(W=w, V=V, r=r, layer_id=i) for i, w in enumerate(W)]
+    with Ctx(layers, extra=1 << 24) as ctx:
+        for kind, want in ((B.KC_RMW, not tensor_cores), (B.KC_RMW_TC, tensor_cores)):
+            B.agzo_set_option(ctx, "time_kernel_class", kind)
+            B.agzo_perturb(ctx, layers, 3, 1e-3)
+            assert (B.agzo_read_counters(ctx)[1] > 0) == want
