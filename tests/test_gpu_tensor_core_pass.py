@@ -35,3 +35,20 @@ def test_items_that_rebuild_the_operand(n, d_out, d_in, pad, r):
         want = O.apply_direction(W0, Vh, seed, i, np.float32(c), "bf16")
         assert_weights_match(to_host(Ws[i]), want, "bf16", frac=tc_mismatch_bound(want, c, seed, i, Vh),
                              floor=cancellation_floor(W0, c, seed, i, Vh, rel=2.0 ** -16))
+
+
+@pytest.mark.parametrize("r", [12, 40])
+def test_last_layers_of_a_few_rounds_have_shorter_items(r):
+    # about one and a half rounds of items over the SMs: the last layers' are cut shorter, with remainders in both directions
+    n, d_out, d_in, seed, c = 9, 1300, 1096, 13, 1e-3
+    W0 = WL.gaussian_weights(d_out, d_in, 0.02, seed=r, bf16=True)
+    Vh = np.linalg.qr(np.random.default_rng(r).standard_normal((d_in, r)))[0].T.astype(np.float32).copy()
+    Ws, V = [to_dev(W0, True)[0] for _ in range(n)], to_dev(Vh, False)[0]
+    layers = [B.make_layer(W=W, V=V, r=r, layer_id=i) for i, W in enumerate(Ws)]
+    with Ctx(layers, extra=1 << 24) as ctx:
+        B.agzo_perturb(ctx, layers, seed, c)
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+    for i in (0, n - 2, n - 1):
+        want = O.apply_direction(W0, Vh, seed, i, np.float32(c), "bf16")
+        assert_weights_match(to_host(Ws[i]), want, "bf16", frac=tc_mismatch_bound(want, c, seed, i, Vh),
+                             floor=cancellation_floor(W0, c, seed, i, Vh, rel=2.0 ** -16))
