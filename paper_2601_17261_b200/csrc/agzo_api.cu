@@ -345,9 +345,10 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     plan->image_bytes = want ? img : 0;
   }
   // Rows per tile of the CUDA-core pass.  The CTAs, all resident, take tiles in turn, so a pass lasts as many rounds as the one with most
-  // tiles has, each a tile's rows and what setting up a tile costs, twelve more (R, the slice of A^T, the record; with the slice in shared
-  // memory as many again as there are ranks); where there are several rounds, CTAs have drifted apart by half a tile at the end.
-  // Multiples of eight, the tallest of the cheapest.  Measured on 18 lists at 14 heights each; against the other rule two fp32 0.6B-shaped blocks,
+  // tiles has, each a tile's rows and what setting up a tile costs beside them: 3, 9, 12 bf16 rows for ranks 1, 2 and more (R, the slice of A^T, the
+  // record; with the slice in shared memory as many again as there are ranks), half as many of 4-byte weights up to rank 8; where there are several
+  // rounds, CTAs have drifted apart by half a tile at the end.
+  // Multiples of eight, the tallest of the cheapest.  Measured on 35 lists at 10 to 14 heights each; against the other rule two fp32 0.6B-shaped blocks,
   // r = 8, 51 -> 45 us, eight 1024 x 1024 pairs 14.7 -> 9.7, a bf16 0.6B-shaped block, r = 3, 16.7 -> 10.3, twelve, r = 2, 125 -> 122.
   // Lists of more than 640 MB are bound by HBM whatever the rounds: the tallest tiles of which each CTA gets sixteen, for rank 1, whose set-up
   // is least, half as tall (sixty 2048 x 2048 fp32 layers, r = 4, at 64 rows 316 us, 336 by rounds; eight 8B-shaped blocks, r = 1, at 256 / 128 / 64
@@ -357,17 +358,19 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     std::vector<Strip> strips;             // 512 columns wide, by height
     int max_r = 0;
     int64_t bytes = 0;
-    bool slow = false;
+    bool slow = false, narrow = false;
     for (int i = 0; i < n; ++i) {
       if (!L[i].W || takes_tc_rmw(L[i])) continue;
       const int count = (L[i].d_in + kRmwTileCols - 1) / kRmwTileCols;
       max_r = std::max(max_r, L[i].r);
       bytes += (int64_t)L[i].d_out * L[i].d_in * ((L[i].w_dtype == AGZO_BF16 ? 2 : 4) + (L[i].W16 ? 2 : 0));
       slow = slow || !vector_rows(L[i]);
+      narrow = narrow || L[i].w_dtype == AGZO_BF16;
       auto same = std::find_if(strips.begin(), strips.end(), [&](const Strip& s) { return s.d_out == L[i].d_out; });
       if (same != strips.end()) same->n += count; else strips.push_back(Strip{L[i].d_out, count});
     }
     const long long ctas = (slow ? 4ll : max_r <= 8 ? 2ll : 1ll) * opts.sm_count;       // element by element: four on an SM
+    const int setup = (max_r == 1 ? 3 : std::min(12, 3 + 3 * max_r)) * (narrow || max_r > 8 ? 2 : 1);
     long long least = -1;
     auto tiles_of = [&](int rows) {
       long long tiles = 0;
@@ -381,7 +384,7 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     }
     for (int rows = slow ? 32 : kRmwMaxTileRows; rows >= 8 && !strips.empty(); rows -= 8) {
       const long long rounds = (tiles_of(rows) + ctas - 1) / ctas;
-      const long long cost = 2 * rounds * (rows + 12 + (max_r > 16 ? max_r : 0)) + (rounds > 1 ? rows : 0);
+      const long long cost = rounds * (2 * rows + setup + (max_r > 16 ? 2 * max_r : 0)) + (rounds > 1 ? rows : 0);     // in half rows
       if (least < 0 || cost < least) { least = cost; plan->tile_rows = rows; }
     }
   }
