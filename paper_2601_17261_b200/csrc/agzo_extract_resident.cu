@@ -16,9 +16,9 @@
 // Accumulation is fp32, over at most 128 tb tokens or 128 cb columns before the sums leave TMEM.
 //
 // What bounds it is the chain of synchronisations of a round: a cluster barrier 0.2 us, all CTAs of a unit at a counter 1.3, the
-// partial sums of Y from L2 1.2, the exchange of T 2.3, the Gram matrix and its exchange 2, the factor 0.5 to 2.4.  Against the
-// chain of launches, K = 3: without workspace 4096 x 2048, r = 16 158 -> 85 us; 8000 x 256 bf16, r = 8 83 -> 51; 1500 x 515 fp32,
-// r = 5 97 -> 51; 613 x 1024 bf16, three layers of r = 8 53 -> 51.
+// partial sums of Y from L2 1.2, the exchange of T 1.4 and the Gram matrix with its exchange 2 (both read from the peers between
+// barriers; sent, 0.3 to 0.9 less together), the factor 0.5 to 2.4.  Against the chain of launches, K = 3: without workspace 4096 x 2048, r = 16 158 -> 85 us;
+// 8000 x 256 bf16, r = 8 83 -> 51; 1500 x 515 fp32, r = 5 97 -> 51; 613 x 1024 bf16, three layers of r = 8 53 -> 48.
 #include "agzo_qr.cuh"
 #include "agzo_resident.cuh"
 
@@ -41,6 +41,7 @@ constexpr size_t kMaxSmem = 226 * 1024;
 
 struct ResShared {
   uint64_t mma;
+  uint64_t gram_in, t_in, t_full;      // what the peers send has come: shares of S, partial T, the T operand
   uint32_t tmem_base;
   int failed;
   DevStatus st;
@@ -387,17 +388,31 @@ __device__ __forceinline__ void issue_product(uint32_t go, uint32_t tmem, uint32
     if (PARTS != 3) d += (uint32_t)NB;
   }
 }
-// element i of a share (tiles of the upper triangle) -> S
+// Row and column in S of element i of a share (tiles of the upper triangle)
 template <int NT>
-__device__ __forceinline__ void place_share(double* A, double* own, int i, double v) {
+__device__ __forceinline__ void share_place(int i, int* row, int* col) {
   int t = i >> 6, bi = 0;
   while (t >= NT - bi) { t -= NT - bi; ++bi; }
-  const int row = 8 * bi + ((i & 63) >> 3), col = 8 * (bi + t) + (i & 7);
+  *row = 8 * bi + ((i & 63) >> 3);
+  *col = 8 * (bi + t) + (i & 7);
+}
+// element i of a share -> S
+template <int NT>
+__device__ __forceinline__ void place_share(double* A, double* own, int i, double v) {
+  int row, col;
+  share_place<NT>(i, &row, &col);
   A[row * QrCfg<NT>::ap + col] = v;
   if (row == col) own[row] = v;
 }
+// Bytes of Y, with which the pieces of T that the warps send take turns
+__host__ __device__ constexpr int push_front(int y_bytes, int parts) { return y_bytes > kWarps * parts * 256 ? y_bytes : kWarps * parts * 256; }
 
-template <int PLANES, int PARTS>
+// PUSH: what a cluster's CTAs exchange is sent (st.async, counted on the receiver's barrier) into buffers that nothing else uses at the
+// time: a way instead of a barrier of the cluster, a round trip, and for T another barrier.  512 x 256 fp32, r = 4 35.3 -> 32.2 us, the
+// layers of a block of width 1024 with 613 tokens 45.3 -> 42.7 on the mean.  No buffer is sent to before its owner is done with it: a
+// CTA sends its shares of a round only after the exchange of T of the last one (or a meeting), which its peers' sums of the shares before
+// precede, and partial T only after the exchange of the shares.  Otherwise it is read from the peers between barriers (resident_plan).
+template <int PLANES, int PARTS, bool PUSH>
 __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __grid_constant__ ResidentParams P) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ ResShared sh;
@@ -421,19 +436,33 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
   // after the product that reads Q, and Q after the one that reads T
   uint8_t* sQ = sX + PLANES * plane;
   uint8_t* sT = sQ;
-  double* sG = reinterpret_cast<double*>(sQ + max(cb, tb) * 2 * NB * 128);       // shares of S, one layer's after another's
-  uint8_t* sAM = reinterpret_cast<uint8_t*>(sG + nl * kShareElems);      // [layer] S / R and M
+  int n_share = 0;                                       // elements of the shares of all layers
+#pragma unroll 1
+  for (int l = 0; l < nl; ++l) n_share += U.layer[l].r <= 8 ? 64 : kShareElems;
+  const int n_gram = U.sub ? cs : cj, gram0 = U.sub ? 0 : row0;          // CTAs whose shares are added up, the first of them
+  const bool wide = U.sub && clusters > 1;               // the clusters' shares meet in global memory
+  // shares of S, one layer's after another's; those of all CTAs where they are sent
+  double* sG = reinterpret_cast<double*>(sQ + max(cb, tb) * 2 * NB * 128);
+  uint8_t* sAM = reinterpret_cast<uint8_t*>(sG + (PUSH ? n_gram * n_share : nl * kShareElems));      // [layer] S / R and M
   uint8_t* sU = sAM + nl * kAmBytes;
   float* sY = reinterpret_cast<float*>(sU);              // [rows][pitch] ...
   double* sPart = reinterpret_cast<double*>(sY + (size_t)U.rows * pitch);        // ... and [layer][warp] shares of S; or
   float* sEx = reinterpret_cast<float*>(sU);             // [rank group][128 tb tokens][8] partial T ...
   __nv_bfloat16* sStage = reinterpret_cast<__nv_bfloat16*>(sEx + (size_t)tb * kBlock * NP);    // ... and pieces to send
+  if (PUSH) {                          // partial T [CTA][token group of mine][8][NP] take turns with the warps' shares, pieces with Y
+    sStage = reinterpret_cast<__nv_bfloat16*>(sU) + warp * (PARTS * 128);
+    sPart = reinterpret_cast<double*>(sU + push_front(U.rows * pitch * 4, PARTS));
+    sEx = reinterpret_cast<float*>(sPart);
+  }
 
   const int y_chunks = PARTS == 3 ? 2 * tb : 1, t_chunks = PARTS == 3 ? 2 * cb : 1;
   uint32_t ncol = 32;
   while ((int)ncol < max(cb * y_chunks, tb * t_chunks) * NB) ncol <<= 1;
   if (tid == 0) {
     mbar_init(&sh.mma, 1);
+    mbar_init(&sh.gram_in, 1);
+    mbar_init(&sh.t_in, 1);
+    mbar_init(&sh.t_full, 1);
     sh.failed = 0;
     sh.st = DevStatus{};
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -450,6 +479,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
 #pragma unroll 1
   for (int k = tid; k < max(cb, tb) * 2 * NB * 8; k += kThreads) reinterpret_cast<uint4*>(sQ)[k] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
+  if (PUSH && cs > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // my barriers can be sent to
   if (!(PLANES == 1 && U.x_vec)) fill_omega<PARTS>(U, sT, t0, tb, P.seed);      // needs nothing from before the launch
   chain_wait();
   load_x<PLANES>(U, sX, plane, t0, col0, tb, cb);
@@ -468,7 +498,41 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
   const int q = warp & 3, half = warp >> 2, groups = NP / 8;
   const uint32_t lanes = (uint32_t)(q * 32) << 16;
   const int gram_split = U.gram_split;
-  uint32_t mma_par = 0;
+  uint32_t mma_par = 0, gram_par = 0, t_par = 0;
+  // element e of the shares of all layers: layer l, element x of its tiles
+  auto share_at = [&](int e, int* l, int* x) {
+    *l = 0;
+#pragma unroll 1
+    for (;; ++*l) {
+      const int n = U.layer[*l].r <= 8 ? 64 : kShareElems;
+      if (e < n) break;
+      e -= n;
+    }
+    *x = e;
+  };
+  // PUSH: this thread's two elements of the shares (at most 512 for 24 ranks in four layers), where they come from and go to
+  const bool has_pair = PUSH && 2 * tid < n_share;
+  const double* pair_src = sPart;
+  double *pair_dst = nullptr, *pair_diag = nullptr;
+  bool diag_second = false;
+  if (has_pair) {
+    int l, x, row, col;
+    share_at(2 * tid, &l, &x);
+    pair_src = sPart + l * gram_split * kShareElems + x;
+    double* A = reinterpret_cast<double*>(sAM + l * kAmBytes);
+    if (U.layer[l].r <= 8) { share_place<1>(x, &row, &col); pair_dst = A + row * QrCfg<1>::ap + col; }
+    else { share_place<2>(x, &row, &col); pair_dst = A + row * QrCfg<2>::ap + col; }
+    diag_second = row == col + 1;
+    if (row == col || diag_second) pair_diag = &sh.own[l][row];
+  }
+  auto place_pair = [&](double2 v) {
+    pair_dst[0] = v.x;
+    pair_dst[1] = v.y;
+    if (pair_diag) *pair_diag = diag_second ? v.y : v.x;
+  };
+  const int own = tb * (kBlock / 8) / cj;                // token groups whose T is added up here: j, j + cj, ... (cj divides 16)
+  __syncwarp();
+  if (PUSH && cs > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   const int width = U.sub ? (i < ni ? max(0, min(U.sub, ncols - i * U.sub)) : 0) : ncols;     // columns of Y that are added up here
   const int c_first = U.sub ? i * U.sub : 0;
   const bool direct = ni == 1;
@@ -595,67 +659,85 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
       }
     }
     __syncthreads();
-    // element e of the shares of all layers: layer l, element x of its tiles
-    int n_share = 0;
+    if constexpr (PUSH) {
+      if (has_pair) {
+        double2 v[kWarps], sum = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w)
+          v[w] = w < gram_split ? *reinterpret_cast<const double2*>(pair_src + w * kShareElems) : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) { sum.x += v[w].x; sum.y += v[w].y; }
+        if (n_gram == 1) {
+          place_pair(sum);
+        } else {
+          const uint32_t to = smem_u32(sG + (rank - gram0) * n_share + 2 * tid), bar = smem_u32(&sh.gram_in);
+          const uint32_t w[4] = {(uint32_t)__double2loint(sum.x), (uint32_t)__double2hiint(sum.x), (uint32_t)__double2loint(sum.y),
+                                 (uint32_t)__double2hiint(sum.y)};
 #pragma unroll 1
-    for (int l = 0; l < nl; ++l) n_share += U.layer[l].r <= 8 ? 64 : kShareElems;
-    auto share_at = [&](int e, int* l, int* x) {
-      *l = 0;
-#pragma unroll 1
-      for (;; ++*l) {
-        const int n = U.layer[*l].r <= 8 ? 64 : kShareElems;
-        if (e < n) break;
-        e -= n;
+          for (int c = 0; c < n_gram; ++c) st_async_u4(mapa_shared(to, (uint32_t)(gram0 + c)), w, mapa_shared(bar, (uint32_t)(gram0 + c)));
+        }
       }
-      *x = e;
-    };
+      if (n_gram > 1) {
+        if (tid == 0) mbar_expect_tx(&sh.gram_in, (uint32_t)(n_gram * n_share * 8));
+        if (!mbar_wait_cluster(&sh.gram_in, gram_par)) product_failed(&sh, clusters == 1 ? cs : 1);
+        gram_par ^= 1u;
+        if (has_pair) {
+          double2 v[8], sum = make_double2(0.0, 0.0);
+#pragma unroll
+          for (int c = 0; c < 8; ++c)
+            v[c] = c < n_gram ? *reinterpret_cast<const double2*>(sG + c * n_share + 2 * tid) : make_double2(0.0, 0.0);
+#pragma unroll
+          for (int c = 0; c < 8; ++c) { sum.x += v[c].x; sum.y += v[c].y; }
+          place_pair(sum);
+        }
+      }
+    } else {
 #pragma unroll 1
-    for (int e = tid; e < n_share; e += kThreads) {
-      int l, x;
-      share_at(e, &l, &x);
-      double v[kWarps], sum = 0.0;
-#pragma unroll
-      for (int w = 0; w < kWarps; ++w) v[w] = w < gram_split ? sPart[(l * gram_split + w) * kShareElems + x] : 0.0;
-#pragma unroll
-      for (int w = 0; w < kWarps; ++w) sum += v[w];
-      sG[e] = sum;
-    }
-    __syncwarp();
-    if (cs > 1) cluster_sync_all(); else __syncthreads();
-    {
-      auto place = [&](int e, double v) {
+      for (int e = tid; e < n_share; e += kThreads) {
         int l, x;
         share_at(e, &l, &x);
-        double* A = reinterpret_cast<double*>(sAM + l * kAmBytes);
-        if (U.layer[l].r <= 8) place_share<1>(A, sh.own[l], x, v); else place_share<2>(A, sh.own[l], x, v);
-      };
-      const int first = U.sub ? 0 : row0, n = U.sub ? cs : cj;
-      const bool wide = U.sub && clusters > 1;
-      if (!wide || rank == 0)
+        double v[kWarps], sum = 0.0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) v[w] = w < gram_split ? sPart[(l * gram_split + w) * kShareElems + x] : 0.0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) sum += v[w];
+        sG[e] = sum;
+      }
+      __syncwarp();
+      if (cs > 1) cluster_sync_all(); else __syncthreads();
+      {
+        auto place = [&](int e, double v) {
+          int l, x;
+          share_at(e, &l, &x);
+          double* A = reinterpret_cast<double*>(sAM + l * kAmBytes);
+          if (U.layer[l].r <= 8) place_share<1>(A, sh.own[l], x, v); else place_share<2>(A, sh.own[l], x, v);
+        };
+        if (!wide || rank == 0)
 #pragma unroll 1
-        for (int e = tid; e < n_share; e += kThreads) {
-          double v[8], sum = 0.0;
+          for (int e = tid; e < n_share; e += kThreads) {
+            double v[8], sum = 0.0;
 #pragma unroll
-          for (int c = 0; c < 8; ++c) v[c] = c < n ? ld_cluster_f64(mapa_shared(smem_u32(sG + e), (uint32_t)(first + c))) : 0.0;
+            for (int c = 0; c < 8; ++c) v[c] = c < n_gram ? ld_cluster_f64(mapa_shared(smem_u32(sG + e), (uint32_t)(gram0 + c))) : 0.0;
 #pragma unroll
-          for (int c = 0; c < 8; ++c) sum += v[c];
-          if (wide) U.gshare[(cluster - U.cluster0) * n_share + e] = sum; else place(e, sum);
-        }
-      if (wide) {
-        unit_barrier(meeting, clusters, cs, P, &sh);
-#pragma unroll 1
-        for (int e = tid; e < n_share; e += kThreads) {
-          double sum = 0.0;
-          constexpr int kP = 16;
-#pragma unroll 1
-          for (int s0 = 0; s0 < clusters; s0 += kP) {
-            double t[kP];
-#pragma unroll
-            for (int c = 0; c < kP; ++c) t[c] = s0 + c < clusters ? __ldcg(U.gshare + (s0 + c) * n_share + e) : 0.0;
-#pragma unroll
-            for (int c = 0; c < kP; ++c) sum += t[c];
+            for (int c = 0; c < 8; ++c) sum += v[c];
+            if (wide) U.gshare[(cluster - U.cluster0) * n_share + e] = sum; else place(e, sum);
           }
-          place(e, sum);
+        if (wide) {
+          unit_barrier(meeting, clusters, cs, P, &sh);
+#pragma unroll 1
+          for (int e = tid; e < n_share; e += kThreads) {
+            double sum = 0.0;
+            constexpr int kP = 16;
+#pragma unroll 1
+            for (int s0 = 0; s0 < clusters; s0 += kP) {
+              double t[kP];
+#pragma unroll
+              for (int c = 0; c < kP; ++c) t[c] = s0 + c < clusters ? __ldcg(U.gshare + (s0 + c) * n_share + e) : 0.0;
+#pragma unroll
+              for (int c = 0; c < kP; ++c) sum += t[c];
+            }
+            place(e, sum);
+          }
         }
       }
     }
@@ -731,13 +813,61 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
 #pragma unroll
             for (int p = 0; p < PARTS; ++p) *reinterpret_cast<__nv_bfloat16*>(box + swz(p * NP + 8 * g + k, (t & 63) >> 3)) = part[p];
           }
+        } else if (PUSH) {                                    // to the CTA that adds up this token's group
+          const int c = (t >> 3) & (cj - 1), o = (t >> 3) / cj;
+          const uint32_t to = mapa_shared(smem_u32(sEx + ((size_t)((j * own + o) * 8 + (t & 7)) * NP + 8 * g)), (uint32_t)(row0 + c));
+          const uint32_t bar = mapa_shared(smem_u32(&sh.t_in), (uint32_t)(row0 + c));
+          st_async_f4(to, make_float4(v[0], v[1], v[2], v[3]), bar);
+          st_async_f4(to + 16u, make_float4(v[4], v[5], v[6], v[7]), bar);
         } else {
           float4* out = reinterpret_cast<float4*>(sEx + ((size_t)g * tb * kBlock + t) * 8);
           out[0] = make_float4(v[0], v[1], v[2], v[3]);
           out[1] = make_float4(v[4], v[5], v[6], v[7]);
         }
       }
-    if (cj > 1) {
+    if (PUSH && cj > 1) {
+      if (tid == 0) {
+        mbar_expect_tx(&sh.t_in, (uint32_t)(tb * kBlock * NP * 4));
+        mbar_expect_tx(&sh.t_full, (uint32_t)(tb * (kBlock / 8) * PARTS * NP * 16));
+      }
+      if (!mbar_wait_cluster(&sh.t_in, t_par)) product_failed(&sh, clusters == 1 ? cs : 1);
+      // lane = (one of two pieces, token of the group, half of a rank group): four ranks of a token; a warp sends what it has split
+#pragma unroll 1
+      for (int e = tid; e < own * 16 * groups; e += kThreads) {
+        const int x = (e >> 1) & 7, kh = e & 1, og = e >> 4, o = og / groups, g = og - o * groups;
+        const float* src = sEx + (size_t)(o * 8 + x) * NP + 8 * g + 4 * kh;
+        float4 z[8], sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          z[c] = c < cj ? *reinterpret_cast<const float4*>(src + (size_t)c * own * 8 * NP) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) { sum.x += z[c].x; sum.y += z[c].y; sum.z += z[c].z; sum.w += z[c].w; }
+        const float v[4] = {sum.x, sum.y, sum.z, sum.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          __nv_bfloat16 part[PARTS];
+          split1<PARTS>(v[k], part);
+#pragma unroll
+          for (int p = 0; p < PARTS; ++p) sStage[(((lane >> 4) * PARTS + p) * 8 + 4 * kh + k) * 8 + x] = part[p];
+        }
+        __syncwarp();
+        // 16 PARTS pieces of eight tokens of an operand row, to every CTA of the row
+#pragma unroll 1
+        for (int n = lane; n < 16 * PARTS; n += 32) {
+          const int h = n / (8 * PARTS), p = (n >> 3) - h * PARTS, og_n = ((e - lane) >> 4) + h, o_n = og_n / groups;
+          const int row = p * NP + 8 * (og_n - o_n * groups) + (n & 7), tg = j + o_n * cj;
+          const uint32_t to = at + (uint32_t)((tg >> 3) * NB * 128) + swz(row, tg & 7), bar = smem_u32(&sh.t_full);
+          const uint4 u = *reinterpret_cast<const uint4*>(sStage + n * 8);
+          const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll 1
+          for (int c = 0; c < cj; ++c)
+            st_async_u4(mapa_shared(to, (uint32_t)(row0 + c)), w, mapa_shared(bar, (uint32_t)(row0 + c)));
+        }
+        __syncwarp();
+      }
+      if (!mbar_wait_cluster(&sh.t_full, t_par)) product_failed(&sh, clusters == 1 ? cs : 1);
+      t_par ^= 1u;
+    } else if (cj > 1) {
       __syncwarp();
       cluster_sync_all();                                    // every CTA's partial T is in its shared memory
       const int n_groups = tb * (kBlock / 8), mine = (n_groups - j + cj - 1) / cj;      // token groups j, j + cj, ...
@@ -780,9 +910,15 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
   }
 
   tc_fence_before();
-  __syncthreads();
-  if (sh.failed) zero_strips(U, i, col0);                    // a wait has run out and the sums are not whole
-  if (cs > 1) cluster_sync_all();                            // nobody leaves while a peer may read its share
+  __syncwarp();
+  if (cs > 1) cluster_sync_all(); else __syncthreads();      // nobody leaves while a peer may read its share
+  if (sh.failed) {                                           // a wait has run out and the sums are not whole
+    zero_strips(U, i, col0);
+    if (PUSH) {                                              // what the peers have sent may be on its way yet
+      const unsigned long long t_end = global_ns() + 100000;
+      while (global_ns() < t_end) {}
+    }
+  }
   if (tid == 0) {
     if (sh.failed && P.status) { atomicExch(&P.status->timeout, 1); atomicExch(&P.status->where, 5); }
     if (i == 0 && j == 0) {
@@ -794,8 +930,9 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
 }
 
 using ResKernel = void (*)(const ResidentParams);
-ResKernel res_kernel(int planes, int parts) {
-  return planes == 3 ? resident_extract_kernel<3, 3> : parts == 3 ? resident_extract_kernel<1, 3> : resident_extract_kernel<1, 2>;
+ResKernel res_kernel(int planes, int parts, bool push) {
+  if (push) return planes == 3 ? resident_extract_kernel<3, 3, true> : parts == 3 ? resident_extract_kernel<1, 3, true> : resident_extract_kernel<1, 2, true>;
+  return planes == 3 ? resident_extract_kernel<3, 3, false> : parts == 3 ? resident_extract_kernel<1, 3, false> : resident_extract_kernel<1, 2, false>;
 }
 
 // Warps of a layer's Gram products: all of them between the layers, fewer where their sums would not fit beside X
@@ -808,6 +945,16 @@ size_t res_smem(const ResidentUnit& u, int planes, int parts) {
   const size_t own = (size_t)(u.tb * (kBlock / 8) + u.cj - 1) / u.cj;
   const size_t ex = u.cj == 1 ? 0 : (size_t)u.tb * kBlock * u.NP * 4 + own * parts * u.NP * 16;
   return x + ops + (size_t)u.n_layers * (kShareElems * 8 + kAmBytes) + std::max(y, ex) + 1024;
+}
+
+// ... of one that is sent what its cluster exchanges (sub is known by then)
+size_t push_smem(const ResidentUnit& u, int planes, int parts, int cs) {
+  const size_t x = (size_t)planes * u.tb * u.cb * 2 * kSlotBytes, ops = (size_t)std::max(u.cb, u.tb) * 2 * u.NB * 128;
+  size_t share = 0;
+  for (int l = 0; l < u.n_layers; ++l) share += u.layer[l].r <= 8 ? 64 : kShareElems;
+  const size_t front = push_front(u.rows * qr_pitch(u.cb * kBlock) * 4, parts);
+  const size_t part = (size_t)u.n_layers * gram_split(u) * kShareElems * 8, ex = u.cj == 1 ? 0 : (size_t)u.tb * kBlock * u.NP * 4;
+  return x + ops + (u.sub ? cs : u.cj) * share * 8 + (size_t)u.n_layers * kAmBytes + front + std::max(part, ex) + 1024;
 }
 
 // One way to lay a unit out over clusters of cs CTAs, and what a round of it is estimated to take (us)
@@ -891,8 +1038,8 @@ bool same_x(const agzo_layer& a, const agzo_layer& b) {
 }  // namespace
 
 cudaError_t resident_init(int sm_count, ResidentCaps* caps) {
-  for (int k = 0; k < 3; ++k) {
-    const void* f = (const void*)res_kernel(k == 2 ? 3 : 1, k == 0 ? 2 : 3);
+  for (int k = 0; k < 6; ++k) {
+    const void* f = (const void*)res_kernel(k % 3 == 2 ? 3 : 1, k % 3 == 0 ? 2 : 3, k >= 3);
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
     if (e != cudaSuccess) return e;
   }
@@ -909,7 +1056,7 @@ cudaError_t resident_init(int sm_count, ResidentCaps* caps) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, (const void*)res_kernel(3, 3), &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+    if (cudaOccupancyMaxActiveClusters(&n, (const void*)res_kernel(3, 3, true), &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
     caps->clusters[cs] = n;
   }
   caps->sm_count = sm_count;
@@ -959,6 +1106,9 @@ bool resident_plan(const ResidentCaps& caps, const agzo_layer* L, int n, bool sh
   p.cs = cs;
   out->planes = planes; out->parts = parts;
   out->n_clusters = 0; out->grid_wide = false; out->smem = 0;
+  size_t sent = 0;
+  int most_sent = 0, most_clusters = 0;
+  bool wide = false;
   for (size_t k = 0; k < units.size(); ++k) {
     ResidentUnit& u = units[k];
     const Shape& s = best[k];
@@ -967,8 +1117,19 @@ bool resident_plan(const ResidentCaps& caps, const agzo_layer* L, int n, bool sh
     out->n_clusters += s.clusters;
     out->grid_wide = out->grid_wide || s.clusters > 1;
     out->smem = std::max(out->smem, res_smem(u, planes, parts));
+    sent = std::max(sent, push_smem(u, planes, parts, cs));
+    wide = wide || (u.sub && u.clusters > 1);
+    most_clusters = std::max(most_clusters, u.clusters);
+    if (u.cj > 1) most_sent = std::max(most_sent, u.tb * u.NP * (16 * parts + 32));
     p.unit[k] = u;
   }
+  // Kernel times of 196 lists, read from the peers -> sent.  Units of one cluster: all faster or even, by 6 % on the mean and up to 23 %
+  // (613 x 280 and smaller; 3 x 128 tokens a CTA 40.1 -> 32.6 us).  Of several, which also meet at a counter: 3 % up to five clusters; from
+  // six on 3 % while a CTA gets up to 1024 messages of 16 bytes for T (two parts: ranks up to 8 on 256 tokens, 16 on 128), beyond those
+  // the receiver's counting of them takes what the barriers did (2560: 88.5 -> 91.1 us, 3840: 77.7 -> 82.3).  Where the clusters' shares
+  // meet in global memory, the round trip is hidden behind that meeting already: 4096 x 2048, r = 16 84.0 -> 87.5.
+  out->push = cs > 1 && !wide && sent <= kMaxSmem && (most_clusters <= 5 || most_sent <= 1024);
+  if (out->push) out->smem = sent;
   resident_bind(out, nullptr);
   return true;
 }
@@ -1092,7 +1253,7 @@ cudaError_t launch_resident(const ResidentLaunch& plan, cudaStream_t s) {
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, res_kernel(plan.planes, plan.parts), plan.p);
+  return cudaLaunchKernelEx(&cfg, res_kernel(plan.planes, plan.parts, plan.push), plan.p);
 }
 
 bool resident_refused(cudaError_t e) {

@@ -69,6 +69,7 @@ struct ResidentLaunch {
   ResidentParams p;
   int planes, parts;                    // bf16 planes of X (1: bf16, 3: fp32), parts of the operands Q and T
   int n_clusters;
+  bool push;                            // the CTAs of a cluster send one another what they exchange
   bool grid_wide;                       // some unit has several clusters, which wait for one another
   size_t smem;
   size_t scratch;                       // bytes behind ypart, y and gshare

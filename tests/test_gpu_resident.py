@@ -98,6 +98,18 @@ def test_columns_in_pieces(units, pieces):
     check(units, 2, pieces=pieces)
 
 
+# What the CTAs of a cluster exchange, sent or read: clusters of two, four and eight side by side, one to three blocks of tokens, shares of
+# all 512 elements, units without an exchange beside others, and both sides of where it is sent (six clusters; 1024 pieces of T)
+@pytest.mark.parametrize("units", [
+    [(128, 256, (4,), True, None)], [(320, 280, (8,), True, None), (1974, 128, (8,), True, None)], [(300, 264, (9, 9, 1, 1), True, None)],
+    [(384, 512, (16,), False, None)], [(44, 136, (6,), True, None)], [(250, 1000, (9, 9, 1, 1), False, None)],
+    [(613, 1024, (8, 8, 8), True, None), (613, 2048, (8,), True, None)], [(640, 1024, (16,), True, None)], [(1000, 1024, (16,), True, None)],
+    [(2500, 1024, (8,), True, None)], [(2500, 1024, (16,), True, None)], [(2385, 1125, (4, 7), True, None), (127, 872, (7, 4), True, None)]])
+@pytest.mark.parametrize("K", [1, 3])
+def test_exchange_within_a_cluster(units, K):
+    check(units, K)
+
+
 def test_a_refused_launch_leaves_the_call_to_the_other_kernels():
     X = to_dev(WL.planted_activations(300, 256, 16, seed=1, bf16=True), True)[0]
     V = torch.zeros(4, 256, device=DEV)
