@@ -1,6 +1,6 @@
 // The two products of Algorithm 1 (SubspaceExtract) with X on CUDA cores in fp32, for any dtype,
 // pitch and size; the tensor-core path (agzo_extract_tc.cu) replaces them when the layer's shape
-// allows it.  qr(Y) is in agzo_panel_qr.cu.
+// allows it, and the products in fp32 precision (agzo_extract_split.cu) where those are estimated the faster ones.  qr(Y) is in agzo_panel_qr.cu.
 //
 // Ypart[s] = X_s^T T_s per token slab s (summed in slab order later, so the result does not
 // depend on scheduling), and T = X Q.

@@ -7,7 +7,7 @@
 // and the tile's slice of A^T lives in registers, so neither R nor Delta ever reaches DRAM.
 // Measured (one pass over six 8B-shaped blocks, bf16, 4.6 GB, copy rate 6541 GB/s): r = 1 6289 GB/s (6182 with loads
 // issued a sub-block at a time and after R), r = 4 6326 (5614), r = 8 5625 (4740); 28 0.6B-shaped blocks r = 4 6246 (5317), fp32
-// r = 8 6194 (4448); eight 1024 x 1024 master/compute pairs, r = 8: 37 -> 13 us; one fp32 256 x 256 layer 16 -> 4 us.
+// r = 8 6194 (4448); eight 1024 x 1024 master/compute pairs, r = 8: 37 -> 9.7 us; one fp32 256 x 256 layer 16 -> 3 us.
 #include "agzo_common.cuh"
 
 namespace agzo {
