@@ -7,7 +7,8 @@
 //   load    Y = sum of the partial sums that the last product left, in order, into shared memory
 //   gram    the slice's share of S on the FP64 tensor cores (mma.sync m8n8k4: true double multiply-adds; tcgen05
 //           has no FP64 form), the warps splitting the columns, partial sums added in a fixed order
-//   -- cluster barrier: every CTA adds the C shares, read through distributed shared memory, in rank order --
+//   -- every CTA sends its share to all (st.async, counted on the receiver's barrier) and adds the C shares in rank order; above rank 16,
+//      or where shared memory has no room for them, they are read from the peers after a cluster barrier --
 //   factor  Cholesky and M = R^-1, by every CTA for itself (what it costs is a dependent chain, so doing it C
 //           times takes no longer than doing it once and saves a second exchange)
 //   apply   Q = Y M on the FP64 tensor cores, from the slice that is still in shared memory, and out: V (fp32) after
@@ -68,7 +69,7 @@ __device__ __forceinline__ void qr_store(const DevLayer& L, const float* sY, int
 
 // kResident: the CTA's whole slice stays in shared memory from load to apply; otherwise it is staged 128 columns at
 // a time and read a second time (from L.Y, through L2) for the apply.
-template <int NT, bool kResident, int kLive = kBlk>
+template <int NT, bool kResident, int kLive, bool kSend>
 __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer* __restrict__ layers, int l0, int C, int pitch,
                                                                  int y_reduced, int after_fused, int last, unsigned* published,
                                                                  DevStatus* status) {
@@ -81,7 +82,13 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
   for (int i = threadIdx.x; i < (int)(sizeof(DevLayer) / 8); i += kQrThreads)
     reinterpret_cast<unsigned long long*>(record)[i] =
         __ldcg(reinterpret_cast<const unsigned long long*>(layers + l0 + (int)blockIdx.x / C) + i);
+  __shared__ uint64_t shares_in;
+  if (kSend && threadIdx.x == 0) {
+    mbar_init(&shares_in, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
   __syncthreads();
+  if (kSend) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");        // my barrier can be sent to
   const DevLayer& L = *reinterpret_cast<const DevLayer*>(record);
   const int rank = (int)cluster_ctarank();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -89,6 +96,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
   double* sU = reinterpret_cast<double*>(qr_smem);                       // warps' partial sums, then S / R and M
   double* sG = reinterpret_cast<double*>(qr_smem + Cfg::u_bytes);        // this CTA's share of S, [tile][8][8]
   float* sY = reinterpret_cast<float*>(qr_smem + Cfg::fixed);            // [r8][pitch]
+  double* sIn = reinterpret_cast<double*>(qr_smem + Cfg::fixed + (size_t)Cfg::r8 * pitch * sizeof(float));      // kSend: the C shares
   double* A = sU;
   double* M = sU + Cfg::r8 * Cfg::ap;
   __shared__ double own[AGZO_MAX_RANK];
@@ -121,28 +129,65 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
   for (int t = 0; t < Cfg::tiles; ++t)
     *reinterpret_cast<double2*>(sU + (warp * Cfg::tiles + t) * 64 + el) = make_double2(acc[t][0], acc[t][1]);
   __syncthreads();
-  for (int i = tid; i < Cfg::tiles * 64; i += kQrThreads) {
-    double s = 0.0;
-#pragma unroll
-    for (int w = 0; w < kQrWarps; ++w) s += sU[w * Cfg::tiles * 64 + i];
-    sG[i] = s;
-  }
-  __syncwarp();
-  cluster_sync_all();                       // every CTA's share is in its shared memory
-  for (int i = tid; i < Cfg::tiles * 64; i += kQrThreads) {
-    double v[kQrMaxCluster], sum = 0.0;
-#pragma unroll
-    for (int c = 0; c < kQrMaxCluster; ++c) v[c] = c < C ? ld_cluster_f64(mapa_shared(smem_u32(sG + i), (uint32_t)c)) : 0.0;
-#pragma unroll
-    for (int c = 0; c < kQrMaxCluster; ++c) sum += v[c];
+  auto place = [&](int i, double v) {
     int t = i >> 6, bi = 0;
     while (t >= NT - bi) { t -= NT - bi; ++bi; }
     const int row = 8 * bi + ((i & 63) >> 3), col = 8 * (bi + t) + (i & 7);
-    A[row * Cfg::ap + col] = sum;
-    if (row == col) own[row] = sum;
+    A[row * Cfg::ap + col] = v;
+    if (row == col) own[row] = v;
+  };
+  if constexpr (kSend) {
+    constexpr int kPairs = Cfg::tiles * 32;
+    static_assert(kPairs <= kQrThreads, "two elements a thread");
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (tid == 0) mbar_expect_tx(&shares_in, (uint32_t)(C * Cfg::tiles * 64 * 8));
+    if (tid < kPairs) {
+      double2 sum = make_double2(0.0, 0.0);
+#pragma unroll
+      for (int w = 0; w < kQrWarps; ++w) {
+        const double2 v = *reinterpret_cast<const double2*>(sU + w * Cfg::tiles * 64 + 2 * tid);
+        sum.x += v.x;
+        sum.y += v.y;
+      }
+      const uint32_t to = smem_u32(sIn + rank * Cfg::tiles * 64 + 2 * tid), bar = smem_u32(&shares_in);
+      const uint32_t w[4] = {(uint32_t)__double2loint(sum.x), (uint32_t)__double2hiint(sum.x), (uint32_t)__double2loint(sum.y),
+                             (uint32_t)__double2hiint(sum.y)};
+#pragma unroll 4
+      for (int c = 0; c < C; ++c) st_async_u4(mapa_shared(to, (uint32_t)c), w, mapa_shared(bar, (uint32_t)c));
+    }
+    __syncthreads();                        // the warps' sums are read: S takes their place
+    if (!mbar_wait_cluster(&shares_in, 0) && lane == 0 && status) { atomicExch(&status->timeout, 1); atomicExch(&status->where, 8); }
+    if (tid < kPairs) {
+      double2 v[kQrMaxCluster], sum = make_double2(0.0, 0.0);
+#pragma unroll
+      for (int c = 0; c < kQrMaxCluster; ++c)
+        v[c] = c < C ? *reinterpret_cast<const double2*>(sIn + c * Cfg::tiles * 64 + 2 * tid) : make_double2(0.0, 0.0);
+#pragma unroll
+      for (int c = 0; c < kQrMaxCluster; ++c) { sum.x += v[c].x; sum.y += v[c].y; }
+      place(2 * tid, sum.x);
+      place(2 * tid + 1, sum.y);
+    }
+  } else {
+    for (int i = tid; i < Cfg::tiles * 64; i += kQrThreads) {
+      double s = 0.0;
+#pragma unroll
+      for (int w = 0; w < kQrWarps; ++w) s += sU[w * Cfg::tiles * 64 + i];
+      sG[i] = s;
+    }
+    __syncwarp();
+    cluster_sync_all();                       // every CTA's share is in its shared memory
+    for (int i = tid; i < Cfg::tiles * 64; i += kQrThreads) {
+      double v[kQrMaxCluster], sum = 0.0;
+#pragma unroll
+      for (int c = 0; c < kQrMaxCluster; ++c) v[c] = c < C ? ld_cluster_f64(mapa_shared(smem_u32(sG + i), (uint32_t)c)) : 0.0;
+#pragma unroll
+      for (int c = 0; c < kQrMaxCluster; ++c) sum += v[c];
+      place(i, sum);
+    }
   }
   __syncthreads();
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // done with the peers' shares
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // done with the peers' shares, or they have come
   qr_factor<NT, kLive>(A, M, own, r, status, rank == 0);
 
   const bool to_v = last || !L.Qb, to_qb = !last && L.Qb;
@@ -336,9 +381,17 @@ cudaError_t launch_qr(const ExtractWave& w, bool last, DevStatus* d_status, cuda
   if (C > w.max_gchunks) C = w.max_gchunks;
   const bool resident = qr_smem<NT>(slice_of(C)) <= kQrResidentSmem;
   const int slice = resident ? slice_of(C) : kQrChunk;
-  return launch_chained(resident ? panel_qr_kernel<NT, true, kLive> : panel_qr_kernel<NT, false, kLive>, dim3((unsigned)(C * nl)),
-                        kQrThreads, qr_smem<NT>(slice), C, s, w.d_layers, w.l0, C, qr_pitch(slice), w.y_reduced, w.after_fused, last ? 1 : 0,
-                        published_at(w, last, d_status), d_status);
+  size_t smem = qr_smem<NT>(slice);
+  auto* kernel = resident ? panel_qr_kernel<NT, true, kLive, false> : panel_qr_kernel<NT, false, kLive, false>;
+  // Sending (up to rank 16, whose C shares are 24 KB at most) leaves out a barrier's wait and a round trip: 120 lists 0.5 % on the mean, eight
+  // 1024 x 1024 layers, r = 8 141.9 -> 139.5 us, two 8B-shaped blocks from hooks 2806 -> 2789.
+  if constexpr (NT <= 2)
+    if (!w.qr_reads && smem + C * QrCfg<NT>::g_bytes <= kQrResidentSmem) {
+      smem += C * QrCfg<NT>::g_bytes;
+      kernel = resident ? panel_qr_kernel<NT, true, kLive, true> : panel_qr_kernel<NT, false, kLive, true>;
+    }
+  return launch_chained(kernel, dim3((unsigned)(C * nl)), kQrThreads, smem, C, s, w.d_layers, w.l0, C, qr_pitch(slice), w.y_reduced,
+                        w.after_fused, last ? 1 : 0, published_at(w, last, d_status), d_status);
 }
 
 constexpr size_t kGramSmem = (size_t)64 * (kQrChunk + 12) * sizeof(float);
@@ -381,17 +434,17 @@ bool allow_wide(K* kernel) {
 }  // namespace
 
 cudaError_t panel_qr_init(bool* wide) {
-  cudaError_t e = allow_smem(panel_qr_kernel<1, true, 4>, kQrResidentSmem);
-  if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<1, false, 4>, kQrResidentSmem);
-  if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<1, true>, kQrResidentSmem);
-  if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<1, false>, kQrResidentSmem);
-  if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<2, true>, kQrResidentSmem);
-  if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<2, false>, kQrResidentSmem);
-  if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<4, true>, kQrResidentSmem);
-  if (e == cudaSuccess) e = allow_smem(panel_qr_kernel<4, false>, kQrResidentSmem);
-  *wide = allow_wide(panel_qr_kernel<1, true, 4>) && allow_wide(panel_qr_kernel<1, false, 4>) && allow_wide(panel_qr_kernel<1, true>) &&
-          allow_wide(panel_qr_kernel<1, false>) && allow_wide(panel_qr_kernel<2, true>) &&
-          allow_wide(panel_qr_kernel<2, false>) && allow_wide(panel_qr_kernel<4, true>) && allow_wide(panel_qr_kernel<4, false>);
+  cudaError_t e = cudaSuccess;
+  *wide = true;
+  auto allow = [&](auto* kernel) {
+    if (e == cudaSuccess) e = allow_smem(kernel, kQrResidentSmem);
+    *wide = *wide && allow_wide(kernel);
+  };
+  allow(panel_qr_kernel<1, true, 4, false>); allow(panel_qr_kernel<1, false, 4, false>); allow(panel_qr_kernel<1, true, kBlk, false>);
+  allow(panel_qr_kernel<1, false, kBlk, false>); allow(panel_qr_kernel<2, true, kBlk, false>); allow(panel_qr_kernel<2, false, kBlk, false>);
+  allow(panel_qr_kernel<4, true, kBlk, false>); allow(panel_qr_kernel<4, false, kBlk, false>);
+  allow(panel_qr_kernel<1, true, 4, true>); allow(panel_qr_kernel<1, false, 4, true>); allow(panel_qr_kernel<1, true, kBlk, true>);
+  allow(panel_qr_kernel<1, false, kBlk, true>); allow(panel_qr_kernel<2, true, kBlk, true>); allow(panel_qr_kernel<2, false, kBlk, true>);
   cudaGetLastError();
   if (e == cudaSuccess) e = allow_smem(panel_factor_kernel, kFactorSmem);
   if (e == cudaSuccess) e = allow_smem(panel_apply_kernel, kApplySmem);

@@ -43,6 +43,14 @@ def test_slices_in_and_out_of_shared_memory(r, dims):
     check(256, dims, r, 1, bf16=True)
 
 
+# Shares of S sent or read: sixteen CTAs with the widest slices that leave room for the shares, and the next ones; two to eight CTAs
+# (8, 9: layers per launch; 200, 300: chunks of columns), one of them without columns of its own
+@pytest.mark.parametrize("r,dims,n_layers", [(16, [18432], 1), (16, [20480], 1), (8, [2176], 8), (8, [2176], 9), (4, [300], 1), (12, [200], 9),
+                                             (16, [1160, 140], 12)])
+def test_shares_sent_and_read(r, dims, n_layers):
+    check(300, dims, r, 2, True, n_layers)
+
+
 @pytest.mark.parametrize("n_layers", [40, 41, 80, 81])
 def test_layers_per_launch(n_layers):
     check(256, [1032, 128, 3080], 12, 1, bf16=True, n_layers=n_layers)
