@@ -216,6 +216,21 @@ def test_static_entry_reports_a_wait_that_ran_out():
         assert flag.item() == 0 and torch.equal(V, want)
 
 
+def test_a_wait_that_ran_out_where_a_cluster_sends():
+    # 96 blocks, twelve clusters of eight that send one another their sums; the rest as above
+    X = to_dev(WL.planted_activations(1500, 1024, 16, seed=3, bf16=True), True)[0]
+    want, V = torch.zeros(8, 1024, device=DEV), torch.zeros(8, 1024, device=DEV)
+    flag = torch.full((1,), -1, dtype=torch.int32, device=DEV)
+    B.agzo_debug_extract_static(X, want, 8, 3, 5, 1, B.STATIC_RESIDENT, flag)
+    assert flag.item() == 0 and want.any()
+    for _ in range(3):
+        V.fill_(7.0)
+        B.agzo_debug_extract_static(X, V, 8, 3, 5, 1, B.STATIC_RESIDENT, flag, wait_ns=0)
+        assert flag.item() == 2 and not V.any()
+        B.agzo_debug_extract_static(X, V, 8, 3, 5, 1, B.STATIC_RESIDENT, flag)
+        assert flag.item() == 0 and torch.equal(V, want)
+
+
 @pytest.mark.parametrize("d_in", [128, 130])
 def test_tiny_fp32_inputs_keep_their_bits(d_in):
     # scaled by a power of two that leaves every element a normal fp32 number: without a power step nothing underflows, so V is that of
