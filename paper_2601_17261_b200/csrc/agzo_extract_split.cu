@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(Cfg<NP, PLANES, XQ>::threads, 1) split_product
     }
     uint32_t s = (uint32_t)(group % kStages), par = 1;     // first round of a stage: free
     while (at.it >= 0) {
-      if (!mbar_wait(&sh.empty[s], par)) { sh.failed = 1; break; }
+      if (!mbar_wait_warp(&sh.empty[s], par)) { sh.failed = 1; break; }
       const uint32_t dst = tiles + s * (uint32_t)kStageBytes;
       const bool moved = at.advance(U, kLoadGroups);
       const bool more = at.it >= 0;
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(Cfg<NP, PLANES, XQ>::threads, 1) split_product
     if (e == 0 && short_launch()) chain_next();
     if (at.it >= 0) { open(); fetch(); }
     while (at.it >= 0) {
-      if (!mbar_wait(&sh.empty[s], par)) { sh.failed = 1; break; }
+      if (!mbar_wait_warp(&sh.empty[s], par)) { sh.failed = 1; break; }
       const uint32_t dst = s * (uint32_t)kStageBytes;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(Cfg<NP, PLANES, XQ>::threads, 1) split_product
 #pragma unroll
         for (int k = 0; k < H / 2; ++k) sum[p][k] = 0;
       for (int k = 0; k < n; ++k) {
-        if (!mbar_wait(&sh.acc_full[b], par)) { ok = false; break; }
+        if (!mbar_wait_warp(&sh.acc_full[b], par)) { ok = false; break; }
         tc_fence_after();
         // two parts at a time, for want of registers
         uint32_t z[2][H];
@@ -472,14 +472,14 @@ __global__ void __launch_bounds__(Cfg<NP, PLANES, XQ>::threads, 1) split_product
         const uint32_t rank = cluster_ctarank(), mine = (uint32_t)((warp - kLoadWarps) * 32 + lane) * 16u, piece = kEpiWarps * 32 * 16;
         const uint32_t peers = tiles + (uint32_t)(kStages * kStageBytes);
         if (rank != 0) {
-          if (i > 0 && !mbar_wait_cluster(&sh.sums_out, (uint32_t)(i - 1) & 1u)) { ok = false; break; }
+          if (i > 0 && !mbar_wait_cluster_warp(&sh.sums_out, (uint32_t)(i - 1) & 1u)) { ok = false; break; }
           const uint32_t dst = mapa_shared(peers + (rank - 1u) * C::peer_bytes + mine, 0), bar = mapa_shared(smem_u32(&sh.sums_in), 0);
 #pragma unroll
           for (int c = 0; c < H; c += 4) st_async_f4(dst + (uint32_t)(c / 4) * piece, make_float4(y[c], y[c + 1], y[c + 2], y[c + 3]), bar);
           continue;
         }
         if (warp == kLoadWarps && lane == 0) mbar_expect_tx(&sh.sums_in, (uint32_t)(U.split - 1) * C::peer_bytes);
-        if (!mbar_wait_cluster(&sh.sums_in, (uint32_t)i & 1u)) { ok = false; break; }
+        if (!mbar_wait_cluster_warp(&sh.sums_in, (uint32_t)i & 1u)) { ok = false; break; }
         for (int p = 0; p < U.split - 1; ++p)
 #pragma unroll
           for (int c = 0; c < H; c += 4) {
