@@ -38,7 +38,8 @@
  *   - Every function returns an agzo_status; nothing throws, traps or aborts.  Argument
  *     errors are detected on the host before anything is launched.  Conditions that only
  *     the device can see (a rank-deficient panel, a wait that ran out) are written to a
- *     status word in the workspace and reported by agzo_poll.
+ *     status word in the workspace and reported by agzo_poll.  An extraction in which a wait ran
+ *     out leaves V = 0 in the layers it concerns, with which a pass changes nothing.
  *   - Random streams: Philox4x32-10 with key = the 64-bit step seed and counter
  *     (b_lo, b_hi, layer_id, tag); b = e >> 2 where e is the row-major index of the element
  *     inside the matrix being drawn, which takes output word e & 3 of that block.

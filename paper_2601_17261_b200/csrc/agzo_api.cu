@@ -1268,7 +1268,7 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
       const bool split = !all_tc && P.split && split_takes(w, P.dev.data(), K);
       auto omega = [&]() -> cudaError_t {
         Timed t(ctx, AGZO_KC_OMEGA, ws);
-        return all_tc ? tc_fill_omega(ctx->tc, w, P.dev.data(), seed, ws) : launch_fill_omega(w, seed, ws);
+        return all_tc ? tc_fill_omega(ctx->tc, w, P.dev.data(), seed, dst, ws) : launch_fill_omega(w, seed, dst, ws);
       };
       // layers served by the fused power-step kernel, by cluster size; the rest take T = X Q, Y = X^T T
       unsigned fz_classes = 0;

@@ -11,8 +11,9 @@ namespace agzo {
 // ------------------------------------------------------------------ Omega -> T
 // Local token t is row row0 + t of the test matrix of the whole batch: element e of the stream is
 // (row0 + t) * r + k, so the Philox blocks that cover the local rows are walked, whatever row0 is.
-__global__ void fill_omega_kernel(const DevLayer* layers, int l0, uint64_t seed, long long row0) {
+__global__ void fill_omega_kernel(const DevLayer* layers, int l0, uint64_t seed, long long row0, DevStatus* status, int region) {
   chain_wait();
+  if (blockIdx.x + blockIdx.y == 0 && threadIdx.x == 0) wave_begins(status, region);
   if (short_launch()) chain_next();
   const DevLayer& L = layers[l0 + blockIdx.y];
   const long long n = (long long)L.m * L.r;
@@ -30,12 +31,12 @@ __global__ void fill_omega_kernel(const DevLayer* layers, int l0, uint64_t seed,
   }
 }
 
-cudaError_t launch_fill_omega(const ExtractWave& w, uint64_t seed, cudaStream_t s) {
+cudaError_t launch_fill_omega(const ExtractWave& w, uint64_t seed, DevStatus* d_status, cudaStream_t s) {
   const long long nb = (((long long)w.max_m * w.max_r + 3) >> 2) + 1;
   int gx = (int)((nb + 255) / 256);
   if (gx > 512) gx = 512;
   if (gx < 1) gx = 1;
-  return launch_chained(fill_omega_kernel, dim3(gx, w.l1 - w.l0), 256, 0, 0, s, w.d_layers, w.l0, seed, w.omega_row0);
+  return launch_chained(fill_omega_kernel, dim3(gx, w.l1 - w.l0), 256, 0, 0, s, w.d_layers, w.l0, seed, w.omega_row0, d_status, w.region);
 }
 
 // ------------------------------------------------------------------ four consecutive columns of one row of X

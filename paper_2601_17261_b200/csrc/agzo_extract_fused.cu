@@ -515,7 +515,7 @@ fused_power_step_kernel(const DevLayer* __restrict__ layers, int l0, int l1, int
   }
   tc_fence_before();
   __syncthreads();
-  if (sh.failed && threadIdx.x == 0) { atomicExch(&status->timeout, 1); atomicExch(&status->where, 4); }
+  if (sh.failed && threadIdx.x == 0) report_timeout(status, 4);
   cluster_sync_all();          // no peer reads my exchange buffer or arrives on my barriers after this
   if (follows) chain_wait();   // complete no earlier than the launches before: the next kernel waits for this one alone
   if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem, tmem_cols); }

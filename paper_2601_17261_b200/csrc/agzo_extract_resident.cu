@@ -90,9 +90,6 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
   asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
   return v;
 }
-__device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t v) {
-  asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
 __device__ __forceinline__ void st_cluster_u4(uint32_t addr, uint4 v) {
   asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
@@ -920,7 +917,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
     }
   }
   if (tid == 0) {
-    if (sh.failed && P.status) { atomicExch(&P.status->timeout, 1); atomicExch(&P.status->where, 5); }
+    if (sh.failed && P.status) report_timeout(P.status, 5);
     if (i == 0 && j == 0) {
       if (P.status && sh.st.rank_deficient) atomicExch(&P.status->rank_deficient, 1);
       if (P.flag) *P.flag = sh.failed ? 2 : sh.st.rank_deficient;

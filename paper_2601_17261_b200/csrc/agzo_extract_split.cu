@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(Cfg<NP, PLANES, XQ>::threads, 1) split_product
   tc_fence_before();
   __syncthreads();
   if (XQ && U.split > 1) cluster_sync_all();               // nobody leaves while a peer sends to it
-  if (sh.failed && threadIdx.x == 0) { atomicExch(&status->timeout, 1); atomicExch(&status->where, XQ ? 6 : 7); }
+  if (sh.failed && threadIdx.x == 0) report_timeout(status, XQ ? 6 : 7);
   if (warp == kMmaWarp) { tc_fence_after(); tmem_dealloc(tmem, C::tmem_cols); }
 }
 

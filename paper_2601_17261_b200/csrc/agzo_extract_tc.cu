@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(tc_threads(MB)) tc_x_q_kernel(const DevLayer* 
   }
   tc_fence_before();
   __syncthreads();
-  if (sh.failed && threadIdx.x == 0) { atomicExch(&status->timeout, 1); atomicExch(&status->where, 1); }
+  if (sh.failed && threadIdx.x == 0) report_timeout(status, 1);
   if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem, ncols); }
 }
 
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(tc_threads(MB)) tc_xt_t_kernel(const DevLayer*
   }
   tc_fence_before();
   __syncthreads();
-  if (sh.failed && threadIdx.x == 0) { atomicExch(&status->timeout, 1); atomicExch(&status->where, 2); }
+  if (sh.failed && threadIdx.x == 0) report_timeout(status, 2);
   if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem, ncols); }
 }
 
@@ -384,8 +384,9 @@ __global__ void __launch_bounds__(tc_threads(MB)) tc_xt_t_kernel(const DevLayer*
 // one where two would leave SMs without work.
 template <int kTok>
 __global__ void __launch_bounds__(256) tc_fill_omega_kernel(const DevLayer* layers, int l0, uint64_t seed,
-                                                            long long row0) {
+                                                            long long row0, DevStatus* status, int region) {
   chain_wait();
+  if (blockIdx.x + blockIdx.y + blockIdx.z == 0 && threadIdx.x == 0) wave_begins(status, region);
   if (short_launch()) chain_next();
   const DevLayer& L = layers[l0 + blockIdx.y];
   const int g = (int)blockIdx.z, r = L.r, rows = L.prow_n;
@@ -440,10 +441,7 @@ __global__ void debug_wait_kernel(DevStatus* status) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  if (threadIdx.x == 0 && !mbar_wait(&bar, 0)) {     // nobody arrives: the wait runs out
-    atomicExch(&status->timeout, 1);
-    atomicExch(&status->where, 100);
-  }
+  if (threadIdx.x == 0 && !mbar_wait(&bar, 0)) report_timeout(status, 100);     // nobody arrives: the wait runs out
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -584,12 +582,12 @@ bool tc_encode_maps(const TcState& st, const DevLayer& D, void* host_maps) {
   return true;
 }
 
-cudaError_t tc_fill_omega(const TcState&, const ExtractWave& w, const DevLayer*, uint64_t seed, cudaStream_t s) {
+cudaError_t tc_fill_omega(const TcState&, const ExtractWave& w, const DevLayer*, uint64_t seed, DevStatus* d_status, cudaStream_t s) {
   const unsigned nl = (unsigned)(w.l1 - w.l0), groups = (unsigned)((w.max_r + 14) >> 3);   // padding rows of a panel included
   const bool pairs = (long long)w.max_m * groups * nl >= 2ll * w.sm_count * 2048;
   const unsigned per = pairs ? 512 : 256;
   return launch_chained(pairs ? tc_fill_omega_kernel<2> : tc_fill_omega_kernel<1>, dim3(((unsigned)w.max_m + per - 1) / per, nl, groups),
-                        256, 0, 0, s, w.d_layers, w.l0, seed, w.omega_row0);
+                        256, 0, 0, s, w.d_layers, w.l0, seed, w.omega_row0, d_status, w.region);
 }
 
 cudaError_t tc_xt_t(const TcState&, const ExtractWave& w, const DevLayer* h_dev, DevStatus* d_status,

@@ -67,12 +67,25 @@ __device__ __forceinline__ void qr_store(const DevLayer& L, const float* sY, int
   }
 }
 
+// A wait for what the peers send has run out: known to all C CTAs of the cluster, and to the round that stores V
+__device__ __noinline__ void qr_wait_failed(int* failed, int C, DevStatus* status) {
+  if ((threadIdx.x & 31) == 0 && atomicExch(failed, 1) == 0) report_timeout(status, 8);
+  if ((int)(threadIdx.x & 31) < C) st_cluster_u32(mapa_shared(smem_u32(failed), threadIdx.x & 31u), 1u);
+}
+// V = 0 in columns [d0, d0 + ncols)
+__device__ __noinline__ void qr_zero(const DevLayer& L, int d0, int ncols) {
+  for (int i = threadIdx.x; i < L.r * ncols; i += kQrThreads) {
+    const int k = i / ncols, d = d0 + i - k * ncols;
+    if (d < L.d_in) L.V[(long long)k * L.ldv + d] = 0.f;
+  }
+}
+
 // kResident: the CTA's whole slice stays in shared memory from load to apply; otherwise it is staged 128 columns at
 // a time and read a second time (from L.Y, through L2) for the apply.
 template <int NT, bool kResident, int kLive, bool kSend>
 __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer* __restrict__ layers, int l0, int C, int pitch,
                                                                  int y_reduced, int after_fused, int last, unsigned* published,
-                                                                 DevStatus* status) {
+                                                                 DevStatus* status, int region) {
   static_assert(NT <= 4, "larger ranks take the three launches");
   using Cfg = QrCfg<NT>;
   // the layer's record comes into shared memory before the wait: read in place, each of its lines would cost the chain a
@@ -83,9 +96,13 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
     reinterpret_cast<unsigned long long*>(record)[i] =
         __ldcg(reinterpret_cast<const unsigned long long*>(layers + l0 + (int)blockIdx.x / C) + i);
   __shared__ uint64_t shares_in;
-  if (kSend && threadIdx.x == 0) {
-    mbar_init(&shares_in, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  __shared__ int failed;                 // a wait of this wave has run out
+  if (threadIdx.x == 0) {
+    failed = 0;
+    if (kSend) {
+      mbar_init(&shares_in, 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
   }
   __syncthreads();
   if (kSend) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");        // my barrier can be sent to
@@ -108,6 +125,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
   chain_wait();
   if (!last && short_launch()) chain_next();
   if (published && blockIdx.x == 0 && tid == 0) *published = 0u;
+  const bool earlier = last && tid == 0 && wave_failed(status, region);       // asked for here, needed behind the Gram products
   double acc[Cfg::my_tiles][2];
 #pragma unroll
   for (int t = 0; t < Cfg::my_tiles; ++t) acc[t][0] = acc[t][1] = 0.0;
@@ -128,6 +146,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
 #pragma unroll
   for (int t = 0; t < Cfg::tiles; ++t)
     *reinterpret_cast<double2*>(sU + (warp * Cfg::tiles + t) * 64 + el) = make_double2(acc[t][0], acc[t][1]);
+  if (earlier) failed = 1;
   __syncthreads();
   auto place = [&](int i, double v) {
     int t = i >> 6, bi = 0;
@@ -157,7 +176,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
       for (int c = 0; c < C; ++c) st_async_u4(mapa_shared(to, (uint32_t)c), w, mapa_shared(bar, (uint32_t)c));
     }
     __syncthreads();                        // the warps' sums are read: S takes their place
-    if (!mbar_wait_cluster(&shares_in, 0) && lane == 0 && status) { atomicExch(&status->timeout, 1); atomicExch(&status->where, 8); }
+    if (!mbar_wait_cluster_warp(&shares_in, 0)) qr_wait_failed(&failed, C, status);
     if (tid < kPairs) {
       double2 v[kQrMaxCluster], sum = make_double2(0.0, 0.0);
 #pragma unroll
@@ -207,6 +226,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
   }
   __syncwarp();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // nobody leaves while a peer may read its share
+  if (last && failed) qr_zero(L, d0, nch * kQrChunk);
 }
 
 // ------------------------------------------------------------------ ranks above 32: three launches
@@ -323,7 +343,7 @@ __global__ void __launch_bounds__(kQrThreads) panel_factor_kernel(const DevLayer
 
 // Q = Y M on 128 columns of a layer
 __global__ void __launch_bounds__(kQrThreads, 2) panel_apply_kernel(const DevLayer* __restrict__ layers, int l0, int last,
-                                                                    unsigned* published) {
+                                                                    unsigned* published, const DevStatus* status, int region) {
   using Cfg = QrCfg<8>;
   const DevLayer& L = layers[l0 + blockIdx.y];
   const int d0 = blockIdx.x * kQrChunk;
@@ -331,6 +351,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_apply_kernel(const DevLay
   if (!last && short_launch()) chain_next();
   if (published && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *published = 0u;
   if (d0 >= L.d_in) return;
+  const bool failed = last && wave_failed(status, region);
   extern __shared__ __align__(16) unsigned char qr_smem[];
   double* M = reinterpret_cast<double*>(qr_smem);
   float* sY = reinterpret_cast<float*>(M + Cfg::r8 * Cfg::mp);
@@ -357,7 +378,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_apply_kernel(const DevLay
   __syncthreads();
   qr_apply<8>(sY, pitch, M, kQrChunk);
   __syncthreads();
-  qr_store(L, sY, pitch, d0, kQrChunk, last || !L.Qb, !last && L.Qb);
+  if (failed) qr_zero(L, d0, kQrChunk); else qr_store(L, sY, pitch, d0, kQrChunk, last || !L.Qb, !last && L.Qb);
 }
 
 // The extraction's last round takes back the number of its last power step (DevStatus::panel_ready): a replayed graph gives the
@@ -386,12 +407,12 @@ cudaError_t launch_qr(const ExtractWave& w, bool last, DevStatus* d_status, cuda
   // Sending (up to rank 16, whose C shares are 24 KB at most) leaves out a barrier's wait and a round trip: 120 lists 0.5 % on the mean, eight
   // 1024 x 1024 layers, r = 8 141.9 -> 139.5 us, two 8B-shaped blocks from hooks 2806 -> 2789.
   if constexpr (NT <= 2)
-    if (!w.qr_reads && smem + C * QrCfg<NT>::g_bytes <= kQrResidentSmem) {
+    if (smem + C * QrCfg<NT>::g_bytes <= kQrResidentSmem) {
       smem += C * QrCfg<NT>::g_bytes;
       kernel = resident ? panel_qr_kernel<NT, true, kLive, true> : panel_qr_kernel<NT, false, kLive, true>;
     }
   return launch_chained(kernel, dim3((unsigned)(C * nl)), kQrThreads, smem, C, s, w.d_layers, w.l0, C, qr_pitch(slice), w.y_reduced,
-                        w.after_fused, last ? 1 : 0, published_at(w, last, d_status), d_status);
+                        w.after_fused, last ? 1 : 0, published_at(w, last, d_status), d_status, w.region);
 }
 
 constexpr size_t kGramSmem = (size_t)64 * (kQrChunk + 12) * sizeof(float);
@@ -405,7 +426,7 @@ cudaError_t launch_qr_large(const ExtractWave& w, bool last, DevStatus* d_status
   if (e == cudaSuccess) e = launch_chained(panel_factor_kernel, dim3(nl), kQrThreads, kFactorSmem, 0, s, w.d_layers, w.l0, d_status);
   if (e == cudaSuccess)
     e = launch_chained(panel_apply_kernel, dim3((unsigned)w.max_gchunks, nl), kQrThreads, kApplySmem, 0, s, w.d_layers, w.l0,
-                       last ? 1 : 0, published_at(w, last, d_status));
+                       last ? 1 : 0, published_at(w, last, d_status), d_status, w.region);
   return e;
 }
 

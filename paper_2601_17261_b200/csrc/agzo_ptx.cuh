@@ -295,6 +295,9 @@ __device__ __forceinline__ uint32_t cluster_count_x() {
 __device__ __forceinline__ uint32_t mapa_shared(uint32_t saddr, uint32_t rank) {
   uint32_t r; asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank)); return r;
 }
+__device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
 // bounded wait with acquire at cluster scope: for barriers that CTAs of the cluster arrive on.  The thread
 // suspends inside try_wait (the hardware wakes it when the phase completes): hundreds of threads polling a
 // barrier keep the shared-memory pipeline busy that the arrivals themselves have to pass through.

@@ -476,7 +476,7 @@ rmw_tc_kernel(const DevLayer* layers, const int* item_start, int n_layers,
   }
   tc_fence_before();
   __syncthreads();
-  if (sh.failed && threadIdx.x == 0) { atomicExch(&status->timeout, 1); atomicExch(&status->where, 3); }
+  if (sh.failed && threadIdx.x == 0) report_timeout(status, 3);
   if (warp == kWarpMma) { tc_fence_after(); tmem_dealloc(tmem, kTmemCols); }
 }
 

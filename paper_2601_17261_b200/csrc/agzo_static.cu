@@ -79,12 +79,10 @@ __global__ void static_begin_kernel(agzo::DevLayer rec, agzo::DevLayer* dst, agz
   st->pad = 0;
 }
 
-// a wait that ran out: V = 0, and the flag says so with a 2
-__global__ void static_end_kernel(const agzo::DevStatus* st, int32_t* flag, float* V, long long ldv, int r, int d_in) {
+// 2: a wait ran out, and the last panel QR has left V = 0
+__global__ void static_end_kernel(const agzo::DevStatus* st, int32_t* flag) {
   agzo::chain_wait();
-  if (flag && threadIdx.x == 0) *flag = st->timeout ? 2 : st->rank_deficient;
-  if (st->timeout)
-    for (long long i = threadIdx.x; i < (long long)r * d_in; i += blockDim.x) V[i / d_in * ldv + i % d_in] = 0.f;
+  *flag = st->timeout ? 2 : st->rank_deficient;
 }
 
 }  // namespace
@@ -167,9 +165,8 @@ agzo_status extract_static(const void* X, int64_t ldx, int32_t x_dtype, int32_t 
   w.l0 = 0; w.l1 = 1;
   w.sm_count = scratch.sm_count;
   w.qr_wide = scratch.qr_wide ? 1 : 0;
-  w.qr_reads = !d_rank_deficient && !split;      // no kernel at the end
   w.max_m = m; w.max_din = d_in; w.max_r = r; w.max_slabs = slabs; w.max_gchunks = (int)gch;
-  if (launch_fill_omega(w, seed, s) != cudaSuccess) return AGZO_ERR_CUDA;     // Omega
+  if (launch_fill_omega(w, seed, d_status, s) != cudaSuccess) return AGZO_ERR_CUDA;     // Omega
   const auto xt_t = [&] { return split ? launch_split_xt_t(w, &rec, true, d_status, s) : launch_xt_t(w, s); };
   const auto x_q = [&] { return split ? launch_split_x_q(w, &rec, true, d_status, s) : launch_x_q(w, s); };
   if (xt_t() != cudaSuccess) return AGZO_ERR_CUDA;                            // Y <- H Omega
@@ -179,9 +176,8 @@ agzo_status extract_static(const void* X, int64_t ldx, int32_t x_dtype, int32_t 
     if (xt_t() != cudaSuccess) return AGZO_ERR_CUDA;                          // Y <- H (H^T Q)
   }
   if (launch_panel_qr(w, true, d_status, s) != cudaSuccess) return AGZO_ERR_CUDA;    // A <- qr(Y)
-  if (d_rank_deficient || split) {
-    if (launch_chained(static_end_kernel, dim3(1), 256, 0, 0, s, d_status, d_rank_deficient, V, (long long)ldv, r, d_in) != cudaSuccess)
-      return AGZO_ERR_CUDA;
+  if (d_rank_deficient) {
+    if (launch_chained(static_end_kernel, dim3(1), 1, 0, 0, s, d_status, d_rank_deficient) != cudaSuccess) return AGZO_ERR_CUDA;
   }
   return AGZO_OK;
 }

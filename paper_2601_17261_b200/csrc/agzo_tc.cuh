@@ -57,7 +57,7 @@ cudaError_t launch_rmw_tc(const DevLayer* d_layers, const int* d_item_start, int
                           uint64_t seed, PassCoef coef, DevStatus* d_status, int sm_count, cudaStream_t s);
 
 cudaError_t tc_fill_omega(const TcState& st, const ExtractWave& w, const DevLayer* h_dev,
-                          uint64_t seed, cudaStream_t s);
+                          uint64_t seed, DevStatus* d_status, cudaStream_t s);
 // skip_fused: leave out the layers that the fused power-step kernel serves (fz_C > 0)
 cudaError_t tc_xt_t(const TcState& st, const ExtractWave& w, const DevLayer* h_dev,
                     DevStatus* d_status, bool skip_fused, cudaStream_t s);
