@@ -180,6 +180,9 @@ agzo_status agzo_destroy(agzo_ctx* ctx);
  * "debug_fail_step_call" = n (test aid, 0 = off): the n-th internal call of agzo_step
  * (extract, perturb, [flip,] ghat, restore_update) returns AGZO_ERR_CUDA on the host before
  * launching anything, so that the step's error path can be exercised without a fault;
+ * "debug_missing_class" = AGZO_KC_PANEL_QR, AGZO_KC_XT_T or AGZO_KC_X_Q (test aid, 0 = off): in that kernel's launches, where
+ * it is the panel QR that sends (ranks up to 16) or a product in parts, a barrier expects more than comes, and the waits
+ * end after 0.1 ms;
  * "debug_refuse_resident" 1 (test aid, 0 = off): launches of the resident kernel end on the host as
  * if the device had refused them for want of SMs, so that the other kernels serve the call. */
 agzo_status agzo_set_option(agzo_ctx* ctx, const char* name, int64_t value);

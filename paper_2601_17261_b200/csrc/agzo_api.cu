@@ -130,6 +130,7 @@ struct agzo_ctx {
   ResidentCaps resident_caps;
   // measurement aid: event pairs around the launches of one kernel class
   int debug_fail_step_call;   // test option: the n-th internal call of agzo_step fails on the host, 0 = off
+  int debug_missing_class;       // test option: in launches of this kernel class a wait runs out (ExtractWave::missing), 0 = off
   int debug_refuse_resident;  // test option: launches of the resident kernel end as if the device had refused them
   int time_class;
   std::vector<cudaEvent_t> events;   // pairs: start, stop
@@ -983,6 +984,7 @@ agzo_status agzo_create(agzo_ctx** out, int device, void* workspace, size_t work
   c->stage_ev = nullptr;
   c->time_class = 0;
   c->debug_fail_step_call = 0;
+  c->debug_missing_class = 0;
   c->debug_refuse_resident = 0;
   c->events_used = 0;
   c->launches = 0;
@@ -1077,6 +1079,10 @@ agzo_status agzo_set_option(agzo_ctx* ctx, const char* name, int64_t value) {
   } else if (std::strcmp(name, "debug_fail_step_call") == 0) {
     if (value < 0 || value > 16) return AGZO_ERR_INVALID_ARG;
     ctx->debug_fail_step_call = (int)value;
+    return AGZO_OK;
+  } else if (std::strcmp(name, "debug_missing_class") == 0) {
+    if (value != 0 && value != AGZO_KC_XT_T && value != AGZO_KC_X_Q && value != AGZO_KC_PANEL_QR) return AGZO_ERR_INVALID_ARG;
+    ctx->debug_missing_class = (int)value;
     return AGZO_OK;
   } else if (std::strcmp(name, "debug_refuse_resident") == 0) {
     if (value < 0 || value > 1) return AGZO_ERR_INVALID_ARG;
@@ -1252,6 +1258,7 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
       DevStatus* dst = dev_status(ctx);
       auto panel_qr = [&](bool last) -> cudaError_t {
         Timed t(ctx, AGZO_KC_PANEL_QR, ws, panel_qr_launches(w.max_r));
+        w.missing = ctx->debug_missing_class == AGZO_KC_PANEL_QR;
         return launch_panel_qr(w, last, dst, ws);
       };
       // token-sharded run: Y = sum over ranks of X_p^T T_p, all panels of the wave in one call
@@ -1278,11 +1285,13 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
       }
       auto xt_t = [&](bool skip_fused) -> cudaError_t {       // Y <- H T
         Timed t(ctx, all_tc ? AGZO_KC_TC_XT_T : AGZO_KC_XT_T, ws);
+        w.missing = ctx->debug_missing_class == AGZO_KC_XT_T;
         if (split) return launch_split_xt_t(w, P.dev.data(), ctx->share_inputs != 0, dst, ws);
         return all_tc ? tc_xt_t(ctx->tc, w, P.dev.data(), dst, skip_fused, ws) : launch_xt_t(w, ws);
       };
       auto x_q = [&]() -> cudaError_t {        // T <- H^T Q
         Timed t(ctx, all_tc ? AGZO_KC_TC_X_Q : AGZO_KC_X_Q, ws);
+        w.missing = ctx->debug_missing_class == AGZO_KC_X_Q;
         if (split) return launch_split_x_q(w, P.dev.data(), ctx->share_inputs != 0, dst, ws);
         return all_tc ? tc_x_q(ctx->tc, w, P.dev.data(), dst, true, ws) : launch_x_q(w, ws);
       };

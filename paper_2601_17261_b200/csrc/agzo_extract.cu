@@ -13,8 +13,8 @@ namespace agzo {
 // (row0 + t) * r + k, so the Philox blocks that cover the local rows are walked, whatever row0 is.
 __global__ void fill_omega_kernel(const DevLayer* layers, int l0, uint64_t seed, long long row0, DevStatus* status, int region) {
   chain_wait();
-  if (blockIdx.x + blockIdx.y == 0 && threadIdx.x == 0) wave_begins(status, region);
   if (short_launch()) chain_next();
+  if (blockIdx.x + blockIdx.y == 0 && threadIdx.x == 0) wave_begins(status, region);
   const DevLayer& L = layers[l0 + blockIdx.y];
   const long long n = (long long)L.m * L.r;
   const long long e0 = row0 * L.r;

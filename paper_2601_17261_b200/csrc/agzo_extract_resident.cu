@@ -911,10 +911,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_extract_kernel(const __g
   if (cs > 1) cluster_sync_all(); else __syncthreads();      // nobody leaves while a peer may read its share
   if (sh.failed) {                                           // a wait has run out and the sums are not whole
     zero_strips(U, i, col0);
-    if (PUSH) {                                              // what the peers have sent may be on its way yet
-      const unsigned long long t_end = global_ns() + 100000;
-      while (global_ns() < t_end) {}
-    }
+    if (PUSH) let_land();
   }
   if (tid == 0) {
     if (sh.failed && P.status) report_timeout(P.status, 5);

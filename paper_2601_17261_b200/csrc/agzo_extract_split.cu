@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(Cfg<NP, PLANES, XQ>::threads, 1) split_product
   const uint32_t tiles = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) { mbar_init(&sh.full[s], kGroupWarps + C::op_warps); mbar_init(&sh.empty[s], 1); }
+    for (int s = 0; s < kStages; ++s) { mbar_init(&sh.full[s], kGroupWarps + C::op_warps + (U.split == 1 ? U.missing : 0u)); mbar_init(&sh.empty[s], 1); }
     for (int b = 0; b < kAcc; ++b) { mbar_init(&sh.acc_full[b], 1); mbar_init(&sh.acc_empty[b], kEpiWarps); }
     mbar_init(&sh.sums_in, 1);
     mbar_init(&sh.sums_out, kEpiWarps);
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(Cfg<NP, PLANES, XQ>::threads, 1) split_product
     }
     uint32_t s = (uint32_t)(group % kStages), par = 1;     // first round of a stage: free
     while (at.it >= 0) {
-      if (!mbar_wait_warp(&sh.empty[s], par)) { sh.failed = 1; break; }
+      if (!mbar_wait_warp(&sh.empty[s], par, U.wait_ns)) { sh.failed = 1; break; }
       const uint32_t dst = tiles + s * (uint32_t)kStageBytes;
       const bool moved = at.advance(U, kLoadGroups);
       const bool more = at.it >= 0;
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(Cfg<NP, PLANES, XQ>::threads, 1) split_product
     for (int i = 0, it; ok && (it = nth_item(U, i)) >= 0; ++i) {
       const int n = __shfl_sync(0xffffffffu, steps_of(item_of<XQ>(U, it)), 0);      // which the compiler knows to be uniform
       for (int k = 0; k < n; ++k) {
-        if (!mbar_wait_warp(&sh.full[s], par) || !mbar_wait_warp(&sh.acc_empty[b], bpar)) { sh.failed = 1; ok = false; break; }
+        if (!mbar_wait_warp(&sh.full[s], par, U.wait_ns) || !mbar_wait_warp(&sh.acc_empty[b], bpar, U.wait_ns)) { sh.failed = 1; ok = false; break; }
         fence_proxy_async();
         tc_fence_after();
         const uint32_t a = tiles + s * (uint32_t)kStageBytes, d = tmem + b * (uint32_t)NB;
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(Cfg<NP, PLANES, XQ>::threads, 1) split_product
     if (e == 0 && short_launch()) chain_next();
     if (at.it >= 0) { open(); fetch(); }
     while (at.it >= 0) {
-      if (!mbar_wait_warp(&sh.empty[s], par)) { sh.failed = 1; break; }
+      if (!mbar_wait_warp(&sh.empty[s], par, U.wait_ns)) { sh.failed = 1; break; }
       const uint32_t dst = s * (uint32_t)kStageBytes;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(Cfg<NP, PLANES, XQ>::threads, 1) split_product
 #pragma unroll
         for (int k = 0; k < H / 2; ++k) sum[p][k] = 0;
       for (int k = 0; k < n; ++k) {
-        if (!mbar_wait_warp(&sh.acc_full[b], par)) { ok = false; break; }
+        if (!mbar_wait_warp(&sh.acc_full[b], par, U.wait_ns)) { ok = false; break; }
         tc_fence_after();
         // two parts at a time, for want of registers
         uint32_t z[2][H];
@@ -472,14 +472,14 @@ __global__ void __launch_bounds__(Cfg<NP, PLANES, XQ>::threads, 1) split_product
         const uint32_t rank = cluster_ctarank(), mine = (uint32_t)((warp - kLoadWarps) * 32 + lane) * 16u, piece = kEpiWarps * 32 * 16;
         const uint32_t peers = tiles + (uint32_t)(kStages * kStageBytes);
         if (rank != 0) {
-          if (i > 0 && !mbar_wait_cluster_warp(&sh.sums_out, (uint32_t)(i - 1) & 1u)) { ok = false; break; }
+          if (i > 0 && !mbar_wait_cluster_warp(&sh.sums_out, (uint32_t)(i - 1) & 1u, U.wait_ns)) { ok = false; break; }
           const uint32_t dst = mapa_shared(peers + (rank - 1u) * C::peer_bytes + mine, 0), bar = mapa_shared(smem_u32(&sh.sums_in), 0);
 #pragma unroll
           for (int c = 0; c < H; c += 4) st_async_f4(dst + (uint32_t)(c / 4) * piece, make_float4(y[c], y[c + 1], y[c + 2], y[c + 3]), bar);
           continue;
         }
-        if (warp == kLoadWarps && lane == 0) mbar_expect_tx(&sh.sums_in, (uint32_t)(U.split - 1) * C::peer_bytes);
-        if (!mbar_wait_cluster_warp(&sh.sums_in, (uint32_t)i & 1u)) { ok = false; break; }
+        if (warp == kLoadWarps && lane == 0) mbar_expect_tx(&sh.sums_in, (uint32_t)(U.split - 1) * C::peer_bytes + U.missing);
+        if (!mbar_wait_cluster_warp(&sh.sums_in, (uint32_t)i & 1u, U.wait_ns)) { ok = false; break; }
         for (int p = 0; p < U.split - 1; ++p)
 #pragma unroll
           for (int c = 0; c < H; c += 4) {
@@ -509,6 +509,7 @@ __global__ void __launch_bounds__(Cfg<NP, PLANES, XQ>::threads, 1) split_product
   tc_fence_before();
   __syncthreads();
   if (XQ && U.split > 1) cluster_sync_all();               // nobody leaves while a peer sends to it
+  if (sh.failed) let_land();
   if (sh.failed && threadIdx.x == 0) report_timeout(status, XQ ? 6 : 7);
   if (warp == kMmaWarp) { tc_fence_after(); tmem_dealloc(tmem, C::tmem_cols); }
 }
@@ -610,7 +611,7 @@ cudaError_t allow_smem(const void* kernel, size_t smem) {
 }
 
 template <int N>
-cudaError_t launch_units(const std::vector<SplitUnit>& units, size_t first, int np, int planes, bool xq, int sm_count, DevStatus* status, cudaStream_t s) {
+cudaError_t launch_units(const std::vector<SplitUnit>& units, size_t first, int np, int planes, bool xq, int sm_count, bool missing, DevStatus* status, cudaStream_t s) {
   SplitUnits<N> U;
   U.n_units = (int)std::min((size_t)N, units.size() - first);
   long long items = 0;
@@ -623,6 +624,8 @@ cudaError_t launch_units(const std::vector<SplitUnit>& units, size_t first, int 
   if (items > 0x3fffffff) return cudaErrorInvalidValue;
   U.n_items = (int)items;
   U.split = 1;
+  U.wait_ns = missing ? kMissingWaitNs : (unsigned)kWaitCapNs;
+  U.missing = missing ? 1 : 0;
   if (xq) {
     std::vector<XqUnit> shapes;
     for (int k = 0; k < U.n_units; ++k) shapes.push_back(XqUnit{U.unit[k].m, U.unit[k].d_in});
@@ -643,9 +646,9 @@ cudaError_t launch(const ExtractWave& w, const DevLayer* dev, bool share, bool x
   const int planes = dev[w.l0].x_dtype == AGZO_F32 ? 3 : 1;
   std::stable_sort(units.begin(), units.end(), [](const SplitUnit& a, const SplitUnit& b) { return a.d_in > b.d_in; });
   if (!xq) std::reverse(units.begin(), units.end());
-  if (units.size() <= kSplitFewUnits) return launch_units<kSplitFewUnits>(units, 0, np, planes, xq, w.sm_count, status, s);
+  if (units.size() <= kSplitFewUnits) return launch_units<kSplitFewUnits>(units, 0, np, planes, xq, w.sm_count, w.missing != 0, status, s);
   for (size_t at = 0; at < units.size(); at += kSplitMaxUnits) {
-    const cudaError_t e = launch_units<kSplitMaxUnits>(units, at, np, planes, xq, w.sm_count, status, s);
+    const cudaError_t e = launch_units<kSplitMaxUnits>(units, at, np, planes, xq, w.sm_count, w.missing != 0, status, s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

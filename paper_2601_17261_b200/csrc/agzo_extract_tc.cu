@@ -386,8 +386,8 @@ template <int kTok>
 __global__ void __launch_bounds__(256) tc_fill_omega_kernel(const DevLayer* layers, int l0, uint64_t seed,
                                                             long long row0, DevStatus* status, int region) {
   chain_wait();
-  if (blockIdx.x + blockIdx.y + blockIdx.z == 0 && threadIdx.x == 0) wave_begins(status, region);
   if (short_launch()) chain_next();
+  if (blockIdx.x + blockIdx.y + blockIdx.z == 0 && threadIdx.x == 0) wave_begins(status, region);
   const DevLayer& L = layers[l0 + blockIdx.y];
   const int g = (int)blockIdx.z, r = L.r, rows = L.prow_n;
   const int t0 = (int)(blockIdx.x * 256 + threadIdx.x) * kTok;

@@ -85,7 +85,7 @@ __device__ __noinline__ void qr_zero(const DevLayer& L, int d0, int ncols) {
 template <int NT, bool kResident, int kLive, bool kSend>
 __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer* __restrict__ layers, int l0, int C, int pitch,
                                                                  int y_reduced, int after_fused, int last, unsigned* published,
-                                                                 DevStatus* status, int region) {
+                                                                 DevStatus* status, int region, unsigned wait_ns, unsigned missing) {
   static_assert(NT <= 4, "larger ranks take the three launches");
   using Cfg = QrCfg<NT>;
   // the layer's record comes into shared memory before the wait: read in place, each of its lines would cost the chain a
@@ -125,7 +125,8 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
   chain_wait();
   if (!last && short_launch()) chain_next();
   if (published && blockIdx.x == 0 && tid == 0) *published = 0u;
-  const bool earlier = last && tid == 0 && wave_failed(status, region);       // asked for here, needed behind the Gram products
+  int timeouts = 0, before = 0;          // asked for here, compared behind the Gram products
+  if (last && tid == 0) { timeouts = __ldcg(&status->timeout); before = __ldcg(&status->before[region]); }
   double acc[Cfg::my_tiles][2];
 #pragma unroll
   for (int t = 0; t < Cfg::my_tiles; ++t) acc[t][0] = acc[t][1] = 0.0;
@@ -146,7 +147,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
 #pragma unroll
   for (int t = 0; t < Cfg::tiles; ++t)
     *reinterpret_cast<double2*>(sU + (warp * Cfg::tiles + t) * 64 + el) = make_double2(acc[t][0], acc[t][1]);
-  if (earlier) failed = 1;
+  if (timeouts != before) failed = 1;
   __syncthreads();
   auto place = [&](int i, double v) {
     int t = i >> 6, bi = 0;
@@ -160,7 +161,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
     static_assert(kPairs <= kQrThreads, "two elements a thread");
     __syncwarp();
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    if (tid == 0) mbar_expect_tx(&shares_in, (uint32_t)(C * Cfg::tiles * 64 * 8));
+    if (tid == 0) mbar_expect_tx(&shares_in, (uint32_t)(C * Cfg::tiles * 64 * 8) + missing);
     if (tid < kPairs) {
       double2 sum = make_double2(0.0, 0.0);
 #pragma unroll
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
       for (int c = 0; c < C; ++c) st_async_u4(mapa_shared(to, (uint32_t)c), w, mapa_shared(bar, (uint32_t)c));
     }
     __syncthreads();                        // the warps' sums are read: S takes their place
-    if (!mbar_wait_cluster_warp(&shares_in, 0)) qr_wait_failed(&failed, C, status);
+    if (!mbar_wait_cluster_warp(&shares_in, 0, wait_ns)) qr_wait_failed(&failed, C, status);
     if (tid < kPairs) {
       double2 v[kQrMaxCluster], sum = make_double2(0.0, 0.0);
 #pragma unroll
@@ -226,7 +227,10 @@ __global__ void __launch_bounds__(kQrThreads, 2) panel_qr_kernel(const DevLayer*
   }
   __syncwarp();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // nobody leaves while a peer may read its share
-  if (last && failed) qr_zero(L, d0, nch * kQrChunk);
+  if (failed) {
+    if (last) qr_zero(L, d0, nch * kQrChunk);
+    if (kSend) let_land();
+  }
 }
 
 // ------------------------------------------------------------------ ranks above 32: three launches
@@ -412,7 +416,8 @@ cudaError_t launch_qr(const ExtractWave& w, bool last, DevStatus* d_status, cuda
       kernel = resident ? panel_qr_kernel<NT, true, kLive, true> : panel_qr_kernel<NT, false, kLive, true>;
     }
   return launch_chained(kernel, dim3((unsigned)(C * nl)), kQrThreads, smem, C, s, w.d_layers, w.l0, C, qr_pitch(slice), w.y_reduced,
-                        w.after_fused, last ? 1 : 0, published_at(w, last, d_status), d_status, w.region);
+                        w.after_fused, last ? 1 : 0, published_at(w, last, d_status), d_status, w.region, w.missing ? kMissingWaitNs : (unsigned)kWaitCapNs,
+                        w.missing ? 1u : 0u);
 }
 
 constexpr size_t kGramSmem = (size_t)64 * (kQrChunk + 12) * sizeof(float);

@@ -73,17 +73,23 @@ __device__ __forceinline__ bool mbar_test_cluster_warp(uint64_t* bar, uint32_t p
       : "memory");
   return __any_sync(0xffffffffu, ok != 0);
 }
-// Bounded wait: false when two seconds have passed without the phase completing.  The
+// Bounded wait: false when `cap` nanoseconds (two seconds) have passed without the phase completing.  The
 // waiting thread sleeps inside try_wait instead of spinning through issue slots.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsigned long long cap = kWaitCapNs) {
   if (mbar_try_wait(bar, parity)) return true;
   const unsigned long long t0 = global_ns();
   for (;;) {
 #pragma unroll 1
     for (int i = 0; i < 16; ++i)
       if (mbar_try_wait_for(bar, parity, 4000u)) return true;
-    if (global_ns() - t0 > kWaitCapNs) return false;
+    if (global_ns() - t0 > cap) return false;
   }
+}
+// A CTA that has given up a wait calls this before it leaves or frees its TMEM: what was on its way to its shared memory (what peers
+// have sent with st.async, which a barrier of the cluster does not order, and its own products) is there when this returns.
+inline __device__ __noinline__ void let_land() {
+  const unsigned long long t_end = global_ns() + 100000;
+  while (global_ns() < t_end) {}
 }
 // What the storing thread has observed of earlier kernels' writes is observed by a thread that sees the value (at gpu scope)
 __device__ __forceinline__ void st_release_gpu(unsigned* p, unsigned v) {
@@ -219,8 +225,8 @@ __device__ __forceinline__ void mma_commit_if(uint32_t go, uint64_t* bar) {
       : "memory");
 }
 // bounded wait by a whole warp; the answer is made the same for all lanes
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity) {
-  const bool ok = mbar_wait(bar, parity);
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, unsigned long long cap = kWaitCapNs) {
+  const bool ok = mbar_wait(bar, parity, cap);
   return __all_sync(0xffffffffu, ok);
 }
 
@@ -301,7 +307,7 @@ __device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t v) {
 // bounded wait with acquire at cluster scope: for barriers that CTAs of the cluster arrive on.  The thread
 // suspends inside try_wait (the hardware wakes it when the phase completes): hundreds of threads polling a
 // barrier keep the shared-memory pipeline busy that the arrivals themselves have to pass through.
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, unsigned long long cap = kWaitCapNs) {
   const unsigned long long t0 = global_ns();
   for (;;) {
 #pragma unroll 1
@@ -316,7 +322,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
           : "memory");
       if (ok) return true;
     }
-    if (global_ns() - t0 > kWaitCapNs) return false;
+    if (global_ns() - t0 > cap) return false;
   }
 }
 // one-way store of four floats into the shared memory of a CTA of the cluster; the bytes are
@@ -336,8 +342,8 @@ __device__ __forceinline__ void st_async_u4(uint32_t remote_addr, const uint32_t
                ::"r"(remote_addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(remote_bar)
                : "memory");
 }
-__device__ __forceinline__ bool mbar_wait_cluster_warp(uint64_t* bar, uint32_t parity) {
-  const bool ok = mbar_wait_cluster(bar, parity);
+__device__ __forceinline__ bool mbar_wait_cluster_warp(uint64_t* bar, uint32_t parity, unsigned long long cap = kWaitCapNs) {
+  const bool ok = mbar_wait_cluster(bar, parity, cap);
   return __all_sync(0xffffffffu, ok);
 }
 // every thread of every CTA of the cluster

@@ -31,9 +31,11 @@ struct SplitUnit {
   SplitLayer layer[kSplitMaxLayers];
 };
 template <int N> struct SplitUnits {
-  int n_units, n_items, split, pad;      // split: CTAs that share an item (T = X Q)
+  int n_units, n_items, split;           // split: CTAs that share an item (T = X Q)
+  unsigned wait_ns, missing, pad;        // limit of a wait; a test's: 1: a barrier expects more than comes
   SplitUnit unit[N];
 };
+static_assert(sizeof(SplitUnits<kSplitMaxUnits>) + sizeof(void*) <= 32764, "kernel parameters");
 
 // Token slabs of Y = X^T T for `units` units of 128 columns on the device: whole steps of 64, the SMs' last items starting
 // together; a step is about 0.7 us, an item's start 1.5 steps, a slab costs the panel QR 0.2 us.
