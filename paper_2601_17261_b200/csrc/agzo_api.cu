@@ -242,16 +242,16 @@ bool same_input(const agzo_layer& a, const agzo_layer& b) {
 // 16384 tokens: every slab costs a partial Y (r x d_in floats written, and read again by the
 // panel QR), and the CTAs' pipelines start and drain less often.
 constexpr int kLongSlabColumnBlocks = 1024;   // 128-column blocks over all layers from which slabs are long
-// cc_blocks: 128-column blocks over the call's layers on the CUDA-core path; 0 = the most slabs the layer can get (sizing).
-// split: cc_blocks counts units of the products in parts.
-void slab_shape(const agzo_layer& a, bool tc, bool long_slabs, long long cc_blocks, bool split, int sm_count, int* slabs, int* slab_rows) {
+// blocks: 128-column blocks over the call's layers on the CUDA-core path, or (split) over the units of the products in parts; 0 = the most
+// slabs the layer can get (sizing).
+void slab_shape(const agzo_layer& a, bool tc, bool long_slabs, long long blocks, bool split, int sm_count, int* slabs, int* slab_rows) {
   int rows;
   if (tc) {
     rows = a.m >= 8192 ? (long_slabs ? (a.m < 16384 ? a.m : 16384) : 2048) : (a.m + 3) / 4;
     rows = (rows + 127) / 128 * 128;      // whole tiles of every tensor-core kernel (64 or 128 tokens)
     if (rows < 256) rows = 256;
-  } else if (cc_blocks > 0) {
-    rows = split ? split_slab_rows(a.m, cc_blocks, sm_count) : cc_slab_rows(a.m, cc_blocks, sm_count);
+  } else if (blocks > 0) {
+    rows = split ? split_slab_rows(a.m, blocks, sm_count) : cc_slab_rows(a.m, blocks, sm_count);
   } else {
     const int most = (a.m + kCcMinSlabRows - 1) / kCcMinSlabRows;
     *slabs = most < kCcMaxSlabs ? most : kCcMaxSlabs;
@@ -515,12 +515,12 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
       if (has_x(L[k]) && !on_tc(L[k])) which.push_back(k);
     plan->split = opts.split == 2 || split_pays(L, which, opts.share_inputs, opts.sm_count);
   }
+  long long split_blocks = 0;
   if (plan->split) {                       // its units are panels of the layers on one X
-    cc_blocks = 0;
     for (int k = 0; k < n;) {
       int run = 1, all = L[k].r;
       while (opts.share_inputs && has_x(L[k]) && k + run < n && has_x(L[k + run]) && same_input(L[k], L[k + run])) all += L[k + run++].r;
-      if (has_x(L[k]) && !on_tc(L[k])) cc_blocks += (long long)((L[k].d_in + 127) / 128) * ((all + kSplitMaxRanks - 1) / kSplitMaxRanks);
+      if (has_x(L[k]) && !on_tc(L[k])) split_blocks += (long long)((L[k].d_in + 127) / 128) * ((all + kSplitMaxRanks - 1) / kSplitMaxRanks);
       k += run;
     }
   }
@@ -533,8 +533,8 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     return (tc ? 0 : align_up((size_t)a.m * a.r * 4)) + align_up((size_t)a.r * a.d_in * 4) + align_up(panel_gram_bytes(a.d_in, a.r, extract_max_r));
   };
   auto ypart_bytes = [&](int parts, int ranks, int d_in) { return align_up((size_t)parts * ranks * (size_t)d_in * 4); };
-  auto slabs_of = [&](const agzo_layer& a, bool tc, int* slabs, int* slab_rows) {
-    slab_shape(a, tc, long_slabs_any, ws ? cc_blocks : 0, plan->split, opts.sm_count, slabs, slab_rows);
+  auto slabs_of = [&](const agzo_layer& a, bool tc, bool split, int* slabs, int* slab_rows) {
+    slab_shape(a, tc, long_slabs_any, !ws ? 0 : split ? split_blocks : cc_blocks, split, opts.sm_count, slabs, slab_rows);
     // a workspace of less than agzo_workspace_bytes takes fewer slabs on the CUDA-core path, as long as one is left
     for (int want = *slabs; ws && !tc && want > 1 && ypart_bytes(*slabs, a.r, a.d_in) + layer_need(a, tc) > scratch_cap;) {
       --want;
@@ -545,7 +545,12 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
   // partial sums of Y that a unit's last product can leave: slabs, or shares of a fused launch
   auto parts_of = [&](const agzo_layer& a, bool tc, bool fused, int ranks) {
     int slabs, slab_rows;
-    slabs_of(a, tc, &slabs, &slab_rows);
+    slabs_of(a, tc, false, &slabs, &slab_rows);
+    if (!tc && plan->split) {              // either product
+      int split_slabs;
+      slabs_of(a, tc, true, &split_slabs, &slab_rows);
+      slabs = std::max(slabs, split_slabs);
+    }
     if (!fused) return slabs;
     const int C = ws ? fused_cluster_size(opts.fused_caps, with_ranks(a, ranks), opts.extract_fused == 2) : fused_min_cluster(a);
     return std::max(slabs, fused_parts_bound(a, C));
@@ -611,7 +616,9 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
         for (int g = 0; g < glen; ++g) {
           DevLayer& D = plan->dev[j + g];
           const agzo_layer& a = L[j + g];
-          slabs_of(a, tc, &D.slabs, &D.slab_rows);
+          slabs_of(a, tc, false, &D.slabs, &D.slab_rows);
+          D.cc_slabs = D.slabs;
+          if (!tc && plan->split) slabs_of(a, tc, true, &D.slabs, &D.slab_rows);
           D.gchunks = (a.d_in + 127) / 128;
           D.Ypart = ypart + (size_t)off * a.d_in;
           D.ypart_stride = (long long)ranks * a.d_in;
@@ -1273,6 +1280,11 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
       };
       // products of this wave in parts: layers of one dtype, and for fp32 a power step (see split_takes)
       const bool split = !all_tc && P.split && split_takes(w, P.dev.data(), K);
+      if (!all_tc && !split) {
+        w.after_fused = 2;
+        w.max_slabs = 0;
+        for (int i = w.l0; i < w.l1; ++i) w.max_slabs = std::max(w.max_slabs, P.dev[i].cc_slabs);
+      }
       auto omega = [&]() -> cudaError_t {
         Timed t(ctx, AGZO_KC_OMEGA, ws);
         return all_tc ? tc_fill_omega(ctx->tc, w, P.dev.data(), seed, dst, ws) : launch_fill_omega(w, seed, dst, ws);

@@ -102,7 +102,7 @@ __device__ __forceinline__ void xt_t_body(const DevLayer& L, float* sT, float* s
   constexpr int kStage = kXtTokens * RC / kXThreads;     // values of T per thread and chunk
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int d = d0 + 4 * lane, r = L.r;
-  const int t_begin = slab * L.slab_rows, t_end = min(L.m, t_begin + L.slab_rows);
+  const int rows = cc_rows(L.m, L.cc_slabs), t_begin = slab * rows, t_end = min(L.m, t_begin + rows);
   for (int k0 = 0; k0 < r; k0 += RC) {
     const int kc = min(RC, r - k0);
     float acc[RC][4];
@@ -229,7 +229,7 @@ template <int RC>
 __global__ void __launch_bounds__(kXThreads, 2) xt_t_kernel(const DevLayer* __restrict__ layers, int l0) {
   const DevLayer& L = layers[l0 + blockIdx.z];
   const int slab = blockIdx.y, d0 = blockIdx.x * kXCols;
-  if (slab >= L.slabs || d0 >= L.d_in) return;
+  if (slab >= L.cc_slabs || d0 >= L.d_in) return;
   __shared__ __align__(16) float sT[kXtTokens * RC * (RC > 8 ? 2 : 1)];
   __shared__ __align__(16) float sRed[kXWarps / 2 * RC * kXCols];
   const int kind = x_kind(L);

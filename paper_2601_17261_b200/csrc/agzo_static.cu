@@ -150,7 +150,7 @@ agzo_status extract_static(const void* X, int64_t ldx, int32_t x_dtype, int32_t 
   DevLayer rec{};
   rec.X = X; rec.V = V; rec.ldx = ldx; rec.ldv = ldv;
   rec.x_dtype = x_dtype; rec.d_in = d_in; rec.m = m; rec.r = r; rec.layer_id = layer_id;
-  rec.slabs = slabs; rec.slab_rows = slab_rows; rec.gchunks = (int)gch;
+  rec.slabs = rec.cc_slabs = slabs; rec.slab_rows = slab_rows; rec.gchunks = (int)gch;
   rec.T = reinterpret_cast<float*>(p);      p += up256(M * R * 4);
   rec.ypart_stride = (long long)r * d_in;
   rec.Ypart = reinterpret_cast<float*>(p);  p += up256((size_t)slabs * R * D * 4);

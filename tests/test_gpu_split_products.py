@@ -86,3 +86,19 @@ def test_small_fp32_inputs_keep_their_bits_without_a_power_step():
         assert B.agzo_poll(ctx) == B.AGZO_OK
     Vo = O.extract_subspace(X.astype(np.float64) * 2.0 ** 118, r, 0, 9, 0)
     assert projector_distance(to_host(V), Vo) <= 1e-6
+
+
+@pytest.mark.parametrize("specs,K", [([(5000, 700, 24, False)] * 2, 0), ([(12000, 512, 16, False)], 0), ([(3000, 516, 9, False), (2000, 1001, 5, True)], 2)])
+def test_what_stays_with_the_cuda_cores_is_cut_for_them(specs, K):
+    # fp32 without a power step, and a wave of both types: the same bits as where there are no products in parts, so the same token slabs
+    X = [torch.randn(m, d, device=DEV).to(torch.bfloat16 if bf16 else torch.float32) for m, d, _, bf16 in specs]
+    V = [[torch.zeros(r, d, device=DEV) for _, d, r, _ in specs] for _ in range(3)]
+    for split in range(3):
+        layers = [B.make_layer(X=x, V=v, r=s[2], layer_id=i) for i, (x, v, s) in enumerate(zip(X, V[split], specs))]
+        with Ctx(layers) as ctx:
+            B.agzo_set_option(ctx, "extract_resident", 0)
+            B.agzo_set_option(ctx, "extract_split", split)
+            B.agzo_extract_subspace(ctx, layers, 9, K)
+            assert B.agzo_poll(ctx) == B.AGZO_OK
+    for split in (1, 2):
+        assert all(torch.equal(a, b) for a, b in zip(V[0], V[split])), split
