@@ -422,6 +422,10 @@ agzo_status agzo_debug_extract_static(const void* X, int64_t ldx, int32_t x_dtyp
 agzo_status agzo_debug_meeting(int32_t n, int32_t first, uint32_t phase, uint64_t value, uint64_t* h_increment, uint32_t* h_phase,
                                uint32_t* h_failures);
 
+/* Test export, host only: h_rows[0] and h_rows[1], the rows of a tile of the CUDA-core in-place pass over the list on a device of
+ * sm_count SMs, for layers whose rows allow 16-byte accesses and for the others.            */
+agzo_status agzo_debug_tile_rows(const agzo_layer* h_layers, int n, int sm_count, int32_t* h_rows);
+
 /* Exercises the bounded device-side wait that every pipeline of the tensor-core kernels uses:
  * launches one small block that waits, with the library's own wait routine, on a barrier that
  * nothing ever completes.  The wait gives up after its time limit (two seconds), the block

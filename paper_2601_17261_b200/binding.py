@@ -36,7 +36,7 @@ EXPORTS = [
     "agzo_extract_subspace_static", "agzo_fill_gaussian_basis", "agzo_set_allreduce",
     "agzo_debug_wait_timeout", "agzo_query_fused", "agzo_query_cluster_capacity", "agzo_debug_fused_split",
     "agzo_debug_early_copy", "agzo_debug_normal_parts", "agzo_debug_meeting",
-    "agzo_debug_extract_static", "agzo_query_resident",
+    "agzo_debug_extract_static", "agzo_query_resident", "agzo_debug_tile_rows",
 ]
 KC_RMW, KC_XT_T, KC_X_Q, KC_PANEL_QR, KC_TC_XT_T, KC_TC_X_Q, KC_OMEGA, KC_RMW_TC, KC_FUSED_POWER, KC_RESIDENT = 1, 2, 3, 4, 5, 6, 7, 8, 9, 10
 
@@ -107,6 +107,7 @@ def lib() -> C.CDLL:
         "agzo_read_counters": (i32, [vp, C.POINTER(C.c_double), C.POINTER(i64), C.POINTER(i64)]),
         "agzo_set_allreduce": (i32, [vp, ALLREDUCE_FN, vp, i64]),
         "agzo_debug_wait_timeout": (i32, [vp, vp]),
+        "agzo_debug_tile_rows": (i32, [LP, i32, i32, C.POINTER(C.c_int32)]),
         "agzo_debug_extract_static": (i32, [vp, i64, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int32, u64, u32, vp, i64, vp,
                                             C.c_int32, i64, vp]),
         "agzo_debug_meeting": (i32, [i32, i32, u32, u64, C.POINTER(u64), C.POINTER(u32), C.POINTER(u32)]),
@@ -275,6 +276,13 @@ def agzo_debug_fused_split(tiles, clusters: int):
     _check(lib().agzo_debug_fused_split(t, n, clusters, tile0, first, parts, begin, C.byref(shares)),
            "agzo_debug_fused_split")
     return list(tile0)[:n], list(first)[:n], list(parts)[:n], list(begin)[:shares.value + 1]
+
+
+def agzo_debug_tile_rows(layers, sm_count: int = 148):
+    """Rows of a tile of the CUDA-core in-place pass: (layers on the vector path, layers element by element); host arithmetic only."""
+    rows = (C.c_int32 * 2)()
+    _check(lib().agzo_debug_tile_rows(layer_array(layers), len(layers), sm_count, rows), "agzo_debug_tile_rows")
+    return tuple(rows)
 
 
 def agzo_query_cluster_capacity(ctx: Context):

@@ -39,9 +39,9 @@ struct Plan {
   std::vector<size_t> wave_y_count;   // floats, alignment gaps included
   int regions = 1;
   int total_tiles = 0;
-  int tile_rows = kRmwMaxTileRows;
+  int tile_rows = kRmwMaxTileRows, slow_rows = 32;     // of layers on the vector path, and of the others
   int max_r = 0;
-  int cc_max_r = 0;                // largest rank among layers of the CUDA-core pass
+  int cc_max_r = 0;                // largest rank among layers on the vector path
   int fast_mode_mask = 0;          // storage modes present among layers on the vector path
   bool any_slow = false;           // some layer needs the scalar kernel
   bool has_extract = false;
@@ -354,18 +354,20 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
   // Lists of more than 640 MB are bound by HBM whatever the rounds: the tallest tiles of which each CTA gets sixteen, for rank 1, whose set-up
   // is least, half as tall (sixty 2048 x 2048 fp32 layers, r = 4, at 64 rows 316 us, 336 by rounds; eight 8B-shaped blocks, r = 1, at 256 / 128 / 64
   // rows 979 / 943 / 969, twenty, r = 4, at 256 / 128 2456 / 2502).
-  {
+  // The element-by-element kernel has heights of its own (32 rows at most): one 1001 x 1001 layer among four fp32 8B-shaped blocks, r = 8,
+  // 1162 us per pass with one height for both, now 998.
+  auto height = [&](bool slow) {
     struct Strip { int d_out, n; };
     std::vector<Strip> strips;             // 512 columns wide, by height
+    int best = slow ? 32 : kRmwMaxTileRows;
     int max_r = 0;
     int64_t bytes = 0;
-    bool slow = false, narrow = false;
+    bool narrow = false;
     for (int i = 0; i < n; ++i) {
-      if (!L[i].W || takes_tc_rmw(L[i])) continue;
+      if (!L[i].W || takes_tc_rmw(L[i]) || vector_rows(L[i]) == slow) continue;
       const int count = (L[i].d_in + kRmwTileCols - 1) / kRmwTileCols;
       max_r = std::max(max_r, L[i].r);
       bytes += (int64_t)L[i].d_out * L[i].d_in * ((L[i].w_dtype == AGZO_BF16 ? 2 : 4) + (L[i].W16 ? 2 : 0));
-      slow = slow || !vector_rows(L[i]);
       narrow = narrow || L[i].w_dtype == AGZO_BF16;
       auto same = std::find_if(strips.begin(), strips.end(), [&](const Strip& s) { return s.d_out == L[i].d_out; });
       if (same != strips.end()) same->n += count; else strips.push_back(Strip{L[i].d_out, count});
@@ -379,16 +381,19 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
       return tiles;
     };
     if (bytes > (640ll << 20)) {
-      plan->tile_rows = slow ? 32 : max_r == 1 ? kRmwMaxTileRows / 2 : kRmwMaxTileRows;
-      while (plan->tile_rows > 32 && tiles_of(plan->tile_rows) < 32ll * opts.sm_count) plan->tile_rows /= 2;
-      strips.clear();
+      best = slow ? 32 : max_r == 1 ? kRmwMaxTileRows / 2 : kRmwMaxTileRows;
+      while (best > 32 && tiles_of(best) < 32ll * opts.sm_count) best /= 2;
+      return best;
     }
     for (int rows = slow ? 32 : kRmwMaxTileRows; rows >= 8 && !strips.empty(); rows -= 8) {
       const long long rounds = (tiles_of(rows) + ctas - 1) / ctas;
       const long long cost = rounds * (2 * rows + setup + (max_r > 16 ? 2 * max_r : 0)) + (rounds > 1 ? rows : 0);     // in half rows
-      if (least < 0 || cost < least) { least = cost; plan->tile_rows = rows; }
+      if (least < 0 || cost < least) { least = cost; best = rows; }
     }
-  }
+    return best;
+  };
+  plan->tile_rows = height(false);
+  plan->slow_rows = height(true);
   // A list with fewer items than three quarters of the SMs gets shorter ones (one 4096 x 4096 layer, r = 64: 64 items of eight
   // row tiles 23.7 us, 128 of four 16.5, 256 of two 20.3; r = 8: 128 of four 14.5, 256 of two 16.7).
   int halvings = 0;
@@ -478,12 +483,17 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
       plan->max_b_bytes = std::max(plan->max_b_bytes, rmw_tc_b_bytes(D));
       if (ws) D.wmap = ws + maps_offset(n) + (size_t)i * kMapBytes + 384;
     } else if (a.W) {
-      if (vec) plan->fast_mode_mask |= 1 << D.rmw_mode; else plan->any_slow = true;
-      plan->cc_max_r = std::max(plan->cc_max_r, a.r);
+      if (vec) {
+        plan->fast_mode_mask |= 1 << D.rmw_mode;
+        plan->cc_max_r = std::max(plan->cc_max_r, a.r);
+      } else {
+        plan->any_slow = true;
+      }
     }
     D.tile0 = tiles;
     D.tiles_c = (a.d_in + kRmwTileCols - 1) / kRmwTileCols;
-    D.tiles_r = (a.W && !tc_rmw) ? (a.d_out + plan->tile_rows - 1) / plan->tile_rows : 0;
+    const int rows = vec ? plan->tile_rows : plan->slow_rows;
+    D.tiles_r = (a.W && !tc_rmw) ? (a.d_out + rows - 1) / rows : 0;
     plan->tile_start[i] = tiles;
     const long long nt = (long long)D.tiles_c * D.tiles_r;
     if (tiles + nt > 0x7fffffff) return AGZO_ERR_INVALID_ARG;
@@ -868,7 +878,7 @@ agzo_status rmw_pass(agzo_ctx* c, const agzo_layer* L, int n, uint64_t seed, Pas
   }
   if (c->plan.total_tiles > 0) {
     Timed t(c, AGZO_KC_RMW, s);
-    CU(c, launch_rmw(dev_layers(c), dev_tiles(c, n), n, c->plan.total_tiles, c->plan.tile_rows, c->plan.cc_max_r,
+    CU(c, launch_rmw(dev_layers(c), dev_tiles(c, n), n, c->plan.total_tiles, c->plan.tile_rows, c->plan.slow_rows, c->plan.cc_max_r,
                      c->plan.fast_mode_mask, c->plan.any_slow, seed, coef, pair_update, c->sm_count, s));
   }
   return AGZO_OK;
@@ -1552,6 +1562,18 @@ agzo_status agzo_debug_meeting(int32_t n, int32_t first, uint32_t phase, uint64_
   *h_increment = meeting_increment(n, first != 0, phase);
   *h_phase = meeting_phase(value);
   *h_failures = meeting_failures(value);
+  return AGZO_OK;
+}
+
+agzo_status agzo_debug_tile_rows(const agzo_layer* h_layers, int n, int sm_count, int32_t* h_rows) {
+  if (sm_count < 1 || !h_rows) return AGZO_ERR_INVALID_ARG;
+  agzo_status st = validate(h_layers, n, 0);
+  if (st != AGZO_OK) return st;
+  Plan plan;
+  st = build_plan(h_layers, n, nullptr, 0, PlanOpts{kDefaultWaveBytes, 0, 0, kRmwTcMinRank, 0, 0, true, 0, false, 2, 0, sm_count, nullptr}, &plan, nullptr);
+  if (st != AGZO_OK) return st;
+  h_rows[0] = plan.tile_rows;
+  h_rows[1] = plan.slow_rows;
   return AGZO_OK;
 }
 

@@ -437,7 +437,7 @@ static cudaError_t launch_mode(const RmwArgs& a, int max_r, cudaStream_t s) {
 }
 
 cudaError_t launch_rmw(const DevLayer* d_layers, const int* d_tile_start, int n_layers,
-                       int total_tiles, int tile_rows, int max_r, int fast_mode_mask, bool any_slow,
+                       int total_tiles, int tile_rows, int slow_rows, int max_r, int fast_mode_mask, bool any_slow,
                        uint64_t seed, PassCoef coef, bool pair_update, int sm_count, cudaStream_t s) {
   if (total_tiles <= 0) return cudaSuccess;
   RmwArgs a{d_layers, d_tile_start, n_layers, total_tiles, tile_rows, seed, coef, pair_update ? 1 : 0, sm_count};
@@ -451,7 +451,7 @@ cudaError_t launch_rmw(const DevLayer* d_layers, const int* d_tile_start, int n_
   if (e == cudaSuccess && any_slow) {
     const int grid = total_tiles < sm_count * 4 ? total_tiles : sm_count * 4;
     e = launch_kernel(rmw_generic_kernel, dim3(grid), kRmwThreads, 0, 0, starts_early(total_tiles, grid), s, d_layers, d_tile_start, n_layers, total_tiles,
-                       tile_rows, seed, coef, pair_update ? 1 : 0);
+                       slow_rows, seed, coef, pair_update ? 1 : 0);
   }
   return e;
 }

@@ -1,0 +1,25 @@
+"""Tiles of the CUDA-core in-place pass (host arithmetic)."""
+import pytest
+
+from paper_2601_17261_b200 import binding as B
+
+BLOCK_0P6B = [(1024, 2048), (1024, 1024), (1024, 1024), (2048, 1024), (1024, 3072), (1024, 3072), (3072, 1024)]
+BLOCK_8B = [(4096, 4096), (4096, 1024), (4096, 1024), (4096, 4096), (4096, 12288), (4096, 12288), (12288, 4096)]
+
+
+def layers_of(shapes, r, f32=True, pair=False):
+    out, at = [], 1 << 32
+    for i, (d_in, d_out) in enumerate(shapes):
+        out.append(B.agzo_layer(at, d_in, at if pair else None, d_in, None, 0, 256, d_in, B.AGZO_F32 if f32 else B.AGZO_BF16, 0, d_out,
+                                d_in, 0, r, i, 0))
+        at += 4 * d_in * d_out + 4096 & -256
+    return out
+
+
+@pytest.mark.parametrize("r", [1, 4, 8, 16, 24])
+@pytest.mark.parametrize("shapes", [BLOCK_0P6B * 2, BLOCK_8B * 4, [(1024, 1024)] * 8])
+def test_a_layer_element_by_element_leaves_the_others_their_tiles(shapes, r):
+    odd = [(1001, 1001)]
+    both = B.agzo_debug_tile_rows(layers_of(shapes + odd, r))
+    assert both == (B.agzo_debug_tile_rows(layers_of(shapes, r))[0], B.agzo_debug_tile_rows(layers_of(odd, r))[1])
+    assert both[1] <= 32
