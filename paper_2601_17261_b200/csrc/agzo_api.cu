@@ -346,14 +346,17 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     plan->image_bytes = want ? img : 0;
   }
   // Rows per tile of the CUDA-core pass.  The CTAs, all resident, take tiles in turn, so a pass lasts as many rounds as the one with most
-  // tiles has, each a tile's rows and what setting up a tile costs beside them: 3, 9, 12 bf16 rows for ranks 1, 2 and more (R, the slice of A^T, the
-  // record; with the slice in shared memory as many again as there are ranks), half as many of 4-byte weights up to rank 8; where there are several
-  // rounds, CTAs have drifted apart by half a tile at the end.
-  // Multiples of eight, the tallest of the cheapest.  Measured on 35 lists at 10 to 14 heights each; against the other rule two fp32 0.6B-shaped blocks,
-  // r = 8, 51 -> 45 us, eight 1024 x 1024 pairs 14.7 -> 9.7, a bf16 0.6B-shaped block, r = 3, 16.7 -> 10.3, twelve, r = 2, 125 -> 122.
-  // Lists of more than 640 MB are bound by HBM whatever the rounds: the tallest tiles of which each CTA gets sixteen, for rank 1, whose set-up
-  // is least, half as tall (sixty 2048 x 2048 fp32 layers, r = 4, at 64 rows 316 us, 336 by rounds; eight 8B-shaped blocks, r = 1, at 256 / 128 / 64
-  // rows 979 / 943 / 969, twenty, r = 4, at 256 / 128 2456 / 2502).
+  // tiles has, each a tile's rows and what setting up a tile costs beside them (R, the slice of A^T, the record; with the slice in shared memory as
+  // many rows again as there are ranks): 32 rows above rank 8, 22 where there are 16-bit weights, five or six of fp32; where there are several
+  // rounds, CTAs have drifted apart by half a tile at the end.  Multiples of eight, the tallest of the cheapest.
+  // From 100 MB of fp32 weights on (ranks up to 4, strips of 512 columns all in use) and 250 MB of bf16 the memory sets the time whatever
+  // the rounds, and takes it best in tiles of 32 and of 128 rows.
+  // Measured on 1377 lists of up to 700 MB at every height and 1148 of up to 4.4 GB at ten: on the mean 1.6 % above the best height (with 2 to 12 rows
+  // for the set-up and without the two lines 2.4); of those above 6 us four are more than 3 % slower than at the height that gives each CTA sixteen
+  // tiles, of at least 32 rows (33 without: two fp32 0.6B-shaped blocks, r = 1, 51 us at 224 rows, 44 at 32; thirty bf16 1024 x 1024, r = 1, 24.6 at
+  // 24 rows, 15.3 at 256).
+  // Other lists of more than 640 MB: the tallest tiles of which each CTA gets sixteen, for rank 1, whose set-up
+  // is least, half as tall.
   // The element-by-element kernel has heights of its own (32 rows at most): one 1001 x 1001 layer among four fp32 8B-shaped blocks, r = 8,
   // 1162 us per pass with one height for both, now 998.
   auto height = [&](bool slow) {
@@ -361,25 +364,32 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     std::vector<Strip> strips;             // 512 columns wide, by height
     int best = slow ? 32 : kRmwMaxTileRows;
     int max_r = 0;
-    int64_t bytes = 0;
-    bool narrow = false;
+    int64_t bytes = 0, weights = 0, strip_rows = 0;
+    bool any_f32 = false, any_bf16 = false, any_pair = false;
     for (int i = 0; i < n; ++i) {
       if (!L[i].W || takes_tc_rmw(L[i]) || vector_rows(L[i]) == slow) continue;
       const int count = (L[i].d_in + kRmwTileCols - 1) / kRmwTileCols;
       max_r = std::max(max_r, L[i].r);
-      bytes += (int64_t)L[i].d_out * L[i].d_in * ((L[i].w_dtype == AGZO_BF16 ? 2 : 4) + (L[i].W16 ? 2 : 0));
-      narrow = narrow || L[i].w_dtype == AGZO_BF16;
+      const int64_t size = (int64_t)L[i].d_out * L[i].d_in;
+      weights += size;
+      strip_rows += (int64_t)count * L[i].d_out;
+      bytes += size * ((L[i].w_dtype == AGZO_BF16 ? 2 : 4) + (L[i].W16 ? 2 : 0));
+      (L[i].w_dtype == AGZO_BF16 ? any_bf16 : L[i].W16 ? any_pair : any_f32) = true;
       auto same = std::find_if(strips.begin(), strips.end(), [&](const Strip& s) { return s.d_out == L[i].d_out; });
       if (same != strips.end()) same->n += count; else strips.push_back(Strip{L[i].d_out, count});
     }
     const long long ctas = (slow ? 4ll : max_r <= 8 ? 2ll : 1ll) * opts.sm_count;       // element by element: four on an SM
-    const int setup = (max_r == 1 ? 3 : std::min(12, 3 + 3 * max_r)) * (narrow || max_r > 8 ? 2 : 1);
+    const int setup = slow ? (max_r == 1 ? 3 : std::min(12, 3 + 3 * max_r)) * (any_bf16 || max_r > 8 ? 2 : 1)
+                           : max_r > 8 ? 64 : any_bf16 || any_pair ? 44 : std::min(12, std::max(9, 3 + 3 * max_r));
     long long least = -1;
     auto tiles_of = [&](int rows) {
       long long tiles = 0;
       for (const Strip& s : strips) tiles += (long long)s.n * ((s.d_out + rows - 1) / rows);
       return tiles;
     };
+    const bool few_ranks = !slow && max_r <= 4;
+    if (few_ranks && !any_bf16 && !any_pair && bytes >= (100ll << 20) && 100 * weights >= 98 * strip_rows * kRmwTileCols) return 32;
+    if (few_ranks && any_bf16 && !any_f32 && !any_pair && bytes >= (250ll << 20)) return 128;
     if (bytes > (640ll << 20)) {
       best = slow ? 32 : max_r == 1 ? kRmwMaxTileRows / 2 : kRmwMaxTileRows;
       while (best > 32 && tiles_of(best) < 32ll * opts.sm_count) best /= 2;

@@ -23,3 +23,15 @@ def test_a_layer_element_by_element_leaves_the_others_their_tiles(shapes, r):
     both = B.agzo_debug_tile_rows(layers_of(shapes + odd, r))
     assert both == (B.agzo_debug_tile_rows(layers_of(shapes, r))[0], B.agzo_debug_tile_rows(layers_of(odd, r))[1])
     assert both[1] <= 32
+
+
+def test_lists_that_memory_bounds():
+    # heights measured as the best ones, or within 2 % of them; by the rounds alone these lists got others
+    assert [B.agzo_debug_tile_rows(layers_of(BLOCK_0P6B * 2, r))[0] for r in (1, 2, 3, 4)] == [32] * 4
+    assert B.agzo_debug_tile_rows(layers_of(BLOCK_8B * 4, 4))[0] == 32
+    assert B.agzo_debug_tile_rows(layers_of([(2048, 2048)] * 24, 2))[0] == 32
+    assert B.agzo_debug_tile_rows(layers_of([(1024, 1024)] * 30, 1, f32=False))[0] > 64
+    assert B.agzo_debug_tile_rows(layers_of(BLOCK_8B, 2, f32=False))[0] == 128
+    # strips of which a fifth is empty stay with the rounds, and so does a list of 60 MB
+    assert B.agzo_debug_tile_rows(layers_of([(1640, 1640)] * 20, 4))[0] > 64
+    assert B.agzo_debug_tile_rows(layers_of(BLOCK_0P6B, 4))[0] > 64
