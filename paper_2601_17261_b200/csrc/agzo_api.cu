@@ -325,16 +325,18 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
       }
     few_weights = weights <= (max_r <= 8 ? 32000000ll : max_r <= 16 ? 3000000ll : 0ll);
   }
-  auto takes_tc_rmw = [&](const agzo_layer& a) {
+  std::vector<char> vector_path((size_t)n), tc_pass((size_t)n);      // of the in-place passes
+  for (int i = 0; i < n; ++i) {
+    vector_path[i] = vector_rows(L[i]);
     // from rank 3 on the element-by-element kernel is no alternative where the vector kernels cannot run
-    return tc_available && opts.rmw_path != 1 && rmw_tc_eligible(a) &&
-           (opts.rmw_path == 2 || (a.r >= opts.rmw_tc_min_rank && !few_weights) || (a.r >= 3 && !vector_rows(a)));
-  };
+    tc_pass[i] = tc_available && opts.rmw_path != 1 && rmw_tc_eligible(L[i]) &&
+                 (opts.rmw_path == 2 || (L[i].r >= opts.rmw_tc_min_rank && !few_weights) || (L[i].r >= 3 && !vector_path[i]));
+  }
   {
     size_t img = 0;
     int max_tiles = 0, max_rp_all = 0;
     for (int i = 0; i < n; ++i) {
-      if (!takes_tc_rmw(L[i])) continue;
+      if (!tc_pass[i]) continue;
       img += rmw_tc_image_bytes(L[i]);
       max_tiles = std::max(max_tiles, (L[i].d_out + 127) / 128);
       max_rp_all = std::max(max_rp_all, (L[i].r + 7) & ~7);
@@ -367,7 +369,7 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     int64_t bytes = 0, weights = 0, strip_rows = 0;
     bool any_f32 = false, any_bf16 = false, any_pair = false;
     for (int i = 0; i < n; ++i) {
-      if (!L[i].W || takes_tc_rmw(L[i]) || vector_rows(L[i]) == slow) continue;
+      if (!L[i].W || tc_pass[i] || (vector_path[i] != 0) == slow) continue;
       const int count = (L[i].d_in + kRmwTileCols - 1) / kRmwTileCols;
       max_r = std::max(max_r, L[i].r);
       const int64_t size = (int64_t)L[i].d_out * L[i].d_in;
@@ -410,7 +412,7 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
   for (; halvings < 3; ++halvings) {
     long long count = 0;
     for (int i = 0; i < n && 4 * count < 3ll * opts.sm_count; ++i) {
-      if (!takes_tc_rmw(L[i])) continue;
+      if (!tc_pass[i]) continue;
       DevLayer D{};
       rmw_tc_shape(L[i], opts.rmw_tc_panels, plan->staged_r, halvings, &D);
       count += (long long)D.rtc_panels * D.rtc_chunks;
@@ -421,44 +423,78 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
   // layers and as short as leave the CTA with most to do the least (row tiles of 128 x 256, an item's set-up counted as one: two 0.6B-shaped
   // blocks, r = 8, with all items half as high 25.8 -> 35 us).  Four 0.6B-shaped blocks, r = 8, 52.4 -> 48.0 us per pass, three, r = 64, 54.0 -> 42.8,
   // five 2048 x 2048 layers, r = 12, 24.8 -> 19.5; 23 of 45 lists unchanged, none slower.
+  // Layers of one shape have the same items, in runs of equal ones, and the layers before the first that gets shorter ones have the same
+  // in all the tries: 9 us for 28 layers of 0.6B shape, 3 for seven of 8B shape; item by item it took 45 and 115.
   int fine_from = n, fine_halvings = 0;
   {
     std::vector<int> which;
     long long count = 0;
-    for (int i = 0; i < n; ++i) {
-      if (!takes_tc_rmw(L[i])) continue;
+    const long long limit = 10ll * opts.sm_count;
+    for (int i = 0; i < n && count <= limit; ++i) {
+      if (!tc_pass[i]) continue;
       DevLayer D{};
       rmw_tc_shape(L[i], opts.rmw_tc_panels, plan->staged_r, halvings, &D);
       which.push_back(i);
       count += (long long)D.rtc_panels * D.rtc_chunks;
     }
-    if (count > opts.sm_count && count <= 10ll * opts.sm_count) {
-      std::vector<float> load;
-      auto most = [&](int from, int more) {
-        load.assign((size_t)opts.sm_count, 0.f);
-        int cta = 0;
-        float max_load = 0.f;
-        for (int i : which) {
-          DevLayer D{};
-          rmw_tc_shape(L[i], opts.rmw_tc_panels, plan->staged_r, halvings + (i >= from ? more : 0), &D);
-          const int row_tiles = (L[i].d_out + 127) / 128, cols = D.rtc_np * D.rtc_cw;
-          for (int c = 0; c < D.rtc_chunks; ++c)
-            for (int g = 0; g < D.rtc_panels; ++g) {
-              const int high = std::min(D.rtc_chunk_blocks, row_tiles - c * D.rtc_chunk_blocks), wide = std::min(cols, L[i].d_in - g * cols);
-              float& l = load[(size_t)cta];
-              l += 1.f + (float)high * (float)wide / 256.f;
-              max_load = std::max(max_load, l);
-              if (++cta == opts.sm_count) cta = 0;
-            }
-        }
-        return max_load;
+    if (count > opts.sm_count && count <= limit) {
+      struct Run { float load; int n; };
+      struct Items { int layer; std::vector<Run> runs[3]; };         // of the layer and those of its shape, by halvings more
+      struct Load { std::vector<float> cta; int next; };
+      auto add_run = [](std::vector<Run>& v, float load, int n) {
+        if (!v.empty() && v.back().load == load) v.back().n += n; else if (n > 0) v.push_back(Run{load, n});
       };
-      float least = 0.97f * most(n, 0);
-      for (size_t k = 1; k <= which.size() && k <= 24; k += k < 4 ? 1 : k / 2)
+      std::vector<Items> items;
+      std::vector<int> items_of;                                     // of which[p]
+      for (int i : which) {
+        const agzo_layer& a = L[i];
+        size_t k = 0;
+        while (k < items.size() && (L[items[k].layer].d_out != a.d_out || L[items[k].layer].d_in != a.d_in || L[items[k].layer].r != a.r)) ++k;
+        items_of.push_back((int)k);
+        if (k < items.size()) continue;
+        items.emplace_back();
+        items[k].layer = i;
+        for (int more = 0; more < 3; ++more) {
+          DevLayer D{};
+          rmw_tc_shape(a, opts.rmw_tc_panels, plan->staged_r, halvings + more, &D);
+          const int row_tiles = (a.d_out + 127) / 128, cols = D.rtc_np * D.rtc_cw;
+          for (int c = 0; c < D.rtc_chunks; ++c) {
+            const float high = (float)std::min(D.rtc_chunk_blocks, row_tiles - c * D.rtc_chunk_blocks);
+            add_run(items[k].runs[more], 1.f + high * (float)cols / 256.f, D.rtc_panels - 1);
+            add_run(items[k].runs[more], 1.f + high * (float)(a.d_in - (D.rtc_panels - 1) * cols) / 256.f, 1);
+          }
+        }
+      }
+      const int G = opts.sm_count;
+      auto add = [&](Load& l, const std::vector<Run>& runs) {        // in turn to the CTAs
+        for (const Run& run : runs) {
+          const float rounds = (float)(run.n / G) * run.load;
+          const int rest = run.n % G, upto = std::min(rest, G - l.next);
+          float* c = l.cta.data();
+          if (rounds > 0.f)
+            for (int x = 0; x < G; ++x) c[x] += rounds;
+          for (int x = 0; x < upto; ++x) c[l.next + x] += run.load;
+          for (int x = 0; x < rest - upto; ++x) c[x] += run.load;
+          l.next = (l.next + rest) % G;
+        }
+      };
+      auto most = [](const Load& l) { return *std::max_element(l.cta.begin(), l.cta.end()); };
+      Load all{std::vector<float>((size_t)G, 0.f), 0}, tried;
+      std::vector<Load> before;                                      // load ahead of which[p], from the last 24 layers on
+      const size_t first = which.size() > 24 ? which.size() - 24 : 0;
+      for (size_t p = 0; p < which.size(); ++p) {
+        if (p >= first) before.push_back(all);
+        add(all, items[items_of[p]].runs[0]);
+      }
+      float least = 0.97f * most(all), sum = 0.f;
+      for (float l : all.cta) sum += l;
+      for (size_t k = 1; k <= before.size() && least * (float)G > sum; k += k < 4 ? 1 : k / 2)      // none can do better than share it evenly
         for (int more = 1; more <= 2; ++more) {
-          const int from = which[which.size() - k];
-          const float m = most(from, more);
-          if (m < least) { least = m; fine_from = from; fine_halvings = more; }
+          const size_t from = which.size() - k;
+          tried = before[from - first];
+          for (size_t p = from; p < which.size(); ++p) add(tried, items[items_of[p]].runs[more]);
+          const float m = most(tried);
+          if (m < least) { least = m; fine_from = which[from]; fine_halvings = more; }
         }
     }
   }
@@ -474,10 +510,10 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     D.d_out = a.d_out; D.d_in = a.d_in; D.m = a.m; D.r = a.r;
     D.layer_id = a.layer_id;
     D.rmw_mode = a.W16 ? RMW_PAIR_COMPUTE : (a.w_dtype == AGZO_BF16 ? RMW_BF16 : RMW_F32);
-    const bool vec = vector_rows(a);
+    const bool vec = vector_path[i] != 0;
     D.vec_ok = vec ? 1 : 0;
     // bf16 weights of sufficient rank go through the tensor-core pass and get no CUDA-core tiles
-    const bool tc_rmw = takes_tc_rmw(a);
+    const bool tc_rmw = tc_pass[i] != 0;
     plan->item_start[i] = (int)items;
     if (tc_rmw) {
       rmw_tc_shape(a, opts.rmw_tc_panels, plan->staged_r, halvings + (i >= fine_from ? fine_halvings : 0), &D);
