@@ -139,10 +139,11 @@ agzo_status agzo_destroy(agzo_ctx* ctx);
  * tensor-core kernels (UNSUPPORTED at call time if a layer cannot use them), 3 = as 2 but
  * without the fused power-step kernel (T = X Q and Y = X^T T as two sweeps over X);
  * "rmw_path" selects the kernel of the in-place passes: 0 = automatic (bf16 weights with
- * 16-byte aligned rows and r >= "rmw_tc_min_rank", default 5 (which lists of few weights do not heed: up to
- * 32 million at ranks up to 8, 3 million up to 16, stay with the CUDA cores), take the tensor-core kernel, and so
+ * 16-byte aligned rows and r >= "rmw_tc_min_rank" take the tensor-core kernel, and so
  * from rank 3 on do those whose d_in or V rules out 16-byte accesses; everything else the CUDA-core
- * kernels), 1 = CUDA-core kernels only, 2 = tensor-core kernel for every layer that allows it;
+ * kernels), 1 = CUDA-core kernels only, 2 = tensor-core kernel for every layer that allows it.  Where "rmw_tc_min_rank" has not
+ * been set it is 5, and lists of few weights (up to 32 million at ranks up to 8, 3 million up to 16) stay with the CUDA
+ * cores: the kernel of a layer then depends on the list it comes in (see agzo_perturb); a value that is set holds for every list;
  * tuning knobs of that kernel, 0 = chosen by rank:
  * "rmw_tc_slots" (shared-memory ring slots), "rmw_tc_inflight" (loads in flight per CTA),
  * "rmw_tc_panels" (column panels per work item, 1 or 2); "rmw_stage_r" 0 = when some layer's rank
@@ -282,7 +283,11 @@ agzo_status agzo_extract_subspace(agzo_ctx* ctx, const agzo_layer* h_layers, int
 /* W_l <- W_l + scale * R_l A_l^T for every layer, R_l regenerated from (seed, layer_id,
  * tag 0): step 2 of Algorithm 2 with scale = mu; the two-point flip is scale = -2 mu.
  * One fused read-modify-write pass; fp32 arithmetic, one rounding to the storage type.
- * With a W16 compute copy: W16 <- bf16(W + scale * Delta), W untouched.                   */
+ * With a W16 compute copy: W16 <- bf16(W + scale * Delta), W untouched.
+ * The kernels that "rmw_path" chooses between form Delta differently, the tensor-core one to about 2^-17 of a term, so the passes
+ * that belong together (perturb, flip, restore, update of one seed) should get a layer in the same list, or
+ * "rmw_tc_min_rank" be set: in an automatic choice a bf16 layer of rank 5 to 16 can take one kernel in a list of its own and
+ * another in a longer one, and a few weights in 10^4 then round the other way.               */
 agzo_status agzo_perturb(agzo_ctx* ctx, const agzo_layer* h_layers, int n, uint64_t seed,
                          float scale, void* stream);
 

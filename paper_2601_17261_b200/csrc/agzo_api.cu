@@ -56,13 +56,13 @@ struct Plan {
   size_t image_bytes = 0;
 };
 
-constexpr int kRmwTcMinRank = 5;   // default of the option
+constexpr int kRmwTcMinRank = 5;   // where the option has not been set
 
 struct PlanOpts {
   int64_t wave_bytes;
   int extract_path;      // 0 auto, 1 CUDA-core only, 2 tensor-core required
   int rmw_path;          // 0 auto, 1 CUDA-core only, 2 tensor cores wherever a layer allows it
-  int rmw_tc_min_rank;   // auto: layers with r >= this use the tensor-core pass
+  int rmw_tc_min_rank;   // auto: layers with r >= this use the tensor-core pass; 0: kRmwTcMinRank, and lists of few weights the CUDA-core pass
   int rmw_tc_panels;     // column panels per work item of the tensor-core pass (1 or 2)
   int rmw_stage_r;       // 0: stage R in scratch when some rank exceeds 16; 1: never; 2: always
   bool tc_available;
@@ -315,7 +315,7 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
   // 0.8 M r = 8 4.8 / 8.6, r = 16 5.0 / 8.5; 8.4 M r = 8 9.5 / 10.9, r = 16 13.0 / 11.2; 31 M r = 5 23.4 / 27.2, r = 8 23.5 / 25.0; 50 M r = 5
   // 41.3 / 40.7, r = 8 43.4 / 37.9).
   bool few_weights = false;
-  if (opts.rmw_path == 0 && opts.rmw_tc_min_rank == kRmwTcMinRank) {
+  if (opts.rmw_path == 0 && opts.rmw_tc_min_rank == 0) {
     int64_t weights = 0;
     int max_r = 0;
     for (int i = 0; i < n; ++i)
@@ -325,12 +325,13 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
       }
     few_weights = weights <= (max_r <= 8 ? 32000000ll : max_r <= 16 ? 3000000ll : 0ll);
   }
+  const int tc_min_rank = opts.rmw_tc_min_rank ? opts.rmw_tc_min_rank : kRmwTcMinRank;
   std::vector<char> vector_path((size_t)n), tc_pass((size_t)n);      // of the in-place passes
   for (int i = 0; i < n; ++i) {
     vector_path[i] = vector_rows(L[i]);
     // from rank 3 on the element-by-element kernel is no alternative where the vector kernels cannot run
     tc_pass[i] = tc_available && opts.rmw_path != 1 && rmw_tc_eligible(L[i]) &&
-                 (opts.rmw_path == 2 || (L[i].r >= opts.rmw_tc_min_rank && !few_weights) || (L[i].r >= 3 && !vector_path[i]));
+                 (opts.rmw_path == 2 || (L[i].r >= tc_min_rank && !few_weights) || (L[i].r >= 3 && !vector_path[i]));
   }
   {
     size_t img = 0;
@@ -1014,7 +1015,7 @@ agzo_status agzo_create(agzo_ctx** out, int device, void* workspace, size_t work
   c->last_cuda = 0;
   c->extract_path = 0;
   c->rmw_path = 0;
-  c->rmw_tc_min_rank = kRmwTcMinRank;   // 8B shapes, six blocks, one pass, CUDA cores / tensor cores: r = 1 736 / 786 us, r = 4 732 / 783,
+  c->rmw_tc_min_rank = 0;   // kRmwTcMinRank: 8B shapes, six blocks, one pass, CUDA cores / tensor cores: r = 1 736 / 786 us, r = 4 732 / 783,
                             // r = 6 822 / 780, r = 8 823 / 783, r = 16 1471 / 770; 0.6B shapes r = 4 282 / 302, r = 6 331 / 316
   c->rmw_tc_slots = 0;
   c->rmw_tc_inflight = 0;
@@ -1616,7 +1617,7 @@ agzo_status agzo_debug_tile_rows(const agzo_layer* h_layers, int n, int sm_count
   agzo_status st = validate(h_layers, n, 0);
   if (st != AGZO_OK) return st;
   Plan plan;
-  st = build_plan(h_layers, n, nullptr, 0, PlanOpts{kDefaultWaveBytes, 0, 0, kRmwTcMinRank, 0, 0, true, 0, false, 2, 0, sm_count, nullptr}, &plan, nullptr);
+  st = build_plan(h_layers, n, nullptr, 0, PlanOpts{kDefaultWaveBytes, 0, 0, 0, 0, 0, true, 0, false, 2, 0, sm_count, nullptr}, &plan, nullptr);
   if (st != AGZO_OK) return st;
   h_rows[0] = plan.tile_rows;
   h_rows[1] = plan.slow_rows;

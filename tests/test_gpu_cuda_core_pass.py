@@ -102,3 +102,23 @@ def test_lists_of_few_weights_stay_with_the_cuda_cores(r, d_out, n, tensor_cores
             B.agzo_set_option(ctx, "time_kernel_class", kind)
             B.agzo_perturb(ctx, layers, 3, 1e-3)
             assert (B.agzo_read_counters(ctx)[1] > 0) == want
+
+
+@pytest.mark.parametrize("min_rank", [5, 9])
+def test_a_rank_that_is_set_holds_for_lists_of_few_weights(min_rank):
+    # the kernel is the layer's then, whatever list it comes in: the same bits for a list and for its layers one by one
+    r, n, d = 8, 6, 512
+    V = torch.linalg.qr(torch.randn(d, r, device=DEV))[0].T.contiguous()
+    W = [[(torch.randn(d, d, generator=torch.Generator(DEV).manual_seed(i), device=DEV) * 0.02).to(torch.bfloat16) for i in range(n)] for _ in range(3)]
+    lists = [[B.make_layer(W=w, V=V, r=r, layer_id=i) for i, w in enumerate(ws)] for ws in W]
+    with Ctx(lists[0], extra=1 << 24) as ctx:
+        B.agzo_set_option(ctx, "rmw_tc_min_rank", min_rank)
+        for kind, want in ((B.KC_RMW_TC, min_rank <= r), (B.KC_RMW, min_rank > r)):
+            B.agzo_set_option(ctx, "time_kernel_class", kind)
+            B.agzo_perturb(ctx, lists[2], 3, 1e-2)
+            assert (B.agzo_read_counters(ctx)[1] > 0) == want
+        B.agzo_perturb(ctx, lists[0], 3, 1e-2)
+        for layer in lists[1]:
+            B.agzo_perturb(ctx, [layer], 3, 1e-2)
+        torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(W[0], W[1]))
