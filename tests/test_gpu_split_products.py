@@ -1,9 +1,11 @@
 """The products in bf16 parts on the tensor cores, at the edges of their steps of 64 and blocks of 128: columns and tokens around them,
-rows that allow accesses of eight columns, of four and of one, ranks around the panels of 8, 16 and 24 and beyond one unit, several
-layers on one X and more units than the short list of a launch holds, clusters of which some CTAs have no columns.
+rows that allow accesses of four columns and of one, ranks around the panels of 8, 16 and 24 and beyond one unit, several
+layers on one X and more units than the short list of a launch holds, clusters of which some CTAs have no columns and clusters with
+several items; their precision, and that they are what ran.
 
 Tolerance: that of the CUDA-core products (fp32 sums over at most 1300 terms), which these replace: 1e-5 orthonormality and 1e-4
-projector distance."""
+projector distance.  Where three parts are to be told from two: 2e-6.  On these inputs, emulated on the CPU with sums in fp32 and an accumulator
+that truncates, three parts are at most 8e-7 from the oracle and two at least 3.8e-6."""
 import numpy as np
 import pytest
 import torch
@@ -102,3 +104,66 @@ def test_what_stays_with_the_cuda_cores_is_cut_for_them(specs, K):
             assert B.agzo_poll(ctx) == B.AGZO_OK
     for split in (1, 2):
         assert all(torch.equal(a, b) for a, b in zip(V[0], V[split])), split
+
+
+def ran_in_parts(ctx, layers, K=2):
+    # a barrier of these kernels that expects more than comes: only where they run does the extraction then end with a wait that ran out
+    found = []
+    for kind in (B.KC_XT_T, B.KC_X_Q):
+        B.agzo_set_option(ctx, "debug_missing_class", kind)
+        B.agzo_extract_subspace(ctx, layers, 9, K)
+        found.append(B.agzo_poll(ctx) == B.AGZO_ERR_TIMEOUT)
+    B.agzo_set_option(ctx, "debug_missing_class", 0)
+    return found
+
+
+def extract_in_parts(specs, K):
+    """specs: (m, d_in, r, bf16, extra columns of the pitch); V of each layer, after the oracle's bounds for three parts"""
+    data, layers = [], []
+    for i, (m, d, r, bf16, extra) in enumerate(specs):
+        X = WL.planted_activations(m, d, min(32, d // 2), seed=m + d, bf16=bf16)
+        Xd, V = to_dev(X, bf16, pitch=d + extra if extra else None)[0], torch.zeros(r, d, device=DEV)
+        data.append((X, Xd, V))
+        layers.append(B.make_layer(X=Xd, V=V, r=r, layer_id=3))
+    with Ctx(layers) as ctx:
+        options(ctx)
+        assert ran_in_parts(ctx, layers, K) == [True, True]
+        B.agzo_extract_subspace(ctx, layers, 9, K)
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+    for (X, _, V), s in zip(data, specs):
+        check(X, V, s[2], K, 9, 3, 2e-6)
+
+
+@pytest.mark.parametrize("r", [1, 8, 17, 25])
+@pytest.mark.parametrize("m,d_in", [(40, 40), (129, 132), (1300, 1032)])
+@pytest.mark.parametrize("bf16,extra", [(False, 0), (False, 3), (True, 1)])
+def test_products_in_parts_have_fp32_precision(r, m, d_in, bf16, extra):
+    extract_in_parts([(m, d_in, r, bf16, extra)], 2)
+
+
+# T = X Q on 148 SMs by clusters of four, whose CTAs have most to do 18 steps of 64 columns (one CTA an item 64, pairs 34): the unit of 4096 columns in
+# one cluster, the 40 items of the other unit in the other 31, so nine of them have two; 64 columns leave three CTAs of four without any
+@pytest.mark.parametrize("d_in", [64, 256])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_clusters_with_empty_shares_and_several_items(d_in, bf16):
+    extra = 1 if bf16 else 0
+    extract_in_parts([(128, 4096, 4, bf16, extra), (5120, d_in, 4, bf16, extra)], 1)
+
+
+def test_products_in_parts_where_they_pay_and_without_workspace():
+    # two uses whose products are the faster ones in parts, in the automatic choice; the call without workspace takes the same route: the bits
+    # of the context's call in parts, which the CUDA-core kernels do not give
+    for m, d_in, bf16 in ((5000, 1001, True), (8000, 1024, False)):
+        r = 8
+        X = torch.randn(m, d_in, device=DEV).to(torch.bfloat16 if bf16 else torch.float32)
+        V = torch.zeros(3, r, d_in, device=DEV)
+        for split in (0, 1):
+            layers = [B.make_layer(X=X, V=V[split], r=r, layer_id=3)]
+            with Ctx(layers) as ctx:
+                B.agzo_set_option(ctx, "extract_resident", 0)
+                B.agzo_set_option(ctx, "extract_split", split)
+                assert ran_in_parts(ctx, layers) == [split == 1] * 2
+                B.agzo_extract_subspace(ctx, layers, 9, 2)
+                assert B.agzo_poll(ctx) == B.AGZO_OK
+        B.agzo_debug_extract_static(X, V[2], r, 2, 9, 3, B.STATIC_CHAIN)
+        assert torch.equal(V[2], V[1]) and not torch.equal(V[2], V[0])
