@@ -265,10 +265,12 @@ __device__ __forceinline__ void unit_barrier(Meeting& m, int clusters, int cs, c
   }
   __syncthreads();
 }
-// A product that did not come: known to the n CTAs of the cluster where that is all of the unit, else to the others by the next meeting
+// A product or a sum that did not come: known to the n CTAs of the cluster where that is all of the unit, else to the others by the next
+// meeting.  By every lane whose wait ran out: near the limit it can be one warp's, or one lane's, and not the first one's.
 __device__ __noinline__ void product_failed(ResShared* sh, int n) {
   sh->failed = 1;
-  if ((int)threadIdx.x < n) st_cluster_u32(mapa_shared(smem_u32(&sh->failed), threadIdx.x), 1u);
+#pragma unroll 1
+  for (int c = 0; c < n; ++c) st_cluster_u32(mapa_shared(smem_u32(&sh->failed), (uint32_t)c), 1u);
 }
 // V = 0, with which a pass changes nothing: the strips of the CTA in row i whose first column is col0
 __device__ __noinline__ void zero_strips(const ResidentUnit& U, int i, int col0) {
