@@ -353,7 +353,9 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
   // many rows again as there are ranks): 32 rows above rank 8, 22 where there are 16-bit weights, five or six of fp32; where there are several
   // rounds, CTAs have drifted apart by half a tile at the end.  Multiples of eight, the tallest of the cheapest.
   // From 100 MB of fp32 weights on (ranks up to 4, strips of 512 columns all in use) and 250 MB of bf16 the memory sets the time whatever
-  // the rounds, and takes it best in tiles of 32 and of 128 rows.
+  // the rounds, and takes it best in tiles of 32 and of 128 rows (bf16 lists of more than 640 MB at ranks 3 and 4 of 256, as below: the same on a cool
+  // chip, 903 and 899 us for 28 1.7B-shaped blocks, r = 4, but with the power cap active, where the set-up's work costs clock, 947 and 920; ranks 1 and
+  // 2 keep 128: r = 2 875 / 898 and 890 / 884).
   // Measured on 1377 lists of up to 700 MB at every height and 1148 of up to 4.4 GB at ten: on the mean 1.6 % above the best height (with 2 to 12 rows
   // for the set-up and without the two lines 2.4); of those above 6 us four are more than 3 % slower than at the height that gives each CTA sixteen
   // tiles, of at least 32 rows (33 without: two fp32 0.6B-shaped blocks, r = 1, 51 us at 224 rows, 44 at 32; thirty bf16 1024 x 1024, r = 1, 24.6 at
@@ -391,9 +393,10 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
       return tiles;
     };
     const bool few_ranks = !slow && max_r <= 4;
+    const bool large = bytes > (640ll << 20);
     if (few_ranks && !any_bf16 && !any_pair && bytes >= (100ll << 20) && 100 * weights >= 98 * strip_rows * kRmwTileCols) return 32;
-    if (few_ranks && any_bf16 && !any_f32 && !any_pair && bytes >= (250ll << 20)) return 128;
-    if (bytes > (640ll << 20)) {
+    if (few_ranks && any_bf16 && !any_f32 && !any_pair && bytes >= (250ll << 20) && !(large && max_r >= 3)) return 128;
+    if (large) {
       best = slow ? 32 : max_r == 1 ? kRmwMaxTileRows / 2 : kRmwMaxTileRows;
       while (best > 32 && tiles_of(best) < 32ll * opts.sm_count) best /= 2;
       return best;

@@ -35,3 +35,9 @@ def test_lists_that_memory_bounds():
     # strips of which a fifth is empty stay with the rounds, and so does a list of 60 MB
     assert B.agzo_debug_tile_rows(layers_of([(1640, 1640)] * 20, 4))[0] > 64
     assert B.agzo_debug_tile_rows(layers_of(BLOCK_0P6B, 4))[0] > 64
+
+
+def test_large_16_bit_lists_of_ranks_3_and_4_keep_the_tallest_tiles():
+    # their set-up is what the power cap takes from the pass: with it active 128 rows are 2 to 3 % slower than 256
+    for blocks in (BLOCK_8B * 10, BLOCK_0P6B * 56):
+        assert [B.agzo_debug_tile_rows(layers_of(blocks, r, f32=False))[0] for r in (1, 2, 3, 4)] == [128, 128, 256, 256]
