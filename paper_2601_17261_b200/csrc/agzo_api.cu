@@ -593,8 +593,16 @@ agzo_status build_plan(const agzo_layer* L, int n, char* ws, size_t ws_bytes, co
     return (tc ? 0 : align_up((size_t)a.m * a.r * 4)) + align_up((size_t)a.r * a.d_in * 4) + align_up(panel_gram_bytes(a.d_in, a.r, extract_max_r));
   };
   auto ypart_bytes = [&](int parts, int ranks, int d_in) { return align_up((size_t)parts * ranks * (size_t)d_in * 4); };
+  // Of the tokens seen last, for either kernel: the layers of a call mostly have as many, and trying the counts takes 0.2 us each time, three times a
+  // layer (a list of 64 layers: 65 -> 30 us, with both kernels' counts 101 -> 31; two fp32 0.6B-shaped blocks, a new state's first step 655 -> 644)
+  struct { int m, slabs, rows; } seen[2] = {};
   auto slabs_of = [&](const agzo_layer& a, bool tc, bool split, int* slabs, int* slab_rows) {
-    slab_shape(a, tc, long_slabs_any, !ws ? 0 : split ? split_blocks : cc_blocks, split, opts.sm_count, slabs, slab_rows);
+    if (!tc && seen[split].m == a.m) {
+      *slabs = seen[split].slabs; *slab_rows = seen[split].rows;
+    } else {
+      slab_shape(a, tc, long_slabs_any, !ws ? 0 : split ? split_blocks : cc_blocks, split, opts.sm_count, slabs, slab_rows);
+      if (!tc) seen[split] = {a.m, *slabs, *slab_rows};
+    }
     // a workspace of less than agzo_workspace_bytes takes fewer slabs on the CUDA-core path, as long as one is left
     for (int want = *slabs; ws && !tc && want > 1 && ypart_bytes(*slabs, a.r, a.d_in) + layer_need(a, tc) > scratch_cap;) {
       --want;

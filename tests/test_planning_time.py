@@ -23,3 +23,27 @@ def test_shorter_items_are_found_quickly(shapes):
             times.append(time.perf_counter() - t)
         return min(times)
     assert best(layers_of(shapes, 8, f32=False)) < 7 * best(layers_of(shapes, 8))
+
+
+@pytest.mark.gpu
+def test_two_kinds_of_token_slabs_are_planned_as_quickly_as_one():
+    # where products run in parts every layer has two slab counts; 64 layers of as many tokens: 31 and 30 us, with each count tried out for each
+    # layer several times 101 and 65
+    import torch
+    X, V = torch.zeros(4000, 256, device="cuda"), torch.zeros(2, 64, 8, 256, device="cuda")
+    lists = [[B.make_layer(X=X, V=V[k, i], r=8, layer_id=i) for i in range(64)] for k in range(2)]
+    ctx = B.agzo_create(lists[0])
+    B.agzo_set_option(ctx, "share_inputs", 0)
+
+    def best(split):
+        B.agzo_set_option(ctx, "extract_split", split)
+        times = []
+        for k in range(60):                    # alternate lists: each is new to the plan
+            t = time.perf_counter()
+            B.agzo_query_fused(ctx, lists[k & 1])
+            times.append(time.perf_counter() - t)
+            torch.cuda.synchronize()
+        return min(times)
+    best(0)
+    assert best(2) < 1.3 * best(0)
+    B.agzo_destroy(ctx)
