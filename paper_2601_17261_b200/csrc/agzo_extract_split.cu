@@ -666,6 +666,7 @@ bool split_pays(const agzo_layer* L, const std::vector<int>& which, bool share, 
   int max_m = 0, max_d = 0, max_r = 0;
   double wide = 0.0;                     // operand rows beyond those of eight ranks, 1 for 24
   double there = 0.0;                    // microseconds of two products X^T T and one X Q
+  double x_bytes = 0.0;
   for (int k : which) max_r = std::max(max_r, L[k].r);
   const bool r4 = max_r > 4, r8 = max_r > 8;
   const int passes = (max_r + 15) / 16;
@@ -687,6 +688,7 @@ bool split_pays(const agzo_layer* L, const std::vector<int>& which, bool share, 
     max_m = std::max(max_m, a.m); max_d = std::max(max_d, a.d_in);
     const bool f32 = a.x_dtype == AGZO_F32, scalar = a.d_in % 4 != 0 || a.ldx % 4 != 0 || (reinterpret_cast<uintptr_t>(a.X) & (f32 ? 15u : 7u)) != 0;
     any_scalar = any_scalar || scalar;
+    x_bytes += (f32 ? 4.0 : 2.0) * a.m * (double)a.d_in;
     const double md = 1e-6 * n * a.m * (double)a.d_in;
     there += md * (scalar ? 2.0 * (1.96 + 0.48 * r4 + 5.30 * (passes - 1)) + 1.70 + 2.43 * r4 + 2.48 * r8 + 4.92 * (passes - 1)
                    : f32 ? 2.0 * (0.21 + 0.31 * r4 + 0.64 * r8 + 1.19 * (passes - 1)) + 1.29 + 0.47 * r8 + 1.82 * (passes - 1)
@@ -699,7 +701,11 @@ bool split_pays(const agzo_layer* L, const std::vector<int>& which, bool share, 
   const int rows = split_slab_rows(max_m, blocks, sm_count);
   const long long slabs = (max_m + rows - 1) / rows, rounds = (slabs * blocks + sm_count - 1) / sm_count;
   const double here = 2.0 * (1.17 + 0.13 * wide) * (double)(rounds * (rows / kStep)) + 0.85 * most_steps(units, sm_count, &split);
-  return here < there;
+  // Inputs that stay in L2 between the products serve fp32 rows of whole 16-byte pieces at ranks up to 8, where the CUDA-core products wait for memory,
+  // sooner than `there` has it: a layer of 7858 x 828, r = 3, 21.7 here and 24.3 there by estimate, takes 101 and 81 us.  From 100 MB on they don't.
+  const bool in_l2 = x_bytes < 100e6 && !any_scalar && L[which[0]].x_dtype == AGZO_F32;
+  const double line = !in_l2 || max_r > 8 ? 1.0 : max_r <= 4 ? 0.8 : 0.92;
+  return here < line * there;
 }
 
 bool split_takes(const ExtractWave& w, const DevLayer* dev, int K) {

@@ -167,3 +167,29 @@ def test_products_in_parts_where_they_pay_and_without_workspace():
                 assert B.agzo_poll(ctx) == B.AGZO_OK
         B.agzo_debug_extract_static(X, V[2], r, 2, 9, 3, B.STATIC_CHAIN)
         assert torch.equal(V[2], V[1]) and not torch.equal(V[2], V[0])
+
+
+@pytest.mark.parametrize("m,d_in,r", [(7858, 828, 3), (9315, 584, 4), (9258, 1992, 5), (3965, 1388, 5)])
+def test_the_cuda_cores_keep_single_fp32_layers_of_low_rank(m, d_in, r):
+    # inputs that L2 holds: 6 to 24 % slower in parts, which the estimates favour by up to 15 %
+    X, V = torch.randn(m, d_in, device=DEV), torch.zeros(2, r, d_in, device=DEV)
+    layers = [B.make_layer(X=X, V=V[0], r=r, layer_id=3)]
+    with Ctx(layers) as ctx:
+        B.agzo_set_option(ctx, "extract_resident", 0)
+        assert ran_in_parts(ctx, layers) == [False, False]
+        B.agzo_extract_subspace(ctx, layers, 9, 2)
+        assert B.agzo_poll(ctx) == B.AGZO_OK
+    B.agzo_debug_extract_static(X, V[1], r, 2, 9, 3, B.STATIC_CHAIN)
+    assert torch.equal(V[0], V[1])
+
+
+def test_larger_fp32_sets_run_in_parts():
+    # two 0.6B-shaped blocks, 229 MB: by estimate 4 % faster in parts, measured 17 %
+    layers, keep = [], []
+    for _ in range(2):
+        for d_in, ranks in ((1024, (8, 8, 8)), (2048, (8,)), (1024, (8, 8)), (3072, (8,))):
+            X = torch.randn(4000, d_in, device=DEV)
+            keep.append((X, [torch.zeros(r, d_in, device=DEV) for r in ranks]))
+            layers += [B.make_layer(X=X, V=v, r=8, layer_id=len(layers) + i) for i, v in enumerate(keep[-1][1])]
+    with Ctx(layers) as ctx:
+        assert ran_in_parts(ctx, layers) == [True, True]
