@@ -39,7 +39,9 @@
  *     errors are detected on the host before anything is launched.  Conditions that only
  *     the device can see (a rank-deficient panel, a wait that ran out) are written to a
  *     status word in the workspace and reported by agzo_poll.  An extraction in which a wait ran
- *     out leaves V = 0 in the layers it concerns, with which a pass changes nothing.
+ *     out leaves V = 0 in the layers it concerns, with which a pass changes nothing (the resident kernel,
+ *     where blocks of several clusters wait in vain after the last time all of them have met: in those
+ *     blocks' columns).
  *   - Random streams: Philox4x32-10 with key = the 64-bit step seed and counter
  *     (b_lo, b_hi, layer_id, tag); b = e >> 2 where e is the row-major index of the element
  *     inside the matrix being drawn, which takes output word e & 3 of that block.

@@ -13,7 +13,9 @@
 // 64 KB are in flight; a warp per four ranks makes the operand's rows, one issues the products, eight take the accumulators in.
 // A step of 32 KB of fp32 takes 1400 to 1800 cycles, of which the copy rate would allow 1400: what bounds it is the round trip of a stage
 // (converted, multiplied, free again) through the two or three others there is room for; leaving out the loads, the conversion or the products
-// changes little.  Two fp32 blocks of 0.6B shape (229 MB), 4000 tokens, r = 8: X^T T 67 -> 57 us, X Q 93 -> 68, the step 694 -> 600;
+// changes little.  All units of a launch run the widest one's instance; with NP = 16 and 24 (928 and 992 threads) a thread has 64 registers, and the
+// instances of X^T T on fp32 spill 28 and 24 bytes, those of NP = 24 on bf16 4 (X^T T) and 8 (X Q).
+// Two fp32 blocks of 0.6B shape (229 MB), 4000 tokens, r = 8: X^T T 67 -> 57 us, X Q 93 -> 68, the step 692 -> 590;
 // r = 16 on 4000 x 3072, two layers, K = 1: 133 -> 100 us for the extraction; 5000 x 1001 in bf16, r = 8: 226 -> 122.
 // Error against 64 bits, 172 bases of 60 lists: 1.2e-7 root mean square, the CUDA-core kernels 1.4e-7.
 // Units go from the widest to the narrowest in T = X Q and back in Y = X^T T, so that what is left of X in L2 serves the next product.

@@ -489,7 +489,7 @@ __global__ void dense_kernel(T* w, long long n, long long b_first, uint64_t seed
 // Vector form for 16-byte aligned vectors: a thread takes eight consecutive elements (two Philox blocks), one 16-byte load and
 // store for bf16, two for fp32.  A long vector is bound by the arithmetic of one Philox + Box-Muller normal per weight, not by HBM
 // (67 M weights: 142 us with logf, sqrtf and sincospif, 119 with one pair of normals after another and a grid that stays resident, 97 now; HBM would
-// allow 43); a short one by its launch, so the normals are made, and the weights asked for as far as L2, before the kernel waits
+// allow 41); a short one by its launch, so the normals are made, and the weights asked for as far as L2, before the kernel waits
 // for its predecessor.  Every thread has one step: with a share of the vector per resident thread the scheduler runs some warps far ahead
 // of others, and the SM ends on few (121 -> 109 us for that alone, 105 with 32-bit block numbers).
 // hi: upper word of the block numbers, the same in the whole launch, so that what the first two rounds of Philox make of it is made once.

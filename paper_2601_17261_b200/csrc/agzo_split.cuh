@@ -26,7 +26,7 @@ struct SplitUnit {
   int m, d_in, slabs, slab_rows;
   int item0, rows;       // first work item; T = X Q: m, Y = X^T T: d_in
   short k0, np;
-  short vec;             // accesses of X that are aligned: 8 columns (2), 4 (1), or element by element (0)
+  short vec;             // accesses of X that are aligned: four columns (1), or element by element (0)
   short quads;           // ranks 4 k to 4 k + 3 of the panel are one layer's, and their source is aligned
   SplitLayer layer[kSplitMaxLayers];
 };
@@ -52,9 +52,10 @@ inline int split_slab_rows(int m, long long blocks, int sm_count) {
 }
 // Whether they are estimated to be the faster ones for the layers `which` of L (ascending): two products X^T T and one X Q.  Both sides fitted
 // to 820 lists of one to 21 layers, 64 to 12000 tokens and 64 to 4096 columns, ranks 1 to 64, all types and alignments, K = 0, 1 and 3.
-// Of the 612 whose inputs the SMs do not hold the rule gains a factor of 1.32 on the mean (1.33 with the faster side each time) and takes
-// the slower side by more than 3 % for 1.5 % (at most 17 %).  The CUDA cores keep ranks up to 4 on layers with an X of their own (their
-// products are at 80 % of the copy rate there, where a step of these takes 0.6 us at best) and lists that do not fill the device.
+// Of 1000 others (one to seven inputs of 1 to 600 MB in all, four fifths of them fp32, K = 3, the resident kernel off) the rule gains a factor of 1.498 on
+// the mean (1.505 with the faster side each time) and takes the slower side by more than 3 % for seven (at most 10 %).  The CUDA cores keep ranks up to
+// 4 on layers with an X of their own (their products are at 80 % of the copy rate there, where a step of these takes 0.6 us at best) and lists
+// that do not fill the device.
 bool split_pays(const agzo_layer* L, const std::vector<int>& which, bool share, int sm_count);
 // Whether the wave's products can run here with a power step or K = 0: below 2^-109 an fp32 value's third part is no bf16 number any
 // more; with a power step such inputs underflow whatever the kernel, without one the CUDA cores keep them.
